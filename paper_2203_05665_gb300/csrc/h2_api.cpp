@@ -53,7 +53,7 @@ static void free_dev(Dev &d) {
   if (d.fbar) cudaFree(d.fbar);
   if (d.grank) cudaFree(d.grank);
   if (d.gpiv) cudaFree(d.gpiv);
-  void *ptrs[] = {d.Vtc, d.tcv_E, d.Ntc, d.xnt, d.ntc_E, d.ntc_xmax, d.Stc, d.xtc, d.tc_E, d.tc_xmax, d.icen, d.adm_dc, d.ihalf, d.colmax, d.nself, d.near_ptr2, d.self_ptr, d.near_col2, d.near_blk2, d.self_col, d.vscale, d.nscale, d.pad_src, d.V, d.Vt, d.Ef,      d.S,       d.near, d.adm_ptr, d.adm_col, d.near_ptr,
+  void *ptrs[] = {d.Vtc, d.tcv_E, d.Ntc, d.xnt, d.ntc_E, d.ntc_s.row, d.ntc_s.ptr, d.ntc_s.col, d.ntc_s.split, d.tc_s.row, d.tc_s.ptr, d.tc_s.col, d.tc_s.split, d.Stc, d.xtc, d.tc_E, d.prec == H2_F64 ? nullptr : (void *)d.tc_xmax, d.icen, d.adm_dc, d.ihalf, d.colmax, d.nself, d.near_ptr2, d.self_ptr, d.near_col2, d.near_blk2, d.self_col, d.vscale, d.nscale, d.pad_src, d.V, d.Vt, d.Ef,      d.S,       d.near, d.adm_ptr, d.adm_col, d.near_ptr,
                   d.near_col, d.cheb, d.xpad, d.ypad, d.xhat, d.yhat, d.io_x,    d.io_y};
   for (void *p : ptrs)
     if (p) cudaFree(p);

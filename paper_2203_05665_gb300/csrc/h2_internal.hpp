@@ -84,6 +84,20 @@ struct GcaParams {
   int green_order = 4, tri_order = 3, max_rank = 128;
 };
 
+// Row order of a block-row kernel (row_schedule, h2_tile.cu): scheduled row i is
+// output row row[i] with blocks ptr[i] .. ptr[i + 1] - 1 in columns col[..]; CTA w
+// takes scheduled rows split[w] .. split[w + 1] - 1
+struct RowSched {
+  int32_t *row = nullptr, *col = nullptr, *split = nullptr;
+  int64_t *ptr = nullptr;
+  int grid = 0;
+};
+// set-up only: the unscheduled block and the output row of every scheduled block
+struct SchedTmp {
+  int32_t *src = nullptr, *brow = nullptr;
+  ~SchedTmp();
+};
+
 // Device representation of one H^2 matrix.
 struct Dev {
   int prec = H2_F64;
@@ -112,29 +126,29 @@ struct Dev {
   // digit planes of every S_b ([nadm][tc_nd][64 x 64] bytes, K-major
   // core-matrix layout), the row exponents ([nclu][64]), the digit planes of
   // the coefficients of one product ([nclu][tc_nd][16 x 64]) and the column
-  // maxima per level ([32][16])
+  // maxima per level ([32][64])
   int tensor = 0;               // 0: use the tensor cores where supported, 1: never
   bool tc = false;              // the digits exist
   int tc_nd = 0;                // digits per value: 10 (FP64-accurate) or 6 (FP32 handles)
   void *Stc = nullptr, *xtc = nullptr;
   int32_t *tc_E = nullptr;
   unsigned *tc_xmax = nullptr;
-  // FP64-accurate nearfield on the tensor cores (leaves of at most 21
-  // triangles): the digit planes of every near block (ntc_ablk bytes each,
-  // two stacked groups of K-major rows), the row exponents ([nleaf][lmax]),
-  // the digit planes of the permuted input of one product ([nleaf][10][16 x
-  // 32]) and its column maxima ([16])
+  // FP64-accurate nearfield on the tensor cores (leaves of at most 32
+  // triangles, h2_tile.cu): the digit planes of every near block, the row
+  // exponents ([nleaf][lmax]), the digit tiles of the permuted input of one
+  // pass ([nleaf][11 x 16 x 32]) and the column maxima of the input ([64])
   bool ntc = false;
   void *Ntc = nullptr, *xnt = nullptr;
   int32_t *ntc_E = nullptr;
+  RowSched ntc_s, tc_s;         // row orders of the nearfield and of the tensor-core coupling
   unsigned *ntc_xmax = nullptr;
-  uint32_t ntc_ablk = 0;
   // tensor-core leaf forward step: the ten E4M3 digit planes of every V_t^T
   // ([leaf][10][64 x 32] bytes, K-major core matrices) and their row powers
   // of two [leaf][64]
   void *Vtc = nullptr;
   int32_t *tcv_E = nullptr;
-  unsigned long long *colmax = nullptr;   // H2_F64: 64 column maxima of x (range guard of double-float)
+  unsigned long long *colmax = nullptr;   // H2_F64: 64 column maxima of x (range guard of double-float), the
+                                          // start of the block of maxima that a product clears (kMaximaBytes)
   bool v32 = false;             // 16-bit handle whose V, Vt and transfer factors are stored in FP32
   float *vscale = nullptr;      // per leaf: power of two dividing the stored V (FP16), or NULL
   float *nscale = nullptr;      // per nearfield block: the same for G_b, or NULL
@@ -235,23 +249,32 @@ int take_device_error(Ctx &c);
 int wait_selftest(Ctx &c, int withhold, uint32_t limit, int *stages_seen);
 
 // FP64-accurate coupling on the tensor cores (h2_tc.cu): eligibility,
-// set-up of the slices (arow_dev: row cluster of every admissible block, on
-// the device), the coupling phase of one product (xhat, yhat: double-float
+// set-up of the slices, the coupling phase of one product (xhat, yhat: double-float
 // coefficient arrays [clusters][k][rp]) and that file's device error word
 bool tc_eligible(const Dev &d);
-int tc_build(Ctx &c, const int32_t *arow_dev);
+int tc_build(Ctx &c);
 // leaf_max: the leaf coefficients' column maxima are in place (written by
 // the tensor-core leaf forward step)
 int tc_upward(Ctx &c, void *xhat, int rp, int64_t *launches, bool leaf_max = false);
 int tc_coupling(Ctx &c, const void *xhat, void *yhat, int rp);
 int tc_take_error(cudaStream_t st);
+// digits of the leaf bases (tensor-core leaf forward step), where eligible
+int tc_leaf_build(Ctx &c);
+// nearfield on the tensor cores (h2_tile.cu); the input's column maxima are
+// taken by the permutation.  wide: digit tiles of 16 columns whatever ncol
+// (the tensor-core leaf step reads those)
 bool ntc_eligible(const Dev &d);
-int ntc_build(Ctx &c, const int32_t *nrow_dev);
+int ntc_build(Ctx &c);
+void ntc_input(Ctx &c, const void *xpad, int rp, int c0, int ncol, bool wide);
 int ntc_near(Ctx &c, const void *xpad, void *ypad, int rp, int accumulate, int64_t *launches,
              bool have_input = false);
-// input column maxima and digit planes per leaf (nearfield, tensor-core leaf step)
-// have_max: the column maxima are in place (taken by the permutation)
-int ntc_input(Ctx &c, const void *xpad, int rp, int64_t *launches, bool have_max = false);
+int tile_take_error(cudaStream_t st);
+int row_schedule(Dev &d, const int64_t *ptr, const int32_t *col, int64_t nrows, RowSched &s, SchedTmp &tmp,
+                 cudaStream_t st);
+// H2_F64 handles: the range guard's column maxima (64 x 8 bytes), the input's
+// (64 x 4) and the coefficients' per level (32 x 64 x 4), one block cleared
+// by one memset per product
+constexpr size_t kMaximaBytes = 64 * 8 + 64 * 4 + 32 * 64 * 4;
 // leaf forward step on the tensor cores (after ntc_input); requires d.Vtc
 int tc_leaf_forward(Ctx &c, void *xhat, int rp);
 

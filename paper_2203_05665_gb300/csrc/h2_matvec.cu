@@ -34,26 +34,30 @@ constexpr int kMaxOut = 16;   // outputs per thread in the block-row kernels
 // lies outside [2^-40, 2^40] is multiplied by the power of two that brings
 // that entry to [1, 2) on the way in and divided by it on the way out (exact;
 // columns inside the range are not touched).  colmax[c] holds the bits of
-// max |x[:, c]| as a double (non-negative doubles order like their bits).
+// max |x[:, c]| as a double (non-negative doubles order like their bits, and
+// infinities and NaN above them).
 template <class Tin>
 __global__ void k_colmax(const Tin *__restrict__ x, int64_t n, unsigned long long *__restrict__ colmax) {
-  __shared__ double wmax[32];
+  __shared__ unsigned long long wmax[32];
   const Tin *xc = x + (int64_t)blockIdx.y * n;
+  auto bits = [&](int64_t i) -> unsigned long long {
+    return (unsigned long long)__double_as_longlong(fabs((double)xc[i]));
+  };
   // four independent maxima per thread keep several loads in flight
-  double m4[4] = {0.0, 0.0, 0.0, 0.0};
+  unsigned long long m4[4] = {0, 0, 0, 0};
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   for (; i + 3 * stride < n; i += 4 * stride)
 #pragma unroll
-    for (int u = 0; u < 4; ++u) m4[u] = fmax(m4[u], fabs((double)xc[i + u * stride]));
-  for (; i < n; i += stride) m4[0] = fmax(m4[0], fabs((double)xc[i]));
-  double mx = fmax(fmax(m4[0], m4[1]), fmax(m4[2], m4[3]));
-  for (int o = 16; o; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    for (int u = 0; u < 4; ++u) m4[u] = max(m4[u], bits(i + u * stride));
+  for (; i < n; i += stride) m4[0] = max(m4[0], bits(i));
+  unsigned long long mx = max(max(m4[0], m4[1]), max(m4[2], m4[3]));
+  for (int o = 16; o; o >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
   if ((threadIdx.x & 31) == 0) wmax[threadIdx.x >> 5] = mx;
   __syncthreads();
   if (threadIdx.x == 0) {
-    for (int w = 1; w < (int)(blockDim.x >> 5); ++w) mx = fmax(mx, wmax[w]);
-    if (mx > 0.0) atomicMax(&colmax[blockIdx.y], (unsigned long long)__double_as_longlong(mx));
+    for (int w = 1; w < (int)(blockDim.x >> 5); ++w) mx = max(mx, wmax[w]);
+    if (mx) atomicMax(&colmax[blockIdx.y], mx);
   }
 }
 
@@ -65,6 +69,11 @@ __device__ __forceinline__ double scale_pow2(double v, int e) {
   const int h = e / 2;
   return v * pow2d(h) * pow2d(e - h);
 }
+
+// a column with an infinity or a NaN: every output depends on every input (the
+// nearfield and the far field cover all pairs), so all its results are NaN;
+// digits cannot carry one, so the last permutation writes them
+__host__ __device__ inline bool not_finite(unsigned long long bits) { return ((bits >> 52) & 0x7ff) == 0x7ff; }
 
 // the power of two by which column c is scaled (0: untouched; zero, infinite
 // and NaN columns are not scaled)
@@ -151,11 +160,14 @@ __global__ void __launch_bounds__(256) k_permute_out(const Tin *__restrict__ ypa
   extern __shared__ __align__(16) unsigned char perm_smem[];
   Tin *tile = reinterpret_cast<Tin *>(perm_smem);
   __shared__ int shift[64];
+  __shared__ float poison[64];   // NaN for the columns with an infinity or a NaN, else 0
   __shared__ int32_t src[kPermRows];
   const int w = rp + 1;
   const int64_t p0 = (int64_t)blockIdx.x * kPermRows;
   if (threadIdx.x < kPermRows) src[threadIdx.x] = p0 + threadIdx.x < npad ? pad_src[p0 + threadIdx.x] : -1;
   if (threadIdx.x < 64) shift[threadIdx.x] = (colmax && (int)threadIdx.x < nrhs) ? range_shift(colmax[threadIdx.x]) : 0;
+  if (threadIdx.x < 64)
+    poison[threadIdx.x] = colmax && (int)threadIdx.x < nrhs && not_finite(colmax[threadIdx.x]) ? __int_as_float(0x7fc00000) : 0.0f;
   const int64_t rows = npad - p0 < kPermRows ? npad - p0 : kPermRows;
   for (int i = threadIdx.x; i < rows * rp; i += blockDim.x) {
     const int q = i / rp, c = i - q * rp;
@@ -168,6 +180,7 @@ __global__ void __launch_bounds__(256) k_permute_out(const Tin *__restrict__ ypa
     if (sp < 0) continue;
     Tout v = convert<Tout, Tin>(tile[q * w + c]);
     if (shift[c]) v = (Tout)scale_pow2((double)v, -shift[c]);
+    if (poison[c] != 0.0f) v = (Tout)poison[c];
     Tout *dst = y + sp + (int64_t)c * n;
     *dst = acc ? *dst + v : v;
   }
@@ -1093,7 +1106,7 @@ int matvec_typed(Ctx &c, const Tio *x, Tio *y, int nrhs, bool acc) {
   // double-float handles: column maxima of x for the range guard
   const unsigned long long *cmx = std::is_same<T, dd>::value ? d.colmax : nullptr;
   if (cmx) {
-    H2_CUDA_TRY(cudaMemsetAsync(d.colmax, 0, sizeof(unsigned long long) * nrhs, st));
+    H2_CUDA_TRY(cudaMemsetAsync(d.colmax, 0, kMaximaBytes, st));
     const int64_t nb = std::min<int64_t>((d.n + 8 * kThreads - 1) / (8 * kThreads), 64);
     k_colmax<Tio><<<dim3((unsigned)std::max<int64_t>(nb, 1), nrhs), kThreads, 0, st>>>(x, d.n, d.colmax);
     mk.count(H2_PH_PERMUTE_IN);
@@ -1102,19 +1115,18 @@ int matvec_typed(Ctx &c, const Tio *x, Tio *y, int nrhs, bool acc) {
   // FP64-accurate with the tensor-core nearfield and coupling: the leaf
   // forward step from the input digits the nearfield reads anyway; the
   // permutation takes the input's column maxima on the way
-  const bool leaf_tc = std::is_same<T, dd>::value && far && d.ntc && d.Vtc && rp <= 16;
-  if (leaf_tc) H2_CUDA_TRY(cudaMemsetAsync(d.ntc_xmax, 0, sizeof(unsigned) * 16, st));
+  const bool near_tc = std::is_same<T, dd>::value && d.ntc;
+  const bool leaf_tc = near_tc && far && d.Vtc && rp <= 16;
   k_permute_in<Tio, T><<<perm_grid, 256, (size_t)kPermRows * (rp + 1) * sizeof(T), st>>>(
-      x, d.n, nrhs, rp, d.pad_src, d.npad, cmx, xpad, leaf_tc ? d.ntc_xmax : nullptr);
+      x, d.n, nrhs, rp, d.pad_src, d.npad, cmx, xpad, near_tc ? d.ntc_xmax : nullptr);
   mk.count(H2_PH_PERMUTE_IN);
   mk.mark(H2_PH_LEAF_FORWARD);
   // leaf steps with one CTA per leaf when the stored values are in the arithmetic type
   const bool leaf_reg = L <= 32 && k <= 64 && rp <= 16;
   if (leaf_tc) {
-    int64_t nl = 0;
-    if ((rc = ntc_input(c, xpad, rp, &nl, true))) return rc;
+    ntc_input(c, xpad, rp, 0, rp, true);
     if ((rc = tc_leaf_forward(c, xhat, rp))) return rc;
-    mk.count(H2_PH_LEAF_FORWARD, nl + 1);
+    mk.count(H2_PH_LEAF_FORWARD, 2);
   } else if (far && leaf_reg) {
     const size_t sm = (size_t)L * (kp + rp) * sizeof(T);
     k_leaf_fwd_reg<TV, T><<<(unsigned)d.nleaf, 256, sm, st>>>((const TV *)d.V, xpad, vscale, L, kp, k, rp,
@@ -1223,7 +1235,7 @@ int matvec_typed(Ctx &c, const Tio *x, Tio *y, int nrhs, bool acc) {
     if ((rc = launch_rows<TV, T>(rows, cf_back, t_back, RL, d.nleaf, 0, ypad, st))) return rc;
     mk.count(H2_PH_LEAF_NEAR);
   }
-  if (std::is_same<T, dd>::value && d.ntc && rp <= 16) {
+  if (near_tc) {
     // FP64-accurate: integer digits on the tensor cores
     int64_t nl = 0;
     if ((rc = ntc_near(c, xpad, ypad, rp, far ? 1 : 0, &nl, leaf_tc))) return rc;
@@ -1327,14 +1339,15 @@ int matvec_gca(Ctx &c, const Tio *x, Tio *y, int nrhs, bool acc) {
   mk.mark(H2_PH_PERMUTE_IN);
   const unsigned long long *cmx = std::is_same<T, dd>::value ? d.colmax : nullptr;
   if (cmx) {
-    H2_CUDA_TRY(cudaMemsetAsync(d.colmax, 0, sizeof(unsigned long long) * nrhs, st));
+    H2_CUDA_TRY(cudaMemsetAsync(d.colmax, 0, kMaximaBytes, st));
     const int64_t nb = std::min<int64_t>((d.n + 8 * kThreads - 1) / (8 * kThreads), 64);
     k_colmax<Tio><<<dim3((unsigned)std::max<int64_t>(nb, 1), nrhs), kThreads, 0, st>>>(x, d.n, d.colmax);
     mk.count(H2_PH_PERMUTE_IN);
   }
   const unsigned perm_grid = (unsigned)((d.npad + kPermRows - 1) / kPermRows);
-  k_permute_in<Tio, T><<<perm_grid, 256, (size_t)kPermRows * (rp + 1) * sizeof(T), st>>>(x, d.n, nrhs, rp, d.pad_src,
-                                                                                        d.npad, cmx, xpad);
+  const bool near_tc = std::is_same<T, dd>::value && d.ntc;
+  k_permute_in<Tio, T><<<perm_grid, 256, (size_t)kPermRows * (rp + 1) * sizeof(T), st>>>(
+      x, d.n, nrhs, rp, d.pad_src, d.npad, cmx, xpad, near_tc ? d.ntc_xmax : nullptr);
   mk.count(H2_PH_PERMUTE_IN);
   auto X = [&](T *base, int l) { return base + d.gX[l] * rp; };
   // FP32: the warp-per-row kernel for the transfer steps and the nearfield,
@@ -1394,7 +1407,7 @@ int matvec_gca(Ctx &c, const Tio *x, Tio *y, int nrhs, bool acc) {
     if ((rc = gca_rows_launch<TS, T>(rows, L, Lp, KD, rp, d.nleaf, 0, ypad, st, wk))) return rc;
     mk.count(H2_PH_LEAF_NEAR);
   }
-  if (std::is_same<T, dd>::value && d.ntc && rp <= 16) {
+  if (near_tc) {
     int64_t nl = 0;
     if ((rc = ntc_near(c, xpad, ypad, rp, far ? 1 : 0, &nl))) return rc;
     mk.count(H2_PH_LEAF_NEAR, nl);
@@ -1800,7 +1813,9 @@ int take_device_error(Ctx &c) {
     H2_CUDA_TRY(cudaStreamSynchronize(c.stream));
     return fail(H2_ETIMEOUT, "a bounded device wait ran out; the last result is not valid");
   }
-  return (c.d.tc || c.d.ntc) ? tc_take_error(c.stream) : H2_OK;
+  int rc = c.d.tc ? tc_take_error(c.stream) : H2_OK;
+  const int rt = c.d.ntc ? tile_take_error(c.stream) : H2_OK;
+  return rc ? rc : rt;
 }
 
 int ensure_work(Ctx &c, int nrhs_req) {

@@ -643,7 +643,7 @@ int build_typed(Ctx &c) {
     H2_CUDA_TRY(cudaGetLastError());
   }
   // FP64 and FP32 handles of order 4: the E4M3 digit planes for the tensor-core coupling
-  if (!d.gca && d.tensor == 0 && tc_eligible(d) && (rc = tc_build(c, (const int32_t *)t_arow.ptr))) return rc;
+  if (!d.gca && d.tensor == 0 && tc_eligible(d) && (rc = tc_build(c))) return rc;
   H2_CUDA_TRY(cudaStreamSynchronize(st));
   c.build_ms[H2_BUILD_COUPLING] = ms_since(tc0) - (d.gca ? c.build_ms[H2_BUILD_BASES] : 0.0);
   const auto tn0 = std::chrono::steady_clock::now();
@@ -731,8 +731,8 @@ int build_typed(Ctx &c) {
       H2_CUDA_TRY(cudaGetLastError());
     }
   }
-  // FP64-accurate handles with leaves of at most 21 triangles: the nearfield digits for the tensor cores
-  if (ntc_eligible(d) && (rc = ntc_build(c, (const int32_t *)t_nrow.ptr))) return rc;
+  // FP64-accurate handles with leaves of at most 32 triangles: the nearfield digits for the tensor cores
+  if (ntc_eligible(d) && (rc = ntc_build(c))) return rc;
   H2_CUDA_TRY(cudaStreamSynchronize(st));
   c.build_ms[H2_BUILD_NEAR] = ms_since(tn0);
   return H2_OK;
@@ -782,8 +782,10 @@ int device_build(Ctx &c) {
   switch (d.prec) {
     case H2_F64: {
       d.esize = 8;
-      int rc = dev_alloc(d, (void **)&d.colmax, 64 * sizeof(unsigned long long));
+      int rc = dev_alloc(d, (void **)&d.colmax, kMaximaBytes);
       if (rc) return rc;
+      d.ntc_xmax = reinterpret_cast<unsigned *>(d.colmax + 64);
+      d.tc_xmax = d.ntc_xmax + 64;
       if (d.fused && (rc = dev_alloc(d, (void **)&d.fbar, 2 * sizeof(unsigned)))) return rc;
       return build_typed<dd>(c);
     }

@@ -1,0 +1,654 @@
+// Block rows with small tiles on the tensor cores (tcgen05, FP8 E4M3
+// operands, FP32 accumulation in tensor memory), FP64 accuracy: output rows
+// of R <= 32 values whose blocks contract over at most 32 values.  The
+// nearfield of H2_F64 handles (R = L triangles per leaf, y|t += sum G_ts x|s,
+// Algorithm 3 over the inadmissible leaf pairs) runs on it for any number of
+// right-hand sides, 16 columns per launch.
+//
+// The arithmetic is the exact digit splitting of h2_tc.cu: every row nu of
+// the blocks of one block row gets a power of two 2^E, every column j of the
+// input a power of two 2^F, a value becomes X = round(v 2^(49-E)), |X| <=
+// 2^49, cut into ten signed 5-bit digits i = 0 .. 9 of weight 2^(-4 - 5 i).
+// All digit pairs of levels i + k <= 10 are summed (and some above), one level
+// more than the tiles of h2_tc.cu sum: the pairs left out stay below 2^-51 of
+// the scales' product, the rounding of X below 2^-50 of each scale, so that
+// the result is as accurate as double-float arithmetic (which it replaces
+// beyond 16 right-hand sides and for leaves of 22 to 32 triangles).
+//
+// Layout.  The digit planes of a block are stacked four to a 128-row MMA
+// operand: digit i (from 0) of row nu lies in group i / 4, row (i mod 4) R +
+// nu (three groups; K = 32 bytes, zero padded, K-major core matrices).  The
+// input digits of a column tile are the N side: digit k (from 0), column j in
+// row W k + j, W = 4, 8 or 16 columns per digit as the right-hand sides ask,
+// followed by an eleventh, zero plane.  Group g multiplies the planes k =
+// 0 .. 10 - 4 g into accumulator columns W (4 g + k) + j: the planes of a
+// group differ in i by their lane quarter only, so column block c = 4 g + k
+// holds, in lanes R q + nu, the sum of every pair of level i + k = c + q
+// (from 0), and the tensor cores add the pairs of a level themselves.  One
+// accumulator set is 11 W columns (176, 88 or 44) instead of one per group,
+// and the epilogue reads 11 column blocks instead of 14.  The last group holds
+// two digits; its other two plane rows are zeros that stay in shared memory.
+//
+// Exactness: a set sums at most three groups of nb blocks of products of
+// magnitude <= 2^8 over R values: 3 x 2^8 x nb R <= 2^18.9 for nb R <= 661, so
+// that two neighbouring column blocks combine exactly in FP32 (32 D_c +
+// D_(c+1) < 2^24) before they enter the double-float sum.  Longer rows are cut
+// into segments of that length.
+//
+// Roles (one CTA per SM, ten warps): warp 0 streams the blocks through a
+// shared-memory ring (bulk copies completing on mbarriers), warp 1 issues the
+// MMAs, warps 2-5 and 6-9 are two epilogue groups that take the rows in turn,
+// each with its own accumulator set and exchange area.
+//
+// What bounds it: the copy stream and the MMA warp's issue.  Nearfield of
+// 327,680 triangles (leaves of 20, 179,008 blocks of 6.4 KB and as many input
+// tiles of 5.6 KB), 16 columns: 480 us before (one epilogue group, separate
+// accumulator columns per plane group, single-stage commits), 354 us now, 6.1
+// TB/s into shared memory.  Leaves of 30 (cube, 30,000 triangles, 5 columns):
+// 161 us in double-float block rows, 47 us now; 32 right-hand sides, 81,920
+// triangles: 414 us in double-float, 215 us now (two passes).
+#include <algorithm>
+#include <functional>
+#include <queue>
+#include <utility>
+#include <vector>
+
+#include "h2_internal.hpp"
+#include "h2_tc.cuh"
+
+namespace h2 {
+namespace {
+
+constexpr int kTileMax = 32;              // rows of a tile, contraction length
+constexpr int kTileThreads = 64 + 256;    // producer, MMA, two epilogue groups
+constexpr uint32_t kTilePad = 4096;       // an MMA reads 128 rows from a group's start: past the last stage at most this far
+constexpr int kTileMaxStages = 24;
+// stages released by one commit: a tcgen05.commit costs its thread about as
+// much as the three MMAs of a block (327,680 triangles, leaves of 20, 16
+// columns: 424 us with one per block, 342 us with one per four)
+constexpr int kTileGroup = 4;
+constexpr int64_t kSchedChunk = 12;       // blocks and rows of a scheduling chunk (see row_schedule)
+constexpr uint32_t kTileSmemMax = 227 * 1024;
+
+// N rows (bytes / 32) of an input digit tile, columns of an accumulator set
+template <int W>
+__host__ __device__ constexpr int tile_n() { return (11 * W + 15) / 16 * 16; }
+
+// bytes of a four-plane group, of the stored last (two-plane) group and of a stored block
+__host__ __device__ inline uint32_t tile_group(int R) { return (uint32_t)((4 * R + 7) / 8 * 8) * 32u; }
+__host__ __device__ inline uint32_t tile_last(int R) { return (uint32_t)((2 * R + 7) / 8 * 8) * 32u; }
+__host__ __device__ inline uint32_t tile_bytes(int R) { return 2 * tile_group(R) + tile_last(R); }
+// blocks per exact segment
+__host__ __device__ inline int tile_seg(int R) { return 661 / R; }
+
+// byte offset of digit i (from 0), row nu, contraction index c of a block
+__device__ __forceinline__ uint32_t tile_off(int R, int i, int nu, int c) {
+  return (uint32_t)(i >> 2) * tile_group(R) + (uint32_t)core_off32((i & 3) * R + nu, c);
+}
+
+struct TileArgs {
+  const unsigned char *A;     // stored blocks, abytes each
+  const unsigned char *X;     // input digit tiles, 32 tile_n<W>() bytes each
+  const int64_t *ptr;         // CSR over the scheduled rows (row_schedule)
+  const int32_t *col;
+  const int32_t *row;         // output row of every scheduled row
+  const int32_t *E;           // [output row][R] powers of two
+  const unsigned *xmax;       // column maxima (bits of a float)
+  const int32_t *split;       // [gridDim.x + 1]: rows of every CTA
+  dd *out;                    // [row][R][rp], at the first column of the pass
+  int R, ncol, rp, nst, accumulate;
+  uint32_t stage, xch;        // bytes of a stage, of one exchange area
+};
+
+template <int W>
+__global__ void __launch_bounds__(kTileThreads, 1) k_tile_tc(const TileArgs a) {
+  constexpr int N0 = tile_n<W>(), SET = W == 16 ? 256 : 128;
+  constexpr uint32_t kX = (uint32_t)N0 * 32u;
+  extern __shared__ __align__(1024) unsigned char smem[];
+  const int R = a.R, nst = a.nst;
+  const uint32_t ga = tile_group(R), ab = tile_bytes(R);
+  dd *xch = reinterpret_cast<dd *>(smem + (size_t)nst * a.stage + kTilePad);
+  uint64_t *full = reinterpret_cast<uint64_t *>(smem + (size_t)nst * a.stage + kTilePad + 2 * a.xch);
+  uint64_t *empty = full + kTileMaxStages;
+  uint64_t *accf = empty + kTileMaxStages;   // [2]: the MMAs of a segment have completed
+  uint64_t *acce = accf + 2;                 // [2]: the epilogue has read the set
+  uint64_t *done = acce + 2;
+  uint32_t *tslot = reinterpret_cast<uint32_t *>(done + 1);
+  volatile int *abort = reinterpret_cast<volatile int *>(tslot + 1);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int64_t r_begin = a.split[blockIdx.x], r_end = a.split[blockIdx.x + 1];
+  const int64_t e_begin = a.ptr[r_begin], e_end = a.ptr[r_end];
+
+  if (tid == 0) {
+    for (int s = 0; s < nst; ++s) {
+      mbar_init(&full[s], 1);
+      mbar_init(&empty[s], 1);
+    }
+    for (int u = 0; u < 2; ++u) {
+      mbar_init(&accf[u], 1);
+      mbar_init(&acce[u], 4);
+    }
+    mbar_init(done, 1);
+    *abort = 0;
+    mbar_fence_init();
+  }
+  if (warp == 1) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tslot)),
+                 "r"(2 * SET)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  // the zero plane rows of the last group, in every stage (the copies never touch them)
+  {
+    const int words = (int)(3 * ga - ab) / 16;
+    for (int i = tid; i < words * nst; i += kTileThreads)
+      *reinterpret_cast<uint4 *>(smem + (size_t)(i / words) * a.stage + ab + 16 * (i % words)) = make_uint4(0, 0, 0, 0);
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tbase = *tslot;
+  const int64_t seg = tile_seg(R);
+
+  if (warp == 0) {
+    // ---------------- producer: the digits of every block of the range and of its column tile
+    if (lane == 0) {
+      int64_t e = e_begin;
+      ColAhead ca(a.col, e, e_end);
+      const uint64_t pol_stream = l2_evict_first(), pol_keep = l2_evict_last();
+      int s = 0;
+      uint32_t ph = 1;   // parity of the stage's previous release
+      bool ok = true;
+      while (e < e_end && ok) {
+        int32_t cb[8];
+        ca.take(e, cb);
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+          if (e >= e_end || !ok) break;
+          if (s % kTileGroup == 0 && e - e_begin >= nst && !mbar_wait_or_abort(&empty[s / kTileGroup], ph, abort)) {
+            ok = false;
+            break;
+          }
+          unsigned char *st = smem + (size_t)s * a.stage;
+          mbar_expect_tx(&full[s], ab + kX);
+          bulk_g2s_hint(st + 3 * ga, a.X + (int64_t)cb[u] * kX, kX, &full[s], pol_keep);
+          bulk_g2s_hint(st, a.A + e * (int64_t)ab, ab, &full[s], pol_stream);
+          ++e;
+          if (++s == nst) {
+            s = 0;
+            ph ^= 1;
+          }
+        }
+      }
+      if (*abort) {
+        // let the copies in flight land before the CTA leaves (bounded)
+        const int64_t j0 = e - nst > e_begin ? e - nst : e_begin;
+        for (int64_t j = j0; j < e; ++j) {
+          const int64_t ij = j - e_begin;
+          mbar_wait_bounded(&full[ij % nst], (uint32_t)((ij / nst) & 1));
+        }
+      }
+    }
+    __syncwarp();
+  } else if (warp == 1) {
+    // ---------------- MMA issuer (the whole warp waits, an elected lane issues)
+    {
+      int s = 0;
+      uint32_t ph = 0, use[2] = {0, 0}, set = 1;
+      bool ok = true;
+      int64_t pnext = a.ptr[r_begin];   // row pointers loaded one row ahead
+      for (int64_t r = r_begin; r < r_end && ok; ++r) {
+        const int64_t b0 = pnext;
+        pnext = a.ptr[r + 1];
+        const int64_t nb = pnext - b0;
+        if (nb > 0) set ^= 1;   // the rows that have blocks alternate between the two groups
+        for (int64_t s0 = 0; s0 < nb && ok; s0 += seg) {
+          const uint32_t u = set ? use[1]++ : use[0]++;
+          if (u > 0 && !mbar_wait_or_abort(&acce[set], (u - 1) & 1, abort)) {
+            ok = false;
+            break;
+          }
+          tc_fence_after();
+          const uint32_t d0 = tbase + set * SET;
+          const int64_t sn = nb - s0 < seg ? nb - s0 : seg;
+          for (int64_t t = 0; t < sn; ++t) {
+            if (!mbar_wait_or_abort(&full[s], ph, abort)) {
+              ok = false;
+              break;
+            }
+            tc_fence_after();
+            const uint32_t A0 = smem_u32(smem + (size_t)s * a.stage);
+            const uint64_t dA = sdesc32(A0), dB = sdesc32(A0 + 3 * ga);
+            // group 0 covers every column of the set, so its MMA of the first block overwrites it
+#pragma unroll
+            for (int g = 0; g < 3; ++g)
+              tc_mma(d0 + 4 * g * W, dA + (uint64_t)((g * ga) >> 4), dB, tc_idesc(((11 - 4 * g) * W + 15) / 16 * 16),
+                     (t > 0 || g > 0) ? 1u : 0u);
+            // the stages of a group are free once these MMAs have read them
+            if (s % kTileGroup == kTileGroup - 1) tc_commit(&empty[s / kTileGroup]);
+            if (++s == nst) {
+              s = 0;
+              ph ^= 1;
+            }
+          }
+          if (ok) tc_commit(&accf[set]);
+        }
+      }
+      // every MMA issued has completed before the tensor memory is released
+      tc_commit(done);
+      mbar_wait_bounded(done, 0);
+    }
+    __syncwarp();
+  } else {
+    // ---------------- epilogue group grp: warps read tensor-memory lanes 32 (warp % 4) ..
+    const uint32_t grp = (uint32_t)(warp - 2) >> 2;
+    const int quad = warp & 3, tl = quad * 32 + lane;
+    const int pitch = 4 * R + 1, nout = R * a.ncol;
+    dd *xg = xch + (size_t)grp * (a.xch / sizeof(dd));
+    const uint32_t bar_or = 1 + 2 * grp, bar_x = 2 + 2 * grp;
+    const uint32_t tset = tbase + ((uint32_t)(quad * 32) << 16) + grp * SET;
+    const bool plane = tl < 4 * R;
+    const float wq = pow2f(-5 * (plane ? tl / R : 0));
+    // this thread's outputs o = tl + 128 u: row o / ncol, column o % ncol
+    constexpr int UO = W / 4;
+    int orow[UO], ocol[UO], fexp[UO];
+#pragma unroll
+    for (int u = 0; u < UO; ++u) {
+      const int o = tl + 128 * u;
+      orow[u] = o < nout ? o / a.ncol : 0;
+      ocol[u] = o < nout ? o % a.ncol : 0;
+      fexp[u] = tc_colexp(a.xmax[ocol[u]]);
+    }
+    uint32_t use = 0, set = 1;
+    int64_t pnext = a.ptr[r_begin];
+    int32_t rnext = r_begin < r_end ? a.row[r_begin] : 0;
+    for (int64_t r = r_begin; r < r_end; ++r) {
+      const int64_t b0 = pnext, orow_id = rnext;
+      pnext = a.ptr[r + 1];
+      if (r + 1 < r_end) rnext = a.row[r + 1];
+      const int64_t nb = pnext - b0;
+      dd *yrow = a.out + orow_id * R * a.rp;
+      if (nb == 0) {
+        if (!a.accumulate && grp == 0)
+#pragma unroll
+          for (int u = 0; u < UO; ++u)
+            if (tl + 128 * u < nout) yrow[orow[u] * a.rp + ocol[u]] = dd{0.0f, 0.0f};
+        continue;
+      }
+      set ^= 1;
+      if (set != grp) continue;
+      bool stop = false;
+      for (int64_t s0 = 0; s0 < nb; s0 += seg, ++use) {
+        // row powers and previous values are loaded before the wait
+        int eo[UO];
+        dd yold[UO];
+#pragma unroll
+        for (int u = 0; u < UO; ++u) {
+          eo[u] = 0;
+          yold[u] = dd{0.0f, 0.0f};
+          if (tl + 128 * u < nout) {
+            eo[u] = a.E[orow_id * R + orow[u]] + fexp[u];
+            if (s0 > 0 || a.accumulate) yold[u] = yrow[orow[u] * a.rp + ocol[u]];
+          }
+        }
+        const bool ready = !*abort && mbar_wait_or_abort(&accf[grp], use & 1, abort);
+        if (named_sync_or_id(bar_or, 128, ready ? 0 : 1)) {
+          stop = true;
+          break;
+        }
+        tc_fence_after();
+        // column blocks c, c + 1 combine exactly; weight 2^(-8 - 5 (c + 1)), times 2^(-5 q) at the end
+        dd acc[W];
+#pragma unroll
+        for (int j = 0; j < W; ++j) acc[j] = dd{0.0f, 0.0f};
+#pragma unroll
+        for (int base = 0; base < N0; base += 64) {
+          uint32_t raw[4][16];
+#pragma unroll
+          for (int u = 0; u < 4; ++u)
+            if (base + 16 * u < N0) tmem_ld16_nw(tset + (uint32_t)(base + 16 * u), raw[u]);
+          tmem_wait();
+#pragma unroll
+          for (int cb = 0; cb < 64 / W; cb += 2) {
+            const int c = base / W + cb;
+            if (c < 11) {
+              const float w = pow2f(-8 - 5 * (c + 1));
+#pragma unroll
+              for (int j = 0; j < W; ++j) {
+                const int p = cb * W + j, p1 = p + W;
+                float v = 32.0f * __uint_as_float(raw[p >> 4][p & 15]);
+                if (c + 1 < 11) v += __uint_as_float(raw[(p1 >> 4) & 3][p1 & 15]);
+                float s, e;
+                two_sum(acc[j].hi, v * w, s, e);
+                acc[j].hi = s;
+                acc[j].lo += e;
+              }
+            }
+          }
+        }
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&acce[grp]);
+        if (plane)
+#pragma unroll
+          for (int j = 0; j < W; ++j) {
+            acc_norm(acc[j]);
+            xg[j * pitch + tl] = dd{acc[j].hi * wq, acc[j].lo * wq};
+          }
+        named_sync_id(bar_x, 128);
+#pragma unroll
+        for (int u = 0; u < UO; ++u) {
+          if (tl + 128 * u >= nout) continue;
+          const dd *xc = xg + ocol[u] * pitch + orow[u];
+          dd v = xc[0];
+#pragma unroll
+          for (int q = 1; q < 4; ++q) v = v + xc[q * R];
+          v = dd_scale(v, eo[u]);
+          if (s0 > 0 || a.accumulate) v = v + yold[u];
+          yrow[orow[u] * a.rp + ocol[u]] = v;
+        }
+        named_sync_id(bar_x, 128);
+      }
+      if (stop) break;
+    }
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  if (warp == 1)
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tbase), "r"(2 * SET) : "memory");
+}
+
+// The input digit tiles of items first .. first + count - 1 (R rows of rp
+// values each, columns 0 .. ncol - 1 of x): 2 W threads per item, thread (g,
+// j) cuts rows 16 g .. 16 g + 15 of column j in registers (zero beyond R and
+// ncol) and writes one 16-byte row of a core matrix per plane, and the zero
+// rows behind the ten planes.
+template <int W>
+__global__ void __launch_bounds__(128) k_tile_cut(const dd *__restrict__ x, int64_t first, int64_t count, int R,
+                                                  int rp, int ncol, const unsigned *__restrict__ xmax,
+                                                  unsigned char *__restrict__ X) {
+  constexpr int N0 = tile_n<W>();
+  const int64_t i = (int64_t)blockIdx.x * (64 / W) + threadIdx.x / (2 * W);
+  if (i >= count) return;
+  const int64_t t = first + i;
+  const int g = (threadIdx.x / W) & 1, j = threadIdx.x % W;
+  const int sc = kTcFixBits - tc_colexp(j < ncol ? xmax[j] : 0u);
+  dd v[16];
+#pragma unroll
+  for (int q = 0; q < 16; ++q) {
+    const int mu = 16 * g + q;
+    v[q] = mu < R && j < ncol ? x[(t * R + mu) * rp + j] : dd{0.0f, 0.0f};
+  }
+  uint4 w[kTcSlices];
+  cut_row16<kTcSlices>(v, sc, w);
+  unsigned char *dst = X + t * (int64_t)(32 * N0) + g * 128;
+#pragma unroll
+  for (int k = 0; k < kTcSlices; ++k) {
+    const int n = W * k + j;
+    *reinterpret_cast<uint4 *>(dst + (n >> 3) * 256 + (n & 7) * 16) = w[k];
+  }
+  for (int n = W * kTcSlices + j; n < N0; n += W)
+    *reinterpret_cast<uint4 *>(dst + (n >> 3) * 256 + (n & 7) * 16) = make_uint4(0, 0, 0, 0);
+}
+
+// E[t][nu] = 1 + floor(log2 max |G_b[nu][mu]|) over the near blocks b of leaf row t (0 if none)
+__global__ void k_near_rowexp(const dd *__restrict__ near, const int64_t *__restrict__ ptr, int64_t nleaf, int L,
+                              int Lp, int32_t *__restrict__ E) {
+  const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (e >= nleaf * L) return;
+  const int64_t t = e / L;
+  const int nu = (int)(e % L);
+  float mx = 0.0f;
+  for (int64_t b = ptr[t]; b < ptr[t + 1]; ++b)
+    for (int mu = 0; mu < L; ++mu) mx = fmaxf(mx, fabsf(near[(b * L + mu) * Lp + nu].hi));
+  E[e] = mx > 0.0f ? ilogbf(mx) + 1 : 0;
+}
+
+// the ten digit planes of scheduled block d (near block src[d], row leaf brow[d]), row nu,
+// contraction indices 16 cg .. 16 cg + 15
+__global__ void k_near_slice(const dd *__restrict__ near, const int32_t *__restrict__ src,
+                             const int32_t *__restrict__ brow, const int32_t *__restrict__ E, int64_t nnear, int L,
+                             int Lp, unsigned char *__restrict__ A) {
+  const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (e >= nnear * L * 2) return;
+  const int64_t d = e / (2 * L), b = src[d];
+  const int nu = (int)((e / 2) % L), cg = (int)(e % 2);
+  const int sc = kTcFixBits - E[(int64_t)brow[d] * L + nu];
+  __align__(16) unsigned char out[kTcSlices][16];
+#pragma unroll
+  for (int q = 0; q < 16; ++q) {
+    const int mu = 16 * cg + q;
+    long long X = 0;
+    if (mu < L) {
+      const dd v = near[(b * L + mu) * Lp + nu];
+      X = llrint(ldexp((double)v.hi + (double)v.lo, sc));
+    }
+    int sl[kTcSlices];
+    split_digits(X, sl);
+#pragma unroll
+    for (int i = 0; i < kTcSlices; ++i) out[i][q] = e4m3(sl[i]);
+  }
+  unsigned char *base = A + d * (int64_t)tile_bytes(L);
+#pragma unroll
+  for (int i = 0; i < kTcSlices; ++i)
+    *reinterpret_cast<uint4 *>(base + tile_off(L, i, nu, 16 * cg)) = *reinterpret_cast<const uint4 *>(out[i]);
+}
+
+// W of a pass over ncol columns
+int tile_width(int ncol) { return ncol <= 4 ? 4 : ncol <= 8 ? 8 : 16; }
+
+template <int W>
+int tile_launch(TileArgs a, int grid, cudaStream_t st) {
+  a.xch = (uint32_t)((W * (4 * a.R + 1) * (int)sizeof(dd) + 127) / 128 * 128);
+  a.stage = 3 * tile_group(a.R) + 32 * tile_n<W>();
+  const uint32_t fixed = kTilePad + 2 * a.xch + 8 * (2 * kTileMaxStages + 5) + 16;
+  a.nst = (int)std::min<uint32_t>(kTileMaxStages, (kTileSmemMax - fixed) / a.stage) / kTileGroup * kTileGroup;
+  H2_CUDA_TRY(cudaFuncSetAttribute((const void *)k_tile_tc<W>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                   (int)kTileSmemMax));
+  k_tile_tc<W><<<grid, kTileThreads, a.nst * a.stage + fixed, st>>>(a);
+  H2_CUDA_TRY(cudaGetLastError());
+  return H2_OK;
+}
+
+int tile_run(const TileArgs &a, int width, int grid, cudaStream_t st) {
+  switch (width) {
+    case 4: return tile_launch<4>(a, grid, st);
+    case 8: return tile_launch<8>(a, grid, st);
+    default: return tile_launch<16>(a, grid, st);
+  }
+}
+
+template <int W>
+void cut_launch(const dd *x, int64_t first, int64_t count, int R, int rp, int ncol, const unsigned *xmax,
+                unsigned char *X, cudaStream_t st) {
+  constexpr int per = 64 / W;
+  k_tile_cut<W><<<(unsigned)((count + per - 1) / per), 128, 0, st>>>(x, first, count, R, rp, ncol, xmax, X);
+}
+
+void tile_cut(const dd *x, int64_t first, int64_t count, int R, int rp, int ncol, const unsigned *xmax,
+              unsigned char *X, int width, cudaStream_t st) {
+  switch (width) {
+    case 4: return cut_launch<4>(x, first, count, R, rp, ncol, xmax, X, st);
+    case 8: return cut_launch<8>(x, first, count, R, rp, ncol, xmax, X, st);
+    default: return cut_launch<16>(x, first, count, R, rp, ncol, xmax, X, st);
+  }
+}
+
+}  // namespace
+
+// The order in which the CTAs of a block-row kernel take their rows, laid out
+// at set-up.  Rows are cut into chunks of neighbouring rows (a few dozen
+// blocks) and every chunk, in row order, goes to the CTA that has the least to
+// do so far: the CTAs work through the rows side by side, so that they read
+// the input tiles of one neighbourhood of the tree at a time (all of them
+// together exceed L2), and their shares differ by less than a chunk.  A row
+// counts its blocks and one more for its epilogue.  The stored blocks follow
+// this order, so that a CTA's blocks are one contiguous stream, and its row
+// range is two loads instead of two binary searches of the row pointers
+// (chains of some 15 dependent loads each).  Chunks of 12 / 32 / 128 / 512
+// blocks and rows at 327,680 triangles, 16 right-hand sides: F64 coupling
+// 1,905 / 1,911 / 1,925 / 2,004 us, nearfield 354 / 361 / 373 / 383 us.
+int row_schedule(Dev &d, const int64_t *ptr, const int32_t *col, int64_t nrows, RowSched &s, SchedTmp &tmp,
+                 cudaStream_t st) {
+  int dev = 0, sms = 0;
+  H2_CUDA_TRY(cudaGetDevice(&dev));
+  H2_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+  const int g = (int)std::max<int64_t>(1, std::min<int64_t>(sms, nrows));
+  const int64_t nblk = ptr[nrows] - ptr[0];
+  const int64_t chunk = std::min<int64_t>(kSchedChunk, (nblk + nrows) / (8 * g));
+  std::vector<std::vector<int32_t>> mine(g);
+  // (load, CTA), least load first, ties to the lower CTA
+  std::priority_queue<std::pair<int64_t, int>, std::vector<std::pair<int64_t, int>>, std::greater<>> next;
+  for (int w = 0; w < g; ++w) next.push({0, w});
+  for (int64_t r = 0; r < nrows;) {
+    auto [load, w] = next.top();
+    next.pop();
+    int64_t c = 0;
+    do {
+      mine[w].push_back((int32_t)r);
+      c += ptr[r + 1] - ptr[r] + 1;
+      ++r;
+    } while (r < nrows && c + (ptr[r + 1] - ptr[r]) + 1 <= chunk);
+    next.push({load + c, w});
+  }
+  std::vector<int32_t> row, split(g + 1), cols, src, brow;
+  std::vector<int64_t> p2;
+  row.reserve(nrows);
+  p2.reserve(nrows + 1);
+  cols.reserve(nblk);
+  src.reserve(nblk);
+  brow.reserve(nblk);
+  for (int w = 0; w < g; ++w) {
+    split[w] = (int32_t)row.size();
+    for (int32_t r : mine[w]) {
+      row.push_back(r);
+      p2.push_back((int64_t)cols.size());
+      for (int64_t e = ptr[r]; e < ptr[r + 1]; ++e) {
+        cols.push_back(col[e]);
+        src.push_back((int32_t)e);
+        brow.push_back(r);
+      }
+    }
+  }
+  split[g] = (int32_t)row.size();
+  p2.push_back((int64_t)cols.size());
+  int rc;
+  auto up = [&](void **dst, const void *from, size_t bytes) -> int {
+    int r = dev_alloc(d, dst, bytes);
+    if (r) return r;
+    if (bytes) H2_CUDA_TRY(cudaMemcpyAsync(*dst, from, bytes, cudaMemcpyHostToDevice, st));
+    return H2_OK;
+  };
+  if ((rc = up((void **)&s.row, row.data(), row.size() * 4)) || (rc = up((void **)&s.ptr, p2.data(), p2.size() * 8)) ||
+      (rc = up((void **)&s.col, cols.data(), cols.size() * 4)) ||
+      (rc = up((void **)&s.split, split.data(), split.size() * 4)))
+    return rc;
+  for (auto [dst, from] : {std::pair<int32_t **, std::vector<int32_t> *>{&tmp.src, &src}, {&tmp.brow, &brow}}) {
+    if (dmalloc(dst, std::max<size_t>(from->size() * 4, 16)) != cudaSuccess) {
+      cudaGetLastError();
+      return fail(H2_ENOMEM, "device set-up buffer");
+    }
+    H2_CUDA_TRY(cudaMemcpyAsync(*dst, from->data(), from->size() * 4, cudaMemcpyHostToDevice, st));
+  }
+  H2_CUDA_TRY(cudaStreamSynchronize(st));
+  s.grid = g;
+  return H2_OK;
+}
+
+SchedTmp::~SchedTmp() {
+  if (src) cudaFree(src);
+  if (brow) cudaFree(brow);
+}
+
+// FP64-accurate handles with leaves of at most 32 triangles, unless the
+// digits would take more than half of the free device memory
+bool ntc_eligible(const Dev &d) {
+  if (!(d.prec == H2_F64 && d.tensor == 0 && d.lmax <= kTileMax && d.nnear > 0)) return false;
+  size_t fr = 0, tot = 0;
+  if (cudaMemGetInfo(&fr, &tot) != cudaSuccess) return false;
+  return (double)d.nnear * tile_bytes((int)d.lmax) + (double)d.nleaf * 32 * tile_n<kTcN>() <= 0.5 * (double)fr;
+}
+
+int ntc_build(Ctx &c) {
+  Dev &d = c.d;
+  cudaStream_t st = c.stream;
+  const int L = (int)d.lmax, Lp = (int)d.lp;
+  const uint32_t ab = tile_bytes(L);
+  int rc;
+  if ((rc = dev_alloc(d, (void **)&d.ntc_E, sizeof(int32_t) * (size_t)d.nleaf * L))) return rc;
+  if ((rc = dev_alloc(d, &d.Ntc, (size_t)d.nnear * ab))) return rc;
+  if ((rc = dev_alloc(d, &d.xnt, (size_t)d.nleaf * 32 * tile_n<kTcN>()))) return rc;
+  SchedTmp tmp;
+  if ((rc = row_schedule(d, c.plan.near_ptr.data(), c.plan.near_col.data(), d.nleaf, d.ntc_s, tmp, st))) return rc;
+  H2_CUDA_TRY(cudaMemsetAsync(d.Ntc, 0, (size_t)d.nnear * ab, st));
+  const int64_t nr = d.nleaf * L;
+  k_near_rowexp<<<(unsigned)((nr + 127) / 128), 128, 0, st>>>((const dd *)d.near, d.near_ptr, d.nleaf, L, Lp,
+                                                              d.ntc_E);
+  const int64_t ns = d.nnear * L * 2;
+  k_near_slice<<<(unsigned)((ns + 255) / 256), 256, 0, st>>>((const dd *)d.near, tmp.src, tmp.brow, d.ntc_E, d.nnear, L,
+                                                             Lp, (unsigned char *)d.Ntc);
+  H2_CUDA_TRY(cudaGetLastError());
+  if ((rc = tc_leaf_build(c))) return rc;
+  H2_CUDA_TRY(cudaStreamSynchronize(st));
+  d.ntc = true;
+  return H2_OK;
+}
+
+// the digit tiles of columns c0 .. c0 + ncol - 1 of the permuted input
+void ntc_input(Ctx &c, const void *xpad, int rp, int c0, int ncol, bool wide) {
+  Dev &d = c.d;
+  tile_cut(static_cast<const dd *>(xpad) + c0, 0, d.nleaf, (int)d.lmax, rp, ncol, d.ntc_xmax + c0,
+           (unsigned char *)d.xnt, wide ? kTcN : tile_width(ncol), c.stream);
+}
+
+// The nearfield phase (y_pad += or = the near sums), 16 columns per pass.
+// The input's column maxima are in place (k_permute_in); have_input: so are
+// the wide digit tiles of the one pass of at most 16 columns.
+int ntc_near(Ctx &c, const void *xpad, void *ypad, int rp, int accumulate, int64_t *launches, bool have_input) {
+  Dev &d = c.d;
+  int64_t nl = 0;
+  for (int c0 = 0; c0 < rp; c0 += kTcN) {
+    const int ncol = std::min(kTcN, rp - c0);
+    if (!have_input) {
+      ntc_input(c, xpad, rp, c0, ncol, false);
+      ++nl;
+    }
+    TileArgs a{};
+    a.A = (const unsigned char *)d.Ntc;
+    a.X = (const unsigned char *)d.xnt;
+    a.ptr = d.ntc_s.ptr;
+    a.col = d.ntc_s.col;
+    a.row = d.ntc_s.row;
+    a.split = d.ntc_s.split;
+    a.E = d.ntc_E;
+    a.xmax = d.ntc_xmax + c0;
+    a.out = static_cast<dd *>(ypad) + c0;
+    a.R = (int)d.lmax;
+    a.ncol = ncol;
+    a.rp = rp;
+    a.accumulate = accumulate;
+    const int rc = tile_run(a, have_input ? kTcN : tile_width(ncol), d.ntc_s.grid, c.stream);
+    if (rc) return rc;
+    ++nl;
+  }
+  H2_CUDA_TRY(cudaGetLastError());
+  if (launches) *launches = nl;
+  return H2_OK;
+}
+
+// this file's device error word (its bounded waits)
+int tile_take_error(cudaStream_t st) {
+  int v = 0, zero = 0;
+  H2_CUDA_TRY(cudaMemcpyFromSymbolAsync(&v, g_h2_device_error, sizeof(int), 0, cudaMemcpyDeviceToHost, st));
+  H2_CUDA_TRY(cudaStreamSynchronize(st));
+  if (v) {
+    H2_CUDA_TRY(cudaMemcpyToSymbolAsync(g_h2_device_error, &zero, sizeof(int), 0, cudaMemcpyHostToDevice, st));
+    H2_CUDA_TRY(cudaStreamSynchronize(st));
+    return fail(H2_ETIMEOUT, "a bounded device wait of the tensor-core block rows ran out");
+  }
+  return H2_OK;
+}
+
+}  // namespace h2

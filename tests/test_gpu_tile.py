@@ -1,0 +1,72 @@
+"""Block rows with small tiles on the tensor cores (h2_tile.cu) at the edges of
+their range: leaves of 2 to 32 triangles, 1 to 64 right-hand sides (every tile
+width and several passes), and rows of many blocks (several exact segments).
+
+Tolerance: the digits are rounded to 2^-50 of their scales and the digit pairs
+left out stay below 2^-51 of them, so the double-float operations around them
+(2^-44 = 5.7e-14 per operation) bound the error; 1e-13 against the FP64 oracle."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_2203_05665_gb300 import H2Matrix, colmajor, inputs as I
+
+pytestmark = pytest.mark.gpu
+TOL = 1e-13
+
+
+def _patch(n):
+    """The first n triangles of a 1,280-triangle sphere."""
+    v, f = I.icosphere(3)
+    return v, np.ascontiguousarray(f[:n])
+
+
+def _rel(a, b):
+    return np.linalg.norm(a - b) / np.linalg.norm(b)
+
+
+@pytest.mark.parametrize("leaf", [2, 7, 8, 9, 16, 17, 21, 22, 31, 32])
+def test_nearfield_leaf_sizes(require_gpu, leaf):
+    v, f = _patch(8 * leaf)
+    o = oracle.Oracle(v, f, leaf_size=leaf, eta=2.0, order=3)
+    h = H2Matrix(v, f, leaf_size=leaf, eta=2.0, order=3, prec="f64")
+    assert h.stats["leaf_max"] == leaf and h.stats["tensor_near"] == 1
+    for nrhs in (1, 4, 5, 8, 9, 16, 17, 24, 33, 64):
+        x = I.uniform_rhs(8 * leaf, nrhs, 5000 + nrhs)
+        assert _rel(h.matvec_host(x), o.matvec(x)) <= TOL, nrhs
+    h.close()
+
+
+@pytest.mark.parametrize("leaf", [3, 21, 32])
+def test_nearfield_long_rows(require_gpu, leaf):
+    """No admissible block (small eta): rows of 32 blocks, one to two exact segments of 661 // leaf blocks,
+    and the rows of a mesh with ragged leaves."""
+    for n in (32 * leaf, 32 * leaf - 5):
+        v, f = _patch(n)
+        o = oracle.Oracle(v, f, leaf_size=leaf, eta=1e-3, order=2)
+        h = H2Matrix(v, f, leaf_size=leaf, eta=1e-3, order=2, prec="f64")
+        assert h.stats["adm_blocks"] == 0 and h.stats["tensor_near"] == 1
+        for nrhs in (3, 7, 20):
+            x = I.uniform_rhs(n, nrhs, 5100 + nrhs)
+            assert _rel(h.matvec_host(x), o.matvec(x)) <= TOL, (n, nrhs)
+        h.close()
+
+
+def test_columns_with_infinity_or_nan(require_gpu):
+    """Every output depends on every input: a column with an infinity or a NaN gives NaN throughout,
+    the other columns are not touched by it."""
+    import torch
+    v, f = I.icosphere(3)
+    n = f.shape[0]
+    for order in (3, 4):
+        h = H2Matrix(v, f, leaf_size=32, eta=2.0, order=order, prec="f64")
+        for nrhs in (4, 20):
+            x = colmajor(torch.from_numpy(I.uniform_rhs(n, nrhs, 5200)).cuda())
+            y0, y1 = colmajor(torch.empty_like(x)), colmajor(torch.empty_like(x))
+            h.matvec(x, y0)
+            x[7, 1], x[n - 1, 3] = float("inf"), float("nan")
+            h.matvec(x, y1)
+            good = [c for c in range(nrhs) if c not in (1, 3)]
+            assert torch.isnan(y1[:, [1, 3]]).all()
+            assert torch.equal(y0[:, good], y1[:, good])
+        h.close()
