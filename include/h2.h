@@ -88,10 +88,13 @@ typedef struct h2_options {
                       * entry, a power of two per row) and runs the coupling phase of products with
                       * up to 16 right-hand sides on the tensor cores (integer digit products summed
                       * exactly, combined in double-float; agrees with the double-float path to
-                      * about 1e-13); an H2_F32 handle of order 4 with stored coupling does the
+                      * about 1e-13); an H2_F64 handle of order 3 with stored coupling does the same for
+                      * any number of right-hand sides (9 KB per block); an H2_F32 handle of order 4 with stored coupling does the
                       * same with 6 digits (6 bytes per entry, FP32 accuracy); any H2_F64 handle
                       * with leaves of at most 32 triangles keeps its nearfield blocks as 10-digit
-                      * planes and runs the nearfield phase on the tensor cores; 1: never */
+                      * planes and runs the nearfield phase on the tensor cores.  Digits that would
+                      * take more than half of the free device memory (order 3, nearfield) are not
+                      * built; 1: never */
   int basis_prec;    /* storage of the leaf bases V (Eq. (6a)) and the transfer factors (Eq. (9))
                       * of H2_BF16 / H2_F16 handles: 0 = the default, H2_F32 for H2_BF16 (V in
                       * bfloat16 costs about 1e-3 of relative accuracy, amplified by the Lebesgue

@@ -376,7 +376,7 @@ int h2_info(h2_handle h, h2_stats *out) {
   out->device_bytes = h->d.bytes;
   out->prec = h->d.prec;
   out->coupling = h->d.coupling == 1 ? H2_COUPLING_REGEN : H2_COUPLING_STORED;
-  out->tensor = h->d.tc ? 1 : 0;
+  out->tensor = h->d.tc || h->d.tct ? 1 : 0;
   out->tensor_near = h->d.ntc ? 1 : 0;
   out->tensor_leaf = h->d.Vtc ? 1 : 0;
   out->basis_prec = h->d.v32 ? H2_F32 : h->d.prec;

@@ -128,7 +128,8 @@ struct Dev {
   // the coefficients of one product ([nclu][tc_nd][16 x 64]) and the column
   // maxima per level ([32][64])
   int tensor = 0;               // 0: use the tensor cores where supported, 1: never
-  bool tc = false;              // the digits exist
+  bool tc = false;              // the digits exist (order 4)
+  bool tct = false;             // the same for order 3: tiles of h2_tile.cu in Stc, xtc ([nclu][11 x 16 x 32])
   int tc_nd = 0;                // digits per value: 10 (FP64-accurate) or 6 (FP32 handles)
   void *Stc = nullptr, *xtc = nullptr;
   int32_t *tc_E = nullptr;
@@ -269,6 +270,12 @@ void ntc_input(Ctx &c, const void *xpad, int rp, int c0, int ncol, bool wide);
 int ntc_near(Ctx &c, const void *xpad, void *ypad, int rp, int accumulate, int64_t *launches,
              bool have_input = false);
 int tile_take_error(cudaStream_t st);
+// FP64-accurate order-3 coupling on the tensor cores (h2_tile.cu)
+bool tct_eligible(const Dev &d);
+int tct_build(Ctx &c);
+void tct_leaf_max(Ctx &c, const void *xhat, int rp);
+int tct_coupling(Ctx &c, const void *xhat, void *yhat, int rp, int64_t *launches);
+constexpr int kLevelCols = 64;   // column maxima per tree level
 int row_schedule(Dev &d, const int64_t *ptr, const int32_t *col, int64_t nrows, RowSched &s, SchedTmp &tmp,
                  cudaStream_t st);
 // H2_F64 handles: the range guard's column maxima (64 x 8 bytes), the input's

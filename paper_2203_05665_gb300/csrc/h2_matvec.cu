@@ -994,13 +994,16 @@ int launch_rows(const Rows &rows, const RowCfg &cfg, int threads, int R, int64_t
 // (nu, jq) forms x^[nu][jq + 4u], in the backward step thread (r, jo) forms
 // y[r][jo + 8u], each as one contraction with a single renormalisation, then
 // multiplied by the leaf's power-of-two scale (16-bit storage) if there is
-// one.  The generic block-row kernel pipelines many terms per row; a leaf
+// one; with MAX the forward step also takes the largest |x^| (|hi|) of every
+// column, as float bits.  The generic block-row kernel pipelines many terms per row; a leaf
 // row has one.
-template <class TS, class T>
+template <class TS, class T, bool MAX>
 __global__ void __launch_bounds__(256) k_leaf_fwd_reg(const TS *__restrict__ V, const T *__restrict__ xpad,
                                                       const float *__restrict__ vscale, int L, int kp, int k, int rp,
-                                                      T *__restrict__ xleaf) {
+                                                      T *__restrict__ xleaf, unsigned *__restrict__ xmax) {
   extern __shared__ __align__(16) unsigned char lsm[];
+  __shared__ unsigned smax[16];
+  if (MAX && threadIdx.x < 16) smax[threadIdx.x] = 0u;
   T *Vs = reinterpret_cast<T *>(lsm);   // [L][kp]
   T *xs = Vs + L * kp;                   // [L][rp]
   const int64_t t = blockIdx.x;
@@ -1010,23 +1013,31 @@ __global__ void __launch_bounds__(256) k_leaf_fwd_reg(const TS *__restrict__ V, 
   for (int i = threadIdx.x; i < L * rp; i += blockDim.x) xs[i] = xt[i];
   __syncthreads();
   const int nu = threadIdx.x >> 2, jq = threadIdx.x & 3;
-  if (nu >= k) return;
-  T acc[4];
+  if (nu < k) {
+    T acc[4];
 #pragma unroll
-  for (int u = 0; u < 4; ++u) acc[u] = zero_of<T>();
-  for (int r = 0; r < L; ++r) {
-    const T v = Vs[r * kp + nu];
+    for (int u = 0; u < 4; ++u) acc[u] = zero_of<T>();
+    for (int r = 0; r < L; ++r) {
+      const T v = Vs[r * kp + nu];
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (jq + 4 * u < rp) acc_fma(acc[u], v, xs[r * rp + jq + 4 * u]);
+    }
+    const float sc = vscale ? vscale[t] : 1.0f;
 #pragma unroll
     for (int u = 0; u < 4; ++u)
-      if (jq + 4 * u < rp) acc_fma(acc[u], v, xs[r * rp + jq + 4 * u]);
+      if (jq + 4 * u < rp) {
+        acc_norm(acc[u]);
+        const T v = vscale ? acc[u] * from_double<T>(sc) : acc[u];
+        xleaf[(t * k + nu) * rp + jq + 4 * u] = v;
+        if (MAX) atomicMax(&smax[jq + 4 * u], __float_as_uint(mag_of(v)));
+      }
   }
-  const float sc = vscale ? vscale[t] : 1.0f;
-#pragma unroll
-  for (int u = 0; u < 4; ++u)
-    if (jq + 4 * u < rp) {
-      acc_norm(acc[u]);
-      xleaf[(t * k + nu) * rp + jq + 4 * u] = vscale ? acc[u] * from_double<T>(sc) : acc[u];
-    }
+  if (MAX) {
+    // one look at the maximum so far spares most CTAs the atomic on a contended word
+    __syncthreads();
+    if (threadIdx.x < 16 && smax[threadIdx.x] > __ldcg(&xmax[threadIdx.x])) atomicMax(&xmax[threadIdx.x], smax[threadIdx.x]);
+  }
 }
 
 // With gself (FP32 self blocks of bfloat16 handles, [leaf][c][Lp]) the
@@ -1117,6 +1128,8 @@ int matvec_typed(Ctx &c, const Tio *x, Tio *y, int nrhs, bool acc) {
   // permutation takes the input's column maxima on the way
   const bool near_tc = std::is_same<T, dd>::value && d.ntc;
   const bool leaf_tc = near_tc && far && d.Vtc && rp <= 16;
+  // order-3 coupling on the tensor cores: the upward pass takes every level's column maxima
+  const bool cpl_tile = std::is_same<T, dd>::value && far && d.tct;
   k_permute_in<Tio, T><<<perm_grid, 256, (size_t)kPermRows * (rp + 1) * sizeof(T), st>>>(
       x, d.n, nrhs, rp, d.pad_src, d.npad, cmx, xpad, near_tc ? d.ntc_xmax : nullptr);
   mk.count(H2_PH_PERMUTE_IN);
@@ -1129,13 +1142,22 @@ int matvec_typed(Ctx &c, const Tio *x, Tio *y, int nrhs, bool acc) {
     mk.count(H2_PH_LEAF_FORWARD, 2);
   } else if (far && leaf_reg) {
     const size_t sm = (size_t)L * (kp + rp) * sizeof(T);
-    k_leaf_fwd_reg<TV, T><<<(unsigned)d.nleaf, 256, sm, st>>>((const TV *)d.V, xpad, vscale, L, kp, k, rp,
-                                                             xhat + leaf0 * (int64_t)k * rp);
+    T *xl = xhat + leaf0 * (int64_t)k * rp;
+    if (cpl_tile)
+      k_leaf_fwd_reg<TV, T, true><<<(unsigned)d.nleaf, 256, sm, st>>>((const TV *)d.V, xpad, vscale, L, kp, k, rp, xl,
+                                                                     d.tc_xmax + D * kLevelCols);
+    else
+      k_leaf_fwd_reg<TV, T, false><<<(unsigned)d.nleaf, 256, sm, st>>>((const TV *)d.V, xpad, vscale, L, kp, k, rp,
+                                                                      xl, nullptr);
     mk.count(H2_PH_LEAF_FORWARD);
   } else if (far) {
     LeafForwardRows<TV, T> rows{(const TV *)d.V, xpad, vscale, L, kp, rp};
     if ((rc = launch_rows<TV, T>(rows, cf_fwd, t_fwd, Rk, d.nleaf, 0, xhat + leaf0 * (int64_t)k * rp, st))) return rc;
     mk.count(H2_PH_LEAF_FORWARD);
+    if (cpl_tile) {
+      tct_leaf_max(c, xhat, rp);
+      mk.count(H2_PH_LEAF_FORWARD);
+    }
   }
   mk.mark(H2_PH_UPWARD);
   const bool tcpath = d.tc && rp <= 16 &&
@@ -1152,11 +1174,12 @@ int matvec_typed(Ctx &c, const Tio *x, Tio *y, int nrhs, bool acc) {
       const int64_t np = (int64_t)1 << l;
       const dim3 grid((unsigned)((np + kRegParents - 1) / kRegParents), (rp + 15) / 16);
       const dim3 grid2((unsigned)((np + kSplitParents - 1) / kSplitParents), (rp + 15) / 16);
+      unsigned *xm = cpl_tile ? d.tc_xmax + l * kLevelCols : nullptr;
       if (np <= kUpSplitMax) {
-        if (m == 4) k_up_split<TE, T, 4><<<grid2, 256, 0, st>>>((const TE *)d.Ef, rp, np - 1, np, xhat, nullptr);
-        else k_up_split<TE, T, 3><<<grid2, 256, 0, st>>>((const TE *)d.Ef, rp, np - 1, np, xhat, nullptr);
-      } else if (m == 4) k_up_reg<TE, T, 4><<<grid, 256, 0, st>>>((const TE *)d.Ef, rp, np - 1, np, xhat, nullptr);
-      else k_up_reg<TE, T, 3><<<grid, 256, 0, st>>>((const TE *)d.Ef, rp, np - 1, np, xhat, nullptr);
+        if (m == 4) k_up_split<TE, T, 4><<<grid2, 256, 0, st>>>((const TE *)d.Ef, rp, np - 1, np, xhat, xm);
+        else k_up_split<TE, T, 3><<<grid2, 256, 0, st>>>((const TE *)d.Ef, rp, np - 1, np, xhat, xm);
+      } else if (m == 4) k_up_reg<TE, T, 4><<<grid, 256, 0, st>>>((const TE *)d.Ef, rp, np - 1, np, xhat, xm);
+      else k_up_reg<TE, T, 3><<<grid, 256, 0, st>>>((const TE *)d.Ef, rp, np - 1, np, xhat, xm);
       mk.count(H2_PH_UPWARD);
     }
   } else if (far) {
@@ -1196,6 +1219,10 @@ int matvec_typed(Ctx &c, const Tio *x, Tio *y, int nrhs, bool acc) {
     } else if (tcpath) {
       // FP64-accurate: integer slices on the tensor cores
       if ((rc = tc_coupling(c, xhat, yhat, rp))) return rc;
+    } else if (cpl_tile) {
+      int64_t nl = 0;
+      if ((rc = tct_coupling(c, xhat, yhat, rp, &nl))) return rc;
+      mk.count(H2_PH_COUPLING, nl - 1);
     } else {
       CouplingRows<TS, T> rows{(const TS *)d.S, d.adm_ptr, d.adm_col, xhat, k, kp, rp, row0};
       if ((rc = launch_rows<TS, T>(rows, cf_cpl, t_cpl, Rk, d.nclu - row0, 0, out, st))) return rc;
@@ -1363,8 +1390,8 @@ int matvec_gca(Ctx &c, const Tio *x, Tio *y, int nrhs, bool acc) {
   mk.mark(H2_PH_LEAF_FORWARD);
   if (far && leaf_reg) {
     const size_t sm = (size_t)L * (KD + rp) * sizeof(T);
-    k_leaf_fwd_reg<TS, T><<<(unsigned)d.nleaf, 256, sm, st>>>((const TS *)d.V, xpad, nullptr, L, KD, KD, rp,
-                                                             X(xhat, D));
+    k_leaf_fwd_reg<TS, T, false><<<(unsigned)d.nleaf, 256, sm, st>>>((const TS *)d.V, xpad, nullptr, L, KD, KD, rp,
+                                                             X(xhat, D), nullptr);
     mk.count(H2_PH_LEAF_FORWARD);
   } else if (far) {
     LeafForwardRows<TS, T> rows{(const TS *)d.V, xpad, nullptr, L, KD, rp};
@@ -1814,7 +1841,7 @@ int take_device_error(Ctx &c) {
     return fail(H2_ETIMEOUT, "a bounded device wait ran out; the last result is not valid");
   }
   int rc = c.d.tc ? tc_take_error(c.stream) : H2_OK;
-  const int rt = c.d.ntc ? tile_take_error(c.stream) : H2_OK;
+  const int rt = c.d.ntc || c.d.tct ? tile_take_error(c.stream) : H2_OK;
   return rc ? rc : rt;
 }
 

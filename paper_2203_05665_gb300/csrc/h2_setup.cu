@@ -644,6 +644,8 @@ int build_typed(Ctx &c) {
   }
   // FP64 and FP32 handles of order 4: the E4M3 digit planes for the tensor-core coupling
   if (!d.gca && d.tensor == 0 && tc_eligible(d) && (rc = tc_build(c))) return rc;
+  // FP64 handles of order 3: digit tiles of the small-tile kernel
+  if (tct_eligible(d) && (rc = tct_build(c))) return rc;
   H2_CUDA_TRY(cudaStreamSynchronize(st));
   c.build_ms[H2_BUILD_COUPLING] = ms_since(tc0) - (d.gca ? c.build_ms[H2_BUILD_BASES] : 0.0);
   const auto tn0 = std::chrono::steady_clock::now();

@@ -6,6 +6,7 @@
 #include <cuda_fp8.h>
 
 #include "h2_dd.cuh"
+#include "h2_internal.hpp"
 #include "h2_digits.hpp"
 #include "h2_ptx.cuh"
 
@@ -16,7 +17,7 @@ constexpr int kTcN = 16;                 // columns of one tensor-core pass (rig
 constexpr int kTcSlices = 10;            // 5-bit digits of an FP64-accurate value
 constexpr int kTcFixBits = 49;           // |X| <= 2^49
 constexpr uint32_t kTmemCols = 512;      // tensor memory of one SM
-constexpr int kXmaxCols = 64;            // column maxima per tree level (one per right-hand side)
+constexpr int kXmaxCols = kLevelCols;
 
 // instruction descriptor of tcgen05.mma kind::f8f6f4: D FP32 (bits 4-5 =
 // 1), A and B E4M3 (bits 7-9 = 0, bits 10-12 = 0), both K-major (bits 15, 16

@@ -2,12 +2,13 @@
 // operands, FP32 accumulation in tensor memory), FP64 accuracy: output rows
 // of R <= 32 values whose blocks contract over at most 32 values.  The
 // nearfield of H2_F64 handles (R = L triangles per leaf, y|t += sum G_ts x|s,
-// Algorithm 3 over the inadmissible leaf pairs) runs on it for any number of
+// Algorithm 3 over the inadmissible leaf pairs) and the coupling of order-3
+// handles (R = 27, y^_t += sum S_ts x^_s) run on it for any number of
 // right-hand sides, 16 columns per launch.
 //
 // The arithmetic is the exact digit splitting of h2_tc.cu: every row nu of
 // the blocks of one block row gets a power of two 2^E, every column j of the
-// input a power of two 2^F, a value becomes X = round(v 2^(49-E)), |X| <=
+// input (of each tree level, for the coupling) a power of two 2^F, a value becomes X = round(v 2^(49-E)), |X| <=
 // 2^49, cut into ten signed 5-bit digits i = 0 .. 9 of weight 2^(-4 - 5 i).
 // All digit pairs of levels i + k <= 10 are summed (and some above), one level
 // more than the tiles of h2_tc.cu sum: the pairs left out stay below 2^-51 of
@@ -46,7 +47,11 @@
 // accumulator columns per plane group, single-stage commits), 354 us now, 6.1
 // TB/s into shared memory.  Leaves of 30 (cube, 30,000 triangles, 5 columns):
 // 161 us in double-float block rows, 47 us now; 32 right-hand sides, 81,920
-// triangles: 414 us in double-float, 215 us now (two passes).
+// triangles: 414 us in double-float, 215 us now (two passes).  Order-3
+// coupling, double-float block rows before: 81,920 triangles, 32 right-hand
+// sides (75,224 blocks of 9.0 KB, two passes) 1,070 us, now 393 us with the
+// digit cuts; cube of 30,000 triangles, 5 columns 195 us, now 62 us; 5,120
+// triangles, one column 35 us, now 22 us.
 #include <algorithm>
 #include <functional>
 #include <queue>
@@ -54,6 +59,7 @@
 #include <vector>
 
 #include "h2_internal.hpp"
+#include "h2_kernel.cuh"
 #include "h2_tc.cuh"
 
 namespace h2 {
@@ -97,6 +103,8 @@ struct TileArgs {
   const int32_t *split;       // [gridDim.x + 1]: rows of every CTA
   dd *out;                    // [row][R][rp], at the first column of the pass
   int R, ncol, rp, nst, accumulate;
+  int64_t row0;               // output row of scheduled row value 0 (E, out, xmax are indexed from it)
+  int by_level;               // xmax holds kXmaxCols maxima per tree level, output rows are clusters
   uint32_t stage, xch;        // bytes of a stage, of one exchange area
 };
 
@@ -264,7 +272,7 @@ __global__ void __launch_bounds__(kTileThreads, 1) k_tile_tc(const TileArgs a) {
     int64_t pnext = a.ptr[r_begin];
     int32_t rnext = r_begin < r_end ? a.row[r_begin] : 0;
     for (int64_t r = r_begin; r < r_end; ++r) {
-      const int64_t b0 = pnext, orow_id = rnext;
+      const int64_t b0 = pnext, orow_id = a.row0 + rnext;
       pnext = a.ptr[r + 1];
       if (r + 1 < r_end) rnext = a.row[r + 1];
       const int64_t nb = pnext - b0;
@@ -288,6 +296,7 @@ __global__ void __launch_bounds__(kTileThreads, 1) k_tile_tc(const TileArgs a) {
           eo[u] = 0;
           yold[u] = dd{0.0f, 0.0f};
           if (tl + 128 * u < nout) {
+            if (a.by_level) fexp[u] = tc_colexp(a.xmax[tc_level(orow_id) * kXmaxCols + ocol[u]]);
             eo[u] = a.E[orow_id * R + orow[u]] + fexp[u];
             if (s0 > 0 || a.accumulate) yold[u] = yrow[orow[u] * a.rp + ocol[u]];
           }
@@ -367,14 +376,14 @@ __global__ void __launch_bounds__(kTileThreads, 1) k_tile_tc(const TileArgs a) {
 // rows behind the ten planes.
 template <int W>
 __global__ void __launch_bounds__(128) k_tile_cut(const dd *__restrict__ x, int64_t first, int64_t count, int R,
-                                                  int rp, int ncol, const unsigned *__restrict__ xmax,
+                                                  int rp, int ncol, const unsigned *__restrict__ xmax, int by_level,
                                                   unsigned char *__restrict__ X) {
   constexpr int N0 = tile_n<W>();
   const int64_t i = (int64_t)blockIdx.x * (64 / W) + threadIdx.x / (2 * W);
   if (i >= count) return;
   const int64_t t = first + i;
   const int g = (threadIdx.x / W) & 1, j = threadIdx.x % W;
-  const int sc = kTcFixBits - tc_colexp(j < ncol ? xmax[j] : 0u);
+  const int sc = kTcFixBits - tc_colexp(j < ncol ? xmax[(by_level ? tc_level(t) * kXmaxCols : 0) + j] : 0u);
   dd v[16];
 #pragma unroll
   for (int q = 0; q < 16; ++q) {
@@ -436,6 +445,83 @@ __global__ void k_near_slice(const dd *__restrict__ near, const int32_t *__restr
     *reinterpret_cast<uint4 *>(base + tile_off(L, i, nu, 16 * cg)) = *reinterpret_cast<const uint4 *>(out[i]);
 }
 
+// ---------------------------------------------------------------- order-3 coupling
+// interpolation point nu of cluster c (tensor Chebyshev points, Eq. (6c))
+__device__ __forceinline__ void cheb_point(const double *cheb, int m, int64_t c, int nu, double *x) {
+  x[0] = cheb[(3 * c + 0) * m + nu % m];
+  x[1] = cheb[(3 * c + 1) * m + (nu / m) % m];
+  x[2] = cheb[(3 * c + 2) * m + nu / (m * m)];
+}
+
+// E[t][nu] = 1 + floor(log2 max |S_ts[nu][mu]|) over the blocks of row t (0 if none)
+__global__ void k_cpl_rowexp(const int64_t *__restrict__ ptr, const int32_t *__restrict__ col,
+                             const double *__restrict__ cheb, int m, int64_t row0, int64_t nclu, KernelFn kf,
+                             int32_t *__restrict__ E) {
+  const int k = m * m * m;
+  const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (e >= (nclu - row0) * k) return;
+  const int64_t t = row0 + e / k;
+  const int nu = (int)(e % k);
+  double x[3], y[3], mx = 0.0;
+  cheb_point(cheb, m, t, nu, x);
+  for (int64_t b = ptr[t]; b < ptr[t + 1]; ++b)
+    for (int mu = 0; mu < k; ++mu) {
+      cheb_point(cheb, m, col[b], mu, y);
+      mx = fmax(mx, fabs(kernel_value(kf, x, y)));
+    }
+  E[t * k + nu] = mx > 0.0 ? ilogb(mx) + 1 : 0;
+}
+
+// the ten digit planes of scheduled block b (row cluster row0 + brow[b], column cluster col[b]), row
+// nu, contraction indices 16 cg .. 16 cg + 15
+__global__ void k_cpl_slice(const int32_t *__restrict__ brow, const int32_t *__restrict__ col, int64_t row0,
+                            const double *__restrict__ cheb, int m, const int32_t *__restrict__ E, int64_t nblk,
+                            KernelFn kf, unsigned char *__restrict__ A) {
+  const int k = m * m * m;
+  const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (e >= nblk * k * 2) return;
+  const int64_t b = e / (2 * k), t = row0 + brow[b];
+  const int nu = (int)((e / 2) % k), cg = (int)(e % 2);
+  const int sc = kTcFixBits - E[t * k + nu];
+  double x[3], y[3];
+  cheb_point(cheb, m, t, nu, x);
+  __align__(16) unsigned char out[kTcSlices][16];
+#pragma unroll
+  for (int q = 0; q < 16; ++q) {
+    const int mu = 16 * cg + q;
+    long long X = 0;
+    if (mu < k) {
+      cheb_point(cheb, m, col[b], mu, y);
+      X = llrint(ldexp(kernel_value(kf, x, y), sc));
+    }
+    int sl[kTcSlices];
+    split_digits(X, sl);
+#pragma unroll
+    for (int i = 0; i < kTcSlices; ++i) out[i][q] = e4m3(sl[i]);
+  }
+  unsigned char *base = A + b * (int64_t)tile_bytes(k);
+#pragma unroll
+  for (int i = 0; i < kTcSlices; ++i)
+    *reinterpret_cast<uint4 *>(base + tile_off(k, i, nu, 16 * cg)) = *reinterpret_cast<const uint4 *>(out[i]);
+}
+
+// xmax[c] = largest |hi| of column c of x ([rows][rp], rp <= 64), as float
+// bits: every thread keeps one column
+__global__ void __launch_bounds__(256) k_row_max(const dd *__restrict__ x, int64_t rows, int rp,
+                                                 unsigned *__restrict__ xmax) {
+  __shared__ unsigned loc[kXmaxCols];
+  if (threadIdx.x < kXmaxCols) loc[threadIdx.x] = 0u;
+  __syncthreads();
+  const int per = (int)blockDim.x / rp, c = (int)threadIdx.x % rp, q = (int)threadIdx.x / rp;
+  float mx = 0.0f;
+  if (q < per)
+    for (int64_t r = blockIdx.x * (int64_t)per + q; r < rows; r += (int64_t)gridDim.x * per)
+      mx = fmaxf(mx, fabsf(x[r * rp + c].hi));
+  if (mx > 0.0f) atomicMax(&loc[c], __float_as_uint(mx));
+  __syncthreads();
+  if ((int)threadIdx.x < rp && loc[threadIdx.x]) atomicMax(&xmax[threadIdx.x], loc[threadIdx.x]);
+}
+
 // W of a pass over ncol columns
 int tile_width(int ncol) { return ncol <= 4 ? 4 : ncol <= 8 ? 8 : 16; }
 
@@ -461,18 +547,18 @@ int tile_run(const TileArgs &a, int width, int grid, cudaStream_t st) {
 }
 
 template <int W>
-void cut_launch(const dd *x, int64_t first, int64_t count, int R, int rp, int ncol, const unsigned *xmax,
+void cut_launch(const dd *x, int64_t first, int64_t count, int R, int rp, int ncol, const unsigned *xmax, int by_level,
                 unsigned char *X, cudaStream_t st) {
   constexpr int per = 64 / W;
-  k_tile_cut<W><<<(unsigned)((count + per - 1) / per), 128, 0, st>>>(x, first, count, R, rp, ncol, xmax, X);
+  k_tile_cut<W><<<(unsigned)((count + per - 1) / per), 128, 0, st>>>(x, first, count, R, rp, ncol, xmax, by_level, X);
 }
 
-void tile_cut(const dd *x, int64_t first, int64_t count, int R, int rp, int ncol, const unsigned *xmax,
+void tile_cut(const dd *x, int64_t first, int64_t count, int R, int rp, int ncol, const unsigned *xmax, int by_level,
               unsigned char *X, int width, cudaStream_t st) {
   switch (width) {
-    case 4: return cut_launch<4>(x, first, count, R, rp, ncol, xmax, X, st);
-    case 8: return cut_launch<8>(x, first, count, R, rp, ncol, xmax, X, st);
-    default: return cut_launch<16>(x, first, count, R, rp, ncol, xmax, X, st);
+    case 4: return cut_launch<4>(x, first, count, R, rp, ncol, xmax, by_level, X, st);
+    case 8: return cut_launch<8>(x, first, count, R, rp, ncol, xmax, by_level, X, st);
+    default: return cut_launch<16>(x, first, count, R, rp, ncol, xmax, by_level, X, st);
   }
 }
 
@@ -599,7 +685,7 @@ int ntc_build(Ctx &c) {
 // the digit tiles of columns c0 .. c0 + ncol - 1 of the permuted input
 void ntc_input(Ctx &c, const void *xpad, int rp, int c0, int ncol, bool wide) {
   Dev &d = c.d;
-  tile_cut(static_cast<const dd *>(xpad) + c0, 0, d.nleaf, (int)d.lmax, rp, ncol, d.ntc_xmax + c0,
+  tile_cut(static_cast<const dd *>(xpad) + c0, 0, d.nleaf, (int)d.lmax, rp, ncol, d.ntc_xmax + c0, 0,
            (unsigned char *)d.xnt, wide ? kTcN : tile_width(ncol), c.stream);
 }
 
@@ -632,6 +718,84 @@ int ntc_near(Ctx &c, const void *xpad, void *ypad, int rp, int accumulate, int64
     const int rc = tile_run(a, have_input ? kTcN : tile_width(ncol), d.ntc_s.grid, c.stream);
     if (rc) return rc;
     ++nl;
+  }
+  H2_CUDA_TRY(cudaGetLastError());
+  if (launches) *launches = nl;
+  return H2_OK;
+}
+
+// Coupling of FP64-accurate order-3 handles with stored coupling (k = 27),
+// unless the digits would take more than half of the free device memory or
+// the handle's products are single launches
+bool tct_eligible(const Dev &d) {
+  if (!(d.prec == H2_F64 && d.tensor == 0 && !d.gca && d.coupling == 0 && d.m == 3 && d.nadm > 0)) return false;
+  if (d.fused && d.n <= kFusedMaxN) return false;
+  size_t fr = 0, tot = 0;
+  if (cudaMemGetInfo(&fr, &tot) != cudaSuccess) return false;
+  return (double)d.nadm * tile_bytes(d.k) + (double)d.nclu * 32 * tile_n<kTcN>() <= 0.5 * (double)fr;
+}
+
+int tct_build(Ctx &c) {
+  Dev &d = c.d;
+  cudaStream_t st = c.stream;
+  const int64_t row0 = ((int64_t)1 << d.first_adm_level) - 1;
+  const uint32_t ab = tile_bytes(d.k);
+  int rc;
+  SchedTmp tmp;
+  if ((rc = row_schedule(d, c.plan.adm_ptr.data() + row0, c.plan.adm_col.data(), d.nclu - row0, d.tc_s, tmp, st)))
+    return rc;
+  if ((rc = dev_alloc(d, (void **)&d.tc_E, sizeof(int32_t) * (size_t)d.nclu * d.k))) return rc;
+  if ((rc = dev_alloc(d, &d.Stc, (size_t)d.nadm * ab))) return rc;
+  if ((rc = dev_alloc(d, &d.xtc, (size_t)d.nclu * 32 * tile_n<kTcN>()))) return rc;
+  H2_CUDA_TRY(cudaMemsetAsync(d.tc_E, 0, sizeof(int32_t) * (size_t)d.nclu * d.k, st));
+  H2_CUDA_TRY(cudaMemsetAsync(d.Stc, 0, (size_t)d.nadm * ab, st));
+  const int64_t nr = (d.nclu - row0) * d.k, ns = d.nadm * d.k * 2;
+  k_cpl_rowexp<<<(unsigned)((nr + 127) / 128), 128, 0, st>>>(d.adm_ptr, d.adm_col, d.cheb, d.m, row0, d.nclu,
+                                                             d.kernel, d.tc_E);
+  k_cpl_slice<<<(unsigned)((ns + 255) / 256), 256, 0, st>>>(tmp.brow, d.tc_s.col, row0, d.cheb, d.m, d.tc_E, d.nadm,
+                                                            d.kernel, (unsigned char *)d.Stc);
+  H2_CUDA_TRY(cudaGetLastError());
+  H2_CUDA_TRY(cudaStreamSynchronize(st));
+  d.tct = true;
+  return H2_OK;
+}
+
+// column maxima of the leaf coefficients (where the leaf step does not take them)
+void tct_leaf_max(Ctx &c, const void *xhat, int rp) {
+  const Dev &d = c.d;
+  const int64_t rows = d.nleaf * d.k, per = 256 / rp;
+  const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>((rows + 8 * per - 1) / (8 * per), 152 * 8));
+  k_row_max<<<grid, 256, 0, c.stream>>>(static_cast<const dd *>(xhat) + (d.nleaf - 1) * d.k * (int64_t)rp, rows, rp,
+                                        d.tc_xmax + d.depth * kXmaxCols);
+}
+
+// the coupling phase, 16 columns per pass; the column maxima of every level are in place
+int tct_coupling(Ctx &c, const void *xhat, void *yhat, int rp, int64_t *launches) {
+  Dev &d = c.d;
+  const int64_t row0 = ((int64_t)1 << d.first_adm_level) - 1;
+  int64_t nl = 0;
+  for (int c0 = 0; c0 < rp; c0 += kTcN) {
+    const int ncol = std::min(kTcN, rp - c0);
+    tile_cut(static_cast<const dd *>(xhat) + c0, row0, d.nclu - row0, d.k, rp, ncol, d.tc_xmax + c0, 1,
+             (unsigned char *)d.xtc, tile_width(ncol), c.stream);
+    TileArgs a{};
+    a.A = (const unsigned char *)d.Stc;
+    a.X = (const unsigned char *)d.xtc;
+    a.ptr = d.tc_s.ptr;
+    a.col = d.tc_s.col;
+    a.row = d.tc_s.row;
+    a.split = d.tc_s.split;
+    a.E = d.tc_E;
+    a.xmax = d.tc_xmax + c0;
+    a.out = static_cast<dd *>(yhat) + c0;
+    a.R = d.k;
+    a.ncol = ncol;
+    a.rp = rp;
+    a.row0 = row0;
+    a.by_level = 1;
+    const int rc = tile_run(a, tile_width(ncol), d.tc_s.grid, c.stream);
+    if (rc) return rc;
+    nl += 2;
   }
   H2_CUDA_TRY(cudaGetLastError());
   if (launches) *launches = nl;

@@ -284,7 +284,7 @@ __global__ void __launch_bounds__(256, 2) k_up_reg(const TS *__restrict__ Ef, in
     mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
     if (act && jz == 0 && mx > 0.0f) atomicMax(&loc[j & 15], __float_as_uint(mx));
     __syncthreads();
-    if (threadIdx.x < 16 && loc[threadIdx.x]) atomicMax(&xmax[threadIdx.x], loc[threadIdx.x]);
+    if (threadIdx.x < 16 && loc[threadIdx.x]) atomicMax(&xmax[16 * blockIdx.y + threadIdx.x], loc[threadIdx.x]);
   }
 }
 
@@ -416,7 +416,7 @@ __global__ void __launch_bounds__(256, 2) k_up_split(const TS *__restrict__ Ef, 
     mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
     if (ch == 0 && act && jz == 0 && mx > 0.0f) atomicMax(&loc[j & 15], __float_as_uint(mx));
     __syncthreads();
-    if (threadIdx.x < 16 && loc[threadIdx.x]) atomicMax(&xmax[threadIdx.x], loc[threadIdx.x]);
+    if (threadIdx.x < 16 && loc[threadIdx.x]) atomicMax(&xmax[16 * blockIdx.y + threadIdx.x], loc[threadIdx.x]);
   }
 }
 

@@ -70,3 +70,29 @@ def test_columns_with_infinity_or_nan(require_gpu):
             assert torch.isnan(y1[:, [1, 3]]).all()
             assert torch.equal(y0[:, good], y1[:, good])
         h.close()
+
+
+@pytest.mark.parametrize("mesh, leaf", [("patch", 32), ("cube", 16), ("cube", 40), ("ellipsoid", 24)])
+def test_order3_coupling(require_gpu, mesh, leaf):
+    """The order-3 coupling: ragged leaves, leaves beyond the tensor-core nearfield (40), rows of up to
+    about 140 blocks (cubes; several exact segments of 24), every tile width and several passes,
+    columns of very different scales; bit-reproducible."""
+    import torch
+    v, f = {"patch": lambda: _patch(1111), "cube": lambda: I.cube(20),
+            "ellipsoid": lambda: I.ellipsoid(3, (2.0, 1.0, 0.5))}[mesh]()
+    n = f.shape[0]
+    o = oracle.Oracle(v, f, leaf_size=leaf, eta=2.0, order=3)
+    h = H2Matrix(v, f, leaf_size=leaf, eta=2.0, order=3, prec="f64")
+    assert h.stats["tensor"] == 1 and h.stats["adm_blocks"] > 0
+    # 64 columns of a leaf of 40 exceed one tile of the leaf backward step
+    for nrhs in (1, 3, 4, 5, 8, 9, 16, 17, 32, 37) + ((64,) if leaf <= 32 else ()):
+        x = I.uniform_rhs(n, nrhs, 5300 + nrhs) * np.logspace(-9, 6, nrhs)
+        y, ref = h.matvec_host(x), o.matvec(x)
+        for c in range(nrhs):
+            assert _rel(y[:, c], ref[:, c]) <= TOL, (nrhs, c)
+    xd = colmajor(torch.from_numpy(I.uniform_rhs(n, 20, 5400)).cuda())
+    y1, y2 = colmajor(torch.empty_like(xd)), colmajor(torch.empty_like(xd))
+    h.matvec(xd, y1)
+    h.matvec(xd, y2)
+    assert torch.equal(y1, y2)
+    h.close()
