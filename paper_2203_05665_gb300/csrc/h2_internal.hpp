@@ -120,8 +120,9 @@ struct Dev {
   int32_t *near_col = nullptr;  // leaf-local
   double *cheb = nullptr;       // nclu x 3 x m (FP64 always)
   double *icen = nullptr;       // nclu x 3 interpolation-box centres (regenerated coupling)
-  float *adm_dc = nullptr;      // nadm x 4: centre of the row cluster minus centre of the column cluster
-  float *ihalf = nullptr;       // nclu x 3 interpolation-box half widths
+  float *adm_dc = nullptr;      // nadm x 4: centre of the row cluster minus centre of the column cluster, times 2^regen_shift
+  float *ihalf = nullptr;       // nclu x 3 interpolation-box half widths, times 2^regen_shift
+  int regen_shift = 0;          // brings the mesh's extent to [1, 2)
   // Coupling on the tensor cores (order 4, FP64 or FP32 handles): the E4M3
   // digit planes of every S_b ([nadm][tc_nd][64 x 64] bytes, K-major
   // core-matrix layout), the row exponents ([nclu][64]), the digit planes of

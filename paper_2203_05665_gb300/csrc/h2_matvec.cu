@@ -272,7 +272,7 @@ __device__ __forceinline__ void scale_by(double &, float) {}
 __device__ __forceinline__ void scale_by(dd &, float) {}
 
 constexpr float kInv4PiF = 0.0795774715459476679f;
-constexpr uint32_t kMetaBytes = 32;   // per-term values at the end of every stage
+constexpr uint32_t kMetaBytes = 16;   // per-term values at the end of every stage
 
 // Launch geometry of the block-row kernel (computed on the host).
 struct RowCfg {
@@ -296,15 +296,12 @@ struct Term {
 // first term, first(nrows) = total), term(e) gives the tiles of flat term e,
 // kdim(e) its contraction length and meta(e) a few values the producer puts
 // beside the tiles: [0] the power of two the stored A tile was divided by
-// (FP16 storage; 1 otherwise), [1..6] the box data of generated A tiles.
-// kGen rows compute their A tiles in the consumer threads instead of loading
-// them.
+// (FP16 storage; 1 otherwise).
 
 // Coupling (Algorithm 3, admissible blocks): row r = cluster row0 + r, terms
 // S_b x^_{s_b} for the admissible blocks b of that row (S_b stored [mu][nu]).
 template <class TS, class TC>
 struct CouplingRows {
-  static constexpr bool kGen = false;
   const TS *S;
   const int64_t *ptr;
   const int32_t *col;
@@ -320,47 +317,10 @@ struct CouplingRows {
   }
 };
 
-// Coupling with S_b regenerated on the fly in FP32 (Eq. (6c)): s_{nu mu} =
-// 1/(4 pi |xi_{t,nu} - xi_{s,mu}|) from the clusters' interpolation boxes
-// (centre c, half width h, Chebyshev nodes c + h t_j); the difference of the
-// centres is formed in FP64 before rounding, so the distance keeps FP32
-// relative accuracy for well-separated small clusters.
-struct CouplingGenRows {
-  static constexpr bool kGen = true;
-  const int64_t *ptr;
-  const int32_t *col;
-  const float *xhat;
-  const float4 *dc;     // [admissible blocks]: centre of t minus centre of s, formed in FP64
-  const float *half;    // [clusters][3]
-  float t[kMaxM];       // reference Chebyshev nodes cos((2j+1) pi / (2m))
-  int m, k, kp, rp;
-  int64_t row0;
-  __device__ int kdim(int64_t) const { return k; }
-  // scale, centre gap (3), half widths of the column cluster (3)
-  __device__ void meta(int64_t e, float *mt) const {
-    const int64_t b = ptr[row0] + e;
-    const int64_t sg = col[b];
-    const float4 g = dc[b];
-    mt[0] = 1.0f;
-    mt[1] = g.x;
-    mt[2] = g.y;
-    mt[3] = g.z;
-    mt[4] = half[3 * sg];
-    mt[5] = half[3 * sg + 1];
-    mt[6] = half[3 * sg + 2];
-  }
-  __device__ int64_t first(int64_t r) const { return ptr[row0 + r] - ptr[row0]; }
-  __device__ Term<float, float> term(int64_t e) const {
-    const int64_t b = ptr[row0] + e;
-    return Term<float, float>{nullptr, xhat + (int64_t)col[b] * k * rp, k};
-  }
-};
-
 // Leaf forward step (Algorithm 1 on the leaves): row j = leaf j, one term
 // V_j^T x|j (V_j stored [t][nu], padded to kp).
 template <class TS, class TC>
 struct LeafForwardRows {
-  static constexpr bool kGen = false;
   const TS *V;
   const TC *xpad;
   const float *vscale;   // per leaf, or NULL
@@ -377,7 +337,6 @@ struct LeafForwardRows {
 // V_j y^_j (V_j stored transposed [nu][t], padded to Lp).
 template <class TS, class TC>
 struct LeafBackwardRows {
-  static constexpr bool kGen = false;
   const TS *Vt;
   const TC *yhat;
   const float *vscale;
@@ -397,7 +356,6 @@ struct LeafBackwardRows {
 // of the blocks), else block e.
 template <class TS, class TC>
 struct NearRows {
-  static constexpr bool kGen = false;
   const TS *near;
   const int64_t *ptr;
   const int32_t *col;
@@ -421,7 +379,6 @@ struct NearRows {
 // cluster ([c - c0][K][rp]).
 template <class TS, class TC>
 struct GcaCouplingRows {
-  static constexpr bool kGen = false;
   const TS *S;
   const int64_t *ptr;
   const int32_t *col;
@@ -442,7 +399,6 @@ struct GcaCouplingRows {
 // [Kc][Kp]: the son's index is the contraction index).
 template <class TS, class TC>
 struct GcaUpRows {
-  static constexpr bool kGen = false;
   const TS *E;
   const TC *xs;
   int Kc, Kp, rp;
@@ -458,7 +414,6 @@ struct GcaUpRows {
 // E_r y^_parent (E_r stored transposed [Kp][Kc]); added to the son's y^.
 template <class TS, class TC>
 struct GcaDownRows {
-  static constexpr bool kGen = false;
   const TS *Et;
   const TC *yp;
   int Kc, Kp, rp;
@@ -630,12 +585,12 @@ __global__ void __launch_bounds__(kThreads + 32, 2)
         if (i >= cfg.nst && !mbar_wait_or_abort(&empty[s], (uint32_t)((i / cfg.nst - 1) & 1), abort)) break;
         unsigned char *st = smem + (size_t)s * cfg.stage_bytes;
         const Term<TS, TC> tm = rows.term(e);
-        const uint32_t ab = Rows::kGen ? 0u : (uint32_t)(sizeof(TS) * tm.K * Mp);
+        const uint32_t ab = (uint32_t)(sizeof(TS) * tm.K * Mp);
         const uint32_t xb = (uint32_t)(sizeof(TC) * tm.K * rp);
         // the term's metadata goes beside the tiles; the arrival below releases it
         rows.meta(e, reinterpret_cast<float *>(st + cfg.stage_bytes - kMetaBytes));
         mbar_expect_tx(&full[s], ab + xb);
-        if (!Rows::kGen) bulk_g2s(st, tm.A, ab, &full[s]);
+        bulk_g2s(st, tm.A, ab, &full[s]);
         bulk_g2s(st + cfg.a_bytes, tm.X, xb, &full[s]);
       }
       if (*abort) {
@@ -663,21 +618,6 @@ __global__ void __launch_bounds__(kThreads + 32, 2)
     for (int a = 0; a < 4 * R; ++a)
 #pragma unroll
       for (int c = 0; c < VN; ++c) acc[a][c] = zero_of<TC>();
-    // generated coupling: node offsets of this thread's rows in the row cluster
-    float gnode[Rows::kGen ? 4 * R : 1][3];
-    bool gvalid[Rows::kGen ? 4 * R : 1];
-    if constexpr (Rows::kGen) {
-      const int64_t grow = rows.row0 + r;
-      const int m = rows.m;
-#pragma unroll
-      for (int a = 0; a < 4 * R; ++a) {
-        const int nu = (a / 4) * gstride + 4 * vg + (a % 4);
-        gvalid[a] = nu < rows.k;
-        const int jj[3] = {nu % m, (nu / m) % m, min(nu / (m * m), m - 1)};
-#pragma unroll
-        for (int d = 0; d < 3; ++d) gnode[a][d] = rows.half[3 * grow + d] * rows.t[jj[d]];
-      }
-    }
     const int64_t e_row_end = rows.first(r + 1);
     for (; e < e_row_end; ++e) {
       const int64_t i = e - e_begin;
@@ -693,35 +633,11 @@ __global__ void __launch_bounds__(kThreads + 32, 2)
         const int kc = (K + cfg.ksplit - 1) / cfg.ksplit;
         const int mu0 = ks * kc, mu1 = min(K, mu0 + kc);
         const float sc = mt[0];
-        float hs[3] = {0.f, 0.f, 0.f};
-        float gbase[Rows::kGen ? 4 * R : 1][3];
-        if constexpr (Rows::kGen) {
-#pragma unroll
-          for (int a = 0; a < 4 * R; ++a) {
-            gbase[a][0] = mt[1] + gnode[a][0];
-            gbase[a][1] = mt[2] + gnode[a][1];
-            gbase[a][2] = mt[3] + gnode[a][2];
-          }
-          hs[0] = mt[4];
-          hs[1] = mt[5];
-          hs[2] = mt[6];
-        }
 #pragma unroll 2
         for (int mu = mu0; mu < mu1; ++mu) {
           TC av[4 * R];
-          if constexpr (Rows::kGen) {
-            const int m = rows.m;
-            const float ox = hs[0] * rows.t[mu % m], oy = hs[1] * rows.t[(mu / m) % m], oz = hs[2] * rows.t[mu / (m * m)];
 #pragma unroll
-            for (int a = 0; a < 4 * R; ++a) {
-              const float dx = gbase[a][0] - ox, dy = gbase[a][1] - oy, dz = gbase[a][2] - oz;
-              const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-              av[a] = gvalid[a] ? kInv4PiF * rsqrtf(r2) : 0.0f;
-            }
-          } else {
-#pragma unroll
-            for (int g = 0; g < R; ++g) load4<TS, TC>(sA + mu * Mp + g * gstride + 4 * vg, av + 4 * g);
-          }
+          for (int g = 0; g < R; ++g) load4<TS, TC>(sA + mu * Mp + g * gstride + 4 * vg, av + 4 * g);
           const XV xv = *reinterpret_cast<const XV *>(sX + mu * rp + VN * cg);
           TC xs[VN];
 #pragma unroll
@@ -763,116 +679,188 @@ __global__ void __launch_bounds__(kThreads + 32, 2)
   }
 }
 
-// Coupling regenerated in FP32, warp per row cluster (for up to 64 rows and
-// 16 columns): lane l owns rows nu = l + 32 q of y^_t for all columns and
-// loops over the admissible blocks of the row; per block the warp stages
-// x^_s and the column cluster's node offsets in its own shared memory and
-// evaluates s_{nu mu} = 1/(4 pi |xi_{t,nu} - xi_{s,mu}|) in registers (the
-// centre gap comes precomputed from FP64).  No cross-warp reduction: each
-// output is summed by one lane in a fixed order.
+// Coupling regenerated in FP32 (Eq. (6c): s_{nu mu} = 1 / (4 pi |xi_{t,nu} -
+// xi_{s,mu}|)), warp per row cluster: lane l owns the rows nu = l + 32 q of
+// y^_t for CP columns (a pass) and loops over the admissible blocks of the
+// row.  The interpolation points are tensor grids, so the three differences
+// of a point pair come from three short tables per block and lane (M values
+// per axis), and a kernel value costs one multiply-add, one reciprocal square
+// root and the CP multiply-adds it feeds; 1 / (4 pi) enters once, at the end.
+// The next block's coefficients x^_s are copied to the warp's second buffer
+// (cp.async) and its box data loaded while the current block is computed.
+// Centre gaps (formed in FP64) and half widths are stored scaled by a power of
+// two that brings the mesh to size 1, so that the squared distances are
+// normal numbers whatever the mesh's scale; the factor goes into 1 / (4 pi).
+// No cross-warp reduction: every output is summed by one lane in block order.
+// Bound by instruction issue and the reciprocal square roots.  1.3 M
+// triangles, order 3, 4 columns (0.89 G kernel values): 1,142 us with the
+// distances formed per value (about 20 instructions each), 360 us now.
 constexpr int kRegenWarps = 4;
+struct RegenArgs {
+  const int64_t *ptr;
+  const int32_t *col;
+  const float4 *dc;     // [admissible blocks]: centre of t minus centre of s (scaled)
+  const float *half;    // [clusters][3] half widths (scaled)
+  const float *xhat;
+  float *yhat;
+  float t[kMaxM];       // reference Chebyshev nodes cos((2j+1) pi / (2m))
+  float factor;         // 1 / (4 pi), times the scale
+  int rp, c0;
+  int64_t row0, nrows;
+};
 
-template <int QR, int CP>
-__global__ void __launch_bounds__(32 * kRegenWarps)
-    k_coupling_regen_warp(const int64_t *__restrict__ ptr, const int32_t *__restrict__ col,
-                          const float4 *__restrict__ dc, const float *__restrict__ half,
-                          const float *__restrict__ xhat, CouplingGenRows g, int64_t nrows, float *__restrict__ yhat) {
+__device__ __forceinline__ float rsqrt_fast(float v) {
+  float r;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(v));
+  return r;
+}
+
+template <int M, int CP>
+__global__ void __launch_bounds__(32 * kRegenWarps) k_coupling_regen(const __grid_constant__ RegenArgs a) {
+  constexpr int K = M * M * M, QR = (K + 31) / 32, C4 = CP / 4;
   extern __shared__ __align__(16) float wsm[];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const int k = g.k, m = g.m, rp = g.rp;
-  float *tn = wsm;                                          // reference nodes
-  float *xs = wsm + 16 + (size_t)w * (64 * CP + 3 * 64);   // [k][rp] then offsets [3][k]
-  float *offs = xs + 64 * CP;
-  if (threadIdx.x == 0) {
-#pragma unroll
-    for (int j = 0; j < kMaxM; ++j) tn[j] = g.t[j];   // constant indices: no local copy of the parameters
-  }
-  __syncthreads();
+  float *buf = wsm + (size_t)w * 2 * K * CP;
   const int64_t r = (int64_t)blockIdx.x * kRegenWarps + w;
-  if (r >= nrows) return;
-  const int64_t t = g.row0 + r;
+  if (r >= a.nrows) return;
+  const int64_t t = a.row0 + r;
   float node[QR][3];
-  bool valid[QR];
 #pragma unroll
   for (int q = 0; q < QR; ++q) {
-    const int nu = lane + 32 * q;
-    valid[q] = nu < k;
-    const int j[3] = {nu % m, (nu / m) % m, min(nu / (m * m), m - 1)};
+    const int nu = min(lane + 32 * q, K - 1);
+    const int j[3] = {nu % M, (nu / M) % M, nu / (M * M)};
 #pragma unroll
-    for (int d = 0; d < 3; ++d) node[q][d] = half[3 * t + d] * tn[j[d]];
+    for (int d = 0; d < 3; ++d) {
+      float tj = a.t[0];
+#pragma unroll
+      for (int i = 1; i < M; ++i) tj = j[d] == i ? a.t[i] : tj;
+      node[q][d] = a.half[3 * t + d] * tj;
+    }
   }
   float acc[QR][CP];
 #pragma unroll
   for (int q = 0; q < QR; ++q)
 #pragma unroll
     for (int c = 0; c < CP; ++c) acc[q][c] = 0.0f;
-  const int64_t b0 = ptr[t], b1 = ptr[t + 1];
+  const int64_t b0 = a.ptr[t], b1 = a.ptr[t + 1];
+  // x^_s (columns c0 .. c0 + CP - 1) of block b into buffer b & 1
+  auto stage = [&](int64_t b, int32_t sg) {
+    float *dst = buf + (size_t)(b & 1) * K * CP;
+    const float *src = a.xhat + (int64_t)sg * K * a.rp + a.c0;
+    for (int i = lane; i < K * C4; i += 32) cp_async16(dst + 4 * i, src + (i / C4) * a.rp + 4 * (i % C4));
+    cp_async_commit();
+  };
+  int32_t sg = b0 < b1 ? a.col[b0] : 0, sg1 = b0 + 1 < b1 ? a.col[b0 + 1] : 0;
+  float4 gap = make_float4(0.f, 0.f, 0.f, 0.f);
+  float h[3] = {0.f, 0.f, 0.f};
+  if (b0 < b1) {
+    stage(b0, sg);
+    gap = a.dc[b0];
+#pragma unroll
+    for (int d = 0; d < 3; ++d) h[d] = a.half[3 * (int64_t)sg + d];
+  }
   for (int64_t b = b0; b < b1; ++b) {
-    const int64_t sg = col[b];
-    const float4 gap = dc[b];
-    __syncwarp();
-    const float *xsrc = xhat + sg * (int64_t)k * rp;
-    for (int i = lane; i < k * rp; i += 32) xs[i] = xsrc[i];
-    for (int i = lane; i < k; i += 32) {
-      offs[i] = half[3 * sg] * tn[i % m];
-      offs[64 + i] = half[3 * sg + 1] * tn[(i / m) % m];
-      offs[128 + i] = half[3 * sg + 2] * tn[i / (m * m)];
+    float4 gap1 = gap;
+    float h1[3] = {h[0], h[1], h[2]};
+    if (b + 1 < b1) {
+      stage(b + 1, sg1);
+      gap1 = a.dc[b + 1];
+#pragma unroll
+      for (int d = 0; d < 3; ++d) h1[d] = a.half[3 * (int64_t)sg1 + d];
+      sg1 = b + 2 < b1 ? a.col[b + 2] : 0;
+      cp_async_wait<1>();
+    } else {
+      cp_async_wait<0>();
     }
     __syncwarp();
-    float base[QR][3];
+    const float4 *xs = reinterpret_cast<const float4 *>(buf + (size_t)(b & 1) * K * CP);
+    float dx[QR][M], dy[QR][M], dz[QR][M];
 #pragma unroll
     for (int q = 0; q < QR; ++q) {
-      base[q][0] = gap.x + node[q][0];
-      base[q][1] = gap.y + node[q][1];
-      base[q][2] = gap.z + node[q][2];
-    }
-#pragma unroll 3
-    for (int mu = 0; mu < k; ++mu) {
-      const float ox = offs[mu], oy = offs[64 + mu], oz = offs[128 + mu];
-      float xv[CP];
+      const float bx = gap.x + node[q][0], by = gap.y + node[q][1], bz = gap.z + node[q][2];
 #pragma unroll
-      for (int c = 0; c < CP; c += 4) {
-        const float4 v = *reinterpret_cast<const float4 *>(xs + mu * rp + c);
-        xv[c] = v.x; xv[c + 1] = v.y; xv[c + 2] = v.z; xv[c + 3] = v.w;
-      }
-#pragma unroll
-      for (int q = 0; q < QR; ++q) {
-        const float dx = base[q][0] - ox, dy = base[q][1] - oy, dz = base[q][2] - oz;
-        const float sv = valid[q] ? kInv4PiF * rsqrtf(fmaf(dx, dx, fmaf(dy, dy, dz * dz))) : 0.0f;
-#pragma unroll
-        for (int c = 0; c < CP; ++c)
-          if (c < rp) acc[q][c] = fmaf(sv, xv[c], acc[q][c]);
+      for (int j = 0; j < M; ++j) {
+        dx[q][j] = bx - h[0] * a.t[j];
+        dy[q][j] = by - h[1] * a.t[j];
+        dz[q][j] = bz - h[2] * a.t[j];
       }
     }
+#pragma unroll
+    for (int jz = 0; jz < M; ++jz)
+#pragma unroll
+      for (int jy = 0; jy < M; ++jy) {
+        float fyz[QR];
+#pragma unroll
+        for (int q = 0; q < QR; ++q) fyz[q] = fmaf(dy[q][jy], dy[q][jy], dz[q][jz] * dz[q][jz]);
+#pragma unroll
+        for (int jx = 0; jx < M; ++jx) {
+          const int mu = jx + M * (jy + M * jz);
+          float4 xv[C4];
+#pragma unroll
+          for (int c = 0; c < C4; ++c) xv[c] = xs[mu * C4 + c];
+#pragma unroll
+          for (int q = 0; q < QR; ++q) {
+            const float sv = rsqrt_fast(fmaf(dx[q][jx], dx[q][jx], fyz[q]));
+#pragma unroll
+            for (int c = 0; c < C4; ++c) {
+              acc[q][4 * c] = fmaf(sv, xv[c].x, acc[q][4 * c]);
+              acc[q][4 * c + 1] = fmaf(sv, xv[c].y, acc[q][4 * c + 1]);
+              acc[q][4 * c + 2] = fmaf(sv, xv[c].z, acc[q][4 * c + 2]);
+              acc[q][4 * c + 3] = fmaf(sv, xv[c].w, acc[q][4 * c + 3]);
+            }
+          }
+        }
+      }
+    __syncwarp();
+    gap = gap1;
+#pragma unroll
+    for (int d = 0; d < 3; ++d) h[d] = h1[d];
   }
-  float *out = yhat + t * (int64_t)k * rp;
+  float *out = a.yhat + t * (int64_t)K * a.rp + a.c0;
 #pragma unroll
-  for (int q = 0; q < QR; ++q)
-    if (valid[q])
+  for (int q = 0; q < QR; ++q) {
+    const int nu = lane + 32 * q;
+    if (nu < K)
 #pragma unroll
-      for (int c = 0; c < CP; ++c)
-        if (c < rp) out[(lane + 32 * q) * rp + c] = acc[q][c];
+      for (int c = 0; c < C4; ++c)
+        *reinterpret_cast<float4 *>(out + nu * a.rp + 4 * c) =
+            make_float4(acc[q][4 * c] * a.factor, acc[q][4 * c + 1] * a.factor, acc[q][4 * c + 2] * a.factor,
+                        acc[q][4 * c + 3] * a.factor);
+  }
 }
 
-template <int QR, int CP>
-int launch_regen_warp(const CouplingGenRows &g, int64_t nrows, float *yhat, cudaStream_t st) {
-  const size_t sm = (16 + (size_t)kRegenWarps * (64 * CP + 3 * 64)) * sizeof(float);
-  const unsigned grid = (unsigned)((nrows + kRegenWarps - 1) / kRegenWarps);
-  k_coupling_regen_warp<QR, CP><<<grid, 32 * kRegenWarps, sm, st>>>(g.ptr, g.col, g.dc, g.half, g.xhat, g, nrows,
-                                                                     yhat);
+constexpr size_t kRegenSmemMax = 4u * 2 * 125 * 16 * sizeof(float);   // order 5, 16 columns
+
+template <int M, int CP>
+int launch_regen(const RegenArgs &a, cudaStream_t st) {
+  const size_t sm = (size_t)kRegenWarps * 2 * M * M * M * CP * sizeof(float);
+  if (sm > 48 * 1024)
+    H2_CUDA_TRY(cudaFuncSetAttribute(k_coupling_regen<M, CP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     (int)kRegenSmemMax));
+  k_coupling_regen<M, CP><<<(unsigned)((a.nrows + kRegenWarps - 1) / kRegenWarps), 32 * kRegenWarps, sm, st>>>(a);
   return H2_OK;
 }
 
-// warp-per-row regenerated coupling when k <= 64 and rp <= 16, else -1;
-// yhat is the base of [clusters][k][rp] (rows g.row0 .. g.row0 + nrows - 1 are written)
-int regen_warp(const CouplingGenRows &g, int64_t nrows, float *yhat, cudaStream_t st) {
-  if (g.k > 64 || g.rp > 16 || nrows <= 0) return -1;
-  const int QR = g.k > 32 ? 2 : 1, CP = g.rp <= 4 ? 4 : (g.rp <= 8 ? 8 : 16);
-  if (QR == 1) return CP == 4 ? launch_regen_warp<1, 4>(g, nrows, yhat, st)
-                              : CP == 8 ? launch_regen_warp<1, 8>(g, nrows, yhat, st)
-                                        : launch_regen_warp<1, 16>(g, nrows, yhat, st);
-  return CP == 4 ? launch_regen_warp<2, 4>(g, nrows, yhat, st)
-                 : CP == 8 ? launch_regen_warp<2, 8>(g, nrows, yhat, st) : launch_regen_warp<2, 16>(g, nrows, yhat, st);
+// one pass of ncol (a multiple of 4, at most 16) columns from a.c0 on
+template <int M>
+int regen_pass(const RegenArgs &a, int ncol, cudaStream_t st) {
+  switch (ncol) {
+    case 4: return launch_regen<M, 4>(a, st);
+    case 8: return launch_regen<M, 8>(a, st);
+    case 12: return launch_regen<M, 12>(a, st);
+    default: return launch_regen<M, 16>(a, st);
+  }
+}
+
+int regen_coupling(RegenArgs a, int m, int64_t *launches, cudaStream_t st) {
+  int rc = H2_OK;
+  *launches = 0;
+  for (a.c0 = 0; a.c0 < a.rp && !rc && a.nrows > 0; a.c0 += 16, ++*launches) {
+    const int ncol = std::min(16, a.rp - a.c0);
+    rc = m == 1 ? regen_pass<1>(a, ncol, st) : m == 2 ? regen_pass<2>(a, ncol, st) : m == 3 ? regen_pass<3>(a, ncol, st)
+         : m == 4 ? regen_pass<4>(a, ncol, st) : regen_pass<5>(a, ncol, st);
+  }
+  return rc;
 }
 
 constexpr size_t kSmemMax = 227 * 1024;
@@ -880,7 +868,7 @@ constexpr size_t kSmemMax = 227 * 1024;
 // geometry for output tiles M x rp and contraction lengths up to Kmax;
 // threads: the number of threads the kernel is launched with
 template <class TS, class T>
-int row_cfg(int M, int Mp, int rp, int Kmax, int threads, int R, bool gen, RowCfg &cfg) {
+int row_cfg(int M, int Mp, int rp, int Kmax, int threads, int R, RowCfg &cfg) {
   constexpr int VN = Vec16<T>::N;
   cfg.M = M;
   cfg.Mp = Mp;
@@ -890,7 +878,7 @@ int row_cfg(int M, int Mp, int rp, int Kmax, int threads, int R, bool gen, RowCf
   cfg.tiles = cfg.nvg * cfg.ncg;
   if (cfg.tiles > threads) return fail(H2_EINVAL, "tile rows x right-hand sides too large for one CTA");
   cfg.ksplit = std::max(1, std::min(threads / cfg.tiles, Kmax));
-  cfg.a_bytes = gen ? 0u : (uint32_t)((sizeof(TS) * Kmax * Mp + 15) / 16 * 16);
+  cfg.a_bytes = (uint32_t)((sizeof(TS) * Kmax * Mp + 15) / 16 * 16);
   cfg.stage_bytes = cfg.a_bytes + (uint32_t)((sizeof(T) * Kmax * rp + 15) / 16 * 16) + kMetaBytes;
   const size_t red = sizeof(T) * (size_t)cfg.ksplit * Mp * rp;   // slice sums, after the ring
   // stages: up to 8, sized so that 512 consumer threads per SM stay resident when possible
@@ -1105,11 +1093,11 @@ int matvec_typed(Ctx &c, const Tio *x, Tio *y, int nrhs, bool acc) {
   const int t_fwd = row_threads(kp, rp, L, sizeof(T), Rk), t_cpl = row_threads(kp, rp, k, sizeof(T), Rk);
   const int t_back = row_threads(Lp, rp, k, sizeof(T), RL), t_near = row_threads(Lp, rp, L, sizeof(T), RL);
   if (far) {
-    if ((rc = row_cfg<TV, T>(k, kp, rp, L, t_fwd, Rk, false, cf_fwd))) return rc;
-    if ((rc = row_cfg<TS, T>(k, kp, rp, k, t_cpl, Rk, gen, cf_cpl))) return rc;
-    if ((rc = row_cfg<TV, T>(L, Lp, rp, k, t_back, RL, false, cf_back))) return rc;
+    if ((rc = row_cfg<TV, T>(k, kp, rp, L, t_fwd, Rk, cf_fwd))) return rc;
+    if ((rc = row_cfg<TS, T>(k, kp, rp, k, t_cpl, Rk, cf_cpl))) return rc;
+    if ((rc = row_cfg<TV, T>(L, Lp, rp, k, t_back, RL, cf_back))) return rc;
   }
-  if ((rc = row_cfg<TS, T>(L, Lp, rp, L, t_near, RL, false, cf_near))) return rc;
+  if ((rc = row_cfg<TS, T>(L, Lp, rp, L, t_near, RL, cf_near))) return rc;
   const float *vscale = (const float *)d.vscale, *nscale = (const float *)d.nscale;
   Marks mk(c);
 
@@ -1198,21 +1186,22 @@ int matvec_typed(Ctx &c, const Tio *x, Tio *y, int nrhs, bool acc) {
     T *out = yhat + row0 * (int64_t)k * rp;
     if (gen) {
       if constexpr (std::is_same<T, float>::value) {
-        CouplingGenRows rows{};
-        rows.ptr = d.adm_ptr;
-        rows.col = d.adm_col;
-        rows.xhat = xhat;
-        rows.dc = (const float4 *)d.adm_dc;
-        rows.half = d.ihalf;
-        for (int j = 0; j < kMaxM; ++j) rows.t[j] = j < m ? (float)std::cos((2 * j + 1) * 3.14159265358979323846 / (2.0 * m)) : 0.f;
-        rows.m = m;
-        rows.k = k;
-        rows.kp = kp;
-        rows.rp = rp;
-        rows.row0 = row0;
-        // the warp kernel indexes y^ by absolute cluster number: give it the base
-        const int wr = regen_warp(rows, d.nclu - row0, yhat, st);
-        if (wr < 0 && (rc = launch_rows<float, T>(rows, cf_cpl, t_cpl, Rk, d.nclu - row0, 0, out, st))) return rc;
+        RegenArgs ra{};
+        ra.ptr = d.adm_ptr;
+        ra.col = d.adm_col;
+        ra.dc = (const float4 *)d.adm_dc;
+        ra.half = d.ihalf;
+        ra.xhat = xhat;
+        ra.yhat = yhat;
+        for (int j = 0; j < kMaxM; ++j)
+          ra.t[j] = j < m ? (float)std::cos((2 * j + 1) * 3.14159265358979323846 / (2.0 * m)) : 0.f;
+        ra.factor = kInv4PiF * std::ldexp(1.0f, d.regen_shift);
+        ra.rp = rp;
+        ra.row0 = row0;
+        ra.nrows = d.nclu - row0;
+        int64_t nl = 0;
+        if ((rc = regen_coupling(ra, m, &nl, st))) return rc;
+        mk.count(H2_PH_COUPLING, nl - 1);
       } else {
         return fail(H2_EINVAL, "the regenerated coupling runs in FP32 arithmetic only");
       }
@@ -1275,7 +1264,7 @@ int matvec_typed(Ctx &c, const Tio *x, Tio *y, int nrhs, bool acc) {
     if constexpr (std::is_same<T, float>::value) {
       if (!self_fused) {
       RowCfg cf_self{};
-      if ((rc = row_cfg<float, T>(L, Lp, rp, L, t_near, RL, false, cf_self))) return rc;
+      if ((rc = row_cfg<float, T>(L, Lp, rp, L, t_near, RL, cf_self))) return rc;
       NearRows<float, T> self{d.nself, d.self_ptr, d.self_col, xpad, nullptr, L, Lp, rp, nullptr};
       if ((rc = launch_rows<float, T>(self, cf_self, t_near, RL, d.nleaf, 1, ypad, st))) return rc;
       mk.count(H2_PH_LEAF_NEAR);
@@ -1340,7 +1329,7 @@ int gca_rows_launch(const Rows &rows, int M, int Mp, int Kmax, int rp, int64_t n
   }
   RowCfg cfg{};
   int rc;
-  if ((rc = row_cfg<TS, T>(M, Mp, rp, Kmax, threads, R, false, cfg))) return rc;
+  if ((rc = row_cfg<TS, T>(M, Mp, rp, Kmax, threads, R, cfg))) return rc;
   return launch_rows<TS, T>(rows, cfg, threads, R, nrows, accumulate, out, st);
 }
 

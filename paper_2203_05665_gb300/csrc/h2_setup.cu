@@ -593,7 +593,12 @@ int build_typed(Ctx &c) {
   const auto tc0 = std::chrono::steady_clock::now();
   if (d.coupling == 1) {
     // regenerated coupling: interpolation-box centres (FP64) and half widths (FP32)
-    std::vector<float> hw(p.ihalf.begin(), p.ihalf.end());
+    // scaled by the power of two that brings the mesh's largest extent to [1, 2)
+    double ext = 0.0;
+    for (int q = 0; q < 3; ++q) ext = std::max(ext, p.hi[q] - p.lo[q]);
+    d.regen_shift = ext > 0.0 ? std::max(-120, std::min(120, -std::ilogb(ext))) : 0;
+    std::vector<float> hw(p.ihalf.size());
+    for (size_t i = 0; i < hw.size(); ++i) hw[i] = (float)std::ldexp(p.ihalf[i], d.regen_shift);
     if ((rc = dev_alloc(d, (void **)&d.icen, p.icen.size() * 8))) return rc;
     H2_CUDA_TRY(cudaMemcpyAsync(d.icen, p.icen.data(), p.icen.size() * 8, cudaMemcpyHostToDevice, st));
     if ((rc = dev_alloc(d, (void **)&d.ihalf, hw.size() * 4))) return rc;
@@ -602,7 +607,7 @@ int build_typed(Ctx &c) {
     std::vector<float> dc(4 * std::max<size_t>(1, p.adm_col.size()), 0.0f);
     for (int64_t t = 0; t < p.nclu; ++t)
       for (int64_t e = p.adm_ptr[t]; e < p.adm_ptr[t + 1]; ++e)
-        for (int q = 0; q < 3; ++q) dc[4 * e + q] = (float)(p.icen[3 * t + q] - p.icen[3 * p.adm_col[e] + q]);
+        for (int q = 0; q < 3; ++q) dc[4 * e + q] = (float)std::ldexp(p.icen[3 * t + q] - p.icen[3 * p.adm_col[e] + q], d.regen_shift);
     if ((rc = dev_alloc(d, (void **)&d.adm_dc, dc.size() * 4))) return rc;
     H2_CUDA_TRY(cudaMemcpyAsync(d.adm_dc, dc.data(), dc.size() * 4, cudaMemcpyHostToDevice, st));
     H2_CUDA_TRY(cudaStreamSynchronize(st));
