@@ -186,20 +186,6 @@ __global__ void __launch_bounds__(256) k_permute_out(const Tin *__restrict__ ypa
   }
 }
 
-// upward step for the parents of level l (Algorithm 1), one CTA per parent
-template <class TS, class T>
-__global__ void k_upward(const TS *__restrict__ Ef, int m, int k, int rp, int64_t par0, T *__restrict__ xhat) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  upward_parent<TS, T>(Ef, m, k, rp, par0 + blockIdx.x, xhat, smem_raw);
-}
-
-// downward step for the children of level l+1 (Algorithm 2), one CTA per parent of level l
-template <class TS, class T>
-__global__ void k_downward(const TS *__restrict__ Ef, int m, int k, int rp, int64_t par0, T *__restrict__ yhat) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  downward_parent<TS, T>(Ef, m, k, rp, par0 + blockIdx.x, yhat, smem_raw);
-}
-
 template <class T>
 struct Vec16;
 template <>
@@ -1156,27 +1142,10 @@ int matvec_typed(Ctx &c, const Tio *x, Tio *y, int nrhs, bool acc) {
     int64_t nl = 0;
     if ((rc = tc_upward(c, xhat, rp, &nl, leaf_tc))) return rc;
     mk.count(H2_PH_UPWARD, nl);
-  } else if (far && (m == 3 || m == 4)) {
-    // orders 3 and 4: register kernels (the z mode product by warp shuffles)
+  } else if (far) {
     for (int l = D - 1; l >= lmin; --l) {
       const int64_t np = (int64_t)1 << l;
-      const dim3 grid((unsigned)((np + kRegParents - 1) / kRegParents), (rp + 15) / 16);
-      const dim3 grid2((unsigned)((np + kSplitParents - 1) / kSplitParents), (rp + 15) / 16);
-      unsigned *xm = cpl_tile ? d.tc_xmax + l * kLevelCols : nullptr;
-      if (np <= kUpSplitMax) {
-        if (m == 4) k_up_split<TE, T, 4><<<grid2, 256, 0, st>>>((const TE *)d.Ef, rp, np - 1, np, xhat, xm);
-        else k_up_split<TE, T, 3><<<grid2, 256, 0, st>>>((const TE *)d.Ef, rp, np - 1, np, xhat, xm);
-      } else if (m == 4) k_up_reg<TE, T, 4><<<grid, 256, 0, st>>>((const TE *)d.Ef, rp, np - 1, np, xhat, xm);
-      else k_up_reg<TE, T, 3><<<grid, 256, 0, st>>>((const TE *)d.Ef, rp, np - 1, np, xhat, xm);
-      mk.count(H2_PH_UPWARD);
-    }
-  } else if (far) {
-    size_t sm = ((size_t)3 * k * rp + 6 * m * m) * sizeof(T);
-    if ((rc = set_smem<T>((const void *)k_upward<TE, T>, sm))) return rc;
-    for (int l = D - 1; l >= lmin; --l) {
-      int64_t par0 = ((int64_t)1 << l) - 1;
-      k_upward<TE, T><<<(unsigned)((int64_t)1 << l), transfer_threads(l), sm, st>>>((const TE *)d.Ef, m, k, rp, par0,
-                                                                                   xhat);
+      launch_up<TE, T>((const TE *)d.Ef, m, rp, np - 1, np, xhat, cpl_tile ? d.tc_xmax + l * kLevelCols : nullptr, st);
       mk.count(H2_PH_UPWARD);
     }
   }
@@ -1219,23 +1188,10 @@ int matvec_typed(Ctx &c, const Tio *x, Tio *y, int nrhs, bool acc) {
     mk.count(H2_PH_COUPLING);
   }
   mk.mark(H2_PH_DOWNWARD);
-  if (far && (m == 3 || m == 4)) {
-    for (int l = lmin; l < D; ++l) {
-      const int64_t np = (int64_t)1 << l;
-      const dim3 grid((unsigned)((np + kSplitParents - 1) / kSplitParents), (rp + 15) / 16);
-      if (m == 4) k_down_split<TE, T, 4><<<grid, 256, 0, st>>>((const TE *)d.Ef, rp, np - 1, np, yhat);
-      else k_down_split<TE, T, 3><<<grid, 256, 0, st>>>((const TE *)d.Ef, rp, np - 1, np, yhat);
-      mk.count(H2_PH_DOWNWARD);
-    }
-  } else if (far) {
-    size_t sm = ((size_t)3 * k * rp + 6 * m * m) * sizeof(T);
-    if ((rc = set_smem<T>((const void *)k_downward<TE, T>, sm))) return rc;
-    for (int l = lmin; l < D; ++l) {
-      int64_t par0 = ((int64_t)1 << l) - 1;
-      k_downward<TE, T><<<(unsigned)((int64_t)1 << l), transfer_threads(l), sm, st>>>((const TE *)d.Ef, m, k, rp,
-                                                                                     par0, yhat);
-      mk.count(H2_PH_DOWNWARD);
-    }
+  for (int l = lmin; far && l < D; ++l) {
+    const int64_t np = (int64_t)1 << l;
+    launch_down<TE, T>((const TE *)d.Ef, m, rp, np - 1, np, yhat, st);
+    mk.count(H2_PH_DOWNWARD);
   }
   mk.mark(H2_PH_LEAF_NEAR);
   // bfloat16 handles: the FP32 self blocks join the leaf backward step when it runs per leaf

@@ -720,12 +720,7 @@ int tc_upward_t(Ctx &c, T *xhat, int rp, int64_t *launches, bool leaf_max) {
   for (int l = D - 1; l >= lmin; --l) {
     // level l from level l + 1, with the column maxima of level l
     const int64_t np = (int64_t)1 << l;
-    if (np <= kUpSplitMax)
-      k_up_split<T, T, 4><<<(unsigned)((np + kSplitParents - 1) / kSplitParents), 256, 0, st>>>(
-          (const T *)d.Ef, rp, np - 1, np, xhat, d.tc_xmax + l * kXmaxCols);
-    else
-      k_up_reg<T, T, 4><<<(unsigned)((np + kRegParents - 1) / kRegParents), 256, 0, st>>>(
-          (const T *)d.Ef, rp, np - 1, np, xhat, d.tc_xmax + l * kXmaxCols);
+    launch_up<T, T>((const T *)d.Ef, 4, rp, np - 1, np, xhat, d.tc_xmax + l * kXmaxCols, st);
     ++nl;
   }
   // the digits of every level at once (all maxima are complete)

@@ -7,6 +7,8 @@
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
+#include <algorithm>
+
 #include "h2_dd.cuh"
 
 namespace h2 {
@@ -61,65 +63,10 @@ __device__ __forceinline__ float to_compute<float, __half>(__half v) {
   return __half2float(v);
 }
 
-// upward step for one parent (Algorithm 1): x^_p = sum over both children c of E_c^T x^_c;
-// smem holds 3 k rp + 6 m^2 values of T
-template <class TS, class T>
-__device__ __forceinline__ void upward_parent(const TS *__restrict__ Ef, int m, int k, int rp, int64_t par,
-                                              T *__restrict__ xhat, unsigned char *smem_raw) {
-  const int kr = k * rp, mm = m * m;
-  T *a = reinterpret_cast<T *>(smem_raw);
-  T *b = a + kr;
-  T *acc = b + kr;
-  T *F = acc + kr;   // 2 children x 3 axes x m x m
-  for (int i = threadIdx.x; i < 6 * mm; i += blockDim.x) F[i] = to_compute<T>(Ef[(2 * par + 1) * 3 * mm + i]);
-  for (int i = threadIdx.x; i < kr; i += blockDim.x) acc[i] = zero_of<T>();
-  for (int ch = 0; ch < 2; ++ch) {
-    const int64_t c = 2 * par + 1 + ch;
-    for (int i = threadIdx.x; i < kr; i += blockDim.x) a[i] = xhat[c * kr + i];
-    __syncthreads();
-    const T *Fc = F + ch * 3 * mm;
-    mode_fibres(Fc, a, b, m, k, rp, 0, true, threadIdx.x, blockDim.x);
-    __syncthreads();
-    mode_fibres(Fc + mm, b, a, m, k, rp, 1, true, threadIdx.x, blockDim.x);
-    __syncthreads();
-    mode_fibres(Fc + 2 * mm, a, b, m, k, rp, 2, true, threadIdx.x, blockDim.x);
-    __syncthreads();
-    for (int i = threadIdx.x; i < kr; i += blockDim.x) acc[i] = acc[i] + b[i];
-    __syncthreads();
-  }
-  for (int i = threadIdx.x; i < kr; i += blockDim.x) xhat[par * kr + i] = acc[i];
-}
-
-// downward step below one parent (Algorithm 2): y^_c += E_c y^_parent for both children
-template <class TS, class T>
-__device__ __forceinline__ void downward_parent(const TS *__restrict__ Ef, int m, int k, int rp, int64_t par,
-                                                T *__restrict__ yhat, unsigned char *smem_raw) {
-  const int kr = k * rp, mm = m * m;
-  T *p = reinterpret_cast<T *>(smem_raw);
-  T *a = p + kr;
-  T *b = a + kr;
-  T *F = b + kr;
-  for (int i = threadIdx.x; i < 6 * mm; i += blockDim.x) F[i] = to_compute<T>(Ef[(2 * par + 1) * 3 * mm + i]);
-  for (int i = threadIdx.x; i < kr; i += blockDim.x) p[i] = yhat[par * kr + i];
-  __syncthreads();
-  for (int ch = 0; ch < 2; ++ch) {
-    const int64_t c = 2 * par + 1 + ch;
-    const T *Fc = F + ch * 3 * mm;
-    mode_fibres(Fc, p, a, m, k, rp, 0, false, threadIdx.x, blockDim.x);
-    __syncthreads();
-    mode_fibres(Fc + mm, a, b, m, k, rp, 1, false, threadIdx.x, blockDim.x);
-    __syncthreads();
-    mode_fibres(Fc + 2 * mm, b, a, m, k, rp, 2, false, threadIdx.x, blockDim.x);
-    __syncthreads();
-    for (int i = threadIdx.x; i < kr; i += blockDim.x) yhat[c * kr + i] = yhat[c * kr + i] + a[i];
-    __syncthreads();
-  }
-}
-
-// Warp-level variants: one warp per parent, the warp's own shared memory
-// (3 k rp + 6 m^2 values of T), warp synchronisation only.  For the small
-// per-parent tensors of low orders and few right-hand sides a whole CTA per
-// parent leaves most threads idle.
+// Steps of one parent by one warp (batched products): the warp's own shared
+// memory (3 k rp + 6 m^2 values of T), warp synchronisation only.
+//   upward (Algorithm 1): x^_p = sum over both children c of E_c^T x^_c
+//   downward (Algorithm 2): y^_c += E_c y^_parent for both children
 template <class TS, class T>
 __device__ __forceinline__ void upward_parent_warp(const TS *__restrict__ Ef, int m, int k, int rp, int64_t par,
                                                    T *__restrict__ xhat, T *ws, int lane) {
@@ -180,7 +127,7 @@ __device__ __forceinline__ void downward_parent_warp(const TS *__restrict__ Ef, 
 // m = 3) holds the m x m slab nu = jx + m jy + m^2 jz of one column in
 // registers.  The x and y mode products run in registers, the z mode product
 // takes the slab entries of the threads of the column (adjacent lanes) by
-// warp shuffles.  Every output is formed exactly as in mode_fibres (m
+// warp shuffles.  Used for the wide upward levels in FP32 (launch_up_m).  Every output is formed exactly as in mode_fibres (m
 // multiply-adds, one renormalisation), in the same axis order, so the
 // results equal those of the shared-memory kernels above; the gain is that
 // no CTA-wide barrier separates the three mode products.
@@ -292,63 +239,12 @@ __global__ void __launch_bounds__(256, 2) k_up_reg(const TS *__restrict__ Ef, in
 // taking one child each (two parents per 256-thread CTA), so every thread
 // forms half the mode products.  On levels with few parents a CTA's time is
 // the latency of one thread's chain of double-float operations, which this
-// halves.  The upward step adds the second child's part to the first through
-// shared memory in the order of k_up_reg (same bits).
-//
-// Downward (Algorithm 2): y^_c += E_c y^_parent for both children of parents
-// par0 .. par0 + npar - 1, the children independent.
+// halves.  The second child's part is added to the first through shared memory
+// in the order of k_up_reg (same bits).
 constexpr int kSplitParents = 2;   // parents per 256-thread CTA
-// upward levels of at most this many parents take the split kernel (the
-// downward pass takes it at every level; both measured at level 7, 16 RHS)
+// upward levels of at most this many parents take the split kernel (measured
+// at 327,680 triangles, 16 right-hand sides)
 constexpr int64_t kUpSplitMax = 4096;
-
-template <class TS, class T, int M>
-__global__ void __launch_bounds__(256, 2) k_down_split(const TS *__restrict__ Ef, int rp, int64_t par0, int64_t npar,
-                                                       T *__restrict__ yhat) {
-  constexpr int K = M * M * M;
-  __shared__ T F[kSplitParents][2][3][M * M];
-  load_factors<TS, T, M, kSplitParents>(Ef, par0, npar, F);
-  const int pl = threadIdx.x >> 7, ch = (threadIdx.x >> 6) & 1, t = threadIdx.x & 63;
-  const int j = (t >> 2) + 16 * blockIdx.y, jz = t & 3;
-  const int64_t pi = (int64_t)blockIdx.x * kSplitParents + pl, par = par0 + pi;
-  const bool act = pi < npar && j < rp && jz < M;
-  const int base = (threadIdx.x & 31) & ~3;
-  const int zq = jz < M ? jz : 0;
-  const T *Fx = F[pl][ch][0], *Fy = F[pl][ch][1], *Fz = F[pl][ch][2];
-  const int64_t c = 2 * par + 1 + ch;
-  T v[M][M], yc[M][M];
-#pragma unroll
-  for (int jy = 0; jy < M; ++jy)
-#pragma unroll
-    for (int jx = 0; jx < M; ++jx) {
-      const int64_t nu = jx + M * jy + M * M * jz;
-      v[jy][jx] = act ? yhat[(par * K + nu) * rp + j] : zero_of<T>();
-      yc[jy][jx] = act ? yhat[(c * K + nu) * rp + j] : zero_of<T>();
-    }
-  T a[M][M], b[M][M];
-#pragma unroll
-  for (int jy = 0; jy < M; ++jy)
-#pragma unroll
-    for (int jx = 0; jx < M; ++jx) a[jy][jx] = modem_out<T, false, M>(Fx, v[jy], jx);
-#pragma unroll
-  for (int jx = 0; jx < M; ++jx) {
-    T col[M];
-#pragma unroll
-    for (int jy = 0; jy < M; ++jy) col[jy] = a[jy][jx];
-#pragma unroll
-    for (int jy = 0; jy < M; ++jy) b[jy][jx] = modem_out<T, false, M>(Fy, col, jy);
-  }
-#pragma unroll
-  for (int jy = 0; jy < M; ++jy)
-#pragma unroll
-    for (int jx = 0; jx < M; ++jx) {
-      T in[M];
-#pragma unroll
-      for (int q = 0; q < M; ++q) in[q] = shfl_t(b[jy][jx], base + q);
-      const T r = modem_out<T, false, M>(Fz, in, zq);
-      if (act) yhat[(c * K + jx + M * jy + M * M * jz) * rp + j] = yc[jy][jx] + r;
-    }
-}
 
 template <class TS, class T, int M>
 __global__ void __launch_bounds__(256, 2) k_up_split(const TS *__restrict__ Ef, int rp, int64_t par0, int64_t npar,
@@ -417,6 +313,214 @@ __global__ void __launch_bounds__(256, 2) k_up_split(const TS *__restrict__ Ef, 
     if (ch == 0 && act && jz == 0 && mx > 0.0f) atomicMax(&loc[j & 15], __float_as_uint(mx));
     __syncthreads();
     if (threadIdx.x < 16 && loc[threadIdx.x]) atomicMax(&xmax[16 * blockIdx.y + threadIdx.x], loc[threadIdx.x]);
+  }
+}
+
+// ---------------------------------------------------------------------------
+// Transfer kernels with one output pair per thread: a parent has M^3 x NP
+// threads, thread (nu, p) forms the coefficient nu of two neighbouring columns
+// (one 16-byte value pair for double-float) in each of the three mode products,
+// which exchange their tensors through shared memory.  The children of a
+// parent are taken in turn.  Threads exist for the columns there are, PP
+// parents share a CTA, and a thread's chain is twelve multiply-adds per child
+// instead of the register kernels' hundreds (whose unrolled code also misses
+// the instruction cache on narrow levels).  Every output is formed by the same
+// operations in the same order as there, so the bits are the same.  Narrow
+// levels: 8 - 9 us per level with the register kernels (order 4, double-float),
+// 4 - 5 us here; 81,920 triangles, order 4, one column, all upward levels 122
+// -> 64 us.
+template <class T>
+struct alignas(2 * sizeof(T)) Pair {
+  T a, b;
+};
+
+// columns of a CTA in pairs (grid.y runs over groups of this many)
+template <int M>
+__host__ __device__ constexpr int pair_max() { return M == 5 ? 4 : 8; }
+
+// sum_b F[b][j] (up) or F[j][b] (down) in[base + b stride], both columns
+template <class T, bool TRANS, int M>
+__device__ __forceinline__ Pair<T> mode_pair(const T *F, int j, const Pair<T> *in, int stride) {
+  Pair<T> o{zero_of<T>(), zero_of<T>()};
+#pragma unroll
+  for (int b = 0; b < M; ++b) {
+    const T f = TRANS ? F[b * M + j] : F[j * M + b];
+    const Pair<T> v = in[b * stride];
+    acc_fma(o.a, f, v.a);
+    acc_fma(o.b, f, v.b);
+  }
+  acc_norm(o.a);
+  acc_norm(o.b);
+  return o;
+}
+
+template <class TS, class T, int M>
+__device__ __forceinline__ void pair_factors(const TS *__restrict__ Ef, int64_t par, int64_t npar_left, int pp, T *F) {
+  constexpr int kPer = 6 * M * M;
+  const int n = npar_left < pp ? (int)npar_left : pp;
+  for (int i = threadIdx.x; i < n * kPer; i += blockDim.x)
+    F[i] = to_compute<T>(Ef[(2 * par + 1) * (3 * M * M) + i]);   // the children of consecutive parents are consecutive
+}
+
+template <class TS, class T, int M>
+__global__ void __launch_bounds__(512, 3) k_up_pair(const TS *__restrict__ Ef, int rp, int np, int pp, int64_t par0,
+                                                    int64_t npar, T *__restrict__ xhat, unsigned *__restrict__ xmax) {
+  constexpr int K = M * M * M;
+  extern __shared__ __align__(16) unsigned char psm[];
+  __shared__ unsigned loc[16];
+  const int tpp = K * np, pl = (int)threadIdx.x / tpp, rem = (int)threadIdx.x - pl * tpp;
+  Pair<T> *buf = reinterpret_cast<Pair<T> *>(psm);          // [2][pp][K][np]
+  T *F = reinterpret_cast<T *>(buf + 2 * pp * tpp);         // [pp][2][3][M x M]
+  if (threadIdx.x < 16) loc[threadIdx.x] = 0u;
+  const int64_t p0 = (int64_t)blockIdx.x * pp, par = par0 + p0 + pl;
+  const int nu = rem / np, p = rem - nu * np, col = 2 * (pair_max<M>() * (int)blockIdx.y + p);
+  const int jx = nu % M, jy = (nu / M) % M, jz = nu / (M * M);
+  const bool act = pl < pp && p0 + pl < npar && col < rp;
+  Pair<T> v[2];
+#pragma unroll
+  for (int ch = 0; ch < 2; ++ch)
+    v[ch] = act ? *reinterpret_cast<const Pair<T> *>(xhat + ((2 * par + 1 + ch) * K + nu) * rp + col)
+                : Pair<T>{zero_of<T>(), zero_of<T>()};
+  pair_factors<TS, T, M>(Ef, par0 + p0, npar - p0, pp, F);
+  const int slot = pl < pp ? (int)threadIdx.x : 0, at = pl < pp ? pl * tpp + p : 0;
+  const T *Fp = F + (pl < pp ? pl : 0) * 6 * M * M;
+  Pair<T> acc{zero_of<T>(), zero_of<T>()};
+#pragma unroll
+  for (int ch = 0; ch < 2; ++ch) {
+    Pair<T> *A = buf + (ch ? pp * tpp : 0), *Bf = buf + (ch ? 0 : pp * tpp);
+    const T *Fc = Fp + ch * 3 * M * M;
+    if (pl < pp) A[slot] = v[ch];
+    __syncthreads();
+    Pair<T> o = mode_pair<T, true, M>(Fc, jx, A + at + (nu - jx) * np, np);
+    if (pl < pp) Bf[slot] = o;
+    __syncthreads();
+    o = mode_pair<T, true, M>(Fc + M * M, jy, Bf + at + (nu - M * jy) * np, M * np);
+    if (pl < pp) A[slot] = o;
+    __syncthreads();
+    o = mode_pair<T, true, M>(Fc + 2 * M * M, jz, A + at + (nu - M * M * jz) * np, M * M * np);
+    acc.a = acc.a + o.a;
+    acc.b = acc.b + o.b;
+  }
+  if (act) *reinterpret_cast<Pair<T> *>(xhat + (par * K + nu) * rp + col) = acc;
+  if (xmax) {
+    if (act) {
+      atomicMax(&loc[2 * p], __float_as_uint(mag_of(acc.a)));
+      atomicMax(&loc[2 * p + 1], __float_as_uint(mag_of(acc.b)));
+    }
+    __syncthreads();
+    unsigned *dst = xmax + 2 * pair_max<M>() * blockIdx.y + threadIdx.x;
+    if (threadIdx.x < 16 && loc[threadIdx.x] && loc[threadIdx.x] > __ldcg(dst)) atomicMax(dst, loc[threadIdx.x]);
+  }
+}
+
+template <class TS, class T, int M>
+__global__ void __launch_bounds__(512, 3) k_down_pair(const TS *__restrict__ Ef, int rp, int np, int pp, int64_t par0,
+                                                      int64_t npar, T *__restrict__ yhat) {
+  constexpr int K = M * M * M;
+  extern __shared__ __align__(16) unsigned char psm[];
+  const int tpp = K * np, pl = (int)threadIdx.x / tpp, rem = (int)threadIdx.x - pl * tpp;
+  Pair<T> *P = reinterpret_cast<Pair<T> *>(psm), *A = P + pp * tpp, *Bf = A + pp * tpp;   // [pp][K][np] each
+  T *F = reinterpret_cast<T *>(Bf + pp * tpp);
+  const int64_t p0 = (int64_t)blockIdx.x * pp, par = par0 + p0 + pl;
+  const int nu = rem / np, p = rem - nu * np, col = 2 * (pair_max<M>() * (int)blockIdx.y + p);
+  const int jx = nu % M, jy = (nu / M) % M, jz = nu / (M * M);
+  const bool act = pl < pp && p0 + pl < npar && col < rp;
+  const Pair<T> zero{zero_of<T>(), zero_of<T>()};
+  const Pair<T> v = act ? *reinterpret_cast<const Pair<T> *>(yhat + (par * K + nu) * rp + col) : zero;
+  Pair<T> yc[2];
+#pragma unroll
+  for (int ch = 0; ch < 2; ++ch)
+    yc[ch] = act ? *reinterpret_cast<const Pair<T> *>(yhat + ((2 * par + 1 + ch) * K + nu) * rp + col) : zero;
+  pair_factors<TS, T, M>(Ef, par0 + p0, npar - p0, pp, F);
+  const int slot = pl < pp ? (int)threadIdx.x : 0, at = pl < pp ? pl * tpp + p : 0;
+  const T *Fp = F + (pl < pp ? pl : 0) * 6 * M * M;
+  if (pl < pp) P[slot] = v;
+  __syncthreads();
+#pragma unroll
+  for (int ch = 0; ch < 2; ++ch) {
+    const T *Fc = Fp + ch * 3 * M * M;
+    Pair<T> o = mode_pair<T, false, M>(Fc, jx, P + at + (nu - jx) * np, np);
+    if (pl < pp) A[slot] = o;
+    __syncthreads();
+    o = mode_pair<T, false, M>(Fc + M * M, jy, A + at + (nu - M * jy) * np, M * np);
+    if (pl < pp) Bf[slot] = o;
+    __syncthreads();
+    o = mode_pair<T, false, M>(Fc + 2 * M * M, jz, Bf + at + (nu - M * M * jz) * np, M * M * np);
+    if (act)
+      *reinterpret_cast<Pair<T> *>(yhat + ((2 * par + 1 + ch) * K + nu) * rp + col) =
+          Pair<T>{yc[ch].a + o.a, yc[ch].b + o.b};
+  }
+}
+
+// parents of a CTA of the pair kernels: 512 threads on wide levels, fewer where
+// that leaves SMs without a CTA
+template <int M>
+inline int pair_parents(int64_t npar, int np) {
+  const int most = std::max(1, 512 / (M * M * M * np));
+  return (int)std::max<int64_t>(1, std::min<int64_t>(most, npar / (2 * 152)));
+}
+
+// Upward levels that take the pair kernel: every level in double-float (and
+// double) arithmetic, orders other than 3 and 4, and in FP32 up to 8 columns
+// and narrow levels.  Wide FP32 levels of more columns are bound by the pair
+// kernel's shared-memory reads (eight per four multiply-adds): 327,680
+// triangles, order 4, 16 columns 210 us with the register kernels, 238 us
+// without; 1.3 M triangles, order 3, 4 columns 150 us with them, 95 us without.
+// Downward the pair kernel was never slower (1.3 M, 4 columns 193 -> 93 us;
+// 327,680, 16 columns FP32 146 -> 133 us, double-float 343 -> 306 us; 81,920,
+// one column, double-float order 4 121 -> 64 us).
+template <class T>
+inline bool pair_up(int m, int64_t npar, int rp) {
+  return sizeof(T) == 8 || (m != 3 && m != 4) || rp <= 8 || npar * rp <= 4096;
+}
+
+template <class TS, class T, int M>
+void launch_up_m(const TS *Ef, int rp, int64_t par0, int64_t npar, T *xhat, unsigned *xmax, cudaStream_t st) {
+  if (pair_up<T>(M, npar, rp)) {
+    const int np = std::min(pair_max<M>(), rp / 2), pp = pair_parents<M>(npar, np), thr = (pp * M * M * M * np + 31) / 32 * 32;
+    const dim3 grid((unsigned)((npar + pp - 1) / pp), (rp / 2 + np - 1) / np);
+    k_up_pair<TS, T, M><<<grid, thr, pp * (2 * M * M * M * np * sizeof(Pair<T>) + 6 * M * M * sizeof(T)), st>>>(
+        Ef, rp, np, pp, par0, npar, xhat, xmax);
+    return;
+  }
+  if constexpr (M == 3 || M == 4) {
+    const int gy = (rp + 15) / 16;
+    if (npar <= kUpSplitMax)
+      k_up_split<TS, T, M><<<dim3((unsigned)((npar + kSplitParents - 1) / kSplitParents), gy), 256, 0, st>>>(
+          Ef, rp, par0, npar, xhat, xmax);
+    else
+      k_up_reg<TS, T, M><<<dim3((unsigned)((npar + kRegParents - 1) / kRegParents), gy), 256, 0, st>>>(
+          Ef, rp, par0, npar, xhat, xmax);
+  }
+}
+
+template <class TS, class T, int M>
+void launch_down_m(const TS *Ef, int rp, int64_t par0, int64_t npar, T *yhat, cudaStream_t st) {
+  const int np = std::min(pair_max<M>(), rp / 2), pp = pair_parents<M>(npar, np), thr = (pp * M * M * M * np + 31) / 32 * 32;
+  const dim3 grid((unsigned)((npar + pp - 1) / pp), (rp / 2 + np - 1) / np);
+  k_down_pair<TS, T, M><<<grid, thr, pp * (3 * M * M * M * np * sizeof(Pair<T>) + 6 * M * M * sizeof(T)), st>>>(
+      Ef, rp, np, pp, par0, npar, yhat);
+}
+
+// the upward step for parents par0 .. par0 + npar - 1, and the downward step below them
+template <class TS, class T>
+void launch_up(const TS *Ef, int m, int rp, int64_t par0, int64_t npar, T *xhat, unsigned *xmax, cudaStream_t st) {
+  switch (m) {
+    case 1: return launch_up_m<TS, T, 1>(Ef, rp, par0, npar, xhat, xmax, st);
+    case 2: return launch_up_m<TS, T, 2>(Ef, rp, par0, npar, xhat, xmax, st);
+    case 3: return launch_up_m<TS, T, 3>(Ef, rp, par0, npar, xhat, xmax, st);
+    case 4: return launch_up_m<TS, T, 4>(Ef, rp, par0, npar, xhat, xmax, st);
+    default: return launch_up_m<TS, T, 5>(Ef, rp, par0, npar, xhat, xmax, st);
+  }
+}
+template <class TS, class T>
+void launch_down(const TS *Ef, int m, int rp, int64_t par0, int64_t npar, T *yhat, cudaStream_t st) {
+  switch (m) {
+    case 1: return launch_down_m<TS, T, 1>(Ef, rp, par0, npar, yhat, st);
+    case 2: return launch_down_m<TS, T, 2>(Ef, rp, par0, npar, yhat, st);
+    case 3: return launch_down_m<TS, T, 3>(Ef, rp, par0, npar, yhat, st);
+    case 4: return launch_down_m<TS, T, 4>(Ef, rp, par0, npar, yhat, st);
+    default: return launch_down_m<TS, T, 5>(Ef, rp, par0, npar, yhat, st);
   }
 }
 
