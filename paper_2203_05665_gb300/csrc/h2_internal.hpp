@@ -180,6 +180,7 @@ struct Dev {
   int gkcap = 0;
   int32_t *grank = nullptr, *gpiv = nullptr;
   int64_t coupling_entries = 0;  // stored coupling entries (padded; GCA handles)
+  int near_longest = 0, adm_longest = 0;   // blocks of the longest row
   // work buffers for up to cap_nrhs right-hand sides
   int cap_nrhs = 0;
   void *xpad = nullptr, *ypad = nullptr, *xhat = nullptr, *yhat = nullptr;
@@ -285,6 +286,27 @@ int row_schedule(Dev &d, const int64_t *ptr, const int32_t *col, int64_t nrows, 
 constexpr size_t kMaximaBytes = 64 * 8 + 64 * 4 + 32 * 64 * 4;
 // leaf forward step on the tensor cores (after ntc_input); requires d.Vtc
 int tc_leaf_forward(Ctx &c, void *xhat, int rp);
+
+// Block rows in FP32 arithmetic, one or four warps per row (h2_lane.cu): row r of
+// out ([row][M][rp]) is the sum of
+//   its blocks e = ptr[r] .. ptr[r + 1] - 1 (ptr NULL: block r): stored block
+//   blk[e] of A ([K][Mp], blk NULL: e) times item col[e] of X ([K][rp], col
+//   NULL: e), times scale[stored block];
+//   V_r ([kv][Mp], NULL: none) times item r of Y ([kv][rp]), times vscale[r];
+//   G_r ([K][Mp] in FP32, NULL: none) times item r of X.
+// prec gives the types of A (the handle's) and V (v32: FP32).  M, K <= 64.
+struct LaneRows {
+  const void *A, *V;
+  const float *G, *X, *Y, *scale, *vscale;
+  const int64_t *ptr;
+  const int32_t *col, *blk;
+  float *out;
+  int64_t nrows;
+  int M, Mp, K, kv, rp;
+  int longest;               // blocks of the longest row
+};
+int lane_rows(const LaneRows &g, int prec, bool v32, int64_t *launches, cudaStream_t st);
+constexpr int kLaneMax = 64;
 
 // h2_build for a given kernel (h2_api.cpp)
 int build_handle(const double *vert, int64_t nv, const int32_t *tri, int64_t nt, int leaf_size, double eta, int order,

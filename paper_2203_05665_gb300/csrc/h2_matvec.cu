@@ -1014,27 +1014,18 @@ __global__ void __launch_bounds__(256) k_leaf_fwd_reg(const TS *__restrict__ V, 
   }
 }
 
-// With gself (FP32 self blocks of bfloat16 handles, [leaf][c][Lp]) the
-// leaf's self block joins the contraction: y|t = V_t y^_t + G_tt x|t.
 template <class TS, class T>
 __global__ void __launch_bounds__(256) k_leaf_bwd_reg(const TS *__restrict__ Vt, const T *__restrict__ yleaf,
                                                       const float *__restrict__ vscale, int L, int Lp, int k, int rp,
-                                                      const float *__restrict__ gself, const T *__restrict__ xpad,
                                                       T *__restrict__ ypad) {
   extern __shared__ __align__(16) unsigned char lsm[];
   T *Vs = reinterpret_cast<T *>(lsm);   // [k][Lp]
   T *ys = Vs + k * Lp;                   // [k][rp]
-  T *Gs = ys + k * rp;                   // [L][Lp] (with gself)
-  T *xs = Gs + L * Lp;                   // [L][rp] (with gself)
   const int64_t t = blockIdx.x;
   const TS *vt = Vt + t * (int64_t)k * Lp;
   const T *yt = yleaf + t * (int64_t)k * rp;
   for (int i = threadIdx.x; i < k * Lp; i += blockDim.x) Vs[i] = to_compute<T>(vt[i]);
   for (int i = threadIdx.x; i < k * rp; i += blockDim.x) ys[i] = yt[i];
-  if (gself) {
-    for (int i = threadIdx.x; i < L * Lp; i += blockDim.x) Gs[i] = from_double<T>(gself[t * (int64_t)L * Lp + i]);
-    for (int i = threadIdx.x; i < L * rp; i += blockDim.x) xs[i] = xpad[t * (int64_t)L * rp + i];
-  }
   __syncthreads();
   const int r = threadIdx.x >> 3, jo = threadIdx.x & 7;
   if (r >= L) return;
@@ -1045,13 +1036,6 @@ __global__ void __launch_bounds__(256) k_leaf_bwd_reg(const TS *__restrict__ Vt,
     for (int u = 0; u < 2; ++u)
       if (jo + 8 * u < rp) acc_fma(acc[u], w, ys[nu * rp + jo + 8 * u]);
   }
-  if (gself)
-    for (int c = 0; c < L; ++c) {
-      const T w = Gs[c * Lp + r];
-#pragma unroll
-      for (int u = 0; u < 2; ++u)
-        if (jo + 8 * u < rp) acc_fma(acc[u], w, xs[c * rp + jo + 8 * u]);
-    }
   const float sc = vscale ? vscale[t] : 1.0f;
 #pragma unroll
   for (int u = 0; u < 2; ++u)
@@ -1108,12 +1092,28 @@ int matvec_typed(Ctx &c, const Tio *x, Tio *y, int nrhs, bool acc) {
       x, d.n, nrhs, rp, d.pad_src, d.npad, cmx, xpad, near_tc ? d.ntc_xmax : nullptr);
   mk.count(H2_PH_PERMUTE_IN);
   mk.mark(H2_PH_LEAF_FORWARD);
-  // leaf steps with one CTA per leaf when the stored values are in the arithmetic type
+  // FP32 arithmetic, tiles of at most 64 rows: one or four warps per block row
+  const bool lane = std::is_same<T, float>::value && L <= kLaneMax && k <= kLaneMax;
+  // leaf steps with one CTA per leaf
   const bool leaf_reg = L <= 32 && k <= 64 && rp <= 16;
   if (leaf_tc) {
     ntc_input(c, xpad, rp, 0, rp, true);
     if ((rc = tc_leaf_forward(c, xhat, rp))) return rc;
     mk.count(H2_PH_LEAF_FORWARD, 2);
+  } else if (far && lane) {
+    LaneRows g{};
+    g.A = d.V;
+    g.scale = vscale;
+    g.X = (const float *)xpad;
+    g.out = (float *)(xhat + leaf0 * (int64_t)k * rp);
+    g.nrows = d.nleaf;
+    g.M = k;
+    g.Mp = kp;
+    g.K = L;
+    g.rp = rp;
+    int64_t nl = 0;
+    if ((rc = lane_rows(g, d.v32 ? (int)H2_F32 : d.prec, false, &nl, st))) return rc;
+    mk.count(H2_PH_LEAF_FORWARD, nl);
   } else if (far && leaf_reg) {
     const size_t sm = (size_t)L * (kp + rp) * sizeof(T);
     T *xl = xhat + leaf0 * (int64_t)k * rp;
@@ -1181,6 +1181,22 @@ int matvec_typed(Ctx &c, const Tio *x, Tio *y, int nrhs, bool acc) {
       int64_t nl = 0;
       if ((rc = tct_coupling(c, xhat, yhat, rp, &nl))) return rc;
       mk.count(H2_PH_COUPLING, nl - 1);
+    } else if (lane) {
+      LaneRows g{};
+      g.A = d.S;
+      g.ptr = d.adm_ptr + row0;
+      g.col = d.adm_col;
+      g.X = (const float *)xhat;
+      g.out = (float *)out;
+      g.nrows = d.nclu - row0;
+      g.M = k;
+      g.Mp = kp;
+      g.K = k;
+      g.rp = rp;
+      g.longest = d.adm_longest;
+      int64_t nl = 0;
+      if ((rc = lane_rows(g, d.prec, false, &nl, st))) return rc;
+      mk.count(H2_PH_COUPLING, nl - 1);
     } else {
       CouplingRows<TS, T> rows{(const TS *)d.S, d.adm_ptr, d.adm_col, xhat, k, kp, rp, row0};
       if ((rc = launch_rows<TS, T>(rows, cf_cpl, t_cpl, Rk, d.nclu - row0, 0, out, st))) return rc;
@@ -1194,13 +1210,13 @@ int matvec_typed(Ctx &c, const Tio *x, Tio *y, int nrhs, bool acc) {
     mk.count(H2_PH_DOWNWARD);
   }
   mk.mark(H2_PH_LEAF_NEAR);
-  // bfloat16 handles: the FP32 self blocks join the leaf backward step when it runs per leaf
-  const bool self_fused = far && leaf_reg && d.nself && std::is_same<T, float>::value;
-  if (far && leaf_reg) {
-    const size_t sm = ((size_t)k * (Lp + rp) + (self_fused ? (size_t)L * (Lp + rp) : 0)) * sizeof(T);
+  if (lane) {
+    // FP32 arithmetic: the leaf backward step, the FP32 self blocks of bfloat16 handles and the
+    // nearfield as one sum per leaf row
+  } else if (far && leaf_reg) {
+    const size_t sm = (size_t)k * (Lp + rp) * sizeof(T);
     k_leaf_bwd_reg<TV, T><<<(unsigned)d.nleaf, 256, sm, st>>>((const TV *)d.Vt, yhat + leaf0 * (int64_t)k * rp,
-                                                             vscale, L, Lp, k, rp, self_fused ? d.nself : nullptr,
-                                                             xpad, ypad);
+                                                             vscale, L, Lp, k, rp, ypad);
     mk.count(H2_PH_LEAF_NEAR);
   } else if (far) {
     LeafBackwardRows<TV, T> rows{(const TV *)d.Vt, yhat, vscale, k, Lp, rp, leaf0};
@@ -1212,19 +1228,40 @@ int matvec_typed(Ctx &c, const Tio *x, Tio *y, int nrhs, bool acc) {
     int64_t nl = 0;
     if ((rc = ntc_near(c, xpad, ypad, rp, far ? 1 : 0, &nl, leaf_tc))) return rc;
     mk.count(H2_PH_LEAF_NEAR, nl);
+  } else if (lane) {
+    LaneRows g{};
+    g.A = d.near;
+    g.scale = nscale;
+    g.ptr = d.nself ? d.near_ptr2 : d.near_ptr;
+    g.col = d.nself ? d.near_col2 : d.near_col;
+    g.blk = d.nself ? d.near_blk2 : nullptr;
+    g.G = d.nself;
+    g.X = (const float *)xpad;
+    g.V = far ? d.Vt : nullptr;
+    g.Y = (const float *)(yhat + leaf0 * (int64_t)k * rp);
+    g.vscale = vscale;
+    g.out = (float *)ypad;
+    g.nrows = d.nleaf;
+    g.M = L;
+    g.Mp = Lp;
+    g.K = L;
+    g.kv = k;
+    g.rp = rp;
+    g.longest = d.near_longest;
+    int64_t nl = 0;
+    if ((rc = lane_rows(g, d.prec, d.v32, &nl, st))) return rc;
+    mk.count(H2_PH_LEAF_NEAR, nl);
   } else if (d.nself) {
     // bfloat16: the blocks of other leaves, then the self blocks G_jj in FP32
     NearRows<TS, T> rows{(const TS *)d.near, d.near_ptr2, d.near_col2, xpad, nscale, L, Lp, rp, d.near_blk2};
     if ((rc = launch_rows<TS, T>(rows, cf_near, t_near, RL, d.nleaf, far ? 1 : 0, ypad, st))) return rc;
     mk.count(H2_PH_LEAF_NEAR);
     if constexpr (std::is_same<T, float>::value) {
-      if (!self_fused) {
       RowCfg cf_self{};
       if ((rc = row_cfg<float, T>(L, Lp, rp, L, t_near, RL, cf_self))) return rc;
       NearRows<float, T> self{d.nself, d.self_ptr, d.self_col, xpad, nullptr, L, Lp, rp, nullptr};
       if ((rc = launch_rows<float, T>(self, cf_self, t_near, RL, d.nleaf, 1, ypad, st))) return rc;
       mk.count(H2_PH_LEAF_NEAR);
-      }
     }
   } else {
     NearRows<TS, T> rows{(const TS *)d.near, d.near_ptr, d.near_col, xpad, nscale, L, Lp, rp, nullptr};
@@ -1372,7 +1409,7 @@ int matvec_gca(Ctx &c, const Tio *x, Tio *y, int nrhs, bool acc) {
   if (far && leaf_reg) {
     const size_t sm = (size_t)KD * (Lp + rp) * sizeof(T);
     k_leaf_bwd_reg<TS, T><<<(unsigned)d.nleaf, 256, sm, st>>>((const TS *)d.Vt, X(yhat, D), nullptr, L, Lp, KD, rp,
-                                                             nullptr, xpad, ypad);
+                                                             ypad);
     mk.count(H2_PH_LEAF_NEAR);
   } else if (far) {
     LeafBackwardRows<TS, T> rows{(const TS *)d.Vt, X(yhat, D), nullptr, KD, Lp, rp, 0};

@@ -778,6 +778,9 @@ int device_build(Ctx &c) {
   d.npad = p.nleaf * p.lmax;
   d.lp = (p.lmax + rowpad - 1) / rowpad * rowpad;
   d.nadm = (int64_t)p.adm_col.size();
+  for (int64_t c = 0; c < p.nclu; ++c) d.adm_longest = std::max(d.adm_longest, (int)(p.adm_ptr[c + 1] - p.adm_ptr[c]));
+  for (int64_t j = 0; j < p.nleaf; ++j)
+    d.near_longest = std::max(d.near_longest, (int)(p.near_ptr[j + 1] - p.near_ptr[j]));
   d.nnear = (int64_t)p.near_col.size();
   if (d.coupling < 0) {
     // automatic: store S unless it would take more than half of the free memory (FP32 only)
