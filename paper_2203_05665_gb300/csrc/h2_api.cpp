@@ -353,6 +353,7 @@ int h2_destroy(h2_handle h) {
   if (h->stream) cudaStreamSynchronize(h->stream);
   else cudaDeviceSynchronize();
   drop_events(h->prof);
+  free_call_graphs(*h);
   free_gmres_work(h->gw);
   free_stream_work(h->sw);
   free_dev(h->d);

@@ -223,7 +223,31 @@ struct StreamWork {
   cudaEvent_t ev_in[2] = {nullptr, nullptr}, ev_done[2] = {nullptr, nullptr}, ev_out[2] = {nullptr, nullptr};
 };
 
+// A product captured as a CUDA graph for repeated calls with the same number of
+// right-hand sides (run_matvec): only the nodes that read x or write y change
+// from call to call
+struct CallGraph {
+  struct Node {
+    cudaGraphNode_t node;
+    int arg;                      // index of the x or y parameter
+    bool out;
+  };
+  int nrhs = 0;
+  bool io64 = false, acc = false;
+  int64_t work_gen = -1;          // work buffers the capture refers to
+  uint64_t used = 0;              // call count of the last use
+  cudaGraph_t graph = nullptr;
+  cudaGraphExec_t exec = nullptr; // NULL until the second call
+  const void *x = nullptr;
+  void *y = nullptr;
+  std::vector<Node> nodes;
+};
+constexpr int kMaxCallGraphs = 4;
+
 struct Ctx {
+  CallGraph calls[kMaxCallGraphs];
+  uint64_t ncalls = 0;
+  bool direct = false;                // launch kernel by kernel (no call graphs)
   double build_ms[H2_NBUILD] = {0};   // wall time of the build phases (h2_build_times)
   StreamWork sw;                      // h2_matvec_host_stream
   GcaParams gp;                       // GCA-H^2 handles: construction parameters
@@ -325,6 +349,7 @@ int gca_build(Ctx &c, const double *vert, const int32_t *tri, const double *area
 // if x64/y64 are given instead the product reads/writes FP64 arrays.
 // accumulate: y += G~ x instead of y = G~ x (the final scatter adds)
 int run_matvec(Ctx &c, const void *x, void *y, int nrhs, bool io64, bool accumulate = false);
+void free_call_graphs(Ctx &c);
 // GMRES (h2_solve.cu); b, z device FP64 arrays
 int run_gmres(Ctx &c, const double *b, double *z, int nrhs, double rtol, int restart, int maxit,
               h2_solve_info *info);

@@ -69,6 +69,8 @@ extern "C" int h2_matvec_noalloc(h2_handle h, const void *x, void *y, int nrhs) 
   d.yhat = b + 2 * vec + coef;
   d.cap_nrhs = rp;        // the buffers fit rp columns: no growth, no allocation
   h->prof.on = false;     // no timing events either
+  const bool sdirect = h->direct;
+  h->direct = true;       // call graphs refer to the handle's own work buffers
   int rc = run_matvec(*h, x, y, nrhs, false);
   d.xpad = sv[0];
   d.ypad = sv[1];
@@ -76,6 +78,7 @@ extern "C" int h2_matvec_noalloc(h2_handle h, const void *x, void *y, int nrhs) 
   d.yhat = sv[3];
   d.cap_nrhs = scap;
   h->prof.on = sprof;
+  h->direct = sdirect;
   d.last_nrhs = slast;    // h2_coefficients keeps reporting the last h2_matvec product
   d.last_rp = slast_rp;
   return rc;
