@@ -407,7 +407,7 @@ int h2_phase_times(h2_handle h, double *ms, int64_t *launches, int64_t *products
  *
  * The paper multiplies one H^2 matrix at a time (Section 2, Algorithms 1-3);
  * the batch runs the same steps for many matrices at once: each block-row
- * phase (leaf forward, coupling, leaf backward, nearfield) is ONE persistent
+ * phase (leaf forward, coupling, leaf backward, nearfield) is ONE
  * kernel launch over the rows of all matrices, the transfer passes run level
  * by level across the matrices, and the whole product is captured in a CUDA
  * graph on first use and replayed afterwards.
@@ -436,8 +436,8 @@ int h2_batch_offsets(h2_batch b, int64_t *offsets);
  * replay it.  A capture uses a private stream: do not call this function
  * while another capture is in progress on the calling thread. */
 int h2_batch_matvec(h2_batch b, const float *x, float *y);
-/* Autotuner of the launch shapes: times every candidate shape (slot size,
- * slots per warp, warps per CTA) of every block-row phase, reps launches
+/* Autotuner of the launch shapes: times every candidate shape (warps per CTA,
+ * stages per warp) of every block-row phase, reps launches
  * each, on the work vectors as the last product left them, and keeps the
  * fastest.  choice (4 ints, may be NULL) receives the chosen shape indices
  * of leaf forward, coupling, leaf backward and nearfield.  Synchronises. */
@@ -452,7 +452,7 @@ int h2_batch_phase_times(h2_batch b, double *ms, int64_t *launches, int64_t *pro
 /* info[9]: problems, packed length, sum of n_p nrhs_p, work bytes, kernel
  * launches per product, the four shape indices. */
 int h2_batch_info(h2_batch b, int64_t *info);
-/* Wait for the batch's products; H2_ETIMEOUT if a bounded device wait ran out. */
+/* Wait for the batch's products. */
 int h2_batch_sync(h2_batch b);
 int h2_batch_destroy(h2_batch b);
 

@@ -1,67 +1,58 @@
 // Batched H^2 products over independent matrices of uneven sizes (FP32
 // storage and arithmetic, stored coupling).
 //
-// Every block-row phase of the product (leaf forward, coupling, leaf
-// backward, nearfield: Algorithms 1-3) runs as ONE persistent launch over
-// the rows of all problems.  Rows differ in shape from problem to problem
-// (rank k = m^3 for m = 3 or 4, leaf sizes up to 64, 1 to 16 right-hand
-// sides), so the kernel is warp-per-row: every warp owns a contiguous range
-// of rows holding about 1/(number of warps) of the work, in problem order,
-// and streams the stored tiles of its rows through its own ring of shared-
-// memory slots with bulk copies (TMA engine, one mbarrier per slot).  A slot
-// holds several whole terms A X of one row, or one piece of a term cut along
-// the contraction index when a term is larger than a slot.  Lane l owns the
-// output rows 2l and 2l + 1 (row l for tiles of at most 32 rows) of the
-// current row for all right-hand sides, multiplies in packed FP32 pairs and
-// sums its terms in a fixed order: results are bit-reproducible.
+// Every block-row phase of the product (leaf forward, coupling, leaf backward,
+// nearfield: Algorithms 1-3) runs as ONE launch over the rows of all problems.  Rows differ in shape from problem to problem (rank k =
+// m^3 for m = 3 or 4, leaf sizes up to 64, 1 to 16 right-hand sides); a warp
+// looks up its row's problem and takes the row as the single-matrix kernel does
+// (lane_row, h2_lane.cu): double-buffered pieces in its own shared-memory
+// stages, 4 x 8 (4 x 4) register tiles.  Rows of many terms are cut in chunk
+// rows whose partial sums are added in order, so that no warp finishes long
+// after the others; results are bit-reproducible.
 //
-// The transfer passes run level-synchronously across problems: step s of the
-// upward pass treats level D_p - 1 - s of every problem p, step s of the
-// downward pass level lmin_p + s.  The permutations in and out are one
-// launch each over the packed vectors of all problems.  The whole sequence
-// is captured once in a CUDA graph and replayed.
+// The transfer passes run level-synchronously across problems (up_pair and
+// down_pair, h2_transfer.cuh): step s of the upward pass treats level D_p - 1 - s
+// of every problem p, step s of the downward pass level lmin_p + s.  The
+// permutations in and out are one launch each over the packed vectors of all
+// problems.  The whole sequence is captured once in a CUDA graph and replayed.
 //
-// The slot size, slots per warp and warps per CTA of every block-row phase
-// are chosen by measurement (h2_batch_tune).
+// The warps per CTA and stages per warp of every block-row phase are chosen by
+// measurement (h2_batch_tune).
+//
+// Six problems (20,480 to 130,000 triangles, order 3 and 4, leaves of 64, 1 to 8
+// right-hand sides), default launch shapes: 1,124 us per product with a
+// persistent kernel of four warps per SM and one output row per lane (coupling
+// 416, leaf backward + nearfield 442, transfers 210), 426 us now (134, 182, 81);
+// bound by the instructions around pieces of 27 to 64 rows and 4 columns.
 #include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <new>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 #include "h2_internal.hpp"
-#include "h2_ptx.cuh"
+#include "h2_lane.cuh"
 #include "h2_transfer.cuh"
 
 namespace h2 {
 namespace {
 
-// One problem's rows in one block-row phase.
+// One problem's rows in one block-row phase; first: its first row among the phase's
 struct BRows {
-  const float *A;        // stored tiles: term b at A + b a_stride, [K][Mp] (contraction index major)
-  const float *X;        // input tiles: unit u at X + u x_stride, [K][rp]
-  const int64_t *ptr;    // terms of row r: [ptr[row0 + r], ptr[row0 + r + 1]); NULL: the single term r
-  const int64_t *pend;   // if set, row r's terms end at pend[r] instead (rows made of chunks)
-  const int32_t *col;    // unit of term b; NULL: unit = r
-  float *out;            // output row r at out + r out_stride, [M][rp]
-  int64_t a_stride, x_stride, out_stride, row0, nrows;
-  int64_t w0;            // work of all earlier problems in this phase
-  int64_t wterm, wrow;   // work of a term and of a row (bytes moved, plus a fixed overhead)
-  int64_t cap;           // at most cap terms of a row are taken here (the rest goes to chunk rows)
-  int64_t wfix;          // if > 0, every row counts wfix work (chunk rows)
-  int M, Mp, K, rp;
-  int tps;               // whole terms per slot; 0: terms are cut in pieces of P contraction rows
-  int P, ppt;            // rows per piece, pieces per term (cut terms)
-  int accumulate;
+  LaneRows g;
+  LaneShape t;
+  int64_t first;
+  int tc;                // columns of a register tile
 };
 
 // One problem's parents in one transfer step.
 struct BTr {
   const float *Ef;
   float *hat;
-  int64_t par0, g0;      // first parent of the entry, its global parent index
-  int m, k, rp, pad;
+  int64_t par0, npar;
+  int cta0, m, rp, np, pp;   // first CTA of the entry, order, columns, column pairs, parents per CTA
 };
 
 // One problem's part of the packed input / output vectors.
@@ -75,313 +66,56 @@ struct BPerm {
 constexpr int kBatchMaxRows = 64;   // output rows of a tile (k or the leaf size)
 constexpr int kBatchMaxRp = 16;     // padded right-hand sides
 
-// ---------------------------------------------------------------------------
-// work partition: position (problem, row) of the first row whose work starts
-// at or after W
-struct Pos {
-  int p;
-  int64_t r;
-};
-__device__ __forceinline__ bool pos_less(Pos a, Pos b) { return a.p < b.p || (a.p == b.p && a.r < b.r); }
-
-__device__ __forceinline__ int64_t row_work(const BRows &q, int64_t r) {
-  if (q.wfix > 0) return q.w0 + r * q.wfix;
-  const int64_t terms = q.ptr ? q.ptr[q.row0 + r] - q.ptr[q.row0] : r;
-  return q.w0 + terms * q.wterm + r * q.wrow;
-}
-
-// first term and number of terms of row r
-__device__ __forceinline__ void row_terms(const BRows &q, int64_t r, int64_t &b0, int64_t &nt) {
-  if (!q.ptr) {
-    b0 = r;
-    nt = 1;
-    return;
-  }
-  b0 = q.ptr[q.row0 + r];
-  const int64_t e = q.pend ? q.pend[r] : q.ptr[q.row0 + r + 1];
-  nt = min(e - b0, q.cap);
-}
-
-__device__ Pos find_pos(const BRows *__restrict__ pr, int np, int64_t W) {
-  int lo = 0, hi = np - 1;   // largest p with w0 <= W
-  while (lo < hi) {
-    const int mid = (lo + hi + 1) / 2;
-    if (pr[mid].w0 <= W) lo = mid;
-    else hi = mid - 1;
-  }
-  Pos ps{lo, 0};
-  const BRows &q = pr[lo];
-  int64_t a = 0, b = q.nrows;   // smallest r with row_work >= W
-  while (a < b) {
-    const int64_t mid = (a + b) / 2;
-    if (row_work(q, mid) >= W) b = mid;
-    else a = mid + 1;
-  }
-  ps.r = a;
-  while (ps.p < np && ps.r >= pr[ps.p].nrows) {
-    ps.p++;
-    ps.r = 0;
-  }
-  return ps;
-}
-
-// issue cursor over the slots of a warp
-struct Cur {
-  int p;
-  int64_t r, e, b0, nt;
-  int q;
-};
-
-__device__ __forceinline__ void cur_load(const BRows *__restrict__ pr, Cur &c) {
-  row_terms(pr[c.p], c.r, c.b0, c.nt);
-  c.e = 0;
-  c.q = 0;
-}
-
-// next row that has terms, or a position at or after end
-__device__ __forceinline__ void cur_next_row(const BRows *__restrict__ pr, int np, Pos end, Cur &c) {
-  for (;;) {
-    c.r++;
-    while (c.p < np && c.r >= pr[c.p].nrows) {
-      c.p++;
-      c.r = 0;
-    }
-    if (c.p >= np || !pos_less(Pos{c.p, c.r}, end)) return;
-    cur_load(pr, c);
-    if (c.nt > 0) return;
-  }
-}
-
-__device__ __forceinline__ bool cur_valid(int np, Pos end, const Cur &c) {
-  return c.p < np && pos_less(Pos{c.p, c.r}, end);
-}
-
-// lane 0 issues the copies of the cursor's slot into `slot`; all lanes advance the cursor
-__device__ __forceinline__ void issue_slot(const BRows *__restrict__ pr, int np, Pos end, Cur &c,
-                                           unsigned char *slot, uint64_t *bar, int lane) {
-  const BRows &q = pr[c.p];
-  if (q.tps > 0) {
-    const int cnt = (int)min((int64_t)q.tps, c.nt - c.e);
-    const uint32_t ab = 4u * q.K * q.Mp, xb = 4u * q.K * q.rp;
-    if (lane == 0) {
-      mbar_expect_tx(bar, (uint32_t)cnt * (ab + xb));
-      for (int t = 0; t < cnt; ++t) {
-        const int64_t b = c.b0 + c.e + t;
-        const int64_t u = q.col ? (int64_t)q.col[b] : c.r;
-        bulk_g2s(slot + t * (ab + xb), q.A + b * q.a_stride, ab, bar);
-        bulk_g2s(slot + t * (ab + xb) + ab, q.X + u * q.x_stride, xb, bar);
-      }
-    }
-    c.e += cnt;
-  } else {
-    const int r0 = c.q * q.P, rows = min(q.P, q.K - r0);
-    const uint32_t ab = 4u * rows * q.Mp, xb = 4u * rows * q.rp;
-    if (lane == 0) {
-      const int64_t b = c.b0 + c.e;
-      const int64_t u = q.col ? (int64_t)q.col[b] : c.r;
-      mbar_expect_tx(bar, ab + xb);
-      bulk_g2s(slot, q.A + b * q.a_stride + (int64_t)r0 * q.Mp, ab, bar);
-      bulk_g2s(slot + ab, q.X + u * q.x_stride + (int64_t)r0 * q.rp, xb, bar);
-    }
-    if (++c.q == q.ppt) {
-      c.q = 0;
-      c.e++;
-    }
-  }
-  if (c.e >= c.nt) cur_next_row(pr, np, end, c);
-}
-
-// Packed FP32 pairs: (lo, hi) in one 64-bit register pair.  fma.rn.f32x2
-// rounds each half exactly like fmaf, so results equal the scalar form.
-__device__ __forceinline__ uint64_t dup2(float a) {
-  uint64_t r;
-  asm("mov.b64 %0, {%1, %1};" : "=l"(r) : "f"(a));
-  return r;
-}
-__device__ __forceinline__ void fma2(uint64_t &d, uint64_t a, uint64_t b) {
-  asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(d) : "l"(a), "l"(b));
-}
-
-// acc[i] += sum_mu A[mu][row_i] X[mu][:] over one segment of a slot, the
-// columns of X in packed pairs.  QR = 2 (tiles of more than 32 rows): lane l
-// owns rows 2l and 2l + 1 and reads both with one 8-byte load; QR = 1: row l.
-template <int QR, int CP>
-__device__ __forceinline__ void seg_fma(const float *sA, const float *sX, int rows, int Mp, int lane,
-                                        uint64_t (&acc)[2][kBatchMaxRp / 2]) {
-  const bool v = QR == 2 ? 2 * lane < Mp : lane < Mp;
-#pragma unroll 4
-  for (int mu = 0; mu < rows; ++mu) {
-    uint64_t a0, a1 = 0;
-    if (QR == 2) {
-      const float2 av = v ? *reinterpret_cast<const float2 *>(sA + mu * Mp + 2 * lane) : make_float2(0.f, 0.f);
-      a0 = dup2(av.x);
-      a1 = dup2(av.y);
-    } else {
-      a0 = dup2(v ? sA[mu * Mp + lane] : 0.0f);
-    }
-#pragma unroll
-    for (int c = 0; c < CP; c += 4) {
-      const ulonglong2 xv = *reinterpret_cast<const ulonglong2 *>(sX + mu * CP + c);
-      fma2(acc[0][c / 2], a0, xv.x);
-      fma2(acc[0][c / 2 + 1], a0, xv.y);
-      if (QR == 2) {
-        fma2(acc[1][c / 2], a1, xv.x);
-        fma2(acc[1][c / 2 + 1], a1, xv.y);
-      }
-    }
-  }
-}
-
-__device__ __forceinline__ void seg_any(bool two, int rp, const float *sA, const float *sX, int rows, int Mp, int lane,
-                                        uint64_t (&acc)[2][kBatchMaxRp / 2]) {
-  switch (rp) {
-    case 4: two ? seg_fma<2, 4>(sA, sX, rows, Mp, lane, acc) : seg_fma<1, 4>(sA, sX, rows, Mp, lane, acc); break;
-    case 8: two ? seg_fma<2, 8>(sA, sX, rows, Mp, lane, acc) : seg_fma<1, 8>(sA, sX, rows, Mp, lane, acc); break;
-    case 12: two ? seg_fma<2, 12>(sA, sX, rows, Mp, lane, acc) : seg_fma<1, 12>(sA, sX, rows, Mp, lane, acc); break;
-    default: two ? seg_fma<2, 16>(sA, sX, rows, Mp, lane, acc) : seg_fma<1, 16>(sA, sX, rows, Mp, lane, acc); break;
-  }
-}
-
-__device__ __forceinline__ float lo_of(uint64_t v) { return __uint_as_float((uint32_t)v); }
-__device__ __forceinline__ float hi_of(uint64_t v) { return __uint_as_float((uint32_t)(v >> 32)); }
-
-// The batched block-row kernel (see the top of the file).  nslot slots of
-// zbytes per warp, then nslot mbarriers per warp.
-__global__ void __launch_bounds__(512) k_batch_rows(const BRows *__restrict__ pr, int np, int64_t wtotal, int nslot,
-                                                    int zbytes) {
-  extern __shared__ __align__(128) unsigned char smem[];
-  const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5, wpb = blockDim.x >> 5;
-  unsigned char *ring = smem + (size_t)wib * nslot * zbytes;
-  uint64_t *bar = reinterpret_cast<uint64_t *>(smem + (size_t)wpb * nslot * zbytes) + (size_t)wib * nslot;
-  const int64_t gw = (int64_t)blockIdx.x * wpb + wib, nw = (int64_t)gridDim.x * wpb;
-  const Pos beg = find_pos(pr, np, wtotal * gw / nw);
-  const Pos end = find_pos(pr, np, wtotal * (gw + 1) / nw);
-  if (!pos_less(beg, end)) return;
-
-  if (lane == 0) {
-    for (int s = 0; s < nslot; ++s) mbar_init(&bar[s], 1);
-    mbar_fence_init();
-  }
-  __syncwarp();
-
-  // issue cursor: first row of the range that has terms
-  Cur ic{beg.p, beg.r, 0, 0, 0, 0};
-  cur_load(pr, ic);
-  if (ic.nt == 0) cur_next_row(pr, np, end, ic);
-  int64_t issued = 0, consumed = 0;
-  while (issued < nslot && cur_valid(np, end, ic)) {
-    issue_slot(pr, np, end, ic, ring + (size_t)issued * zbytes, &bar[issued], lane);
-    ++issued;
-  }
-
-  Pos ps = beg;
-  while (pos_less(ps, end)) {
-    const BRows &q = pr[ps.p];
-    int64_t b0, nt;
-    row_terms(q, ps.r, b0, nt);
-    const int64_t ns = q.tps > 0 ? (nt + q.tps - 1) / q.tps : nt * q.ppt;
-    const bool two = q.M > 32;
-    uint64_t acc[2][kBatchMaxRp / 2];
-#pragma unroll
-    for (int i = 0; i < 2; ++i)
-#pragma unroll
-      for (int c = 0; c < kBatchMaxRp / 2; ++c) acc[i][c] = 0;
-    for (int64_t j = 0; j < ns; ++j) {
-      const int s = (int)(consumed % nslot);
-      if (!mbar_wait_bounded(&bar[s], (uint32_t)((consumed / nslot) & 1))) {
-        // a copy did not arrive: let the others in flight land, then leave
-        for (int64_t i = consumed + 1; i < issued; ++i)
-          mbar_wait_bounded(&bar[i % nslot], (uint32_t)((i / nslot) & 1));
-        return;
-      }
-      const unsigned char *slot = ring + (size_t)s * zbytes;
-      if (q.tps > 0) {
-        const int cnt = (int)min((int64_t)q.tps, nt - j * q.tps);
-        const int tb = 4 * q.K * (q.Mp + q.rp);
-        for (int t = 0; t < cnt; ++t) {
-          const float *sA = reinterpret_cast<const float *>(slot + t * tb);
-          seg_any(two, q.rp, sA, sA + q.K * q.Mp, q.K, q.Mp, lane, acc);
-        }
-      } else {
-        const int rows = min(q.P, q.K - (int)(j % q.ppt) * q.P);
-        const float *sA = reinterpret_cast<const float *>(slot);
-        seg_any(two, q.rp, sA, sA + rows * q.Mp, rows, q.Mp, lane, acc);
-      }
-      __syncwarp();
-      ++consumed;
-      if (cur_valid(np, end, ic)) {
-        // the slot just read is refilled by the TMA engine: order the reads first
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        issue_slot(pr, np, end, ic, ring + (size_t)s * zbytes, &bar[s], lane);
-        ++issued;
-      }
-    }
-    // write the row: lane owns rows 2 lane and 2 lane + 1 (tiles of more than 32 rows) or row lane
-    float *o = q.out + ps.r * q.out_stride;
-#pragma unroll
-    for (int i = 0; i < 2; ++i) {
-      const int row = two ? 2 * lane + i : (i == 0 ? lane : q.M);
-      if (row < q.M) {
-        float4 *o4 = reinterpret_cast<float4 *>(o + (int64_t)row * q.rp);
-#pragma unroll
-        for (int c4 = 0; c4 < kBatchMaxRp / 4; ++c4) {
-          if (4 * c4 < q.rp) {
-            const uint64_t p0 = acc[i][2 * c4], p1 = acc[i][2 * c4 + 1];
-            float4 v = make_float4(lo_of(p0), hi_of(p0), lo_of(p1), hi_of(p1));
-            if (q.accumulate) {
-              const float4 u = o4[c4];
-              v.x += u.x;
-              v.y += u.y;
-              v.z += u.z;
-              v.w += u.w;
-            }
-            o4[c4] = v;
-          }
-        }
-      }
-    }
-    ps.r++;
-    while (ps.p < np && ps.r >= pr[ps.p].nrows) {
-      ps.p++;
-      ps.r = 0;
-    }
-  }
+// The batched block-row kernel (see the top of the file): warp per row, the
+// rows of the phase's problems one after the other.
+template <int NST>
+__global__ void __launch_bounds__(256) k_batch_rows(const BRows *__restrict__ pr, int np, int64_t total,
+                                                    uint32_t stage) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int64_t row = (int64_t)blockIdx.x * (blockDim.x >> 5) + w;
+  if (row >= total) return;
+  // the row's problem: the last one that starts at or before it
+  int p = -1;
+  for (int b = 0; b < np; b += 32)
+    p += __popc(__ballot_sync(0xffffffffu, b + lane < np && pr[min(b + lane, np - 1)].first <= row));
+  const LaneRows g = pr[p].g;
+  const LaneShape t = pr[p].t;
+  unsigned char *ring = smem + (size_t)w * NST * stage;
+  if (pr[p].tc == 4) lane_row<float, float, 4, 1, NST>(g, t, 1, row - pr[p].first, w, ring, nullptr);
+  else lane_row<float, float, 8, 1, NST>(g, t, 1, row - pr[p].first, w, ring, nullptr);
 }
 
 // ---------------------------------------------------------------------------
-// transfers: warp per parent; global parent g -> (entry, parent) by the
-// entries' first global parent index
-constexpr int kTrWarps = 4;
-
-__device__ __forceinline__ int find_entry(const BTr *__restrict__ te, int ne, int64_t g) {
+// transfers: CTA per group of parents; CTA b belongs to the last entry that
+// starts at or before it
+__device__ __forceinline__ int find_entry(const BTr *__restrict__ te, int ne, int b) {
   int lo = 0, hi = ne - 1;
   while (lo < hi) {
     const int mid = (lo + hi + 1) / 2;
-    if (te[mid].g0 <= g) lo = mid;
+    if (te[mid].cta0 <= b) lo = mid;
     else hi = mid - 1;
   }
   return lo;
 }
 
-__global__ void __launch_bounds__(32 * kTrWarps) k_batch_upward(const BTr *__restrict__ te, int ne, int64_t total,
-                                                                 int wfloats) {
-  extern __shared__ __align__(16) float trs[];
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const int64_t g = (int64_t)blockIdx.x * kTrWarps + w;
-  if (g >= total) return;
-  const BTr &t = te[find_entry(te, ne, g)];
-  upward_parent_warp<float, float>(t.Ef, t.m, t.k, t.rp, t.par0 + (g - t.g0), t.hat, trs + (size_t)w * wfloats, lane);
-}
-
-__global__ void __launch_bounds__(32 * kTrWarps) k_batch_downward(const BTr *__restrict__ te, int ne, int64_t total,
-                                                                   int wfloats) {
-  extern __shared__ __align__(16) float trs[];
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const int64_t g = (int64_t)blockIdx.x * kTrWarps + w;
-  if (g >= total) return;
-  const BTr &t = te[find_entry(te, ne, g)];
-  downward_parent_warp<float, float>(t.Ef, t.m, t.k, t.rp, t.par0 + (g - t.g0), t.hat, trs + (size_t)w * wfloats,
-                                     lane);
+template <bool UP>
+__global__ void __launch_bounds__(512, 3) k_batch_transfer(const BTr *__restrict__ te, int ne) {
+  extern __shared__ __align__(16) unsigned char psm[];
+  __shared__ unsigned loc[16];
+  const BTr t = te[find_entry(te, ne, (int)blockIdx.x)];
+  const int bx = (int)blockIdx.x - t.cta0;
+  auto go = [&](auto order) {
+    constexpr int M = decltype(order)::value;
+    if (UP) up_pair<float, float, M>(t.Ef, t.rp, t.np, t.pp, t.par0, t.npar, t.hat, nullptr, bx, 0, psm, loc);
+    else down_pair<float, float, M>(t.Ef, t.rp, t.np, t.pp, t.par0, t.npar, t.hat, bx, 0, psm);
+  };
+  switch (t.m) {
+    case 1: return go(std::integral_constant<int, 1>{});
+    case 2: return go(std::integral_constant<int, 2>{});
+    case 3: return go(std::integral_constant<int, 3>{});
+    default: return go(std::integral_constant<int, 4>{});
+  }
 }
 
 // rows cut in chunks: out (+)= the partial sums of the chunk rows, in chunk order
@@ -443,34 +177,19 @@ __global__ void k_batch_permute_out(const BPerm *__restrict__ pp, int np, int64_
   }
 }
 
-int take_batch_error(cudaStream_t st) {
-  int v = 0, zero = 0;
-  H2_CUDA_TRY(cudaMemcpyFromSymbolAsync(&v, g_h2_device_error, sizeof(int), 0, cudaMemcpyDeviceToHost, st));
-  H2_CUDA_TRY(cudaStreamSynchronize(st));
-  if (v) {
-    H2_CUDA_TRY(cudaMemcpyToSymbolAsync(g_h2_device_error, &zero, sizeof(int), 0, cudaMemcpyHostToDevice, st));
-    H2_CUDA_TRY(cudaStreamSynchronize(st));
-    return fail(H2_ETIMEOUT, "a bounded device wait ran out; the last batched result is not valid");
-  }
-  return H2_OK;
-}
-
 constexpr int kRowPhases = 4;   // leaf forward, coupling, leaf backward, nearfield
 constexpr int64_t kChunkTerms = 24;   // rows with more terms are cut in chunks of this many terms
-constexpr int64_t kNoCap = (int64_t)1 << 62;
 constexpr int kPermThreads = 256;
 constexpr size_t kBatchSmemMax = 227 * 1024;
 
 // launch shapes of the block-row kernel the tuner chooses from
 struct Shape {
-  int wpb, nslot, zbytes;
+  int wpb, nst;   // warps per CTA, stages per warp
 };
-constexpr Shape kShapes[] = {
-    {4, 6, 8192}, {8, 6, 4096}, {8, 4, 6144}, {4, 6, 4096}, {12, 4, 4096}, {16, 3, 4096}, {6, 4, 8192}, {2, 8, 6144},
-};
+constexpr Shape kShapes[] = {{4, 2}, {8, 2}, {2, 2}, {1, 2}, {4, 3}, {2, 3}, {6, 2}, {6, 3}};
 constexpr int kNumShapes = sizeof(kShapes) / sizeof(kShapes[0]);
-
-size_t shape_smem(const Shape &s) { return (size_t)s.wpb * s.nslot * (s.zbytes + 8); }
+// the largest stage (a piece of 32 x 64 entries, 16 columns) fits every shape
+static_assert(6 * 3 * (32 * 64 * 4 + 32 * 16 * 4 + 16) <= 227 * 1024, "batched block-row stages");
 
 }  // namespace
 }  // namespace h2
@@ -495,9 +214,9 @@ struct h2_batch_s {
   // block-row phases
   std::vector<BRows> rows[kRowPhases];
   BRows *d_rows[kRowPhases] = {};
-  int64_t wtotal[kRowPhases] = {};
+  int64_t total[kRowPhases] = {};      // rows
+  uint32_t stage[kRowPhases] = {};     // bytes of the largest stage
   int shape[kRowPhases] = {0, 0, 0, 0};
-  int grid[kRowPhases] = {};
   // rows cut in chunks (coupling and nearfield): chunk bounds, partial sums, reductions
   int64_t *d_chunks[kRowPhases] = {};
   float *scratch[kRowPhases] = {};
@@ -505,9 +224,11 @@ struct h2_batch_s {
   int nred[kRowPhases] = {};
   // transfers: per step, entries (device arrays) and parents
   std::vector<BTr *> d_up, d_down;
-  std::vector<int> n_up, n_down;
-  std::vector<int64_t> tot_up, tot_down;
-  int tr_wfloats = 0;
+  struct Step {
+    int entries, ctas, threads;
+    size_t smem;
+  };
+  std::vector<Step> s_up, s_down;
   // permutations
   BPerm *d_perm_in = nullptr, *d_perm_out = nullptr;
   int64_t perm_total = 0;
@@ -528,62 +249,37 @@ struct h2_batch_s {
 namespace h2 {
 namespace {
 
-// work per term / row: bytes moved plus a fixed overhead
-void set_rows_shape(BRows &q, int zbytes) {
-  const int64_t tb = 4LL * q.K * (q.Mp + q.rp);
-  q.wterm = tb + 64;
-  q.wrow = 4LL * q.M * q.rp * (1 + q.accumulate) + 128;
-  if (tb <= zbytes) {
-    q.tps = (int)(zbytes / tb);
-    q.P = q.K;
-    q.ppt = 1;
-  } else {
-    q.tps = 0;
-    q.P = std::max(1, (int)(zbytes / (4LL * (q.Mp + q.rp))));
-    q.ppt = (q.K + q.P - 1) / q.P;
-  }
-}
-
+// shapes, row offsets and device copies of a phase's rows
 int upload_rows(h2_batch_s &b, int ph) {
-  const Shape &s = kShapes[b.shape[ph]];
-  // work prefix over the problems, from the host copies of the block lists
-  int64_t w = 0;
-  for (size_t p = 0; p < b.rows[ph].size(); ++p) {
-    BRows &q = b.rows[ph][p];
-    set_rows_shape(q, s.zbytes);
-    q.w0 = w;
-    if (q.pend) {   // chunk rows
-      q.wfix = kChunkTerms * q.wterm + q.wrow;
-      w += q.nrows * q.wfix;
-      continue;
-    }
-    const Plan &pl = b.probs[p].h->plan;
-    int64_t terms = q.nrows;
-    if (q.nrows > 0 && q.ptr) {
-      if (ph == 1) terms = pl.adm_ptr[q.row0 + q.nrows] - pl.adm_ptr[q.row0];
-      else terms = pl.near_ptr[q.nrows] - pl.near_ptr[0];
-    }
-    w += terms * q.wterm + q.nrows * q.wrow;
+  b.total[ph] = 0;
+  b.stage[ph] = 0;
+  for (BRows &q : b.rows[ph]) {
+    q.first = b.total[ph];
+    b.total[ph] += q.g.nrows;
+    q.t = LaneShape{};
+    lane_pieces(q.g, q.t);
+    q.tc = lane_columns(q.g.rp, q.t);
+    q.t.stage = lane_stage(q.g, sizeof(float), sizeof(float), q.t.xp, &q.t.xoff);
+    if (q.g.nrows > 0) b.stage[ph] = std::max(b.stage[ph], q.t.stage);
   }
-  b.wtotal[ph] = w;
+  if (b.rows[ph].empty()) return H2_OK;
   H2_CUDA_TRY(cudaMemcpy(b.d_rows[ph], b.rows[ph].data(), sizeof(BRows) * b.rows[ph].size(), cudaMemcpyHostToDevice));
-  // persistent grid: as many CTAs as stay resident
-  const size_t sm = shape_smem(s);
-  H2_CUDA_TRY(cudaFuncSetAttribute((const void *)k_batch_rows, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  H2_CUDA_TRY(cudaFuncSetAttribute((const void *)k_batch_rows<2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                    (int)kBatchSmemMax));
-  int per_sm = 0, sms = 0;
-  H2_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, b.device));
-  H2_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, (const void *)k_batch_rows, 32 * s.wpb, sm));
-  if (per_sm < 1) return fail(H2_EINVAL, "batched block-row kernel cannot be resident");
-  b.grid[ph] = per_sm * sms;
+  H2_CUDA_TRY(cudaFuncSetAttribute((const void *)k_batch_rows<3>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                   (int)kBatchSmemMax));
   return H2_OK;
 }
 
 void launch_rows_phase(h2_batch_s &b, int ph, cudaStream_t st) {
-  if (b.wtotal[ph] == 0) return;
+  if (b.total[ph] == 0) return;
   const Shape &s = kShapes[b.shape[ph]];
-  k_batch_rows<<<b.grid[ph], 32 * s.wpb, shape_smem(s), st>>>(b.d_rows[ph], (int)b.rows[ph].size(), b.wtotal[ph],
-                                                              s.nslot, s.zbytes);
+  const unsigned grid = (unsigned)((b.total[ph] + s.wpb - 1) / s.wpb);
+  const size_t sm = (size_t)s.wpb * s.nst * b.stage[ph];
+  if (s.nst == 2)
+    k_batch_rows<2><<<grid, 32 * s.wpb, sm, st>>>(b.d_rows[ph], (int)b.rows[ph].size(), b.total[ph], b.stage[ph]);
+  else
+    k_batch_rows<3><<<grid, 32 * s.wpb, sm, st>>>(b.d_rows[ph], (int)b.rows[ph].size(), b.total[ph], b.stage[ph]);
 }
 
 // enqueue one product on st; returns the number of kernel launches
@@ -599,26 +295,24 @@ int64_t enqueue(h2_batch_s &b, const float *x, float *y, cudaStream_t st, bool e
   k_batch_permute_in<<<pgrid, kPermThreads, 0, st>>>(b.d_perm_in, np, b.perm_total, x);
   ++nl;
   mark(H2_PH_LEAF_FORWARD);
-  if (b.wtotal[0]) launch_rows_phase(b, 0, st), ++nl;
-  const size_t trs = (size_t)kTrWarps * b.tr_wfloats * sizeof(float);
+  if (b.total[0]) launch_rows_phase(b, 0, st), ++nl;
   mark(H2_PH_UPWARD);
-  for (size_t s = 0; s < b.d_up.size(); ++s) {
-    k_batch_upward<<<(unsigned)((b.tot_up[s] + kTrWarps - 1) / kTrWarps), 32 * kTrWarps, trs, st>>>(
-        b.d_up[s], b.n_up[s], b.tot_up[s], b.tr_wfloats);
+  for (size_t i = 0; i < b.d_up.size(); ++i) {
+    k_batch_transfer<true><<<b.s_up[i].ctas, b.s_up[i].threads, b.s_up[i].smem, st>>>(b.d_up[i], b.s_up[i].entries);
     ++nl;
   }
   mark(H2_PH_COUPLING);
-  if (b.wtotal[1]) launch_rows_phase(b, 1, st), ++nl;
+  if (b.total[1]) launch_rows_phase(b, 1, st), ++nl;
   if (b.nred[1]) k_batch_reduce<<<b.nred[1], 128, 0, st>>>(b.d_red[1]), ++nl;
   mark(H2_PH_DOWNWARD);
-  for (size_t s = 0; s < b.d_down.size(); ++s) {
-    k_batch_downward<<<(unsigned)((b.tot_down[s] + kTrWarps - 1) / kTrWarps), 32 * kTrWarps, trs, st>>>(
-        b.d_down[s], b.n_down[s], b.tot_down[s], b.tr_wfloats);
+  for (size_t i = 0; i < b.d_down.size(); ++i) {
+    k_batch_transfer<false><<<b.s_down[i].ctas, b.s_down[i].threads, b.s_down[i].smem, st>>>(b.d_down[i],
+                                                                                            b.s_down[i].entries);
     ++nl;
   }
   mark(H2_PH_LEAF_NEAR);
-  if (b.wtotal[2]) launch_rows_phase(b, 2, st), ++nl;
-  if (b.wtotal[3]) launch_rows_phase(b, 3, st), ++nl;
+  if (b.total[2]) launch_rows_phase(b, 2, st), ++nl;
+  if (b.total[3]) launch_rows_phase(b, 3, st), ++nl;
   if (b.nred[3]) k_batch_reduce<<<b.nred[3], 128, 0, st>>>(b.d_red[3]), ++nl;
   mark(H2_PH_PERMUTE_OUT);
   k_batch_permute_out<<<pgrid, kPermThreads, 0, st>>>(b.d_perm_out, np, b.perm_total, y);
@@ -759,57 +453,36 @@ int h2_batch_create(const h2_handle *hs, int nprob, const int *nrhs, void *strea
     const int k = d.k, kp = d.kp, L = (int)d.lmax, Lp = (int)d.lp, rp = P.rp;
     const bool far = d.first_adm_level <= d.depth;
     const int64_t leaf0 = d.nleaf - 1, row0 = ((int64_t)1 << d.first_adm_level) - 1;
-    BRows z{};
-    z.rp = rp;
-    BRows &fw = b->rows[0][p];
-    fw = z;
-    fw.A = (const float *)d.V;
-    fw.a_stride = (int64_t)L * kp;
+    LaneRows &fw = b->rows[0][p].g;
+    fw.A = d.V;
     fw.X = P.xpad;
-    fw.x_stride = (int64_t)L * rp;
     fw.out = P.xhat + leaf0 * k * rp;
-    fw.out_stride = (int64_t)k * rp;
     fw.nrows = far ? d.nleaf : 0;
-    fw.M = k, fw.Mp = kp, fw.K = L;
-    BRows &cp = b->rows[1][p];
-    cp = z;
-    cp.A = (const float *)d.S;
-    cp.a_stride = (int64_t)k * kp;
+    fw.M = k, fw.Mp = kp, fw.K = L, fw.rp = rp;
+    LaneRows &cp = b->rows[1][p].g;
+    cp.A = d.S;
     cp.X = P.xhat;
-    cp.x_stride = (int64_t)k * rp;
-    cp.ptr = d.adm_ptr;
+    cp.ptr = d.adm_ptr + row0;
     cp.col = d.adm_col;
     cp.out = P.yhat + row0 * k * rp;
-    cp.out_stride = (int64_t)k * rp;
-    cp.row0 = row0;
     cp.nrows = far ? d.nclu - row0 : 0;
-    cp.M = k, cp.Mp = kp, cp.K = k;
-    BRows &bw = b->rows[2][p];
-    bw = z;
-    bw.A = (const float *)d.Vt;
-    bw.a_stride = (int64_t)k * Lp;
+    cp.M = k, cp.Mp = kp, cp.K = k, cp.rp = rp;
+    LaneRows &bw = b->rows[2][p].g;
+    bw.A = d.Vt;
     bw.X = P.yhat + leaf0 * k * rp;
-    bw.x_stride = (int64_t)k * rp;
     bw.out = P.ypad;
-    bw.out_stride = (int64_t)L * rp;
     bw.nrows = far ? d.nleaf : 0;
-    bw.M = L, bw.Mp = Lp, bw.K = k;
-    BRows &nr = b->rows[3][p];
-    nr = z;
-    nr.A = (const float *)d.near;
-    nr.a_stride = (int64_t)L * Lp;
+    bw.M = L, bw.Mp = Lp, bw.K = k, bw.rp = rp;
+    LaneRows &nr = b->rows[3][p].g;
+    nr.A = d.near;
     nr.X = P.xpad;
-    nr.x_stride = (int64_t)L * rp;
     nr.ptr = d.near_ptr;
     nr.col = d.near_col;
-    nr.out = P.ypad;
-    nr.out_stride = (int64_t)L * rp;
-    nr.nrows = d.nleaf;
-    nr.M = L, nr.Mp = Lp, nr.K = L;
     nr.accumulate = far ? 1 : 0;
+    nr.out = P.ypad;
+    nr.nrows = d.nleaf;
+    nr.M = L, nr.Mp = Lp, nr.K = L, nr.rp = rp;
     if (far) max_steps = std::max(max_steps, d.depth - d.first_adm_level);
-    b->tr_wfloats = std::max(b->tr_wfloats, (3 * k * rp + 6 * d.m * d.m + 3) / 4 * 4);
-    for (int ph = 0; ph < kRowPhases; ++ph) b->rows[ph][p].cap = kNoCap;
   }
 
   // rows of the coupling and the nearfield with more than kChunkTerms terms
@@ -819,13 +492,13 @@ int h2_batch_create(const h2_handle *hs, int nprob, const int *nrhs, void *strea
   for (int ph : {1, 3}) {
     std::vector<int64_t> cb, ce_;
     std::vector<BRed> red;
-    std::vector<BRows> extra;
+    std::vector<LaneRows> extra;
     for (int p = 0; p < nprob; ++p) {
-      BRows &q = b->rows[ph][p];
+      LaneRows &q = b->rows[ph][p].g;
       if (q.nrows == 0) continue;
       const Plan &pl = b->probs[p].h->plan;
-      const int64_t *hp = ph == 1 ? pl.adm_ptr.data() + q.row0 : pl.near_ptr.data();
-      BRows x = q;
+      const int64_t *hp = ph == 1 ? pl.adm_ptr.data() + (((int64_t)1 << pl.first_adm_level) - 1) : pl.near_ptr.data();
+      LaneRows x = q;
       x.nrows = 0;
       const int64_t first_chunk = (int64_t)cb.size();
       for (int64_t r = 0; r < q.nrows; ++r) {
@@ -833,7 +506,7 @@ int h2_batch_create(const h2_handle *hs, int nprob, const int *nrhs, void *strea
         if (nt <= kChunkTerms) continue;
         const int64_t nch = (nt - 1) / kChunkTerms;   // chunks beyond the first
         BRed rd{};
-        rd.out = q.out + r * q.out_stride;
+        rd.out = q.out + r * q.M * q.rp;
         rd.part = nullptr;   // set once the partial rows are allocated
         rd.nch = (int)nch;
         rd.len = q.M * q.rp;
@@ -847,11 +520,8 @@ int h2_batch_create(const h2_handle *hs, int nprob, const int *nrhs, void *strea
       if (x.nrows == 0) continue;
       q.cap = kChunkTerms;
       x.ptr = reinterpret_cast<const int64_t *>(first_chunk);   // rebased below
-      x.row0 = 0;
-      x.pend = nullptr;
       x.accumulate = 0;
-      x.out_stride = (int64_t)q.M * q.rp;
-      x.cap = kNoCap;
+      x.cap = kChunkTerms;
       extra.push_back(x);
     }
     if (extra.empty()) continue;
@@ -875,7 +545,7 @@ int h2_batch_create(const h2_handle *hs, int nprob, const int *nrhs, void *strea
     // rebase: chunk bounds and partial rows of each extra entry
     size_t ri = 0;
     for (size_t i = 0; i < extra.size(); ++i) {
-      BRows &x = extra[i];
+      LaneRows &x = extra[i];
       const int64_t c0 = reinterpret_cast<int64_t>(x.ptr);
       x.ptr = b->d_chunks[ph] + c0;
       x.pend = b->d_chunks[ph] + nc + c0;
@@ -887,7 +557,9 @@ int h2_batch_create(const h2_handle *hs, int nprob, const int *nrhs, void *strea
         row_in_entry += red[ri].nch;
         ++ri;
       }
-      b->rows[ph].push_back(x);
+      BRows br{};
+      br.g = x;
+      b->rows[ph].push_back(br);
     }
     if ((ce = cudaMemcpy(b->d_red[ph], red.data(), red.size() * sizeof(BRed), cudaMemcpyHostToDevice)) != cudaSuccess)
       return bail(cuda_fail(ce, "chunk reductions"));
@@ -904,7 +576,7 @@ int h2_batch_create(const h2_handle *hs, int nprob, const int *nrhs, void *strea
   for (int up = 0; up < 2; ++up) {
     for (int s = 0; s < max_steps; ++s) {
       std::vector<BTr> ent;
-      int64_t tot = 0;
+      h2_batch_s::Step step{0, 0, 32, 0};
       for (int p = 0; p < nprob; ++p) {
         const auto &P = b->probs[p];
         const Dev &d = P.h->d;
@@ -913,34 +585,28 @@ int h2_batch_create(const h2_handle *hs, int nprob, const int *nrhs, void *strea
         BTr t{};
         t.Ef = (const float *)d.Ef;
         t.hat = up ? P.xhat : P.yhat;
-        t.par0 = ((int64_t)1 << l) - 1;
-        t.g0 = tot;
+        t.npar = (int64_t)1 << l;
+        t.par0 = t.npar - 1;
+        t.cta0 = step.ctas;
         t.m = d.m;
-        t.k = d.k;
         t.rp = P.rp;
+        t.np = P.rp / 2;
+        t.pp = pair_parents(d.m, t.npar, t.np);
         ent.push_back(t);
-        tot += (int64_t)1 << l;
+        step.ctas += (int)((t.npar + t.pp - 1) / t.pp);
+        step.threads = std::max(step.threads, (t.pp * d.k * t.np + 31) / 32 * 32);
+        step.smem = std::max(step.smem, pair_smem<float>(d.m, t.np, t.pp, !up));
       }
+      step.entries = (int)ent.size();
       BTr *dp = nullptr;
       if ((ce = dmalloc((void **)&dp, sizeof(BTr) * ent.size())) != cudaSuccess)
         return bail(cuda_fail(ce, "transfer descriptors"));
       (up ? b->d_up : b->d_down).push_back(dp);
       if ((ce = cudaMemcpy(dp, ent.data(), sizeof(BTr) * ent.size(), cudaMemcpyHostToDevice)) != cudaSuccess)
         return bail(cuda_fail(ce, "transfer descriptors"));
-      (up ? b->n_up : b->n_down).push_back((int)ent.size());
-      (up ? b->tot_up : b->tot_down).push_back(tot);
+      (up ? b->s_up : b->s_down).push_back(step);
     }
   }
-  {
-    const int trs = kTrWarps * b->tr_wfloats * (int)sizeof(float);
-    if ((size_t)trs > kBatchSmemMax) return bail(fail(H2_EINVAL, "transfer work space does not fit in shared memory"));
-    if (trs > 48 * 1024) {   // one value for all batches (they may be created from several threads)
-      cudaFuncSetAttribute((const void *)k_batch_upward, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBatchSmemMax);
-      cudaFuncSetAttribute((const void *)k_batch_downward, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)kBatchSmemMax);
-    }
-  }
-
   // permutations
   std::vector<BPerm> pin(nprob), pout(nprob);
   int64_t e0 = 0;
@@ -1005,13 +671,11 @@ int h2_batch_tune(h2_batch b, int reps, int *choice) {
   H2_CUDA_TRY(cudaEventCreate(&t1));
   int rc = H2_OK;
   for (int ph = 0; ph < kRowPhases && !rc; ++ph) {
-    if (b->wtotal[ph] == 0) continue;
+    if (b->total[ph] == 0) continue;
     int best = b->shape[ph];
     float best_ms = 1e30f;
     for (int s = 0; s < kNumShapes && !rc; ++s) {
-      if (shape_smem(kShapes[s]) > kBatchSmemMax) continue;
       b->shape[ph] = s;
-      if ((rc = upload_rows(*b, ph))) break;
       launch_rows_phase(*b, ph, b->cap);   // warm-up
       cudaEventRecord(t0, b->cap);
       for (int i = 0; i < reps; ++i) launch_rows_phase(*b, ph, b->cap);
@@ -1029,13 +693,11 @@ int h2_batch_tune(h2_batch b, int reps, int *choice) {
       }
     }
     b->shape[ph] = best;
-    if (!rc) rc = upload_rows(*b, ph);
     // a phase that accumulates was run repeatedly: the next product rewrites it
   }
   cudaEventDestroy(t0);
   cudaEventDestroy(t1);
   if (rc) return rc;
-  if ((rc = take_batch_error(b->cap))) return rc;
   if (choice)
     for (int ph = 0; ph < kRowPhases; ++ph) choice[ph] = b->shape[ph];
   return H2_OK;
@@ -1044,15 +706,13 @@ int h2_batch_tune(h2_batch b, int reps, int *choice) {
 int h2_batch_set_shapes(h2_batch b, const int *choice) {
   if (!b || !choice) return fail(H2_EINVAL, "NULL argument");
   for (int ph = 0; ph < kRowPhases; ++ph)
-    if (choice[ph] < 0 || choice[ph] >= kNumShapes || shape_smem(kShapes[choice[ph]]) > kBatchSmemMax)
+    if (choice[ph] < 0 || choice[ph] >= kNumShapes)
       return fail(H2_EINVAL, "unknown launch shape");
   H2_CUDA_TRY(cudaSetDevice(b->device));
   H2_CUDA_TRY(cudaStreamSynchronize(b->stream));
   drop_graph(*b);
   for (int ph = 0; ph < kRowPhases; ++ph) {
     b->shape[ph] = choice[ph];
-    int rc = upload_rows(*b, ph);
-    if (rc) return rc;
   }
   return H2_OK;
 }
@@ -1069,17 +729,15 @@ int h2_batch_phase_times(h2_batch b, double *ms, int64_t *launches, int64_t *pro
   if (!b) return fail(H2_EINVAL, "NULL batch");
   H2_CUDA_TRY(cudaSetDevice(b->device));
   H2_CUDA_TRY(cudaStreamSynchronize(b->stream));
-  int rc = take_batch_error(b->cap);
-  if (rc) return rc;
   if (ms)
     for (int i = 0; i < H2_NPHASE; ++i) ms[i] = b->ms[i];
   if (launches) {
     launches[H2_PH_PERMUTE_IN] = 1;
-    launches[H2_PH_LEAF_FORWARD] = b->wtotal[0] ? 1 : 0;
+    launches[H2_PH_LEAF_FORWARD] = b->total[0] ? 1 : 0;
     launches[H2_PH_UPWARD] = (int64_t)b->d_up.size();
-    launches[H2_PH_COUPLING] = (b->wtotal[1] ? 1 : 0) + (b->nred[1] ? 1 : 0);
+    launches[H2_PH_COUPLING] = (b->total[1] ? 1 : 0) + (b->nred[1] ? 1 : 0);
     launches[H2_PH_DOWNWARD] = (int64_t)b->d_down.size();
-    launches[H2_PH_LEAF_NEAR] = (b->wtotal[2] ? 1 : 0) + (b->wtotal[3] ? 1 : 0) + (b->nred[3] ? 1 : 0);
+    launches[H2_PH_LEAF_NEAR] = (b->total[2] ? 1 : 0) + (b->total[3] ? 1 : 0) + (b->nred[3] ? 1 : 0);
     launches[H2_PH_PERMUTE_OUT] = 1;
   }
   if (products) *products = b->products;
@@ -1093,7 +751,7 @@ int h2_batch_info(h2_batch b, int64_t *info) {
   info[2] = b->dofs;
   info[3] = b->work_bytes;
   int64_t nl = 2 + (int64_t)b->d_up.size() + (int64_t)b->d_down.size();
-  for (int ph = 0; ph < kRowPhases; ++ph) nl += (b->wtotal[ph] ? 1 : 0) + (b->nred[ph] ? 1 : 0);
+  for (int ph = 0; ph < kRowPhases; ++ph) nl += (b->total[ph] ? 1 : 0) + (b->nred[ph] ? 1 : 0);
   info[4] = nl;
   for (int ph = 0; ph < kRowPhases; ++ph) info[5 + ph] = b->shape[ph];
   return H2_OK;
@@ -1103,7 +761,7 @@ int h2_batch_sync(h2_batch b) {
   if (!b) return fail(H2_EINVAL, "NULL batch");
   H2_CUDA_TRY(cudaSetDevice(b->device));
   H2_CUDA_TRY(cudaStreamSynchronize(b->stream));
-  return take_batch_error(b->cap);
+  return H2_OK;
 }
 
 int h2_batch_destroy(h2_batch b) {

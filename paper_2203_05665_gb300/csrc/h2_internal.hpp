@@ -313,7 +313,8 @@ int tc_leaf_forward(Ctx &c, void *xhat, int rp);
 
 // Block rows in FP32 arithmetic, one or four warps per row (h2_lane.cu): row r of
 // out ([row][M][rp]) is the sum of
-//   its blocks e = ptr[r] .. ptr[r + 1] - 1 (ptr NULL: block r): stored block
+//   its blocks e = ptr[r] .. ptr[r + 1] - 1 (pend given: pend[r] - 1; at most
+//   cap blocks; ptr NULL: block r): stored block
 //   blk[e] of A ([K][Mp], blk NULL: e) times item col[e] of X ([K][rp], col
 //   NULL: e), times scale[stored block];
 //   V_r ([kv][Mp], NULL: none) times item r of Y ([kv][rp]), times vscale[r];
@@ -322,12 +323,13 @@ int tc_leaf_forward(Ctx &c, void *xhat, int rp);
 struct LaneRows {
   const void *A, *V;
   const float *G, *X, *Y, *scale, *vscale;
-  const int64_t *ptr;
+  const int64_t *ptr, *pend;
   const int32_t *col, *blk;
   float *out;
-  int64_t nrows;
+  int64_t nrows, cap = (int64_t)1 << 40;
   int M, Mp, K, kv, rp;
   int longest;               // blocks of the longest row
+  int accumulate;            // out += instead of out =
 };
 int lane_rows(const LaneRows &g, int prec, bool v32, int64_t *launches, cudaStream_t st);
 constexpr int kLaneMax = 64;

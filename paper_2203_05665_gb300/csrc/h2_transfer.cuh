@@ -14,40 +14,7 @@
 namespace h2 {
 namespace {
 
-// One mode product of the factored transfer on a [k][rp] coefficient tensor
-// (nu = jx + m jy + m^2 jz): every thread owns one fibre along axis d for one
-// column, reads its m entries once and writes m results.
-//   trans: out[.., j, ..] = sum_{j'} F[j'][j] in[.., j', ..]   (E^T, upward)
-//   plain: out[.., j', ..] = sum_{j} F[j'][j] in[.., j, ..]    (E, downward)
 constexpr int kMaxM = 5;
-
-template <class T>
-__device__ __forceinline__ void mode_fibres(const T *F, const T *in, T *out, int m, int k, int rp, int d, bool trans,
-                                            int tid, int nthr) {
-  const int stride = d == 0 ? 1 : (d == 1 ? m : m * m);
-  const int items = (k / m) * rp;
-  for (int it = tid; it < items; it += nthr) {
-    const int c = it % rp, f = it / rp;
-    const int lo = f % stride, hi = f / stride;
-    const int base = lo + hi * stride * m;
-    T v[kMaxM];
-#pragma unroll
-    for (int i = 0; i < kMaxM; ++i)
-      if (i < m) v[i] = in[(base + i * stride) * rp + c];
-#pragma unroll
-    for (int j = 0; j < kMaxM; ++j) {
-      if (j >= m) break;
-      // double-float: the low word collects the exact errors of the m terms,
-      // one renormalisation per output
-      T acc = zero_of<T>();
-#pragma unroll
-      for (int i = 0; i < kMaxM; ++i)
-        if (i < m) acc_fma(acc, trans ? F[i * m + j] : F[j * m + i], v[i]);
-      acc_norm(acc);
-      out[(base + j * stride) * rp + c] = acc;
-    }
-  }
-}
 
 // storage -> compute conversion of a transfer factor
 template <class TC, class TS>
@@ -63,63 +30,6 @@ __device__ __forceinline__ float to_compute<float, __half>(__half v) {
   return __half2float(v);
 }
 
-// Steps of one parent by one warp (batched products): the warp's own shared
-// memory (3 k rp + 6 m^2 values of T), warp synchronisation only.
-//   upward (Algorithm 1): x^_p = sum over both children c of E_c^T x^_c
-//   downward (Algorithm 2): y^_c += E_c y^_parent for both children
-template <class TS, class T>
-__device__ __forceinline__ void upward_parent_warp(const TS *__restrict__ Ef, int m, int k, int rp, int64_t par,
-                                                   T *__restrict__ xhat, T *ws, int lane) {
-  const int kr = k * rp, mm = m * m;
-  T *a = ws;
-  T *b = a + kr;
-  T *acc = b + kr;
-  T *F = acc + kr;
-  for (int i = lane; i < 6 * mm; i += 32) F[i] = to_compute<T>(Ef[(2 * par + 1) * 3 * mm + i]);
-  for (int ch = 0; ch < 2; ++ch) {
-    const int64_t c = 2 * par + 1 + ch;
-    for (int i = lane; i < kr; i += 32) a[i] = xhat[c * kr + i];
-    __syncwarp();
-    const T *Fc = F + ch * 3 * mm;
-    mode_fibres(Fc, a, b, m, k, rp, 0, true, lane, 32);
-    __syncwarp();
-    mode_fibres(Fc + mm, b, a, m, k, rp, 1, true, lane, 32);
-    __syncwarp();
-    mode_fibres(Fc + 2 * mm, a, b, m, k, rp, 2, true, lane, 32);
-    __syncwarp();
-    for (int i = lane; i < kr; i += 32) acc[i] = ch == 0 ? b[i] : acc[i] + b[i];
-    __syncwarp();
-  }
-  for (int i = lane; i < kr; i += 32) xhat[par * kr + i] = acc[i];
-  __syncwarp();
-}
-
-template <class TS, class T>
-__device__ __forceinline__ void downward_parent_warp(const TS *__restrict__ Ef, int m, int k, int rp, int64_t par,
-                                                     T *__restrict__ yhat, T *ws, int lane) {
-  const int kr = k * rp, mm = m * m;
-  T *p = ws;
-  T *a = p + kr;
-  T *b = a + kr;
-  T *F = b + kr;
-  for (int i = lane; i < 6 * mm; i += 32) F[i] = to_compute<T>(Ef[(2 * par + 1) * 3 * mm + i]);
-  for (int i = lane; i < kr; i += 32) p[i] = yhat[par * kr + i];
-  __syncwarp();
-  for (int ch = 0; ch < 2; ++ch) {
-    const int64_t c = 2 * par + 1 + ch;
-    const T *Fc = F + ch * 3 * mm;
-    mode_fibres(Fc, p, a, m, k, rp, 0, false, lane, 32);
-    __syncwarp();
-    mode_fibres(Fc + mm, a, b, m, k, rp, 1, false, lane, 32);
-    __syncwarp();
-    mode_fibres(Fc + 2 * mm, b, a, m, k, rp, 2, false, lane, 32);
-    __syncwarp();
-    for (int i = lane; i < kr; i += 32) yhat[c * kr + i] = yhat[c * kr + i] + a[i];
-    __syncwarp();
-  }
-}
-
-
 // ---------------------------------------------------------------------------
 // Register transfer kernels for m = 3 and m = 4 (k = m^3): 64 threads per
 // parent and 16 columns (grid.y runs over groups of 16 columns), thread
@@ -127,10 +37,9 @@ __device__ __forceinline__ void downward_parent_warp(const TS *__restrict__ Ef, 
 // m = 3) holds the m x m slab nu = jx + m jy + m^2 jz of one column in
 // registers.  The x and y mode products run in registers, the z mode product
 // takes the slab entries of the threads of the column (adjacent lanes) by
-// warp shuffles.  Used for the wide upward levels in FP32 (launch_up_m).  Every output is formed exactly as in mode_fibres (m
-// multiply-adds, one renormalisation), in the same axis order, so the
-// results equal those of the shared-memory kernels above; the gain is that
-// no CTA-wide barrier separates the three mode products.
+// warp shuffles, so no barrier separates the three mode products.  Every output
+// is formed by m multiply-adds and one renormalisation, axes x, y, z in turn.
+// Used for the wide upward levels in FP32 (launch_up_m).
 constexpr int kRegParents = 4;   // parents per 256-thread CTA
 
 __device__ __forceinline__ float shfl_t(float v, int src) { return __shfl_sync(0xffffffffu, v, src); }
@@ -362,18 +271,19 @@ __device__ __forceinline__ void pair_factors(const TS *__restrict__ Ef, int64_t 
     F[i] = to_compute<T>(Ef[(2 * par + 1) * (3 * M * M) + i]);   // the children of consecutive parents are consecutive
 }
 
+// The bodies: CTA bx of the launch (or of its part of a batched launch), column
+// group by; psm: shared memory of pair_smem bytes, loc: 16 shared words.
 template <class TS, class T, int M>
-__global__ void __launch_bounds__(512, 3) k_up_pair(const TS *__restrict__ Ef, int rp, int np, int pp, int64_t par0,
-                                                    int64_t npar, T *__restrict__ xhat, unsigned *__restrict__ xmax) {
+__device__ __forceinline__ void up_pair(const TS *__restrict__ Ef, int rp, int np, int pp, int64_t par0, int64_t npar,
+                                        T *__restrict__ xhat, unsigned *__restrict__ xmax, int bx, int by,
+                                        unsigned char *psm, unsigned *loc) {
   constexpr int K = M * M * M;
-  extern __shared__ __align__(16) unsigned char psm[];
-  __shared__ unsigned loc[16];
   const int tpp = K * np, pl = (int)threadIdx.x / tpp, rem = (int)threadIdx.x - pl * tpp;
   Pair<T> *buf = reinterpret_cast<Pair<T> *>(psm);          // [2][pp][K][np]
   T *F = reinterpret_cast<T *>(buf + 2 * pp * tpp);         // [pp][2][3][M x M]
   if (threadIdx.x < 16) loc[threadIdx.x] = 0u;
-  const int64_t p0 = (int64_t)blockIdx.x * pp, par = par0 + p0 + pl;
-  const int nu = rem / np, p = rem - nu * np, col = 2 * (pair_max<M>() * (int)blockIdx.y + p);
+  const int64_t p0 = (int64_t)bx * pp, par = par0 + p0 + pl;
+  const int nu = rem / np, p = rem - nu * np, col = 2 * (pair_max<M>() * by + p);
   const int jx = nu % M, jy = (nu / M) % M, jz = nu / (M * M);
   const bool act = pl < pp && p0 + pl < npar && col < rp;
   Pair<T> v[2];
@@ -408,21 +318,28 @@ __global__ void __launch_bounds__(512, 3) k_up_pair(const TS *__restrict__ Ef, i
       atomicMax(&loc[2 * p + 1], __float_as_uint(mag_of(acc.b)));
     }
     __syncthreads();
-    unsigned *dst = xmax + 2 * pair_max<M>() * blockIdx.y + threadIdx.x;
+    unsigned *dst = xmax + 2 * pair_max<M>() * by + threadIdx.x;
     if (threadIdx.x < 16 && loc[threadIdx.x] && loc[threadIdx.x] > __ldcg(dst)) atomicMax(dst, loc[threadIdx.x]);
   }
 }
 
 template <class TS, class T, int M>
-__global__ void __launch_bounds__(512, 3) k_down_pair(const TS *__restrict__ Ef, int rp, int np, int pp, int64_t par0,
-                                                      int64_t npar, T *__restrict__ yhat) {
-  constexpr int K = M * M * M;
+__global__ void __launch_bounds__(512, 3) k_up_pair(const TS *__restrict__ Ef, int rp, int np, int pp, int64_t par0,
+                                                    int64_t npar, T *__restrict__ xhat, unsigned *__restrict__ xmax) {
   extern __shared__ __align__(16) unsigned char psm[];
+  __shared__ unsigned loc[16];
+  up_pair<TS, T, M>(Ef, rp, np, pp, par0, npar, xhat, xmax, (int)blockIdx.x, (int)blockIdx.y, psm, loc);
+}
+
+template <class TS, class T, int M>
+__device__ __forceinline__ void down_pair(const TS *__restrict__ Ef, int rp, int np, int pp, int64_t par0,
+                                          int64_t npar, T *__restrict__ yhat, int bx, int by, unsigned char *psm) {
+  constexpr int K = M * M * M;
   const int tpp = K * np, pl = (int)threadIdx.x / tpp, rem = (int)threadIdx.x - pl * tpp;
   Pair<T> *P = reinterpret_cast<Pair<T> *>(psm), *A = P + pp * tpp, *Bf = A + pp * tpp;   // [pp][K][np] each
   T *F = reinterpret_cast<T *>(Bf + pp * tpp);
-  const int64_t p0 = (int64_t)blockIdx.x * pp, par = par0 + p0 + pl;
-  const int nu = rem / np, p = rem - nu * np, col = 2 * (pair_max<M>() * (int)blockIdx.y + p);
+  const int64_t p0 = (int64_t)bx * pp, par = par0 + p0 + pl;
+  const int nu = rem / np, p = rem - nu * np, col = 2 * (pair_max<M>() * by + p);
   const int jx = nu % M, jy = (nu / M) % M, jz = nu / (M * M);
   const bool act = pl < pp && p0 + pl < npar && col < rp;
   const Pair<T> zero{zero_of<T>(), zero_of<T>()};
@@ -452,11 +369,23 @@ __global__ void __launch_bounds__(512, 3) k_down_pair(const TS *__restrict__ Ef,
   }
 }
 
+template <class TS, class T, int M>
+__global__ void __launch_bounds__(512, 3) k_down_pair(const TS *__restrict__ Ef, int rp, int np, int pp, int64_t par0,
+                                                      int64_t npar, T *__restrict__ yhat) {
+  extern __shared__ __align__(16) unsigned char psm[];
+  down_pair<TS, T, M>(Ef, rp, np, pp, par0, npar, yhat, (int)blockIdx.x, (int)blockIdx.y, psm);
+}
+
+// shared memory of a CTA: two (up) or three (down) tensors per parent and the factors
+template <class T>
+inline size_t pair_smem(int m, int np, int pp, bool down) {
+  return (size_t)pp * ((down ? 3 : 2) * m * m * m * np * sizeof(Pair<T>) + 6 * m * m * sizeof(T));
+}
+
 // parents of a CTA of the pair kernels: 512 threads on wide levels, fewer where
 // that leaves SMs without a CTA
-template <int M>
-inline int pair_parents(int64_t npar, int np) {
-  const int most = std::max(1, 512 / (M * M * M * np));
+inline int pair_parents(int m, int64_t npar, int np) {
+  const int most = std::max(1, 512 / (m * m * m * np));
   return (int)std::max<int64_t>(1, std::min<int64_t>(most, npar / (2 * 152)));
 }
 
@@ -477,9 +406,9 @@ inline bool pair_up(int m, int64_t npar, int rp) {
 template <class TS, class T, int M>
 void launch_up_m(const TS *Ef, int rp, int64_t par0, int64_t npar, T *xhat, unsigned *xmax, cudaStream_t st) {
   if (pair_up<T>(M, npar, rp)) {
-    const int np = std::min(pair_max<M>(), rp / 2), pp = pair_parents<M>(npar, np), thr = (pp * M * M * M * np + 31) / 32 * 32;
+    const int np = std::min(pair_max<M>(), rp / 2), pp = pair_parents(M, npar, np), thr = (pp * M * M * M * np + 31) / 32 * 32;
     const dim3 grid((unsigned)((npar + pp - 1) / pp), (rp / 2 + np - 1) / np);
-    k_up_pair<TS, T, M><<<grid, thr, pp * (2 * M * M * M * np * sizeof(Pair<T>) + 6 * M * M * sizeof(T)), st>>>(
+    k_up_pair<TS, T, M><<<grid, thr, pair_smem<T>(M, np, pp, false), st>>>(
         Ef, rp, np, pp, par0, npar, xhat, xmax);
     return;
   }
@@ -496,9 +425,9 @@ void launch_up_m(const TS *Ef, int rp, int64_t par0, int64_t npar, T *xhat, unsi
 
 template <class TS, class T, int M>
 void launch_down_m(const TS *Ef, int rp, int64_t par0, int64_t npar, T *yhat, cudaStream_t st) {
-  const int np = std::min(pair_max<M>(), rp / 2), pp = pair_parents<M>(npar, np), thr = (pp * M * M * M * np + 31) / 32 * 32;
+  const int np = std::min(pair_max<M>(), rp / 2), pp = pair_parents(M, npar, np), thr = (pp * M * M * M * np + 31) / 32 * 32;
   const dim3 grid((unsigned)((npar + pp - 1) / pp), (rp / 2 + np - 1) / np);
-  k_down_pair<TS, T, M><<<grid, thr, pp * (3 * M * M * M * np * sizeof(Pair<T>) + 6 * M * M * sizeof(T)), st>>>(
+  k_down_pair<TS, T, M><<<grid, thr, pair_smem<T>(M, np, pp, true), st>>>(
       Ef, rp, np, pp, par0, npar, yhat);
 }
 
