@@ -177,6 +177,185 @@ __global__ void k_residual(const double *__restrict__ b, const double *__restric
     r[e] = b[e] - Az[e];
 }
 
+// One Arnoldi step of a small system in one launch: classical Gram-Schmidt
+// applied twice against V_0 .. V_j, the norm, the next basis vector and the
+// Givens update of k_givens, by a cluster of 16 CTAs per column.  A thread keeps
+// its rows of w in registers; the dot products are reduced eight at a time
+// (transposed within a warp: nine FP64 additions instead of forty, FP64 being the
+// scarce unit), across the CTA in shared memory and across the cluster through
+// distributed shared memory, always in the same order.  The eleven launches it
+// replaces take 55 to 70 us per iteration whatever the size: 5,120 triangles,
+// one column, 138 us per iteration with the product, 107 us now.  Taken up to
+// 32,768 rows (16 rows per thread) and 9 columns (all clusters resident);
+// larger systems fill the GPU with the separate kernels.
+constexpr int kArnCtas = 16, kArnThreads = 128, kArnRows = 16, kArnVecs = 208;
+constexpr int64_t kArnMaxN = (int64_t)kArnCtas * kArnThreads * kArnRows;
+constexpr int kArnMaxCols = 9;
+
+__device__ __forceinline__ uint32_t cluster_rank() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.aligned;\n\tbarrier.cluster.wait.aligned;" ::: "memory");
+}
+// *p of CTA rank of the cluster
+__device__ __forceinline__ double ld_cluster(const double *p, uint32_t rank) {
+  uint32_t a = (uint32_t)__cvta_generic_to_shared(p), m;
+  double v;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(m) : "r"(a), "r"(rank));
+  asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v) : "r"(m) : "memory");
+  return v;
+}
+
+// s[0..7] of every lane summed over the warp: lane l returns sum (l >> 2)
+__device__ __forceinline__ double warp_sum8(double (&s)[8]) {
+  const int l = threadIdx.x & 31;
+#pragma unroll
+  for (int h = 4; h >= 1; h >>= 1) {   // lanes 4 h apart exchange h values
+    const bool up = l & (4 * h);
+#pragma unroll
+    for (int i = 0; i < h; ++i) {
+      const double give = up ? s[i] : s[i + h], keep = up ? s[i + h] : s[i];
+      s[i] = keep + __shfl_xor_sync(0xffffffffu, give, 4 * h);
+    }
+  }
+  double v = s[0];
+  v += __shfl_xor_sync(0xffffffffu, v, 2);
+  v += __shfl_xor_sync(0xffffffffu, v, 1);
+  return v;
+}
+
+__global__ void __launch_bounds__(kArnThreads) k_arnoldi(
+    double *__restrict__ Vb, const double *__restrict__ W, int64_t n, int nrhs, int j, int mr, double *__restrict__ H,
+    double *__restrict__ cs, double *__restrict__ sn, double *__restrict__ g, double *__restrict__ resid,
+    int *__restrict__ active, const double *__restrict__ tolv, const int *__restrict__ maxv, int *__restrict__ itc,
+    int *__restrict__ jc) {
+  __shared__ double red[kArnVecs][kArnThreads / 32], part[3][kArnVecs], hv[2][kArnVecs], nrm;
+  const int c = blockIdx.x / kArnCtas, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nv = j + 1;
+  const uint32_t q = cluster_rank();
+  const int64_t tot = n * nrhs, r0 = n * q / kArnCtas, r1 = n * (q + 1) / kArnCtas;
+  const double *V = Vb + (int64_t)c * n;
+  const int on = active[c];
+  double w[kArnRows];
+#pragma unroll
+  for (int k = 0; k < kArnRows; ++k) {
+    const int64_t r = r0 + tid + k * kArnThreads;
+    w[k] = r < r1 ? W[(int64_t)c * n + r] : 0.0;
+  }
+  for (int pass = 0; pass < 2; ++pass) {
+    for (int i0 = 0; i0 < nv; i0 += 8) {
+      double s[8];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) s[i] = 0.0;
+#pragma unroll
+      for (int k = 0; k < kArnRows; ++k) {
+        const int64_t r = r0 + tid + k * kArnThreads;
+        if (r0 + k * kArnThreads >= r1) break;
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+          if (i0 + i < nv && r < r1) s[i] = fma(V[(i0 + i) * tot + r], w[k], s[i]);
+      }
+      const double v = warp_sum8(s);
+      if ((lane & 3) == 0 && i0 + (lane >> 2) < nv) red[i0 + (lane >> 2)][warp] = v;
+    }
+    __syncthreads();
+    for (int i = tid; i < nv; i += kArnThreads) {
+      double v = red[i][0];
+#pragma unroll
+      for (int u = 1; u < kArnThreads / 32; ++u) v += red[i][u];
+      part[pass][i] = v;
+    }
+    cluster_sync();
+    for (int i = tid; i < nv; i += kArnThreads) {
+      double p[kArnCtas], v = 0.0;
+#pragma unroll
+      for (int u = 0; u < kArnCtas; ++u) p[u] = ld_cluster(&part[pass][i], u);
+#pragma unroll
+      for (int u = 0; u < kArnCtas; ++u) v += p[u];
+      hv[pass][i] = v;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < kArnRows; ++k) {
+      const int64_t r = r0 + tid + k * kArnThreads;
+      if (r0 + k * kArnThreads >= r1) break;
+      if (r < r1)
+        for (int i = 0; i < nv; ++i) w[k] -= hv[pass][i] * V[i * tot + r];
+    }
+  }
+  double s = 0.0;
+#pragma unroll
+  for (int k = 0; k < kArnRows; ++k) s = fma(w[k], w[k], s);
+  for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  if (lane == 0) red[0][warp] = s;
+  __syncthreads();
+  if (tid == 0) {
+    double v = red[0][0];
+    for (int u = 1; u < kArnThreads / 32; ++u) v += red[0][u];
+    part[2][0] = v;
+  }
+  cluster_sync();
+  if (tid == 0) {
+    double v = 0.0;
+    for (int u = 0; u < kArnCtas; ++u) v += ld_cluster(&part[2][0], u);
+    nrm = sqrt(v);
+  }
+  __syncthreads();
+  const double hn = nrm, inv = on && hn > 0.0 ? 1.0 / hn : 0.0;
+#pragma unroll
+  for (int k = 0; k < kArnRows; ++k) {
+    const int64_t r = r0 + tid + k * kArnThreads;
+    if (r < r1) Vb[(int64_t)(j + 1) * tot + (int64_t)c * n + r] = w[k] * inv;
+  }
+  // no CTA leaves while another may read its sums (and active[c] has been read by all)
+  cluster_sync();
+  if (q == 0 && tid == 0 && on) {
+    for (int i = 0; i <= j; ++i) hv[0][i] += hv[1][i];
+    for (int i = 0; i < j; ++i) {
+      const double a = hv[0][i], b = hv[0][i + 1], ci = cs[i * nrhs + c], si = sn[i * nrhs + c];
+      hv[0][i] = ci * a + si * b;
+      hv[0][i + 1] = -si * a + ci * b;
+    }
+    const double a = hv[0][j], b = hn, den = sqrt(a * a + b * b);
+    const double cj = den > 0 ? a / den : 1.0, sj = den > 0 ? b / den : 0.0;
+    cs[j * nrhs + c] = cj;
+    sn[j * nrhs + c] = sj;
+    hv[0][j] = cj * a + sj * b;
+    for (int i = 0; i <= j; ++i) H[((int64_t)i * mr + j) * nrhs + c] = hv[0][i];
+    H[((int64_t)(j + 1) * mr + j) * nrhs + c] = 0.0;
+    const double gj = g[j * nrhs + c], rc = fabs(sj * gj);
+    g[(j + 1) * nrhs + c] = -sj * gj;
+    g[j * nrhs + c] = cj * gj;
+    resid[c] = rc;
+    const int it = itc[c] + 1;
+    itc[c] = it;
+    jc[c] = j + 1;
+    if (rc <= tolv[c] || hn == 0.0 || it >= maxv[c]) active[c] = 0;
+  }
+}
+
+// launch configuration of k_arnoldi for nrhs columns; false where the step does not take it
+bool arnoldi_config(int64_t n, int nrhs, int mr, cudaStream_t st, cudaLaunchConfig_t &cfg, cudaLaunchAttribute &attr) {
+  if (n > kArnMaxN || nrhs > kArnMaxCols || mr > 200) return false;
+  attr.id = cudaLaunchAttributeClusterDimension;
+  attr.val.clusterDim.x = kArnCtas;
+  attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+  cfg = cudaLaunchConfig_t{};
+  cfg.gridDim = dim3((unsigned)(kArnCtas * nrhs));
+  cfg.blockDim = dim3(kArnThreads);
+  cfg.stream = st;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  int clusters = 0;
+  const bool ok = cudaFuncSetAttribute((const void *)k_arnoldi, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) ==
+                      cudaSuccess &&
+                  cudaOccupancyMaxActiveClusters(&clusters, (const void *)k_arnoldi, &cfg) == cudaSuccess && clusters > 0;
+  if (!ok) cudaGetLastError();
+  return ok;
+}
+
 int grid1(int64_t n) {
   int64_t g = (n + kT - 1) / kT;
   return (int)std::max<int64_t>(1, std::min<int64_t>(g, 152 * 16));
@@ -313,18 +492,26 @@ int gmres_cycle(const LinOp &op, GmresWork &w, const double *R, double *D, int n
   // stopped changes nothing (all its updates are masked by `active`).
   const int check = tot >= ((int64_t)1 << 20) ? 1 : 4;
   bool pending = false;
+  cudaLaunchConfig_t acfg;
+  cudaLaunchAttribute aattr;
+  const bool small = arnoldi_config(n, nrhs, mr, st, acfg, aattr);
   for (int j = 0; j < mr; ++j) {
     double *Vj = w.Vb + (int64_t)j * tot, *Vj1 = w.Vb + (int64_t)(j + 1) * tot;
     if ((rc = op.apply(Vj, w.W, nrhs))) return rc;
-    dots(w.Vb, w.W, n, nrhs, j + 1, w.h1, w.dpart, st);
-    k_orth<<<grid1(tot), kT, 0, st>>>(w.Vb, w.h1, j + 1, n, nrhs, w.W);
-    dots(w.Vb, w.W, n, nrhs, j + 1, w.h2, w.dpart, st);
-    k_orth<<<grid1(tot), kT, 0, st>>>(w.Vb, w.h2, j + 1, n, nrhs, w.W);
-    dots(w.W, w.W, n, nrhs, 1, w.hn, w.dpart, st);
-    k_sqrt<<<(nrhs + 63) / 64, 64, 0, st>>>(w.hn, nrhs);
-    launch_scale(w.W, w.hn, w.active, n, nrhs, Vj1, st);
-    k_givens<<<(nrhs + 63) / 64, 64, 0, st>>>(w.h1, w.h2, w.hn, j, mr, nrhs, w.H, w.cs, w.sn, w.g, w.resid,
-                                              w.active, w.tolv, w.maxv, w.itc, w.jc);
+    if (small) {
+      H2_CUDA_TRY(cudaLaunchKernelEx(&acfg, k_arnoldi, w.Vb, (const double *)w.W, n, nrhs, j, mr, w.H, w.cs, w.sn, w.g,
+                                     w.resid, w.active, (const double *)w.tolv, (const int *)w.maxv, w.itc, w.jc));
+    } else {
+      dots(w.Vb, w.W, n, nrhs, j + 1, w.h1, w.dpart, st);
+      k_orth<<<grid1(tot), kT, 0, st>>>(w.Vb, w.h1, j + 1, n, nrhs, w.W);
+      dots(w.Vb, w.W, n, nrhs, j + 1, w.h2, w.dpart, st);
+      k_orth<<<grid1(tot), kT, 0, st>>>(w.Vb, w.h2, j + 1, n, nrhs, w.W);
+      dots(w.W, w.W, n, nrhs, 1, w.hn, w.dpart, st);
+      k_sqrt<<<(nrhs + 63) / 64, 64, 0, st>>>(w.hn, nrhs);
+      launch_scale(w.W, w.hn, w.active, n, nrhs, Vj1, st);
+      k_givens<<<(nrhs + 63) / 64, 64, 0, st>>>(w.h1, w.h2, w.hn, j, mr, nrhs, w.H, w.cs, w.sn, w.g, w.resid,
+                                                w.active, w.tolv, w.maxv, w.itc, w.jc);
+    }
     H2_CUDA_TRY(cudaGetLastError());
     if (pending) {
       H2_CUDA_TRY(cudaEventSynchronize(w.ev));
