@@ -34,6 +34,7 @@
 
 #include "h2_internal.hpp"
 #include "h2_lane.cuh"
+#include "h2_launch.cuh"
 #include "h2_transfer.cuh"
 
 namespace h2 {
@@ -71,6 +72,8 @@ constexpr int kBatchMaxRp = 16;     // padded right-hand sides
 template <int NST>
 __global__ void __launch_bounds__(256) k_batch_rows(const BRows *__restrict__ pr, int np, int64_t total,
                                                     uint32_t stage) {
+  pdl_wait();
+  pdl_go();
   extern __shared__ __align__(16) unsigned char smem[];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int64_t row = (int64_t)blockIdx.x * (blockDim.x >> 5) + w;
@@ -126,6 +129,8 @@ struct BRed {
 };
 
 __global__ void k_batch_reduce(const BRed *__restrict__ rd) {
+  pdl_wait();
+  pdl_go();
   const BRed &q = rd[blockIdx.x];
   for (int i = threadIdx.x; i < q.len; i += blockDim.x) {
     float v = q.out[i];
@@ -148,6 +153,8 @@ __device__ __forceinline__ int perm_problem(const BPerm *__restrict__ pp, int np
 }
 
 __global__ void k_batch_permute_in(const BPerm *__restrict__ pp, int np, int64_t total, const float *__restrict__ x) {
+  pdl_wait();
+  pdl_go();
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= total) return;
@@ -163,6 +170,8 @@ __global__ void k_batch_permute_in(const BPerm *__restrict__ pp, int np, int64_t
 }
 
 __global__ void k_batch_permute_out(const BPerm *__restrict__ pp, int np, int64_t total, float *__restrict__ y) {
+  pdl_wait();
+  pdl_go();
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= total) return;
@@ -277,9 +286,9 @@ void launch_rows_phase(h2_batch_s &b, int ph, cudaStream_t st) {
   const unsigned grid = (unsigned)((b.total[ph] + s.wpb - 1) / s.wpb);
   const size_t sm = (size_t)s.wpb * s.nst * b.stage[ph];
   if (s.nst == 2)
-    k_batch_rows<2><<<grid, 32 * s.wpb, sm, st>>>(b.d_rows[ph], (int)b.rows[ph].size(), b.total[ph], b.stage[ph]);
+    pdl(k_batch_rows<2>, grid, 32 * s.wpb, sm, st, b.d_rows[ph], (int)b.rows[ph].size(), b.total[ph], b.stage[ph]);
   else
-    k_batch_rows<3><<<grid, 32 * s.wpb, sm, st>>>(b.d_rows[ph], (int)b.rows[ph].size(), b.total[ph], b.stage[ph]);
+    pdl(k_batch_rows<3>, grid, 32 * s.wpb, sm, st, b.d_rows[ph], (int)b.rows[ph].size(), b.total[ph], b.stage[ph]);
 }
 
 // enqueue one product on st; returns the number of kernel launches
@@ -292,30 +301,30 @@ int64_t enqueue(h2_batch_s &b, const float *x, float *y, cudaStream_t st, bool e
   };
   const int pgrid = (int)std::max<int64_t>(1, std::min<int64_t>((b.perm_total + kPermThreads - 1) / kPermThreads, 152 * 16));
   mark(H2_PH_PERMUTE_IN);
-  k_batch_permute_in<<<pgrid, kPermThreads, 0, st>>>(b.d_perm_in, np, b.perm_total, x);
+  pdl(k_batch_permute_in, pgrid, kPermThreads, 0, st, b.d_perm_in, np, b.perm_total, x);
   ++nl;
   mark(H2_PH_LEAF_FORWARD);
   if (b.total[0]) launch_rows_phase(b, 0, st), ++nl;
   mark(H2_PH_UPWARD);
   for (size_t i = 0; i < b.d_up.size(); ++i) {
-    k_batch_transfer<true><<<b.s_up[i].ctas, b.s_up[i].threads, b.s_up[i].smem, st>>>(b.d_up[i], b.s_up[i].entries);
+    pdl(k_batch_transfer<true>, b.s_up[i].ctas, b.s_up[i].threads, b.s_up[i].smem, st, b.d_up[i], b.s_up[i].entries);
     ++nl;
   }
   mark(H2_PH_COUPLING);
   if (b.total[1]) launch_rows_phase(b, 1, st), ++nl;
-  if (b.nred[1]) k_batch_reduce<<<b.nred[1], 128, 0, st>>>(b.d_red[1]), ++nl;
+  if (b.nred[1]) pdl(k_batch_reduce, b.nred[1], 128, 0, st, b.d_red[1]), ++nl;
   mark(H2_PH_DOWNWARD);
   for (size_t i = 0; i < b.d_down.size(); ++i) {
-    k_batch_transfer<false><<<b.s_down[i].ctas, b.s_down[i].threads, b.s_down[i].smem, st>>>(b.d_down[i],
+    pdl(k_batch_transfer<false>, b.s_down[i].ctas, b.s_down[i].threads, b.s_down[i].smem, st, b.d_down[i],
                                                                                             b.s_down[i].entries);
     ++nl;
   }
   mark(H2_PH_LEAF_NEAR);
   if (b.total[2]) launch_rows_phase(b, 2, st), ++nl;
   if (b.total[3]) launch_rows_phase(b, 3, st), ++nl;
-  if (b.nred[3]) k_batch_reduce<<<b.nred[3], 128, 0, st>>>(b.d_red[3]), ++nl;
+  if (b.nred[3]) pdl(k_batch_reduce, b.nred[3], 128, 0, st, b.d_red[3]), ++nl;
   mark(H2_PH_PERMUTE_OUT);
-  k_batch_permute_out<<<pgrid, kPermThreads, 0, st>>>(b.d_perm_out, np, b.perm_total, y);
+  pdl(k_batch_permute_out, pgrid, kPermThreads, 0, st, b.d_perm_out, np, b.perm_total, y);
   ++nl;
   mark(H2_NPHASE);
   return nl;

