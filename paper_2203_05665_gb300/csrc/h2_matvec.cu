@@ -977,31 +977,35 @@ int launch_rows(const Rows &rows, const RowCfg &cfg, int threads, int R, int64_t
 
 
 // Leaf steps (Algorithm 1 at the leaves, x^_t = V_t^T x|t; Algorithm 2 at the
-// leaves, y|t = V_t y^_t) for leaves of at most 32 triangles, k <= 64 and
-// rp <= 16: one CTA per leaf stages V_t (converted to the arithmetic type)
-// and the leaf's vector block in shared memory; in the forward step thread
+// leaves, y|t = V_t y^_t) for leaves of at most 32 triangles and k <= 64, up to
+// 16 columns (c0 .. c0 + nc - 1) per launch: one CTA per leaf stages V_t
+// (converted to the arithmetic type) and the leaf's vector block in shared
+// memory; in the forward step thread
 // (nu, jq) forms x^[nu][jq + 4u], in the backward step thread (r, jo) forms
 // y[r][jo + 8u], each as one contraction with a single renormalisation, then
 // multiplied by the leaf's power-of-two scale (16-bit storage) if there is
 // one; with MAX the forward step also takes the largest |x^| (|hi|) of every
-// column, as float bits.  The generic block-row kernel pipelines many terms per row; a leaf
-// row has one.
+// column, as float bits.  The generic block-row kernel pipelines many terms
+// per row; a leaf row has one (more than 16 columns took one block-row launch
+// before: 81,920 triangles, order 3, 32 columns, FP64-accurate: product 891 ->
+// 881 us with two passes here).
 template <class TS, class T, bool MAX>
 __global__ void __launch_bounds__(256) k_leaf_fwd_reg(const TS *__restrict__ V, const T *__restrict__ xpad,
                                                       const float *__restrict__ vscale, int L, int kp, int k, int rp,
-                                                      T *__restrict__ xleaf, unsigned *__restrict__ xmax) {
+                                                      int c0, int nc, T *__restrict__ xleaf,
+                                                      unsigned *__restrict__ xmax) {
   pdl_wait();
   pdl_go();
   extern __shared__ __align__(16) unsigned char lsm[];
   __shared__ unsigned smax[16];
   if (MAX && threadIdx.x < 16) smax[threadIdx.x] = 0u;
   T *Vs = reinterpret_cast<T *>(lsm);   // [L][kp]
-  T *xs = Vs + L * kp;                   // [L][rp]
+  T *xs = Vs + L * kp;                   // [L][nc]
   const int64_t t = blockIdx.x;
   const TS *vt = V + t * (int64_t)L * kp;
-  const T *xt = xpad + t * (int64_t)L * rp;
+  const T *xt = xpad + t * (int64_t)L * rp + c0;
   for (int i = threadIdx.x; i < L * kp; i += blockDim.x) Vs[i] = to_compute<T>(vt[i]);
-  for (int i = threadIdx.x; i < L * rp; i += blockDim.x) xs[i] = xt[i];
+  for (int i = threadIdx.x; i < L * nc; i += blockDim.x) xs[i] = xt[i / nc * rp + i % nc];
   __syncthreads();
   const int nu = threadIdx.x >> 2, jq = threadIdx.x & 3;
   if (nu < k) {
@@ -1012,15 +1016,15 @@ __global__ void __launch_bounds__(256) k_leaf_fwd_reg(const TS *__restrict__ V, 
       const T v = Vs[r * kp + nu];
 #pragma unroll
       for (int u = 0; u < 4; ++u)
-        if (jq + 4 * u < rp) acc_fma(acc[u], v, xs[r * rp + jq + 4 * u]);
+        if (jq + 4 * u < nc) acc_fma(acc[u], v, xs[r * nc + jq + 4 * u]);
     }
     const float sc = vscale ? vscale[t] : 1.0f;
 #pragma unroll
     for (int u = 0; u < 4; ++u)
-      if (jq + 4 * u < rp) {
+      if (jq + 4 * u < nc) {
         acc_norm(acc[u]);
         const T v = vscale ? acc[u] * from_double<T>(sc) : acc[u];
-        xleaf[(t * k + nu) * rp + jq + 4 * u] = v;
+        xleaf[(t * k + nu) * rp + c0 + jq + 4 * u] = v;
         if (MAX) atomicMax(&smax[jq + 4 * u], __float_as_uint(mag_of(v)));
       }
   }
@@ -1034,17 +1038,17 @@ __global__ void __launch_bounds__(256) k_leaf_fwd_reg(const TS *__restrict__ V, 
 template <class TS, class T>
 __global__ void __launch_bounds__(256) k_leaf_bwd_reg(const TS *__restrict__ Vt, const T *__restrict__ yleaf,
                                                       const float *__restrict__ vscale, int L, int Lp, int k, int rp,
-                                                      T *__restrict__ ypad) {
+                                                      int c0, int nc, T *__restrict__ ypad) {
   pdl_wait();
   pdl_go();
   extern __shared__ __align__(16) unsigned char lsm[];
   T *Vs = reinterpret_cast<T *>(lsm);   // [k][Lp]
-  T *ys = Vs + k * Lp;                   // [k][rp]
+  T *ys = Vs + k * Lp;                   // [k][nc]
   const int64_t t = blockIdx.x;
   const TS *vt = Vt + t * (int64_t)k * Lp;
-  const T *yt = yleaf + t * (int64_t)k * rp;
+  const T *yt = yleaf + t * (int64_t)k * rp + c0;
   for (int i = threadIdx.x; i < k * Lp; i += blockDim.x) Vs[i] = to_compute<T>(vt[i]);
-  for (int i = threadIdx.x; i < k * rp; i += blockDim.x) ys[i] = yt[i];
+  for (int i = threadIdx.x; i < k * nc; i += blockDim.x) ys[i] = yt[i / nc * rp + i % nc];
   __syncthreads();
   const int r = threadIdx.x >> 3, jo = threadIdx.x & 7;
   if (r >= L) return;
@@ -1053,14 +1057,14 @@ __global__ void __launch_bounds__(256) k_leaf_bwd_reg(const TS *__restrict__ Vt,
     const T w = Vs[nu * Lp + r];
 #pragma unroll
     for (int u = 0; u < 2; ++u)
-      if (jo + 8 * u < rp) acc_fma(acc[u], w, ys[nu * rp + jo + 8 * u]);
+      if (jo + 8 * u < nc) acc_fma(acc[u], w, ys[nu * nc + jo + 8 * u]);
   }
   const float sc = vscale ? vscale[t] : 1.0f;
 #pragma unroll
   for (int u = 0; u < 2; ++u)
-    if (jo + 8 * u < rp) {
+    if (jo + 8 * u < nc) {
       acc_norm(acc[u]);
-      ypad[(t * L + r) * rp + jo + 8 * u] = vscale ? acc[u] * from_double<T>(sc) : acc[u];
+      ypad[(t * L + r) * rp + c0 + jo + 8 * u] = vscale ? acc[u] * from_double<T>(sc) : acc[u];
     }
 }
 
@@ -1104,17 +1108,25 @@ int matvec_typed(Ctx &c, const Tio *x, Tio *y, int nrhs, bool acc) {
   // forward step from the input digits the nearfield reads anyway; the
   // permutation takes the input's column maxima on the way
   const bool near_tc = std::is_same<T, dd>::value && d.ntc;
-  const bool leaf_tc = near_tc && far && d.Vtc && rp <= 16;
+  // more than 8 columns: the digit tiles have 16 columns whatever the width (81,920
+  // triangles, one column: 54 us with the wide input digits, 37 us in double-float;
+  // 327,680 triangles, 16 columns: 217 us with the input digits that the nearfield
+  // needs as well, in double-float 215 us and 50 us for those digits)
+  const bool leaf_tc = near_tc && far && d.Vtc && rp > 8 && rp <= 16;
   // order-3 coupling on the tensor cores: the upward pass takes every level's column maxima
   const bool cpl_tile = std::is_same<T, dd>::value && far && d.tct;
   pdl(k_permute_in<Tio, T>, perm_grid, 256, (size_t)kPermRows * (rp + 1) * sizeof(T), st, 
       x, d.n, nrhs, rp, d.pad_src, d.npad, cmx, xpad, near_tc ? d.ntc_xmax : nullptr);
   mk.count(H2_PH_PERMUTE_IN);
   mk.mark(H2_PH_LEAF_FORWARD);
+  const bool tcpath = d.tc && rp <= 16 &&
+                      ((std::is_same<T, dd>::value && d.tc_nd == 10) ||
+                       (std::is_same<T, float>::value && std::is_same<TS, float>::value && d.tc_nd == 6));
+  bool leaf_max = leaf_tc;   // the leaf step takes its coefficients' column maxima
   // FP32 arithmetic, tiles of at most 64 rows: one or four warps per block row
   const bool lane = std::is_same<T, float>::value && L <= kLaneMax && k <= kLaneMax;
   // leaf steps with one CTA per leaf
-  const bool leaf_reg = L <= 32 && k <= 64 && rp <= 16;
+  const bool leaf_reg = L <= 32 && k <= 64;
   if (leaf_tc) {
     ntc_input(c, xpad, rp, 0, rp, true);
     if ((rc = tc_leaf_forward(c, xhat, rp))) return rc;
@@ -1134,15 +1146,19 @@ int matvec_typed(Ctx &c, const Tio *x, Tio *y, int nrhs, bool acc) {
     if ((rc = lane_rows(g, d.v32 ? (int)H2_F32 : d.prec, false, &nl, st))) return rc;
     mk.count(H2_PH_LEAF_FORWARD, nl);
   } else if (far && leaf_reg) {
-    const size_t sm = (size_t)L * (kp + rp) * sizeof(T);
     T *xl = xhat + leaf0 * (int64_t)k * rp;
-    if (cpl_tile)
-      pdl(k_leaf_fwd_reg<TV, T, true>, (unsigned)d.nleaf, 256, sm, st, (const TV *)d.V, xpad, vscale, L, kp, k, rp, xl,
-                                                                     d.tc_xmax + D * kLevelCols);
-    else
-      pdl(k_leaf_fwd_reg<TV, T, false>, (unsigned)d.nleaf, 256, sm, st, (const TV *)d.V, xpad, vscale, L, kp, k, rp,
-                                                                      xl, nullptr);
-    mk.count(H2_PH_LEAF_FORWARD);
+    leaf_max = cpl_tile || (std::is_same<T, dd>::value && tcpath && d.prec == H2_F64);
+    for (int c0 = 0; c0 < rp; c0 += 16) {
+      const int nc = std::min(16, rp - c0);
+      const size_t sm = (size_t)L * (kp + nc) * sizeof(T);
+      if (leaf_max)
+        pdl(k_leaf_fwd_reg<TV, T, true>, (unsigned)d.nleaf, 256, sm, st, (const TV *)d.V, xpad, vscale, L, kp, k, rp,
+            c0, nc, xl, d.tc_xmax + D * kLevelCols + c0);
+      else
+        pdl(k_leaf_fwd_reg<TV, T, false>, (unsigned)d.nleaf, 256, sm, st, (const TV *)d.V, xpad, vscale, L, kp, k, rp,
+            c0, nc, xl, nullptr);
+      mk.count(H2_PH_LEAF_FORWARD);
+    }
   } else if (far) {
     LeafForwardRows<TV, T> rows{(const TV *)d.V, xpad, vscale, L, kp, rp};
     if ((rc = launch_rows<TV, T>(rows, cf_fwd, t_fwd, Rk, d.nleaf, 0, xhat + leaf0 * (int64_t)k * rp, st))) return rc;
@@ -1153,13 +1169,10 @@ int matvec_typed(Ctx &c, const Tio *x, Tio *y, int nrhs, bool acc) {
     }
   }
   mk.mark(H2_PH_UPWARD);
-  const bool tcpath = d.tc && rp <= 16 &&
-                      ((std::is_same<T, dd>::value && d.tc_nd == 10) ||
-                       (std::is_same<T, float>::value && std::is_same<TS, float>::value && d.tc_nd == 6));
   if (far && tcpath) {
     // with the column maxima and coefficient slices of the tensor-core coupling
     int64_t nl = 0;
-    if ((rc = tc_upward(c, xhat, rp, &nl, leaf_tc))) return rc;
+    if ((rc = tc_upward(c, xhat, rp, &nl, leaf_max))) return rc;
     mk.count(H2_PH_UPWARD, nl);
   } else if (far) {
     for (int l = D - 1; l >= lmin; --l) {
@@ -1233,10 +1246,13 @@ int matvec_typed(Ctx &c, const Tio *x, Tio *y, int nrhs, bool acc) {
     // FP32 arithmetic: the leaf backward step, the FP32 self blocks of bfloat16 handles and the
     // nearfield as one sum per leaf row
   } else if (far && leaf_reg) {
-    const size_t sm = (size_t)k * (Lp + rp) * sizeof(T);
-    pdl(k_leaf_bwd_reg<TV, T>, (unsigned)d.nleaf, 256, sm, st, (const TV *)d.Vt, yhat + leaf0 * (int64_t)k * rp,
-                                                             vscale, L, Lp, k, rp, ypad);
-    mk.count(H2_PH_LEAF_NEAR);
+    for (int c0 = 0; c0 < rp; c0 += 16) {
+      const int nc = std::min(16, rp - c0);
+      const size_t sm = (size_t)k * (Lp + nc) * sizeof(T);
+      pdl(k_leaf_bwd_reg<TV, T>, (unsigned)d.nleaf, 256, sm, st, (const TV *)d.Vt, yhat + leaf0 * (int64_t)k * rp,
+          vscale, L, Lp, k, rp, c0, nc, ypad);
+      mk.count(H2_PH_LEAF_NEAR);
+    }
   } else if (far) {
     LeafBackwardRows<TV, T> rows{(const TV *)d.Vt, yhat, vscale, k, Lp, rp, leaf0};
     if ((rc = launch_rows<TV, T>(rows, cf_back, t_back, RL, d.nleaf, 0, ypad, st))) return rc;
@@ -1392,7 +1408,7 @@ int matvec_gca(Ctx &c, const Tio *x, Tio *y, int nrhs, bool acc) {
   if (far && leaf_reg) {
     const size_t sm = (size_t)L * (KD + rp) * sizeof(T);
     pdl(k_leaf_fwd_reg<TS, T, false>, (unsigned)d.nleaf, 256, sm, st, (const TS *)d.V, xpad, nullptr, L, KD, KD, rp,
-                                                             X(xhat, D), nullptr);
+        0, rp, X(xhat, D), nullptr);
     mk.count(H2_PH_LEAF_FORWARD);
   } else if (far) {
     LeafForwardRows<TS, T> rows{(const TS *)d.V, xpad, nullptr, L, KD, rp};
@@ -1427,8 +1443,8 @@ int matvec_gca(Ctx &c, const Tio *x, Tio *y, int nrhs, bool acc) {
   mk.mark(H2_PH_LEAF_NEAR);
   if (far && leaf_reg) {
     const size_t sm = (size_t)KD * (Lp + rp) * sizeof(T);
-    pdl(k_leaf_bwd_reg<TS, T>, (unsigned)d.nleaf, 256, sm, st, (const TS *)d.Vt, X(yhat, D), nullptr, L, Lp, KD, rp,
-                                                             ypad);
+    pdl(k_leaf_bwd_reg<TS, T>, (unsigned)d.nleaf, 256, sm, st, (const TS *)d.Vt, X(yhat, D), nullptr, L, Lp, KD, rp, 0,
+        rp, ypad);
     mk.count(H2_PH_LEAF_NEAR);
   } else if (far) {
     LeafBackwardRows<TS, T> rows{(const TS *)d.Vt, X(yhat, D), nullptr, KD, Lp, rp, 0};

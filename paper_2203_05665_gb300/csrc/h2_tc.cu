@@ -79,25 +79,31 @@ constexpr uint32_t kSliceA = kTcK * kTcK;              // 4096 bytes: one digit 
 // 2^29, pairs i + k <= 7: the dropped pairs stay below 2^-27 of the row's
 // scale).  Group g pairs S digits 2g+1 (accumulator lanes 0-63) and 2g+2
 // (lanes 64-127) with x^ digits k = 1 .. ND - 2g (N = 16 (ND - 2g)) and
-// writes them from accumulator column 32 g on: x^ digit k of group g lands in
+// writes them from accumulator column 2 W g on: x^ digit k of group g lands in
 // column block 2g + k - 1, so column block c holds, in lanes 0-63, the sum of
 // every pair of level i + k = c + 2 and, in lanes 64-127, of level c + 3.  The
 // tensor cores thus add the pairs of one level themselves (exactly: at most
-// five sums of at most 2^20 each), an accumulator set is 16 ND columns wide
-// (160 or 96) and kSets sets rotate, so that the MMAs of the next row segment
+// five sums of at most 2^20 each), an accumulator set is W ND columns wide
+// (160 or 96 for W = 16) and kSets sets rotate, so that the MMAs of the next row segment
 // run while the epilogue reads the previous one.
 //
 // KB is the contraction length of one block in bytes: 64 for the coupling
 // matrices (two MMA K steps), 32 for the leaf bases V_t^T of the leaf forward
 // step (the L <= 32 triangles of a leaf, zero padded; one K step).
-template <int ND, int KB = kTcK>
+//
+// W is the columns of a product the tiles are laid out for: 16, or 8 for up to
+// 8 right-hand sides of the coupling (half the coefficient digits, accumulator
+// columns and epilogue arithmetic).  FP64-accurate, 81,920 triangles, with the leaf
+// forward step in double-float and narrow nearfield tiles at these widths: one
+// column 705 -> 648 us, Helmholtz with 8 real columns 1,651 -> 1,559 us.
+template <int ND, int KB = kTcK, int W = kTcN>
 struct Dig {
   static constexpr int kFix = 5 * ND - 1;
   static constexpr int kTop = ND + 1;
   static constexpr int kGroups = ND / 2;
   static constexpr int kKSteps = KB / 32;
   static constexpr uint32_t kPlaneA = kTcK * KB;   // one digit plane of a block: 64 rows x KB
-  static constexpr uint32_t kPlaneB = kTcN * KB;   // one digit plane of the coefficients: 16 rows x KB
+  static constexpr uint32_t kPlaneB = W * KB;      // one digit plane of the coefficients: W rows x KB
   static constexpr uint32_t kTileA = ND * kPlaneA;
   static constexpr uint32_t kTileB = ND * kPlaneB;
   static constexpr uint32_t kStage = kTileA + kTileB;
@@ -106,10 +112,10 @@ struct Dig {
   // coupling: FP32, 327,680 triangles, 16 right-hand sides 1,457 us, per two 1,415 us;
   // one-block rows wait for every block's results anyway)
   static constexpr int kRel = KB == kTcK ? 2 : 1;
-  static constexpr uint32_t kW = kTcN * ND;      // columns of an accumulator set
+  static constexpr uint32_t kW = W * ND;         // columns of an accumulator set
   static constexpr int kSets = 3;   // one per epilogue group
   __host__ __device__ static constexpr int nx(int g) { return ND - 2 * g; }
-  __host__ __device__ static constexpr uint32_t col(int g) { return (uint32_t)(2 * kTcN * g); }
+  __host__ __device__ static constexpr uint32_t col(int g) { return (uint32_t)(2 * W * g); }
 };
 static_assert(Dig<10>::kSets * Dig<10>::kW <= 512 && Dig<6>::kSets * Dig<6>::kW <= 512, "accumulator sets");
 // epilogue warp groups, one per accumulator set (one group for all three sets held up
@@ -117,14 +123,13 @@ static_assert(Dig<10>::kSets * Dig<10>::kW <= 512 && Dig<6>::kSets * Dig<6>::kW 
 // right-hand sides took 2,018 instead of 2,118 us)
 constexpr int kRowGroups = 3;
 constexpr int kTcThreads = 64 + kRowGroups * 128;   // producer, MMA, epilogue warps
-constexpr uint32_t kXch = 64 * kTcN * 8; // epilogue exchange: 64 rows x 16 double-float values
-// EG: epilogue warp groups, each with its own exchange area
-template <int ND, int KB = kTcK, int EG = kRowGroups>
+// each epilogue group has an exchange area of 64 rows x W double-float values
+template <int ND, int KB = kTcK, int W = kTcN>
 __host__ __device__ constexpr uint32_t tc_bar_off() {
-  return Dig<ND, KB>::kStages * Dig<ND, KB>::kStage + EG * kXch;
+  return Dig<ND, KB, W>::kStages * Dig<ND, KB, W>::kStage + kRowGroups * (64 * W * 8);
 }
-template <int ND, int KB = kTcK, int EG = kRowGroups>
-__host__ __device__ constexpr uint32_t tc_smem() { return tc_bar_off<ND, KB, EG>() + 40 * 8 + 16; }
+template <int ND, int KB = kTcK, int W = kTcN>
+__host__ __device__ constexpr uint32_t tc_smem() { return tc_bar_off<ND, KB, W>() + 40 * 8 + 16; }
 
 // byte offset of (row r, contraction index c) in a K-major one-byte operand
 // of 64 contraction values per row: core matrices of 8 rows x 16 bytes, four
@@ -240,18 +245,18 @@ __global__ void k_tc_levmax(const T *__restrict__ x, int64_t rows, int rp, unsig
 
 // The ND E4M3 digit planes of the coefficients x^_c ([64][rp]) of clusters
 // c0 .. c0 + ncl - 1, each with the column maxima of its own tree level:
-// 64 threads per cluster (four per CTA), thread (g, j) cuts the values
+// 4 W threads per cluster (64 / W per CTA), thread (g, j) cuts the values
 // mu = 16 g .. 16 g + 15 of column j in registers and writes one 16-byte row
 // of a core matrix per plane (zero digits for the columns j >= rp).
-template <class T, int ND>
+template <class T, int ND, int W>
 __global__ void __launch_bounds__(256) k_tc_slice_x(const T *__restrict__ xhat, int64_t c0, int64_t ncl, int rp,
                                                     const unsigned *__restrict__ xmax, unsigned char *__restrict__ xtc) {
   pdl_wait();
   pdl_go();
-  const int64_t ci = (int64_t)blockIdx.x * 4 + (threadIdx.x >> 6);
+  const int64_t ci = (int64_t)blockIdx.x * (64 / W) + threadIdx.x / (4 * W);
   if (ci >= ncl) return;
   const int64_t c = c0 + ci;
-  const int g = (threadIdx.x >> 4) & 3, j = threadIdx.x & 15;
+  const int g = (threadIdx.x / W) & 3, j = threadIdx.x % W;
   const T *xc = xhat + c * kTcK * rp;
   const int sc = Dig<ND>::kFix - tc_colexp(xmax[tc_level(c) * kXmaxCols + j]);
   T v[16];
@@ -259,9 +264,9 @@ __global__ void __launch_bounds__(256) k_tc_slice_x(const T *__restrict__ xhat, 
   for (int q = 0; q < 16; ++q) v[q] = j < rp ? xc[(16 * g + q) * rp + j] : T{};
   uint4 w[ND];
   cut_row16<ND>(v, sc, w);
-  unsigned char *dst = xtc + c * (int64_t)Dig<ND>::kTileB + core_off(j, 16 * g);
+  unsigned char *dst = xtc + c * (int64_t)Dig<ND, kTcK, W>::kTileB + core_off(j, 16 * g);
 #pragma unroll
-  for (int i = 0; i < ND; ++i) *reinterpret_cast<uint4 *>(dst + i * Dig<ND>::kPlaneB) = w[i];
+  for (int i = 0; i < ND; ++i) *reinterpret_cast<uint4 *>(dst + i * Dig<ND, kTcK, W>::kPlaneB) = w[i];
 }
 
 // The coupling kernel (see the top of the file).  Rows t = row0 + r for r
@@ -283,13 +288,14 @@ __device__ __forceinline__ dd to_dd(float v) { return dd{v, 0.0f}; }
 __device__ __forceinline__ void store_as(dd v, dd *p) { *p = v; }
 __device__ __forceinline__ void store_as(dd v, float *p) { *p = v.hi + v.lo; }
 
-template <int ND, class T, int KB = kTcK, bool DIAG = false>
+template <int ND, class T, int KB = kTcK, bool DIAG = false, int W = kTcN>
 __global__ void __launch_bounds__(kTcThreads, 1)
     k_coupling_tc(const unsigned char *__restrict__ Stc, const unsigned char *__restrict__ xtc,
                   const int64_t *__restrict__ ptr, const int32_t *__restrict__ col, const int32_t *__restrict__ row,
                   const int32_t *__restrict__ split, const int32_t *__restrict__ E, const unsigned *__restrict__ xmax,
-                  int64_t row0, int64_t nrows, int rp, T *__restrict__ yhat, unsigned *__restrict__ ymax = nullptr, uint32_t xstride = Dig<ND, KB>::kTileB) {
-  using D = Dig<ND, KB>;
+                  int64_t row0, int64_t nrows, int rp, T *__restrict__ yhat, unsigned *__restrict__ ymax, uint32_t xstride) {
+  using D = Dig<ND, KB, W>;
+  static_assert(!DIAG || W == kTcN, "one-block rows read tiles of 16 columns");
   // first block of scheduled row r; one block per row without ptr
   auto pt = [&](int64_t r) -> int64_t { return DIAG ? r : ptr[r]; };
   constexpr int kTcStages = D::kStages, kTcGroups = D::kGroups;
@@ -297,7 +303,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
   extern __shared__ __align__(1024) unsigned char smem[];
   dd *xch = reinterpret_cast<dd *>(smem + kTcStages * kStage);
   constexpr int kSets = D::kSets;
-  uint64_t *full = reinterpret_cast<uint64_t *>(smem + tc_bar_off<ND, KB, kRowGroups>());
+  uint64_t *full = reinterpret_cast<uint64_t *>(smem + tc_bar_off<ND, KB, W>());
   uint64_t *empty = full + kTcStages;
   uint64_t *accf = empty + kTcStages;   // [kSets]: the MMAs of a segment have completed
   uint64_t *acce = accf + kSets;        // [kSets]: the epilogue has read the set
@@ -422,7 +428,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
 #pragma unroll
               for (int g = 0; g < kTcGroups; ++g)
                 tc_mma(dset + D::col(g), dA + (uint64_t)((2 * g * D::kPlaneA + kk * 256) >> 4),
-                       dB + (uint64_t)(kk * 16), tc_idesc(kTcN * D::nx(g)), (t > 0 || kk > 0 || g > 0) ? 1u : 0u);
+                       dB + (uint64_t)(kk * 16), tc_idesc(W * D::nx(g)), (t > 0 || kk > 0 || g > 0) ? 1u : 0u);
             // the stages of a release group are free once these MMAs have read them
             if (s % D::kRel == D::kRel - 1) tc_commit(&empty[s / D::kRel]);
             if (++s == kTcStages) {
@@ -524,7 +530,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     // turn, each with its own accumulator set
     const int grp = (warp - 2) >> 2;
     const int quad = warp & 3, tl = quad * 32 + lane, half = tl >> 6, nu = tl & 63;
-    dd *xg = xch + grp * (64 * kTcN);
+    dd *xg = xch + grp * (64 * W);
     const uint32_t bar_or = 1 + 2 * grp, bar_x = 2 + 2 * grp;
     uint32_t use = 0;
     int turn = kSets - 1;
@@ -545,9 +551,9 @@ __global__ void __launch_bounds__(kTcThreads, 1)
       if (turn != grp) continue;
       const int Er = E[t * kTcK + nu];
       const int lvl = tc_level(t);
-      int Fc[kTcN];
+      int Fc[W];
 #pragma unroll
-      for (int j = 0; j < kTcN; ++j) Fc[j] = Er + tc_colexp(xmax[lvl * kXmaxCols + j]);
+      for (int j = 0; j < W; ++j) Fc[j] = Er + tc_colexp(xmax[lvl * kXmaxCols + j]);
       bool stop = false;
       for (int64_t s0 = 0; s0 < nb; s0 += kTcSegBlocks, ++use) {
         const int set = grp;
@@ -557,9 +563,9 @@ __global__ void __launch_bounds__(kTcThreads, 1)
           break;
         }
         tc_fence_after();
-        dd acc[kTcN];
+        dd acc[W];
 #pragma unroll
-        for (int j = 0; j < kTcN; ++j) acc[j] = dd{0.0f, 0.0f};
+        for (int j = 0; j < W; ++j) acc[j] = dd{0.0f, 0.0f};
         // column block c of lane nu (+ 64) holds the sum of every digit pair of level
         // L = c + 2 (+ 1) (integers, exact in FP32); the levels share the weight
         // 2^(2-5L) and enter the double-float result once each, in increasing order
@@ -567,10 +573,10 @@ __global__ void __launch_bounds__(kTcThreads, 1)
         const uint32_t tset = tbase + ((uint32_t)(quad * 32) << 16) + (uint32_t)set * D::kW;
 #pragma unroll
         for (int c0 = 0; c0 < ND; c0 += 4) {
-          uint32_t raw[4][16];
+          uint32_t raw[4 * W / 16][16];   // four column blocks
 #pragma unroll
-          for (int u = 0; u < 4; ++u)
-            if (c0 + u < ND) tmem_ld16_nw(tset + (uint32_t)((c0 + u) * kTcN), raw[u]);
+          for (int u = 0; u < 4 * W / 16; ++u)
+            if (c0 * W + 16 * u < ND * W) tmem_ld16_nw(tset + (uint32_t)(c0 * W + 16 * u), raw[u]);
           tmem_wait();
 #pragma unroll
           for (int u = 0; u < 4; ++u) {
@@ -578,7 +584,8 @@ __global__ void __launch_bounds__(kTcThreads, 1)
             if (c0 + u < ND && L <= D::kTop) {
               const float w = pow2f(2 - 5 * L);
 #pragma unroll
-              for (int j = 0; j < kTcN; ++j) acc[j] = acc[j] + dd{__uint_as_float(raw[u][j]) * w, 0.0f};
+              for (int j = 0; j < W; ++j)
+                acc[j] = acc[j] + dd{__uint_as_float(raw[(u * W + j) >> 4][(u * W + j) & 15]) * w, 0.0f};
             }
           }
         }
@@ -587,11 +594,11 @@ __global__ void __launch_bounds__(kTcThreads, 1)
         if (lane == 0) mbar_arrive(&acce[set]);
         if (half == 1)
 #pragma unroll
-          for (int j = 0; j < kTcN; ++j) xg[j * 64 + nu] = acc[j];   // consecutive lanes, consecutive words
+          for (int j = 0; j < W; ++j) xg[j * 64 + nu] = acc[j];   // consecutive lanes, consecutive words
         named_sync_id(bar_x, 128);
         if (half == 0) {
 #pragma unroll
-          for (int j = 0; j < kTcN; ++j) {
+          for (int j = 0; j < W; ++j) {
             if (j >= rp) break;
             dd v = dd_scale(acc[j] + xg[j * 64 + nu], Fc[j]);
             if (s0 > 0) v = v + to_dd(yrow[j]);
@@ -732,28 +739,36 @@ int tc_upward_t(Ctx &c, T *xhat, int rp, int64_t *launches, bool leaf_max) {
   }
   // the digits of every level at once (all maxima are complete)
   const int64_t c0 = ((int64_t)1 << lmin) - 1, ncl = d.nclu - c0;
-  pdl(k_tc_slice_x<T, ND>, (unsigned)((ncl + 3) / 4), 256, 0, st, xhat, c0, ncl, rp, d.tc_xmax,
-                                                                 (unsigned char *)d.xtc);
+  if (rp <= 8)
+    pdl(k_tc_slice_x<T, ND, 8>, (unsigned)((ncl + 7) / 8), 256, 0, st, xhat, c0, ncl, rp, d.tc_xmax,
+        (unsigned char *)d.xtc);
+  else
+    pdl(k_tc_slice_x<T, ND, kTcN>, (unsigned)((ncl + 3) / 4), 256, 0, st, xhat, c0, ncl, rp, d.tc_xmax,
+        (unsigned char *)d.xtc);
   ++nl;
   H2_CUDA_TRY(cudaGetLastError());
   if (launches) *launches = nl;
   return H2_OK;
 }
 
-template <class T, int ND>
-int tc_coupling_t(Ctx &c, T *yhat, int rp) {
+template <class T, int ND, int W>
+int tc_coupling_w(Ctx &c, T *yhat, int rp) {
   Dev &d = c.d;
-  cudaStream_t st = c.stream;
   const int64_t row0 = ((int64_t)1 << d.first_adm_level) - 1, nrows = d.nclu - row0;
   if (nrows <= 0) return H2_OK;
-  static_assert(tc_smem<ND>() <= 227 * 1024, "tensor-core coupling does not fit in shared memory");
-  H2_CUDA_TRY(cudaFuncSetAttribute((const void *)k_coupling_tc<ND, T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                   (int)(227 * 1024)));
-  pdl(k_coupling_tc<ND, T>, d.tc_s.grid, kTcThreads, tc_smem<ND>(), st, 
+  static_assert(tc_smem<ND, kTcK, W>() <= 227 * 1024, "tensor-core coupling does not fit in shared memory");
+  H2_CUDA_TRY(cudaFuncSetAttribute((const void *)k_coupling_tc<ND, T, kTcK, false, W>,
+                                   cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(227 * 1024)));
+  pdl(k_coupling_tc<ND, T, kTcK, false, W>, d.tc_s.grid, kTcThreads, tc_smem<ND, kTcK, W>(), c.stream,
       (const unsigned char *)d.Stc, (const unsigned char *)d.xtc, d.tc_s.ptr, d.tc_s.col, d.tc_s.row, d.tc_s.split,
-      d.tc_E, d.tc_xmax, row0, nrows, rp, yhat, nullptr, Dig<ND>::kTileB);
+      d.tc_E, d.tc_xmax, row0, nrows, rp, yhat, nullptr, Dig<ND, kTcK, W>::kTileB);
   H2_CUDA_TRY(cudaGetLastError());
   return H2_OK;
+}
+
+template <class T, int ND>
+int tc_coupling_t(Ctx &c, T *yhat, int rp) {
+  return rp <= 8 ? tc_coupling_w<T, ND, 8>(c, yhat, rp) : tc_coupling_w<T, ND, kTcN>(c, yhat, rp);
 }
 
 }  // namespace
@@ -804,7 +819,7 @@ int tc_leaf_forward(Ctx &c, void *xhat_v, int rp) {
   cudaStream_t st = c.stream;
   if (rp > kTcN || !d.Vtc) return fail(H2_EINVAL, "no tensor-core leaf forward step for this handle");
   constexpr int KB = 32;
-  constexpr uint32_t sm = tc_smem<kTcSlices, KB, kRowGroups>();
+  constexpr uint32_t sm = tc_smem<kTcSlices, KB>();
   static_assert(sm <= 227 * 1024, "tensor-core leaf step does not fit in shared memory");
   H2_CUDA_TRY(cudaFuncSetAttribute((const void *)k_coupling_tc<kTcSlices, dd, KB, true>,
                                    cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(227 * 1024)));

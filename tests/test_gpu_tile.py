@@ -96,3 +96,37 @@ def test_order3_coupling(require_gpu, mesh, leaf):
     h.matvec(xd, y2)
     assert torch.equal(y1, y2)
     h.close()
+
+
+@pytest.mark.parametrize("prec, tol", [("f64", 4e-13), ("f32", 1e-6)])
+@pytest.mark.parametrize("leaf", [20, 32])
+def test_order4_coupling_widths(require_gpu, prec, tol, leaf):
+    """Digit tiles of 8 and of 16 columns (up to 8 and up to 16 right-hand sides), with the leaf forward
+    step in double-float or on the tensor cores (leaves of at most 21 triangles, more than 8 columns).
+    The digit pairs left out stay below 2^-46 of a row's scale (FP64) and 2^-27 (FP32); a row's scale is
+    at most some 25 times its entries' typical size (1,280 triangles)."""
+    v, f = I.icosphere(3)
+    o = oracle.Oracle(v, f, leaf_size=leaf, eta=2.0, order=4)
+    h = H2Matrix(v, f, leaf_size=leaf, eta=2.0, order=4, prec=prec)
+    assert h.stats["tensor"] == 1
+    for nrhs in (1, 2, 3, 4, 5, 7, 8, 9, 12, 16):
+        x = I.uniform_rhs(f.shape[0], nrhs, 5400 + nrhs)
+        x[:, 0] *= 1e6
+        y, r = h.matvec_host(x), o.matvec(x)
+        for j in range(nrhs):
+            assert _rel(y[:, j], r[:, j]) <= tol, (nrhs, j)
+    h.close()
+
+
+def test_leaf_steps_in_column_passes(require_gpu):
+    """FP64 leaf steps in passes of 16 columns (leaves of at most 32 triangles), order 2 and 3, padded
+    and full last passes."""
+    v, f = _patch(1000)
+    for order, leaf in ((2, 32), (3, 17), (4, 32)):
+        o = oracle.Oracle(v, f, leaf_size=leaf, eta=2.0, order=order)
+        for prec in ("f64", "f64n"):
+            h = H2Matrix(v, f, leaf_size=leaf, eta=2.0, order=order, prec=prec)
+            for nrhs in (17, 31, 32) + ((33, 64) if order < 4 else ()):   # order 4 takes at most 32
+                x = I.uniform_rhs(1000, nrhs, 5500 + nrhs)
+                assert _rel(h.matvec_host(x), o.matvec(x)) <= (TOL if order < 4 else 4e-13), (order, prec, nrhs)
+            h.close()
