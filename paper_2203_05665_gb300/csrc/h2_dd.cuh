@@ -10,6 +10,8 @@
 // single-precision components).  Relative error per operation < 2^-44.
 #pragma once
 
+#include "h2_convert.hpp"
+
 namespace h2 {
 
 struct __align__(8) dd {
@@ -110,11 +112,13 @@ __device__ __forceinline__ To convert(From v) {
 }
 template <>
 __device__ __forceinline__ dd convert<dd, double>(double v) {
-  return dd_from_double(v);
+  dd r;
+  double_to_pair(v, r.hi, r.lo);
+  return r;
 }
 template <>
 __device__ __forceinline__ double convert<double, dd>(dd v) {
-  return dd_to_double(v);
+  return widen(v.hi) + widen(v.lo);
 }
 template <>
 __device__ __forceinline__ dd convert<dd, dd>(dd v) {

@@ -909,11 +909,6 @@ inline int row_threads(int Mp, int rp, int Kmax, size_t esize, int R) {
   return 256;
 }
 
-int grid_for(int64_t n) {
-  int64_t g = (n + kThreads - 1) / kThreads;
-  return (int)std::max<int64_t>(1, std::min<int64_t>(g, 152 * 32));
-}
-
 // Allow the kernel the largest dynamic shared memory once it needs more than
 // the default 48 KB.  Always the same value: products of different handles
 // run concurrently from several threads (serving), and a smaller limit set
