@@ -268,7 +268,7 @@ int upload_rows(h2_batch_s &b, int ph) {
     q.t = LaneShape{};
     lane_pieces(q.g, q.t);
     q.tc = lane_columns(q.g.rp, q.t);
-    q.t.stage = lane_stage(q.g, sizeof(float), sizeof(float), q.t.xp, &q.t.xoff);
+    q.t.stage = lane_stage(q.g, sizeof(float), sizeof(float), q.t.xp, 1, &q.t.xoff);
     if (q.g.nrows > 0) b.stage[ph] = std::max(b.stage[ph], q.t.stage);
   }
   if (b.rows[ph].empty()) return H2_OK;

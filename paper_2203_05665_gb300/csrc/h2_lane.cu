@@ -4,12 +4,13 @@
 // backward step, of FP32, bfloat16 and half handles with tiles of at most 64
 // rows.
 //
-// A row is a sequence of pieces of at most 32 contraction values.  The warp
-// copies the next piece (a tile A, stored [contraction][row], and the rows of X
-// it meets) into the other of its two shared-memory stages (cp.async) while it
-// multiplies the current one (deeper rings cost more in resident warps than
-// they hide: four stages 217 us, three 164, two 162 for the coupling below).  A lane owns a register tile of 4 output rows by
-// TC = 8 (4 for up to 4 columns) columns, two of them for large tiles; lanes
+// A row is a sequence of pieces of at most 32 contraction values (or of two
+// whole blocks).  The warp copies the next piece (a tile A, stored
+// [contraction][row], and the rows of X it meets) into the other of its two
+// shared-memory stages (cp.async) while it multiplies the current one (deeper
+// rings cost more in resident warps than they hide: four stages 217 us, three
+// 164, two 162 for the coupling below).  A lane owns a register tile of 4 output
+// rows by TC = 8 (4 for up to 4 columns) columns, two of them for large tiles; lanes
 // that are left take further slices of the contraction.  The tile shape is set
 // by the shared-memory return bandwidth (128 bytes per cycle and SM, also for
 // broadcasts): 12 words feed 32 multiply-adds (packed pairs, fma.rn.f32x2, each
@@ -27,10 +28,12 @@
 // 20 to 32 rows leave it bound by latency (16 to 25 % of the issue slots).
 // Before -> now: FP32, 81,920 triangles, order 3, 32 columns: coupling 308 ->
 // 149 us, leaf backward + nearfield 124 -> 85 us; FP32, 327,680, order 4, 16
-// columns: leaf forward 88 -> 44 us, leaf backward + nearfield 356 -> 174 us;
-// bfloat16, 1.3 M, order 3, 4 columns: leaf forward 158 -> 61 us, leaf backward +
-// nearfield 896 -> 359 us (bound by the instructions around the 20 x 20 pieces:
-// half of the issue slots at 24 warps per SM).
+// columns: leaf forward 88 -> 43 us, leaf backward + nearfield 356 -> 156 us;
+// bfloat16, 1.3 M, order 3, 4 columns: leaf forward 158 -> 62 us, leaf backward +
+// nearfield 896 -> 305 us (bound by the instructions around the 20 x 20 pieces:
+// half of the issue slots at 24 warps per SM).  The last two take two blocks per
+// piece, which spares half of the waits, copies' set-up and additions of pieces
+// (one block per piece: 178 and 347 us).
 #include <algorithm>
 
 #include "h2_internal.hpp"
@@ -41,6 +44,7 @@ namespace h2 {
 namespace {
 
 constexpr size_t kLaneSmemMax = 227 * 1024;
+constexpr size_t kLaneSmemAll = 220 * 1024;   // shared memory of an SM's CTAs (each takes 1 KB more)
 
 struct LaneArgs {
   LaneRows r;
@@ -48,31 +52,46 @@ struct LaneArgs {
   int wpr;                   // warps per row
 };
 
-template <class TS, class TV, int TC, int TPL>
-__global__ void __launch_bounds__(32 * kLaneWarps, TC == 4 ? 6 : TPL == 1 ? 4 : 2) k_lane_rows(const __grid_constant__ LaneArgs a) {
+// CTAs an SM holds
+constexpr int lane_ctas(int tc, int tpl) { return tc == 4 ? 6 : tpl == 1 ? 4 : 2; }
+
+template <class TS, class TV, int TC, int TPL, int BPP>
+__global__ void __launch_bounds__(32 * kLaneWarps, lane_ctas(TC, TPL)) k_lane_rows(const __grid_constant__ LaneArgs a) {
   pdl_wait();
   pdl_go();
   extern __shared__ __align__(16) unsigned char lsm[];
   const int w = threadIdx.x >> 5;
   const int64_t row = a.wpr == 1 ? (int64_t)blockIdx.x * kLaneWarps + w : (int64_t)blockIdx.x;
   if (row >= a.r.nrows) return;   // whole warps; with four warps per row every row exists
-  lane_row<TS, TV, TC, TPL, 2>(a.r, a.t, a.wpr, row, w, lsm + (size_t)w * 2 * a.t.stage, lsm);
+  lane_row<TS, TV, TC, TPL, 2, BPP>(a.r, a.t, a.wpr, row, w, lsm + (size_t)w * 2 * a.t.stage, lsm);
 }
 
-template <class TS, class TV, int TC, int TPL>
-int lane_launch(LaneArgs a, cudaStream_t st) {
+template <class TS, class TV, int TC, int TPL, int BPP>
+int lane_start(LaneArgs a, cudaStream_t st) {
   const LaneRows &g = a.r;
-  a.t.stage = lane_stage(g, sizeof(TS), sizeof(TV), a.t.xp, &a.t.xoff);
+  a.t.stage = lane_stage(g, sizeof(TS), sizeof(TV), a.t.xp, BPP, &a.t.xoff);
   const size_t sm = std::max<size_t>((size_t)kLaneWarps * 2 * a.t.stage,
                                      a.wpr > 1 ? (size_t)kLaneWarps * TPL * 4 * TC * 32 * sizeof(float) : 0);
   if (sm > kLaneSmemMax) return fail(H2_EINVAL, "block-row tile does not fit in shared memory");
   if (sm > 48 * 1024)
-    H2_CUDA_TRY(cudaFuncSetAttribute((const void *)k_lane_rows<TS, TV, TC, TPL>,
+    H2_CUDA_TRY(cudaFuncSetAttribute((const void *)k_lane_rows<TS, TV, TC, TPL, BPP>,
                                      cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kLaneSmemMax));
   const int64_t grid = a.wpr == 1 ? (g.nrows + kLaneWarps - 1) / kLaneWarps : g.nrows;
-  pdl(k_lane_rows<TS, TV, TC, TPL>, (unsigned)grid, 32 * kLaneWarps, sm, st, a);
+  pdl(k_lane_rows<TS, TV, TC, TPL, BPP>, (unsigned)grid, 32 * kLaneWarps, sm, st, a);
   H2_CUDA_TRY(cudaGetLastError());
   return H2_OK;
+}
+
+template <class TS, class TV, int TC, int TPL>
+int lane_launch(const LaneArgs &a, cudaStream_t st) {
+  // two blocks per piece where the rows have blocks (ptr) of at most kPiece contraction
+  // values and the larger stages leave the SM its CTAs (measured above; with 32 columns
+  // they would not, and one block per piece measured the same, 87 us)
+  uint32_t xoff;
+  const LaneRows &g = a.r;
+  const size_t stage2 = lane_stage(g, sizeof(TS), sizeof(TV), a.t.xp, 2, &xoff);
+  const bool two = g.ptr && a.t.ppb == 1 && lane_ctas(TC, TPL) * kLaneWarps * 2 * stage2 <= kLaneSmemAll;
+  return two ? lane_start<TS, TV, TC, TPL, 2>(a, st) : lane_start<TS, TV, TC, TPL, 1>(a, st);
 }
 
 template <class TS, class TV>

@@ -6,6 +6,7 @@
 #include <cuda_fp16.h>
 
 #include <cstdint>
+#include <type_traits>
 
 #include "h2_internal.hpp"
 #include "h2_ptx.cuh"
@@ -63,14 +64,15 @@ struct LaneShape {
 
 // Output row `row` of g by one warp (wpr = 1) or, as warp w, by four (wpr = 4,
 // all warps of the CTA; red: shared memory for their sums).  ring: the warp's NST
-// stages.
-template <class TS, class TV, int TC, int TPL, int NST>
+// stages.  BPP: whole blocks of a piece (more than one only for K <= kPiece, ppb = 1).
+template <class TS, class TV, int TC, int TPL, int NST, int BPP = 1>
 __device__ __forceinline__ void lane_row(const LaneRows &g, const LaneShape &a, int wpr, int64_t row, int w,
                                          unsigned char *ring, unsigned char *red_smem) {
   const int lane = threadIdx.x & 31;
   const int64_t e0 = g.ptr ? g.ptr[row] : row;
   const int64_t e1 = min(g.ptr ? (g.pend ? g.pend[row] : g.ptr[row + 1]) : row + 1, e0 + g.cap);
-  const int lead = a.vpieces + a.gpieces, np = lead + (int)(e1 - e0) * a.ppb;
+  const int nb = (int)(e1 - e0), lead = a.vpieces + a.gpieces;
+  const int np = lead + (BPP == 1 ? nb * a.ppb : (nb + BPP - 1) / BPP);
   const int first = wpr == 1 ? 0 : w, n = (np - first + wpr - 1) / wpr;
   const int M = g.M, Mp = g.Mp, K = g.K, rp = g.rp, xp = a.xp;
 
@@ -89,6 +91,21 @@ __device__ __forceinline__ void lane_row(const LaneRows &g, const LaneShape &a, 
   };
   batch(0);
 
+  // copies of kc rows of A (ab bytes) and of X as block u of stage st
+  auto copy = [&](unsigned char *st, int u, const unsigned char *src, uint32_t ab, const float *x, int kc) {
+    unsigned char *sa = st + u * ab;
+    for (uint32_t o = 16u * lane; o < ab; o += 512u) cp_async16(sa + o, src + o);
+    float *sx = reinterpret_cast<float *>(st + a.xoff) + u * kc * xp;
+    if (rp == xp) {
+      for (int o = 4 * lane; o < kc * xp; o += 128) cp_async16(sx + o, x + o);
+    } else {
+      const int c4 = a.ncol / 4;
+      for (int o = lane; o < kc * c4; o += 32) {
+        const int mu = o / c4, q = o - mu * c4;
+        cp_async16(sx + mu * xp + 4 * q, x + (int64_t)mu * rp + a.c0 + 4 * q);
+      }
+    }
+  };
   // copies of the warp's i-th piece
   auto issue = [&](int i) {
     if (i < n) {
@@ -96,7 +113,7 @@ __device__ __forceinline__ void lane_row(const LaneRows &g, const LaneShape &a, 
       unsigned char *st = ring + ((uint32_t)i % NST) * (size_t)a.stage;
       const unsigned char *src;
       const float *x;
-      int kc;
+      int kc, b = nb;   // b: the piece's first block
       uint32_t ab;
       float sc = 1.0f;
       if (p < a.vpieces) {
@@ -113,7 +130,9 @@ __device__ __forceinline__ void lane_row(const LaneRows &g, const LaneShape &a, 
         ab = (uint32_t)(sizeof(float) * kc * Mp);
         x = g.X + (row * K + k0) * (int64_t)rp;
       } else {
-        const int t = p - lead, b = a.ppb == 1 ? t : t / a.ppb, k0 = kPiece * (t - b * a.ppb);
+        const int t = p - lead;
+        b = BPP > 1 ? BPP * t : a.ppb == 1 ? t : t / a.ppb;
+        const int k0 = BPP > 1 ? 0 : kPiece * (t - b * a.ppb);
         if (b - base >= 32) batch(b & ~31);
         const int32_t c = __shfl_sync(0xffffffffu, bc, b - base), k = __shfl_sync(0xffffffffu, bb, b - base);
         sc = __shfl_sync(0xffffffffu, bs, b - base);
@@ -122,18 +141,17 @@ __device__ __forceinline__ void lane_row(const LaneRows &g, const LaneShape &a, 
         ab = (uint32_t)(sizeof(TS) * kc * Mp);
         x = g.X + ((int64_t)c * K + k0) * rp;
       }
-      for (uint32_t o = 16u * lane; o < ab; o += 512u) cp_async16(st + o, src + o);
-      float *sx = reinterpret_cast<float *>(st + a.xoff);
-      if (rp == xp) {
-        for (int o = 4 * lane; o < kc * xp; o += 128) cp_async16(sx + o, x + o);
-      } else {
-        const int c4 = a.ncol / 4;
-        for (int o = lane; o < kc * c4; o += 32) {
-          const int mu = o / c4, q = o - mu * c4;
-          cp_async16(sx + mu * xp + 4 * q, x + (int64_t)mu * rp + a.c0 + 4 * q);
-        }
-      }
+      copy(st, 0, src, ab, x, kc);
       if (lane == 0) *reinterpret_cast<float *>(st + a.stage - 16) = sc;
+#pragma unroll
+      for (int u = 1; u < BPP; ++u) {   // BPP divides 32: the blocks share a batch of columns
+        if (b + u >= nb) break;
+        const int32_t c = __shfl_sync(0xffffffffu, bc, b + u - base), k = __shfl_sync(0xffffffffu, bb, b + u - base);
+        sc = __shfl_sync(0xffffffffu, bs, b + u - base);
+        copy(st, u, reinterpret_cast<const unsigned char *>(static_cast<const TS *>(g.A) + (int64_t)k * K * Mp), ab,
+             g.X + (int64_t)c * K * rp, kc);
+        if (lane == 0) *reinterpret_cast<float *>(st + a.stage - 16 + 4 * u) = sc;
+      }
     }
     cp_async_commit();
   };
@@ -206,7 +224,17 @@ __device__ __forceinline__ void lane_row(const LaneRows &g, const LaneShape &a, 
       multiply(reinterpret_cast<const float *>(st), sX, min(kPiece, K - kPiece * (p - a.vpieces)), 1.0f);
     } else {
       const int t = p - lead, k0 = a.ppb == 1 ? 0 : kPiece * (t % a.ppb);
-      multiply(reinterpret_cast<const TS *>(st), sX, min(kPiece, K - k0), sc);
+      const TS *sA = reinterpret_cast<const TS *>(st);
+      if (BPP == 1) {
+        multiply(sA, sX, min(kPiece, K - k0), sc);
+      } else {
+        const int m = min(BPP, nb - BPP * t);
+        if (std::is_same<TS, __half>::value)   // a scale per block
+          for (int u = 0; u < m; ++u)
+            multiply(sA + u * K * Mp, sX + u * K * xp, K, *reinterpret_cast<const float *>(st + a.stage - 16 + 4 * u));
+        else
+          multiply(sA, sX, m * K, sc);
+      }
     }
   }
   cp_async_wait<0>();
@@ -277,12 +305,12 @@ __device__ __forceinline__ void lane_row(const LaneRows &g, const LaneShape &a, 
 }
 
 // bytes of a stage (and the offset of its X region): the largest piece of A, V or G, the rows of X
-// beside it, and the scale
-inline uint32_t lane_stage(const LaneRows &g, size_t sa, size_t sv, int xp, uint32_t *xoff) {
-  const int kb = g.K < kPiece ? g.K : kPiece, kvb = g.V ? (g.kv < kPiece ? g.kv : kPiece) : 0;
+// beside it, and the scales
+inline uint32_t lane_stage(const LaneRows &g, size_t sa, size_t sv, int xp, int bpp, uint32_t *xoff) {
+  const int k1 = g.K < kPiece ? g.K : kPiece, kb = bpp * k1, kvb = g.V ? (g.kv < kPiece ? g.kv : kPiece) : 0;
   size_t ab = sa * kb * g.Mp;
   if (sv * kvb * g.Mp > ab) ab = sv * kvb * g.Mp;
-  if (g.G && sizeof(float) * kb * g.Mp > ab) ab = sizeof(float) * kb * g.Mp;
+  if (g.G && sizeof(float) * k1 * g.Mp > ab) ab = sizeof(float) * k1 * g.Mp;
   *xoff = (uint32_t)((ab + 15) / 16 * 16);
   return *xoff + (uint32_t)((kb > kvb ? kb : kvb) * xp * sizeof(float)) + 16;
 }
