@@ -983,7 +983,11 @@ int launch_rows(const Rows &rows, const RowCfg &cfg, int threads, int R, int64_t
 // column, as float bits.  The generic block-row kernel pipelines many terms
 // per row; a leaf row has one (more than 16 columns took one block-row launch
 // before: 81,920 triangles, order 3, 32 columns, FP64-accurate: product 891 ->
-// 881 us with two passes here).
+// 881 us with two passes here).  Bound by the FP32 pipe.  The columns of a
+// thread are fixed at compile time, with indices clamped to the last column: a
+// test per column and term kept the double-float chains of a thread apart
+// (327,680 triangles, order 4, 16 columns: backward 215 -> 201 us; 15,000,
+// order 3, 5 columns: forward 14.5 -> 12.3 us).
 template <class TS, class T, bool MAX>
 __global__ void __launch_bounds__(256) k_leaf_fwd_reg(const TS *__restrict__ V, const T *__restrict__ xpad,
                                                       const float *__restrict__ vscale, int L, int kp, int k, int rp,
@@ -1004,24 +1008,37 @@ __global__ void __launch_bounds__(256) k_leaf_fwd_reg(const TS *__restrict__ V, 
   __syncthreads();
   const int nu = threadIdx.x >> 2, jq = threadIdx.x & 3;
   if (nu < k) {
-    T acc[4];
-#pragma unroll
-    for (int u = 0; u < 4; ++u) acc[u] = zero_of<T>();
-    for (int r = 0; r < L; ++r) {
-      const T v = Vs[r * kp + nu];
-#pragma unroll
-      for (int u = 0; u < 4; ++u)
-        if (jq + 4 * u < nc) acc_fma(acc[u], v, xs[r * nc + jq + 4 * u]);
-    }
     const float sc = vscale ? vscale[t] : 1.0f;
+    // NU columns jq + 4u; those beyond nc repeat the last one
+    auto sum = [&](auto nuc) {
+      constexpr int NU = decltype(nuc)::value;
+      T acc[NU];
+      int at[NU];
 #pragma unroll
-    for (int u = 0; u < 4; ++u)
-      if (jq + 4 * u < nc) {
-        acc_norm(acc[u]);
-        const T v = vscale ? acc[u] * from_double<T>(sc) : acc[u];
-        xleaf[(t * k + nu) * rp + c0 + jq + 4 * u] = v;
-        if (MAX) atomicMax(&smax[jq + 4 * u], __float_as_uint(mag_of(v)));
+      for (int u = 0; u < NU; ++u) {
+        at[u] = min(jq + 4 * u, nc - 1);
+        acc_mul(acc[u], Vs[nu], xs[at[u]]);
       }
+      for (int r = 1; r < L; ++r) {
+        const T v = Vs[r * kp + nu];
+#pragma unroll
+        for (int u = 0; u < NU; ++u) acc_fma(acc[u], v, xs[r * nc + at[u]]);
+      }
+#pragma unroll
+      for (int u = 0; u < NU; ++u)
+        if (jq + 4 * u < nc) {
+          acc_norm(acc[u]);
+          const T v = vscale ? acc[u] * from_double<T>(sc) : acc[u];
+          xleaf[(t * k + nu) * rp + c0 + jq + 4 * u] = v;
+          if (MAX) atomicMax(&smax[jq + 4 * u], __float_as_uint(mag_of(v)));
+        }
+    };
+    if (nc > 8)
+      sum(std::integral_constant<int, 4>{});
+    else if (nc > 4)
+      sum(std::integral_constant<int, 2>{});
+    else
+      sum(std::integral_constant<int, 1>{});
   }
   if (MAX) {
     // one look at the maximum so far spares most CTAs the atomic on a contended word
@@ -1047,20 +1064,32 @@ __global__ void __launch_bounds__(256) k_leaf_bwd_reg(const TS *__restrict__ Vt,
   __syncthreads();
   const int r = threadIdx.x >> 3, jo = threadIdx.x & 7;
   if (r >= L) return;
-  T acc[2] = {zero_of<T>(), zero_of<T>()};
-  for (int nu = 0; nu < k; ++nu) {
-    const T w = Vs[nu * Lp + r];
-#pragma unroll
-    for (int u = 0; u < 2; ++u)
-      if (jo + 8 * u < nc) acc_fma(acc[u], w, ys[nu * nc + jo + 8 * u]);
-  }
   const float sc = vscale ? vscale[t] : 1.0f;
+  auto sum = [&](auto nuc) {
+    constexpr int NU = decltype(nuc)::value;
+    T acc[NU];
+    int at[NU];
 #pragma unroll
-  for (int u = 0; u < 2; ++u)
-    if (jo + 8 * u < nc) {
-      acc_norm(acc[u]);
-      ypad[(t * L + r) * rp + c0 + jo + 8 * u] = vscale ? acc[u] * from_double<T>(sc) : acc[u];
+    for (int u = 0; u < NU; ++u) {
+      at[u] = min(jo + 8 * u, nc - 1);
+      acc_mul(acc[u], Vs[r], ys[at[u]]);
     }
+    for (int nu = 1; nu < k; ++nu) {
+      const T w = Vs[nu * Lp + r];
+#pragma unroll
+      for (int u = 0; u < NU; ++u) acc_fma(acc[u], w, ys[nu * nc + at[u]]);
+    }
+#pragma unroll
+    for (int u = 0; u < NU; ++u)
+      if (jo + 8 * u < nc) {
+        acc_norm(acc[u]);
+        ypad[(t * L + r) * rp + c0 + jo + 8 * u] = vscale ? acc[u] * from_double<T>(sc) : acc[u];
+      }
+  };
+  if (nc > 8)
+    sum(std::integral_constant<int, 2>{});
+  else
+    sum(std::integral_constant<int, 1>{});
 }
 
 // TS: storage type of S and the nearfield; TV: of the leaf bases V; TE: of

@@ -52,9 +52,10 @@ __device__ __forceinline__ dd shfl_t(dd v, int src) {
 // out[a] = sum_b F[a][b] in[b] (plain, E) or sum_b F[b][a] in[b] (trans, E^T)
 template <class T, bool TRANS, int M>
 __device__ __forceinline__ T modem_out(const T *F, const T (&in)[M], int a) {
-  T acc = zero_of<T>();
+  T acc;
+  acc_mul(acc, F[TRANS ? a : a * M], in[0]);
 #pragma unroll
-  for (int b = 0; b < M; ++b) acc_fma(acc, TRANS ? F[b * M + a] : F[a * M + b], in[b]);
+  for (int b = 1; b < M; ++b) acc_fma(acc, TRANS ? F[b * M + a] : F[a * M + b], in[b]);
   acc_norm(acc);
   return acc;
 }
@@ -252,16 +253,24 @@ struct alignas(2 * sizeof(T)) Pair {
 template <int M>
 __host__ __device__ constexpr int pair_max() { return M == 5 ? 4 : 8; }
 
-// sum_b F[b][j] (up) or F[j][b] (down) in[base + b stride], both columns
+// sum_b F[b][j] (up) or F[j][b] (down) in[base + b stride], both columns.  The
+// first term is a plain product: added to zero like the others it cost 8 of 54
+// FP32 instructions per double-float sum (327,680 triangles, order 4, 16 columns:
+// upward 409 -> 386 us with the digit cut, downward 291 -> 271 us).
 template <class T, bool TRANS, int M>
 __device__ __forceinline__ Pair<T> mode_pair(const T *F, int j, const Pair<T> *in, int stride) {
-  Pair<T> o{zero_of<T>(), zero_of<T>()};
+  Pair<T> o;
 #pragma unroll
   for (int b = 0; b < M; ++b) {
     const T f = TRANS ? F[b * M + j] : F[j * M + b];
     const Pair<T> v = in[b * stride];
-    acc_fma(o.a, f, v.a);
-    acc_fma(o.b, f, v.b);
+    if (b == 0) {
+      acc_mul(o.a, f, v.a);
+      acc_mul(o.b, f, v.b);
+    } else {
+      acc_fma(o.a, f, v.a);
+      acc_fma(o.b, f, v.b);
+    }
   }
   acc_norm(o.a);
   acc_norm(o.b);
@@ -301,7 +310,7 @@ __device__ __forceinline__ void up_pair(const TS *__restrict__ Ef, int rp, int n
                 : Pair<T>{zero_of<T>(), zero_of<T>()};
   const int slot = pl < pp ? (int)threadIdx.x : 0, at = pl < pp ? pl * tpp + p : 0;
   const T *Fp = F + (pl < pp ? pl : 0) * 6 * M * M;
-  Pair<T> acc{zero_of<T>(), zero_of<T>()};
+  Pair<T> acc;
 #pragma unroll
   for (int ch = 0; ch < 2; ++ch) {
     Pair<T> *A = buf + (ch ? pp * tpp : 0), *Bf = buf + (ch ? 0 : pp * tpp);
@@ -315,8 +324,7 @@ __device__ __forceinline__ void up_pair(const TS *__restrict__ Ef, int rp, int n
     if (pl < pp) A[slot] = o;
     __syncthreads();
     o = mode_pair<T, true, M>(Fc + 2 * M * M, jz, A + at + (nu - M * M * jz) * np, M * M * np);
-    acc.a = acc.a + o.a;
-    acc.b = acc.b + o.b;
+    acc = ch == 0 ? o : Pair<T>{acc.a + o.a, acc.b + o.b};
   }
   if (act) *reinterpret_cast<Pair<T> *>(xhat + (par * K + nu) * rp + col) = acc;
   if (xmax) {
@@ -406,7 +414,7 @@ inline int pair_parents(int m, int64_t npar, int np) {
 // without; 1.3 M triangles, order 3, 4 columns 150 us with them, 95 us without.
 // Downward the pair kernel was never slower (1.3 M, 4 columns 193 -> 93 us;
 // 327,680, 16 columns FP32 146 -> 133 us, double-float 343 -> 306 us; 81,920,
-// one column, double-float order 4 121 -> 64 us).
+// one column, double-float order 4 121 -> 64 us; now 113, 271 and 33 us).
 template <class T>
 inline bool pair_up(int m, int64_t npar, int rp) {
   return sizeof(T) == 8 || (m != 3 && m != 4) || rp <= 8 || npar * rp <= 4096;
