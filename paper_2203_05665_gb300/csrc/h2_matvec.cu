@@ -433,8 +433,6 @@ struct GcaDownRows {
 template <class TS, class TC, int TPL, class Rows>
 __global__ void __launch_bounds__(128) k_rows_warp(Rows rows, int M, int Mp, int rp, int Kmax, int64_t nrows,
                                                    int accumulate, TC *__restrict__ out) {
-  pdl_wait();
-  pdl_go();
   using XV = typename Vec16<TC>::V;
   constexpr int VN = Vec16<TC>::N;
   extern __shared__ __align__(16) unsigned char rwsm[];
@@ -534,8 +532,6 @@ __global__ void __launch_bounds__(128) k_rows_warp(Rows rows, int M, int Mp, int
 template <class TS, class TC, int R, class Rows>
 __global__ void __launch_bounds__(kThreads + 32, 2)
     k_blockrow(Rows rows, RowCfg cfg, int64_t nrows, int accumulate, TC *__restrict__ out) {
-  pdl_wait();
-  pdl_go();
   using XV = typename Vec16<TC>::V;
   constexpr int VN = Vec16<TC>::N;
   extern __shared__ __align__(128) unsigned char smem[];
@@ -958,7 +954,10 @@ int launch_rows_r(const Rows &rows, const RowCfg &cfg, int threads, int64_t nrow
   H2_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, threads, sm));
   if (per_sm < 1) return fail(H2_EINVAL, "block-row kernel cannot be resident");
   const int64_t grid = std::min<int64_t>(nrows, (int64_t)per_sm * sms);
-  pdl(k_blockrow<TS, TC, R, Rows>, (unsigned)grid, threads, sm, st, rows, cfg, nrows, accumulate, out);
+  // launched without the early start of h2_launch.cuh: CTAs set up beside the previous kernel's
+  // are spread unevenly over the SMs, and these own fixed shares of the rows (FP32 GCA coupling
+  // of 327,680 triangles, 16 columns: 880 us, with it 1,034; its transfers in double-float 558, 721)
+  k_blockrow<TS, TC, R, Rows><<<(unsigned)grid, threads, sm, st>>>(rows, cfg, nrows, accumulate, out);
   return H2_OK;
 }
 
@@ -986,7 +985,7 @@ int launch_rows(const Rows &rows, const RowCfg &cfg, int threads, int R, int64_t
 // 881 us with two passes here).  Bound by the FP32 pipe.  The columns of a
 // thread are fixed at compile time, with indices clamped to the last column: a
 // test per column and term kept the double-float chains of a thread apart
-// (327,680 triangles, order 4, 16 columns: backward 215 -> 201 us; 15,000,
+// (327,680 triangles, order 4, 16 columns: backward and nearfield 578 -> 563 us; 15,000,
 // order 3, 5 columns: forward 14.5 -> 12.3 us).
 template <class TS, class T, bool MAX>
 __global__ void __launch_bounds__(256) k_leaf_fwd_reg(const TS *__restrict__ V, const T *__restrict__ xpad,
@@ -1363,7 +1362,7 @@ int gca_rows_launch(const Rows &rows, int M, int Mp, int Kmax, int rp, int64_t n
         H2_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 128, sm));
         if (per_sm < 1) return fail(H2_EINVAL, "warp block-row kernel cannot be resident");
         const int64_t grid = std::min<int64_t>((nrows + 3) / 4, (int64_t)per_sm * sms);
-        pdl(kern, (unsigned)grid, 128, sm, st, rows, M, Mp, rp, Kmax, nrows, accumulate, out);
+        kern<<<(unsigned)grid, 128, sm, st>>>(rows, M, Mp, rp, Kmax, nrows, accumulate, out);
         return H2_OK;
       };
       if (tiles <= 32) return go(k_rows_warp<TS, T, 1, Rows>);
