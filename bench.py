@@ -194,7 +194,7 @@ def run_ours(args):
     if args.prec == "f64n":
         roof = {"bound": "alu", "achieved": alg["coupling_flops"] / (cpl_ms * 1e-3) / 1e12, "peak": FP64_TFLOPS,
                 "unit": "TFLOP/s", "kernel": "k_blockrow (coupling, FP64 FMA pipe)"}
-    elif args.prec == "f64" and st.get("tensor", 0):
+    elif args.prec == "f64" and st.get("tensor", 0) and args.order == 4:
         # tensor-core coupling: a stream of the stored slices; algorithmic bytes are
         # those of the FP64 coupling matrices (k^2 x 8 B per block) and coefficients
         # stored_stream_frac: the E4M3 digit planes of S alone (10 B per entry), the part
@@ -208,7 +208,8 @@ def run_ours(args):
                                        / peaks["hbm_gbs"])}
     elif args.prec == "f64":
         roof = {"bound": "alu", "achieved": alg["coupling_flops"] / (cpl_ms * 1e-3) / 1e12, "peak": DD_TFLOPS,
-                "unit": "TFLOP/s", "kernel": "k_blockrow (coupling, double-float on the FP32 pipe)",
+                "unit": "TFLOP/s", "kernel": ("k_tile_tc (coupling, tcgen05 digits)" if st.get("tensor", 0) else
+                                              "k_blockrow (coupling, double-float on the FP32 pipe)"),
                 "hbm_frac": alg["coupling_bytes"] / (cpl_ms * 1e-3) / 1e9 / peaks["hbm_gbs"]}
     elif args.prec in ("bf16", "f16"):
         # regenerated coupling: 2 k^2 nrhs multiply-adds plus one kernel evaluation
@@ -216,16 +217,17 @@ def run_ours(args):
         k = st["rank"]
         flops = alg["coupling_flops"] + 10.0 * st["adm_blocks"] * k * k
         roof = {"bound": "alu", "achieved": flops / (cpl_ms * 1e-3) / 1e12, "peak": FP32_TFLOPS,
-                "unit": "TFLOP/s", "kernel": "k_blockrow (coupling regenerated in FP32)"}
+                "unit": "TFLOP/s", "kernel": "k_coupling_regen (coupling regenerated in FP32)"}
     else:
         roof = {"bound": "hbm", "achieved": alg["coupling_bytes"] / (cpl_ms * 1e-3) / 1e9, "peak": peaks["hbm_gbs"],
-                "unit": "GB/s", "kernel": "k_blockrow (coupling, stored S stream)"}
+                "unit": "GB/s", "kernel": ("k_coupling_tc (six 5-bit E4M3 digits)" if st.get("tensor", 0) else
+                                           "k_lane_rows (coupling, stored S stream)")}
     roof["frac"] = roof["achieved"] / roof["peak"]
     # DRAM bytes (read + write) per coupling launch from the ncu capture of the
     # same kernel at level 5 (profiles/k_coupling_tc_icosphere_L5_m4_16rhs_f64.md,
     # profiles/k_blockrow_coupling_icosphere_L5_m4_16rhs_f64.md), scaled by
     # admissible blocks; None where no capture of the current kernel exists
-    tc = args.prec == "f64" and st.get("tensor", 0)
+    tc = args.prec == "f64" and st.get("tensor", 0) and args.order == 4
     traffic_per_block = {"f64": 691.93e6 / 18876, "f64-tc": (794.690048e6 + 7.657472e6) / 18876}
     key = "f64-tc" if tc else args.prec
     roof["traffic"] = (traffic_per_block[key] * st["adm_blocks"]

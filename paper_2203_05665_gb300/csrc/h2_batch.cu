@@ -22,7 +22,7 @@
 // Six problems (20,480 to 130,000 triangles, order 3 and 4, leaves of 64, 1 to 8
 // right-hand sides), default launch shapes: 1,124 us per product with a
 // persistent kernel of four warps per SM and one output row per lane (coupling
-// 416, leaf backward + nearfield 442, transfers 210), 426 us now (134, 182, 81);
+// 416, leaf backward + nearfield 442, transfers 210), 415 us now (136, 183, 68);
 // bound by the instructions around pieces of 27 to 64 rows and 4 columns.
 #include <algorithm>
 #include <cmath>

@@ -1,8 +1,8 @@
-// Coupling and nearfield phases on the tensor cores (tcgen05, FP8 E4M3
-// operands, FP32 accumulation in tensor memory), up to 16 right-hand sides:
-// the coupling of order-4 handles (k = 64) in FP64 accuracy (ten digits per
-// value) or FP32 accuracy (six digits), and the FP64-accurate nearfield of
-// handles whose leaves hold at most 21 triangles (second part of the file).
+// Coupling phase of order-4 handles (k = 64) on the tensor cores (tcgen05, FP8
+// E4M3 operands, FP32 accumulation in tensor memory), up to 16 right-hand sides,
+// in FP64 accuracy (ten digits per value) or FP32 accuracy (six digits), and the
+// FP64-accurate leaf forward step of leaves of at most 21 triangles.  Block rows
+// with smaller tiles (nearfield, order-3 coupling) are in h2_tile.cu.
 //
 // GB300 runs FP64 at 1/58 of its FP32 rate, and double-float arithmetic on
 // the FP32 pipe leaves the coupling (Algorithm 3, y^_t = sum S_ts x^_s)
@@ -35,8 +35,8 @@
 // each, 10 instructions per block.  The groups write their pairs so that the
 // pairs of one level i + k land in the same accumulator columns (the tensor
 // cores add them, exactly), so a segment's results take 160 columns and
-// three accumulator sets rotate: the MMAs of one row segment overlap the
-// epilogue of the previous one.
+// there are three accumulator sets, one per epilogue group: the MMAs of one row
+// overlap the epilogues of the two before it.
 //
 // Kernel roles (one CTA per SM, 14 warps): warp 0 streams the digits of each
 // block through a shared-memory ring (bulk copies completing on mbarriers;
@@ -84,8 +84,8 @@ constexpr uint32_t kSliceA = kTcK * kTcK;              // 4096 bytes: one digit 
 // every pair of level i + k = c + 2 and, in lanes 64-127, of level c + 3.  The
 // tensor cores thus add the pairs of one level themselves (exactly: at most
 // five sums of at most 2^20 each), an accumulator set is W ND columns wide
-// (160 or 96 for W = 16) and kSets sets rotate, so that the MMAs of the next row segment
-// run while the epilogue reads the previous one.
+// (160 or 96 for W = 16), and each epilogue group has a set of its own, so that the
+// MMAs of the next rows run while it reads its row.
 //
 // KB is the contraction length of one block in bytes: 64 for the coupling
 // matrices (two MMA K steps), 32 for the leaf bases V_t^T of the leaf forward
@@ -621,11 +621,11 @@ __global__ void __launch_bounds__(kTcThreads, 1)
 
 // Leaf forward step on the tensor cores (Algorithm 1 at the leaves,
 // x^_t = V_t^T x|t, FP64-accurate handles of order 4 with leaves of at most
-// 32 triangles): the blocks are V_t^T (64 rows nu, the leaf's triangles r as
+// 21 triangles and 9 to 16 columns): the blocks are V_t^T (64 rows nu, the leaf's triangles r as
 // the contraction index, zero padded to 32 bytes), cut once into the ten
 // digit planes of the coupling with a power of two per row,
 // Ev[t][nu] = 1 + floor(log2 max_r |V_t[r][nu]|); the coefficients are the
-// input digit planes of leaf t that the nearfield cuts (k_ntc_slice_x).
+// wide input digit tiles of leaf t that the nearfield reads too (ntc_input).
 __global__ void k_tcv_rowexp(const dd *__restrict__ V, int64_t nleaf, int L, int kp, int32_t *__restrict__ Ev) {
   const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (e >= nleaf * kTcK) return;
