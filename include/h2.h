@@ -211,7 +211,11 @@ int h2_build_times(h2_handle h, double *ms);
  * stream.  1 <= nrhs <= 64.  H2_F64 handles accept any finite double: a
  * column whose largest entry lies outside [2^-40, 2^40] is scaled by a power
  * of two on the way in and back on the way out (exact), so it keeps FP64-level
- * relative accuracy; zero, infinite and NaN columns are passed as they are.
+ * relative accuracy.  Values far below their column's largest keep 48 bits of
+ * their own where a column's values span many orders of magnitude, except in order-4
+ * products of up to 16 columns with the coupling on the tensor cores: there
+ * coefficients are rounded to 2^-48 of the column's largest of their tree level
+ * (options.tensor = 1 has none of this).  Zero, infinite and NaN columns are passed as they are.
  * Errors: H2_EINVAL (NULL, nrhs out of range), H2_ENOMEM (work buffers),
  * H2_ECUDA (launch failure). */
 int h2_matvec(h2_handle h, const void *x, void *y, int nrhs);

@@ -31,22 +31,23 @@ namespace h2 {
 // remainder (0 or 1) carries into A, and A's remainder after four digits is
 // the top digit, within [-16, 16] because |A| <= 2^24 + 2.
 // The same for six digits of |X| <= 2^29 (one 32-bit value; the top digit
-// stays within [-16, 16] by the same bound).
+// stays within [-16, 16] by the same bound), and for eleven of |X| <= 2^54 (A
+// takes six digits: |A| <= 2^29 + 2).
 template <int ND>
 __host__ __device__ __forceinline__ void split_digits(long long X, int (&s)[ND]) {
-  static_assert(ND == 10 || ND == 6, "digit counts");
-  if (ND == 10) {
+  static_assert(ND == 11 || ND == 10 || ND == 6, "digit counts");
+  if (ND >= 10) {
     int b = (int)(((X + (1LL << 24)) & ((1LL << 25) - 1)) - (1LL << 24));
     int a = (int)((X - b) >> 25);
 #pragma unroll
-    for (int i = ND - 1; i >= ND / 2; --i) {
+    for (int i = ND - 1; i >= ND - 5; --i) {
       const int d = ((b + 16) & 31) - 16;
       s[i] = d;
       b = (b - d) >> 5;
     }
     a += b;
 #pragma unroll
-    for (int i = ND / 2 - 1; i >= 1; --i) {
+    for (int i = ND - 6; i >= 1; --i) {
       const int d = ((a + 16) & 31) - 16;
       s[i] = d;
       a = (a - d) >> 5;
@@ -67,7 +68,7 @@ __host__ __device__ __forceinline__ void split_digits(long long X, int (&s)[ND])
 // The same digits, as exact FP32 values, of X = rint(hs) + rint(ls) (hs, ls
 // the two words of a double-float value, or an FP32 value and 0, already
 // scaled by 2^sc: power-of-two products, exact), formed with 32-bit
-// operations only.  For ten digits: H = rint(hs) is an integer-valued float,
+// operations only.  For ten or eleven digits: H = rint(hs) is an integer-valued float,
 // A = rint(H 2^-25) and B = H - A 2^25 (|B| <= 2^24, an exact float
 // difference) split it, and L = rint(ls) fits in 32 bits, so X = A 2^25 + bt
 // with bt = B + L, whose low 25 bits are those of X: the halves (a, b) of
@@ -92,8 +93,8 @@ __host__ __device__ __forceinline__ float digit_f(int &v) {
 
 template <int ND>
 __host__ __device__ __forceinline__ void split_digits_f(float hs, float ls, float (&f)[ND]) {
-  static_assert(ND == 10 || ND == 6, "digit counts");
-  if (ND == 10) {
+  static_assert(ND == 11 || ND == 10 || ND == 6, "digit counts");
+  if (ND >= 10) {
     const float H = rintf(hs);
     const float A = rintf(H * 0x1p-25f);
     const float B = fmaf(-A, 0x1p25f, H);
@@ -101,10 +102,10 @@ __host__ __device__ __forceinline__ void split_digits_f(float hs, float ls, floa
     int b = ((bt + (1 << 24)) & ((1 << 25) - 1)) - (1 << 24);
     int a = (int)A + ((bt - b) >> 25);
 #pragma unroll
-    for (int i = ND - 1; i >= ND / 2; --i) f[i] = digit_f(b);
+    for (int i = ND - 1; i >= ND - 5; --i) f[i] = digit_f(b);
     a += b;
 #pragma unroll
-    for (int i = ND / 2 - 1; i >= 1; --i) f[i] = digit_f(a);
+    for (int i = ND - 6; i >= 1; --i) f[i] = digit_f(a);
     f[0] = (float)a;
   } else {
     int a = (int)rintf(hs) + (int)rintf(ls);

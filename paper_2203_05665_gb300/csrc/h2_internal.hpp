@@ -144,6 +144,9 @@ struct Dev {
   int32_t *ntc_E = nullptr;
   RowSched ntc_s, tc_s;         // row orders of the nearfield and of the tensor-core coupling
   unsigned *ntc_xmax = nullptr;
+  // per column of the input: twice its entries of at least 2^-5 of the largest, less its
+  // non-zero entries ([64]); negative: the small tiles are summed in double-float (h2_tile.cu)
+  int *spread = nullptr;
   // tensor-core leaf forward step: the ten E4M3 digit planes of every V_t^T
   // ([leaf][10][64 x 32] bytes, K-major core matrices) and their row powers
   // of two [leaf][64]
@@ -293,7 +296,7 @@ int tc_leaf_build(Ctx &c);
 bool ntc_eligible(const Dev &d);
 int ntc_build(Ctx &c);
 void ntc_input(Ctx &c, const void *xpad, int rp, int c0, int ncol, bool wide);
-int ntc_near(Ctx &c, const void *xpad, void *ypad, int rp, int accumulate, int64_t *launches,
+int ntc_near(Ctx &c, const void *xpad, void *ypad, int rp, int accumulate, int64_t *launches, bool ranged,
              bool have_input = false);
 int tile_take_error(cudaStream_t st);
 // FP64-accurate order-3 coupling on the tensor cores (h2_tile.cu)
@@ -305,9 +308,9 @@ constexpr int kLevelCols = 64;   // column maxima per tree level
 int row_schedule(Dev &d, const int64_t *ptr, const int32_t *col, int64_t nrows, RowSched &s, SchedTmp &tmp,
                  cudaStream_t st);
 // H2_F64 handles: the range guard's column maxima (64 x 8 bytes), the input's
-// (64 x 4) and the coefficients' per level (32 x 64 x 4), one block cleared
-// by one memset per product
-constexpr size_t kMaximaBytes = 64 * 8 + 64 * 4 + 32 * 64 * 4;
+// (64 x 4), the coefficients' per level (32 x 64 x 4) and the input's range counts
+// (64 x 4), one block cleared by one memset per product
+constexpr size_t kMaximaBytes = 64 * 8 + 64 * 4 + 32 * 64 * 4 + 64 * 4;
 // leaf forward step on the tensor cores (after ntc_input); requires d.Vtc
 int tc_leaf_forward(Ctx &c, void *xhat, int rp);
 

@@ -101,20 +101,30 @@ constexpr int kPermRows = 64;
 // xpad[p][c] (zero beyond nrhs and for padding rows) from x[src][c], scaled by
 // the column's range-guard power of two; with xmax also the largest |xpad|
 // (|hi| for double-float) of every column, as float bits (atomicMax), the
-// maxima the nearfield's input digits are cut with
-template <class Tin, class Tout>
+// maxima the nearfield's input digits are cut with; with COUNT in spread twice the number
+// of a column's entries of at least 2^-5 of its largest, less that of its non-zero
+// entries (finite columns; whole numbers, so that the sums do not depend on their order)
+template <class Tin, class Tout, bool COUNT>
 __global__ void __launch_bounds__(256) k_permute_in(const Tin *__restrict__ x, int64_t n, int nrhs, int rp,
                                                     const int32_t *__restrict__ pad_src, int64_t npad,
                                                     const unsigned long long *__restrict__ colmax,
-                                                    Tout *__restrict__ xpad, unsigned *__restrict__ xmax = nullptr) {
+                                                    Tout *__restrict__ xpad, unsigned *__restrict__ xmax,
+                                                    int *__restrict__ spread) {
   pdl_wait();
   pdl_go();
   extern __shared__ __align__(16) unsigned char perm_smem[];
   Tout *tile = reinterpret_cast<Tout *>(perm_smem);
-  __shared__ int shift[64];
+  __shared__ int shift[64], cnt[COUNT ? 64 : 1];
+  __shared__ float most[COUNT ? 64 : 1];   // 2^-5 of the column's largest value, as scaled
   __shared__ unsigned smax[64];
   __shared__ int32_t src[kPermRows];
   if (threadIdx.x < 64) smax[threadIdx.x] = 0u;
+  if (COUNT && threadIdx.x < 64) {
+    cnt[threadIdx.x] = 0;
+    const unsigned long long b = (int)threadIdx.x < nrhs ? colmax[threadIdx.x] : 0ull;
+    // an infinite or NaN column counts nothing: the last permutation writes it
+    most[threadIdx.x] = not_finite(b) ? -1.0f : (float)scale_pow2(__longlong_as_double((long long)b), range_shift(b) - 5);
+  }
   const int w = rp + 1;
   const int64_t p0 = (int64_t)blockIdx.x * kPermRows;
   if (threadIdx.x < kPermRows) src[threadIdx.x] = p0 + threadIdx.x < npad ? pad_src[p0 + threadIdx.x] : -1;
@@ -137,7 +147,14 @@ __global__ void __launch_bounds__(256) k_permute_in(const Tin *__restrict__ x, i
       const int c = i / kPermRows, q = i - c * kPermRows;
       Tin v = u[a];
       if (c < nrhs && shift[c]) v = (Tin)scale_pow2((double)v, shift[c]);
-      tile[q * w + c] = (src[q] >= 0 && c < nrhs) ? convert<Tout, Tin>(v) : zero_of<Tout>();
+      const Tout o = (src[q] >= 0 && c < nrhs) ? convert<Tout, Tin>(v) : zero_of<Tout>();
+      tile[q * w + c] = o;
+      if (COUNT) {   // c is the same in all lanes
+        const float m = mag_of(o);
+        const bool any = m > 0.0f && most[c] >= 0.0f;
+        const int k = 2 * __popc(__ballot_sync(0xffffffffu, any && m >= most[c])) - __popc(__ballot_sync(0xffffffffu, any));
+        if ((threadIdx.x & 31) == 0 && k) atomicAdd(&cnt[c], k);
+      }
     }
   }
   __syncthreads();
@@ -155,6 +172,21 @@ __global__ void __launch_bounds__(256) k_permute_in(const Tin *__restrict__ x, i
     __syncthreads();
     if ((int)threadIdx.x < rp && smax[threadIdx.x]) atomicMax(&xmax[threadIdx.x], smax[threadIdx.x]);
   }
+  if (COUNT && (int)threadIdx.x < nrhs && cnt[threadIdx.x]) atomicAdd(&spread[threadIdx.x], cnt[threadIdx.x]);
+}
+
+// the launch; ranged: with the range counts (double-float)
+template <class Tin, class Tout>
+void permute_in(Ctx &c, bool ranged, unsigned grid, const Tin *x, int nrhs, int rp, const unsigned long long *colmax,
+                Tout *xpad, unsigned *xmax) {
+  const Dev &d = c.d;
+  const size_t sm = (size_t)kPermRows * (rp + 1) * sizeof(Tout);
+  if constexpr (std::is_same<Tout, dd>::value)
+    if (ranged)
+      return pdl(k_permute_in<Tin, Tout, true>, grid, 256, sm, c.stream, x, d.n, nrhs, rp, d.pad_src, d.npad, colmax,
+                 xpad, xmax, d.spread);
+  pdl(k_permute_in<Tin, Tout, false>, grid, 256, sm, c.stream, x, d.n, nrhs, rp, d.pad_src, d.npad, colmax, xpad, xmax,
+      nullptr);
 }
 
 // y[src][c] (caller order) from ypad[p][c], divided by the column's range-guard
@@ -1138,13 +1170,15 @@ int matvec_typed(Ctx &c, const Tio *x, Tio *y, int nrhs, bool acc) {
   const bool leaf_tc = near_tc && far && d.Vtc && rp > 8 && rp <= 16;
   // order-3 coupling on the tensor cores: the upward pass takes every level's column maxima
   const bool cpl_tile = std::is_same<T, dd>::value && far && d.tct;
-  pdl(k_permute_in<Tio, T>, perm_grid, 256, (size_t)kPermRows * (rp + 1) * sizeof(T), st, 
-      x, d.n, nrhs, rp, d.pad_src, d.npad, cmx, xpad, near_tc ? d.ntc_xmax : nullptr);
-  mk.count(H2_PH_PERMUTE_IN);
-  mk.mark(H2_PH_LEAF_FORWARD);
   const bool tcpath = d.tc && rp <= 16 &&
                       ((std::is_same<T, dd>::value && d.tc_nd == 10) ||
                        (std::is_same<T, float>::value && std::is_same<TS, float>::value && d.tc_nd == 6));
+  // the small tiles sum columns of wide range in double-float, unless the order-4 coupling
+  // cuts their coefficients into digits in any case
+  const bool ranged = (near_tc || cpl_tile) && !tcpath;
+  permute_in<Tio, T>(c, ranged, perm_grid, x, nrhs, rp, cmx, xpad, near_tc ? d.ntc_xmax : nullptr);
+  mk.count(H2_PH_PERMUTE_IN);
+  mk.mark(H2_PH_LEAF_FORWARD);
   bool leaf_max = leaf_tc;   // the leaf step takes its coefficients' column maxima
   // FP32 arithmetic, tiles of at most 64 rows: one or four warps per block row
   const bool lane = std::is_same<T, float>::value && L <= kLaneMax && k <= kLaneMax;
@@ -1284,7 +1318,7 @@ int matvec_typed(Ctx &c, const Tio *x, Tio *y, int nrhs, bool acc) {
   if (near_tc) {
     // FP64-accurate: integer digits on the tensor cores
     int64_t nl = 0;
-    if ((rc = ntc_near(c, xpad, ypad, rp, far ? 1 : 0, &nl, leaf_tc))) return rc;
+    if ((rc = ntc_near(c, xpad, ypad, rp, far ? 1 : 0, &nl, ranged, leaf_tc))) return rc;
     mk.count(H2_PH_LEAF_NEAR, nl);
   } else if (lane) {
     LaneRows g{};
@@ -1413,8 +1447,7 @@ int matvec_gca(Ctx &c, const Tio *x, Tio *y, int nrhs, bool acc) {
   }
   const unsigned perm_grid = (unsigned)((d.npad + kPermRows - 1) / kPermRows);
   const bool near_tc = std::is_same<T, dd>::value && d.ntc;
-  pdl(k_permute_in<Tio, T>, perm_grid, 256, (size_t)kPermRows * (rp + 1) * sizeof(T), st, 
-      x, d.n, nrhs, rp, d.pad_src, d.npad, cmx, xpad, near_tc ? d.ntc_xmax : nullptr);
+  permute_in<Tio, T>(c, near_tc, perm_grid, x, nrhs, rp, cmx, xpad, near_tc ? d.ntc_xmax : nullptr);
   mk.count(H2_PH_PERMUTE_IN);
   auto X = [&](T *base, int l) { return base + d.gX[l] * rp; };
   // FP32: the warp-per-row kernel for the transfer steps and the nearfield,
@@ -1476,7 +1509,7 @@ int matvec_gca(Ctx &c, const Tio *x, Tio *y, int nrhs, bool acc) {
   }
   if (near_tc) {
     int64_t nl = 0;
-    if ((rc = ntc_near(c, xpad, ypad, rp, far ? 1 : 0, &nl))) return rc;
+    if ((rc = ntc_near(c, xpad, ypad, rp, far ? 1 : 0, &nl, true))) return rc;
     mk.count(H2_PH_LEAF_NEAR, nl);
   } else {
     NearRows<TS, T> rows{(const TS *)d.near, d.near_ptr, d.near_col, xpad, nullptr, L, Lp, rp, nullptr};
@@ -1990,8 +2023,10 @@ static bool capture_call(Ctx &c, CallGraph &g, const void *x, void *y) {
   ok = ok && cudaGraphGetNodes(g.graph, nullptr, &n) == cudaSuccess;
   std::vector<cudaGraphNode_t> nodes(ok ? n : 0);
   ok = ok && cudaGraphGetNodes(g.graph, nodes.data(), &n) == cudaSuccess;
-  const void *ins[] = {(const void *)k_permute_in<double, dd>, (const void *)k_permute_in<double, double>,
-                       (const void *)k_permute_in<double, float>, (const void *)k_permute_in<float, float>};
+  const void *ins[] = {(const void *)k_permute_in<double, dd, false>, (const void *)k_permute_in<double, dd, true>,
+                       (const void *)k_permute_in<double, double, false>,
+                       (const void *)k_permute_in<double, float, false>,
+                       (const void *)k_permute_in<float, float, false>};
   const void *outs[] = {(const void *)k_permute_out<dd, double>, (const void *)k_permute_out<double, double>,
                         (const void *)k_permute_out<float, double>, (const void *)k_permute_out<float, float>};
   int nin = 0, nout = 0, nmax = 0;
@@ -2035,7 +2070,7 @@ static cudaError_t aim_call(CallGraph &g, const void *x, void *y) {
     if (e != cudaSuccess) return e;
     // the node's own parameter values, with x or y exchanged
     void *args[10];
-    const int count = nd.out ? 9 : nd.arg + (p.func == (void *)k_colmax<double> ? 3 : 9);
+    const int count = nd.out ? 9 : nd.arg + (p.func == (void *)k_colmax<double> ? 3 : 10);
     for (int i = 0; i < count; ++i) args[i] = p.kernelParams[i];
     args[nd.arg] = nd.out ? (void *)&y : (void *)&x;
     p.kernelParams = args;

@@ -796,6 +796,7 @@ int device_build(Ctx &c) {
       if (rc) return rc;
       d.ntc_xmax = reinterpret_cast<unsigned *>(d.colmax + 64);
       d.tc_xmax = d.ntc_xmax + 64;
+      d.spread = reinterpret_cast<int *>(d.tc_xmax + 32 * kLevelCols);
       if (d.fused && (rc = dev_alloc(d, (void **)&d.fbar, 2 * sizeof(unsigned)))) return rc;
       return build_typed<dd>(c);
     }

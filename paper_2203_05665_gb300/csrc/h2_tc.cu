@@ -262,11 +262,12 @@ __global__ void __launch_bounds__(256) k_tc_slice_x(const T *__restrict__ xhat, 
   T v[16];
 #pragma unroll
   for (int q = 0; q < 16; ++q) v[q] = j < rp ? xc[(16 * g + q) * rp + j] : T{};
-  uint4 w[ND];
-  cut_row16<ND>(v, sc, w);
+  uint32_t w[ND][4];
+  cut_row<ND, 16>(v, sc, w);
   unsigned char *dst = xtc + c * (int64_t)Dig<ND, kTcK, W>::kTileB + core_off(j, 16 * g);
 #pragma unroll
-  for (int i = 0; i < ND; ++i) *reinterpret_cast<uint4 *>(dst + i * Dig<ND, kTcK, W>::kPlaneB) = w[i];
+  for (int i = 0; i < ND; ++i)
+    *reinterpret_cast<uint4 *>(dst + i * Dig<ND, kTcK, W>::kPlaneB) = make_uint4(w[i][0], w[i][1], w[i][2], w[i][3]);
 }
 
 // The coupling kernel (see the top of the file).  Rows t = row0 + r for r

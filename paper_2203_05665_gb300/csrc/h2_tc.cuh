@@ -16,6 +16,8 @@ namespace {
 constexpr int kTcN = 16;                 // columns of one tensor-core pass (right-hand sides, padded)
 constexpr int kTcSlices = 10;            // 5-bit digits of an FP64-accurate value
 constexpr int kTcFixBits = 49;           // |X| <= 2^49
+constexpr int kTileDigits = 11;          // digits of the input values of the small tiles (h2_tile.cu)
+constexpr int kTileFixBits = 54;         // |X| <= 2^54: the first ten digits are those of the rounding to 49 bits
 constexpr uint32_t kTmemCols = 512;      // tensor memory of one SM
 constexpr int kXmaxCols = kLevelCols;
 
@@ -128,14 +130,13 @@ __device__ __forceinline__ uint32_t e4m3x2(float a, float b) {
   return (uint32_t)__nv_cvt_float2_to_fp8x2(make_float2(a, b), __NV_SATFINITE, __NV_E4M3);
 }
 
-// The digit planes of 16 consecutive values v[0..15] of one column, each
-// scaled by 2^sc: plane i as one 16-byte word (the bytes in value order), a
-// row of one core matrix of the MMA layout.
-template <int ND, class T>
-__device__ __forceinline__ void cut_row16(const T (&v)[16], int sc, uint4 (&w)[ND]) {
-  uint32_t u[ND][4];
+// The digit planes of NV (8 or 16) consecutive values of one column, each scaled by
+// 2^sc: plane i as NV / 4 words (the bytes in value order), a row, or half a row, of
+// one core matrix of the MMA layout.
+template <int ND, int NV, class T>
+__device__ __forceinline__ void cut_row(const T (&v)[NV], int sc, uint32_t (&u)[ND][NV / 4]) {
 #pragma unroll
-  for (int q = 0; q < 8; ++q) {
+  for (int q = 0; q < NV / 2; ++q) {
     float f0[ND], f1[ND];
     digits_of<ND>(v[2 * q], sc, f0);
     digits_of<ND>(v[2 * q + 1], sc, f1);
@@ -145,8 +146,6 @@ __device__ __forceinline__ void cut_row16(const T (&v)[16], int sc, uint4 (&w)[N
       u[i][q >> 1] = (q & 1) ? (u[i][q >> 1] | (h << 16)) : h;
     }
   }
-#pragma unroll
-  for (int i = 0; i < ND; ++i) w[i] = make_uint4(u[i][0], u[i][1], u[i][2], u[i][3]);
 }
 
 __device__ __forceinline__ dd dd_scale(dd v, int e) {

@@ -8,20 +8,33 @@
 //
 // The arithmetic is the exact digit splitting of h2_tc.cu: every row nu of
 // the blocks of one block row gets a power of two 2^E, every column j of the
-// input (of each tree level, for the coupling) a power of two 2^F, a value becomes X = round(v 2^(49-E)), |X| <=
-// 2^49, cut into ten signed 5-bit digits i = 0 .. 9 of weight 2^(-4 - 5 i).
-// All digit pairs of levels i + k <= 10 are summed (and some above), one level
-// more than the tiles of h2_tc.cu sum: the pairs left out stay below 2^-51 of
-// the scales' product, the rounding of X below 2^-50 of each scale, so that
-// the result is as accurate as double-float arithmetic (which it replaces
-// beyond 16 right-hand sides and for leaves of 22 to 32 triangles).
+// input (of each tree level, for the coupling) a power of two 2^F.  A block's value
+// becomes X = round(v 2^(49-E)), |X| <= 2^49, cut into ten signed 5-bit digits i =
+// 0 .. 9 of weight 2^(-4 - 5 i), an input value X = round(v 2^(54-F)) and eleven
+// digits.  All digit pairs of levels i + k <= 10 are summed (and some above): the
+// pairs left out stay below 2^-53 of the scales' product, the rounding of a block's
+// value below 2^-50 of its row's scale, that of an input value below 2^-55 of its
+// column's scale (at most four times the largest value).
+//
+// Range.  Double-float arithmetic, which this replaces, rounds every input value to
+// 2^-48 of itself, the digits to 2^-53 of the column's largest.  A column takes the
+// digits if at least half of its non-zero entries reach 2^-5 of the largest
+// (k_permute_in counts): those keep their 48 bits, and in the 2-norm the rounding
+// is at most 2^-53 2^5 sqrt(2) = 2^-47.5 of the column.  Evenly distributed columns do by a wide margin (uniform 97 %, normal
+// 87 % at 10^6 entries), and so do unit vectors; a pass with a column that
+// does not (a few entries far above the rest, values over many orders of magnitude)
+// is summed in double-float by the same CTAs over the same rows (rows_dd).
+// Errors in the 2-norm, 5,120 triangles graded 55 : 1 in size, order 3, 20
+// columns of entries in [-1, 1] and one of 1e8: 1.0e-10 without that rule, 1.3e-14
+// now, 1.7e-14 in double-float block rows.  The rule and the eleventh digit cost even
+// columns 0 to 1 % (81,920 triangles, 32 columns 853 -> 862 us; 5,120, one 62 us).
 //
 // Layout.  The digit planes of a block are stacked four to a 128-row MMA
 // operand: digit i (from 0) of row nu lies in group i / 4, row (i mod 4) R +
 // nu (three groups; K = 32 bytes, zero padded, K-major core matrices).  The
 // input digits of a column tile are the N side: digit k (from 0), column j in
 // row W k + j, W = 4, 8 or 16 columns per digit as the right-hand sides ask,
-// followed by an eleventh, zero plane.  Group g multiplies the planes k =
+// (the rows up to a multiple of 16 are zero).  Group g multiplies the planes k =
 // 0 .. 10 - 4 g into accumulator columns W (4 g + k) + j: the planes of a
 // group differ in i by their lane quarter only, so column block c = 4 g + k
 // holds, in lanes R q + nu, the sum of every pair of level i + k = c + q
@@ -79,7 +92,7 @@ constexpr uint32_t kTileSmemMax = 227 * 1024;
 
 // N rows (bytes / 32) of an input digit tile, columns of an accumulator set
 template <int W>
-__host__ __device__ constexpr int tile_n() { return (11 * W + 15) / 16 * 16; }
+__host__ __device__ constexpr int tile_n() { return (kTileDigits * W + 15) / 16 * 16; }
 
 // bytes of a four-plane group, of the stored last (two-plane) group and of a stored block
 __host__ __device__ inline uint32_t tile_group(int R) { return (uint32_t)((4 * R + 7) / 8 * 8) * 32u; }
@@ -103,14 +116,132 @@ struct TileArgs {
   const unsigned *xmax;       // column maxima (bits of a float)
   const int32_t *split;       // [gridDim.x + 1]: rows of every CTA
   dd *out;                    // [row][R][rp], at the first column of the pass
+  // the same rows in double-float (rows_dd), for the passes that need it; spread NULL: never
+  const int *spread;          // per column: negative where too few entries come near the largest
+  const dd *B, *Xd;           // blocks [K = R][Bp] (contraction index major), inputs [item][R][rp]
+  const int64_t *bptr;        // CSR over the output rows (from row0 on)
+  const int32_t *bcol;
+  int Bp;
   int R, ncol, rp, nst, accumulate;
   int64_t row0;               // output row of scheduled row value 0 (E, out, xmax are indexed from it)
   int by_level;               // xmax holds kXmaxCols maxima per tree level, output rows are clusters
   uint32_t stage, xch;        // bytes of a stage, of one exchange area
 };
 
+// The CTA's rows in double-float: two blocks and their inputs at a time, staged three
+// deep (cp.async); one of 256 threads sums four output rows of two columns, spare ones
+// take further slices of the contraction, added in order.  Every four blocks are summed
+// from zero and then added to the row, so that long rows keep the rounding error of
+// short sums.  Bound by the FP32 pipe (two warps per scheduler; the other two warps only
+// copy).  Whole products of wide columns, 81,920 triangles, order 3, 1 / 5 / 16 / 32
+// columns: 558 / 694 / 1,178 / 2,298 us; pipelined block rows on the same sums 531 / 637 / 1,053 / 1,871 us
+// (every product, before the digits).
+constexpr int kDdStages = 3, kDdThreads = 256;
+__host__ __device__ inline uint32_t rows_dd_stage(int R, int Bp, int ncol) {
+  return (uint32_t)(2 * R * (Bp + ncol) * (int)sizeof(dd));
+}
+__device__ __noinline__ void rows_dd(const TileArgs &a, int64_t r_begin, int64_t r_end, unsigned char *smem) {
+  const int R = a.R, Bp = a.Bp, nc = a.ncol, tid = threadIdx.x;
+  const uint32_t stage = rows_dd_stage(R, Bp, nc);
+  dd *red = reinterpret_cast<dd *>(smem + kDdStages * stage);   // [slice][tile][8], at most 8 values per thread
+  const int rg = (R + 3) / 4, tiles = rg * (nc / 2), slices = max(1, min(kDdThreads / tiles, R));
+  const int ks = tid / tiles, q = tid - ks * tiles, nu = 4 * (q % rg), c = 2 * (q / rg);
+  const int xo = 2 * tid / nc * a.rp + 2 * tid % nc;   // this thread's two values of an input
+  // The copies run ahead of the sums across rows: block pb (of blocks to pe - 1 of scheduled
+  // row pr) comes next; the bounds of the row after and the row after that are on their way.
+  int64_t pr = r_begin - 1, pb = 0, pe = 0, nb0 = 0, nb1 = 0;
+  int32_t t1 = r_begin < r_end ? a.row[r_begin] : 0, t2 = r_begin + 1 < r_end ? a.row[r_begin + 1] : 0, col[2];
+  if (r_begin < r_end) {
+    nb0 = a.bptr[t1];
+    nb1 = a.bptr[t1 + 1];
+  }
+  auto next_row = [&] {
+    pb = nb0;
+    pe = nb1;
+    if (++pr + 1 < r_end) {
+      nb0 = a.bptr[t2];
+      nb1 = a.bptr[t2 + 1];
+      if (pr + 2 < r_end) t2 = a.row[pr + 2];
+    }
+  };
+  auto seek = [&] {   // the next block's row and the columns of the next copy
+    while (pb >= pe && pr < r_end) next_row();
+#pragma unroll
+    for (int u = 0; u < 2; ++u) col[u] = pb + u < pe ? a.bcol[pb + u] : -1;
+  };
+  auto copy = [&](uint32_t i) {
+    if (pr < r_end) {
+      dd *sB = reinterpret_cast<dd *>(smem + (i % kDdStages) * stage), *sX = sB + 2 * R * Bp;
+      const dd *B = a.B + pb * R * Bp;
+      const int vals = (pb + 1 < pe ? 2 : 1) * R * Bp;
+      for (int o = 2 * tid; o < vals; o += 2 * kTileThreads) cp_async16(sB + o, B + o);
+      if (2 * tid < R * nc)
+#pragma unroll
+        for (int u = 0; u < 2; ++u)
+          if (col[u] >= 0) cp_async16(sX + u * R * nc + 2 * tid, a.Xd + (int64_t)col[u] * R * a.rp + xo);
+      pb = min(pb + 2, pe);
+    }
+    cp_async_commit();
+    seek();
+  };
+  seek();
+  for (int i = 0; i < kDdStages - 1; ++i) copy(i);
+  uint32_t step = 0;
+  for (int64_t r = r_begin; r < r_end; ++r) {
+    const int32_t t = t1;
+    const int nb = (int)(a.bptr[t + 1] - a.bptr[t]);
+    if (r + 1 < r_end) t1 = a.row[r + 1];
+    dd s[4][2] = {}, p[4][2] = {};
+    for (int i = 0; i < nb; i += 2, ++step) {
+      cp_async_wait<kDdStages - 2>();
+      __syncthreads();
+      copy(step + kDdStages - 1);   // into the stage before this one
+      if (ks < slices) {
+        const dd *sB = reinterpret_cast<const dd *>(smem + (step % kDdStages) * stage), *sX = sB + 2 * R * Bp;
+        const int K = (i + 1 < nb ? 2 : 1) * R;
+#pragma unroll 2
+        for (int mu = ks; mu < K; mu += slices) {
+          const float4 v0 = *reinterpret_cast<const float4 *>(sB + mu * Bp + nu);
+          const float4 v1 = *reinterpret_cast<const float4 *>(sB + mu * Bp + nu + 2);
+          const float4 x = *reinterpret_cast<const float4 *>(sX + mu * nc + c);
+          const dd v[4] = {{v0.x, v0.y}, {v0.z, v0.w}, {v1.x, v1.y}, {v1.z, v1.w}};
+#pragma unroll
+          for (int u = 0; u < 4; ++u) {
+            acc_fma(p[u][0], v[u], dd{x.x, x.y});
+            acc_fma(p[u][1], v[u], dd{x.z, x.w});
+          }
+        }
+        if ((i & 2) || i + 2 >= nb)
+#pragma unroll
+          for (int u = 0; u < 4; ++u)
+#pragma unroll
+            for (int w = 0; w < 2; ++w) {
+              acc_norm(p[u][w]);
+              s[u][w] = s[u][w] + p[u][w];
+              p[u][w] = dd{0.0f, 0.0f};
+            }
+      }
+    }
+    // the slices' sums, added in order by a thread per output
+    if (ks < slices)
+#pragma unroll
+      for (int u = 0; u < 8; ++u) red[(ks * tiles + q) * 8 + u] = s[u >> 1][u & 1];
+    __syncthreads();
+    for (int o = tid; o < R * nc; o += kTileThreads) {
+      const int ro = o / nc, co = o - ro * nc;
+      const dd *v = red + ((co >> 1) * rg + (ro >> 2)) * 8 + (ro & 3) * 2 + (co & 1);
+      dd sum = v[0];
+      for (int z = 1; z < slices; ++z) sum = sum + v[z * tiles * 8];
+      dd *y = a.out + ((a.row0 + t) * R + ro) * a.rp + co;
+      *y = a.accumulate ? *y + sum : sum;
+    }
+    __syncthreads();   // red is free again
+  }
+  cp_async_wait<0>();
+}
+
 template <int W>
-__global__ void __launch_bounds__(kTileThreads, 1) k_tile_tc(const TileArgs a) {
+__global__ void __launch_bounds__(kTileThreads, 1) k_tile_tc(const __grid_constant__ TileArgs a) {
   constexpr int N0 = tile_n<W>(), SET = W == 16 ? 256 : 128;
   constexpr uint32_t kX = (uint32_t)N0 * 32u;
   extern __shared__ __align__(1024) unsigned char smem[];
@@ -163,8 +294,12 @@ __global__ void __launch_bounds__(kTileThreads, 1) k_tile_tc(const TileArgs a) {
   // narrow tiles: CTAs of the next kernel beside a long tail cost more than their early start gives
   // (cube of 30,000 triangles, 5 columns 166 us with, 161 us without)
   if (W == 16) pdl_go();
+  const bool wide =
+      a.spread && __any_sync(0xffffffffu, lane < a.ncol && a.spread[min(lane, a.ncol - 1)] < 0);   // the same in every warp
 
-  if (warp == 0) {
+  if (wide) {
+    rows_dd(a, r_begin, r_end, smem);
+  } else if (warp == 0) {
     // ---------------- producer: the digits of every block of the range and of its column tile
     if (lane == 0) {
       int64_t e = e_begin;
@@ -375,10 +510,10 @@ __global__ void __launch_bounds__(kTileThreads, 1) k_tile_tc(const TileArgs a) {
 }
 
 // The input digit tiles of items first .. first + count - 1 (R rows of rp
-// values each, columns 0 .. ncol - 1 of x): 2 W threads per item, thread (g,
-// j) cuts rows 16 g .. 16 g + 15 of column j in registers (zero beyond R and
-// ncol) and writes one 16-byte row of a core matrix per plane, and the zero
-// rows behind the ten planes.
+// values each, columns 0 .. ncol - 1 of x): 4 W threads per item, thread (j, g)
+// cuts rows 8 g .. 8 g + 7 of column j in registers (zero beyond R and ncol) and
+// writes half a 16-byte row of a core matrix per plane, and of the zero rows behind the
+// eleven planes.  (Sixteen values per thread took 168 registers.)
 template <int W>
 __global__ void __launch_bounds__(128) k_tile_cut(const dd *__restrict__ x, int64_t first, int64_t count, int R,
                                                   int rp, int ncol, const unsigned *__restrict__ xmax, int by_level,
@@ -386,27 +521,28 @@ __global__ void __launch_bounds__(128) k_tile_cut(const dd *__restrict__ x, int6
   pdl_wait();
   pdl_go();
   constexpr int N0 = tile_n<W>();
-  const int64_t i = (int64_t)blockIdx.x * (64 / W) + threadIdx.x / (2 * W);
+  const int64_t i = (int64_t)blockIdx.x * (32 / W) + threadIdx.x / (4 * W);
   if (i >= count) return;
   const int64_t t = first + i;
-  const int g = (threadIdx.x / W) & 1, j = threadIdx.x % W;
-  const int sc = kTcFixBits - tc_colexp(j < ncol ? xmax[(by_level ? tc_level(t) * kXmaxCols : 0) + j] : 0u);
-  dd v[16];
+  // the halves of a core-matrix row are neighbouring lanes, then the columns
+  const int h = threadIdx.x & 1, j = (threadIdx.x >> 1) % W, c = (threadIdx.x / (2 * W)) & 1, g = 2 * c + h;
+  const int sc = kTileFixBits - tc_colexp(j < ncol ? xmax[(by_level ? tc_level(t) * kXmaxCols : 0) + j] : 0u);
+  dd v[8];
 #pragma unroll
-  for (int q = 0; q < 16; ++q) {
-    const int mu = 16 * g + q;
+  for (int q = 0; q < 8; ++q) {
+    const int mu = 8 * g + q;
     v[q] = mu < R && j < ncol ? x[(t * R + mu) * rp + j] : dd{0.0f, 0.0f};
   }
-  uint4 w[kTcSlices];
-  cut_row16<kTcSlices>(v, sc, w);
-  unsigned char *dst = X + t * (int64_t)(32 * N0) + g * 128;
+  uint32_t w[kTileDigits][2];
+  cut_row<kTileDigits, 8>(v, sc, w);
+  unsigned char *dst = X + t * (int64_t)(32 * N0) + c * 128 + h * 8;
 #pragma unroll
-  for (int k = 0; k < kTcSlices; ++k) {
+  for (int k = 0; k < kTileDigits; ++k) {
     const int n = W * k + j;
-    *reinterpret_cast<uint4 *>(dst + (n >> 3) * 256 + (n & 7) * 16) = w[k];
+    *reinterpret_cast<uint2 *>(dst + (n >> 3) * 256 + (n & 7) * 16) = make_uint2(w[k][0], w[k][1]);
   }
-  for (int n = W * kTcSlices + j; n < N0; n += W)
-    *reinterpret_cast<uint4 *>(dst + (n >> 3) * 256 + (n & 7) * 16) = make_uint4(0, 0, 0, 0);
+  for (int n = W * kTileDigits + j; n < N0; n += W)
+    *reinterpret_cast<uint2 *>(dst + (n >> 3) * 256 + (n & 7) * 16) = make_uint2(0, 0);
 }
 
 // E[t][nu] = 1 + floor(log2 max |G_b[nu][mu]|) over the near blocks b of leaf row t (0 if none)
@@ -540,6 +676,9 @@ int tile_launch(TileArgs a, int grid, cudaStream_t st) {
   a.stage = 3 * tile_group(a.R) + 32 * tile_n<W>();
   const uint32_t fixed = kTilePad + 2 * a.xch + 8 * (2 * kTileMaxStages + 5) + 16;
   a.nst = (int)std::min<uint32_t>(kTileMaxStages, (kTileSmemMax - fixed) / a.stage) / kTileGroup * kTileGroup;
+  // rows_dd's stages and sums take less than the ring's stages
+  if (a.spread && kDdStages * rows_dd_stage(a.R, a.Bp, a.ncol) + 8 * kDdThreads * sizeof(dd) > a.nst * a.stage + fixed)
+    return fail(H2_EINVAL, "double-float rows do not fit in shared memory");
   H2_CUDA_TRY(cudaFuncSetAttribute((const void *)k_tile_tc<W>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                    (int)kTileSmemMax));
   pdl(k_tile_tc<W>, grid, kTileThreads, a.nst * a.stage + fixed, st, a);
@@ -558,7 +697,7 @@ int tile_run(const TileArgs &a, int width, int grid, cudaStream_t st) {
 template <int W>
 void cut_launch(const dd *x, int64_t first, int64_t count, int R, int rp, int ncol, const unsigned *xmax, int by_level,
                 unsigned char *X, cudaStream_t st) {
-  constexpr int per = 64 / W;
+  constexpr int per = 32 / W;
   pdl(k_tile_cut<W>, (unsigned)((count + per - 1) / per), 128, 0, st, x, first, count, R, rp, ncol, xmax, by_level, X);
 }
 
@@ -700,8 +839,10 @@ void ntc_input(Ctx &c, const void *xpad, int rp, int c0, int ncol, bool wide) {
 
 // The nearfield phase (y_pad += or = the near sums), 16 columns per pass.
 // The input's column maxima are in place (k_permute_in); have_input: so are
-// the wide digit tiles of the one pass of at most 16 columns.
-int ntc_near(Ctx &c, const void *xpad, void *ypad, int rp, int accumulate, int64_t *launches, bool have_input) {
+// the wide digit tiles of the one pass of at most 16 columns.  ranged: columns of
+// wide range in double-float (their counts are in place too).
+int ntc_near(Ctx &c, const void *xpad, void *ypad, int rp, int accumulate, int64_t *launches, bool ranged,
+             bool have_input) {
   Dev &d = c.d;
   int64_t nl = 0;
   for (int c0 = 0; c0 < rp; c0 += kTcN) {
@@ -719,6 +860,12 @@ int ntc_near(Ctx &c, const void *xpad, void *ypad, int rp, int accumulate, int64
     a.split = d.ntc_s.split;
     a.E = d.ntc_E;
     a.xmax = d.ntc_xmax + c0;
+    a.spread = ranged ? d.spread + c0 : nullptr;
+    a.B = static_cast<const dd *>(d.near);
+    a.Bp = (int)d.lp;
+    a.bptr = d.near_ptr;
+    a.bcol = d.near_col;
+    a.Xd = static_cast<const dd *>(xpad) + c0;
     a.out = static_cast<dd *>(ypad) + c0;
     a.R = (int)d.lmax;
     a.ncol = ncol;
@@ -778,7 +925,8 @@ void tct_leaf_max(Ctx &c, const void *xhat, int rp) {
                                         d.tc_xmax + d.depth * kXmaxCols);
 }
 
-// the coupling phase, 16 columns per pass; the column maxima of every level are in place
+// the coupling phase, 16 columns per pass; the column maxima of every level and the input's
+// counts are in place
 int tct_coupling(Ctx &c, const void *xhat, void *yhat, int rp, int64_t *launches) {
   Dev &d = c.d;
   const int64_t row0 = ((int64_t)1 << d.first_adm_level) - 1;
@@ -796,6 +944,12 @@ int tct_coupling(Ctx &c, const void *xhat, void *yhat, int rp, int64_t *launches
     a.split = d.tc_s.split;
     a.E = d.tc_E;
     a.xmax = d.tc_xmax + c0;
+    a.spread = d.spread + c0;
+    a.B = static_cast<const dd *>(d.S);
+    a.Bp = d.kp;
+    a.bptr = d.adm_ptr + row0;
+    a.bcol = d.adm_col;
+    a.Xd = static_cast<const dd *>(xhat) + c0;
     a.out = static_cast<dd *>(yhat) + c0;
     a.R = d.k;
     a.ncol = ncol;

@@ -3,8 +3,10 @@
 // the digits reconstruct X exactly, each digit is an exact FP8 E4M3 value,
 // and the digit-pair products kept by the kernels (levels i + k <= ND, digits
 // counted from 0) reproduce X * Y to within the bound quoted there
-// (2^52 of 2^98 for ten digits, 2^31 of 2^58 for six).  Exit status 0 on
-// success.
+// (2^52 of 2^98 for ten digits, 2^31 of 2^58 for six).  For the small tiles, ten
+// digits of X (|X| <= 2^49) against eleven of Y (|Y| <= 2^54), pairs k <= 10 - 4
+// (i / 4): 2^50 of 2^103; the first ten of the eleven digits are Y rounded to ten.
+// Exit status 0 on success.
 #include <cuda_fp8.h>
 
 #include <cmath>
@@ -52,6 +54,37 @@ static int check(long long lim, int samples, long long bound) {
   return bad;
 }
 
+static int check_tile(int samples) {
+  std::mt19937_64 g(31337);
+  int bad = 0;
+  auto one = [&](long long X, long long Y) {
+    int s[10], t[11];
+    h2::split_digits<10>(X, s);
+    h2::split_digits<11>(Y, t);
+    long long ry = 0, head = 0;
+    for (int k = 0; k < 11; ++k) {
+      if (t[k] < -16 || t[k] > 16) ++bad;
+      if (k == 10) head = ry;
+      ry = ry * 32 + t[k];
+    }
+    if (ry != Y || std::llabs(32 * head - Y) > 16) ++bad;
+    __int128 kept = 0;
+    for (int i = 0; i < 10; ++i)
+      for (int k = 0; k <= 10 - 4 * (i / 4); ++k) kept += (__int128)(s[i] * t[k]) << (5 * (9 - i) + 5 * (10 - k));
+    __int128 err = (__int128)X * Y - kept;
+    if (err < 0) err = -err;
+    if (err > ((__int128)1 << 50)) ++bad;
+  };
+  const long long lx = 1LL << 49, ly = 1LL << 54;
+  for (long long a : {0LL, 1LL, -1LL, 16LL, -17LL, lx, -lx, lx - 1, 1 - lx})
+    for (long long b : {0LL, 1LL, -1LL, 16LL, -17LL, ly, -ly, ly - 1, 1 - ly, ly - 16, ly - 15}) one(a, b);
+  for (int e = 0; e < 54; ++e)
+    for (long long d = -17; d <= 17; ++d) one(lx - 7, (1LL << e) + d), one(3 - lx, -(1LL << e) + d);
+  std::uniform_int_distribution<long long> ux(-lx, lx), uy(-ly, ly);
+  for (int n = 0; n < samples; ++n) one(ux(g), uy(g));
+  return bad;
+}
+
 // split_digits_f (32-bit operations, float digits) against split_digits of
 // the 64-bit integer rint(hs) + rint(ls), for double-float pairs (hi, lo) and
 // FP32 values scaled as the kernels scale them (|hs| < 2^(5 ND - 2)), on
@@ -83,7 +116,7 @@ static int check_f(int samples) {
   for (int n = 0; n < samples; ++n) {
     const float hi = std::ldexp(u(g), ex(g));   // |hi| < 2^(5 ND - 2)
     float lo = 0.0f;
-    if (ND == 10) {
+    if (ND >= 10) {
       const float ul = std::nextafter(std::fabs(hi), INFINITY) - std::fabs(hi);
       lo = u(g) * ul * 0.5f;
     }
@@ -110,7 +143,9 @@ int main() {
   const int b10 = check<10>(1LL << 49, 2000000, 1LL << 52);
   const int b6 = check<6>(1LL << 29, 2000000, 1LL << 31);
   const int f10 = check_f<10>(2000000);
-  const int f6 = check_f<6>(2000000);
-  std::printf("e4m3 %d, ten digits %d, six digits %d, 32-bit cut %d / %d\n", bad, b10, b6, f10, f6);
-  return bad + b10 + b6 + f10 + f6 != 0;
+  const int f6 = check_f<6>(2000000), f11 = check_f<11>(2000000);
+  const int bt = check_tile(2000000);
+  std::printf("e4m3 %d, ten digits %d, six digits %d, ten by eleven %d, 32-bit cut %d / %d / %d\n", bad, b10, b6, bt, f10,
+              f6, f11);
+  return bad + b10 + b6 + bt + f10 + f6 + f11 != 0;
 }

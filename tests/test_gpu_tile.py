@@ -3,7 +3,7 @@ their range: leaves of 2 to 32 triangles, 1 to 64 right-hand sides (every tile
 width and several passes), and rows of many blocks (several exact segments).
 
 Tolerance: the digits are rounded to 2^-50 of their scales and the digit pairs
-left out stay below 2^-51 of them, so the double-float operations around them
+left out stay below 2^-53 of them, so the double-float operations around them
 (2^-44 = 5.7e-14 per operation) bound the error; 1e-13 against the FP64 oracle."""
 import numpy as np
 import pytest
@@ -50,6 +50,45 @@ def test_nearfield_long_rows(require_gpu, leaf):
             x = I.uniform_rhs(n, nrhs, 5100 + nrhs)
             assert _rel(h.matvec_host(x), o.matvec(x)) <= TOL, (n, nrhs)
         h.close()
+
+
+def _wide_columns(n, nrhs, seed):
+    """Columns whose values span many orders of magnitude, in turn: one entry far above the rest, two
+    opposite ones, values falling by 1e-12 over the mesh, log-normal values, and an even one."""
+    r = np.random.default_rng(seed)
+    x = r.uniform(-1.0, 1.0, (n, nrhs))
+    for j in range(nrhs):
+        kind, i = j % 5, int(r.integers(n - 1))
+        if kind == 0:
+            x[i, j] = 1e8
+        elif kind == 1:
+            x[i, j], x[i + 1, j] = 1e8, -1e8
+        elif kind == 2:
+            x[:, j] *= np.logspace(0, -12, n)
+        elif kind == 3:
+            x[:, j] = np.sign(x[:, j]) * np.exp(6 * r.standard_normal(n))
+    return x
+
+
+@pytest.mark.parametrize("order, leaf", [(3, 2), (3, 9), (3, 20), (3, 30), (2, 32), (4, 32)])
+def test_columns_of_wide_range(require_gpu, order, leaf):
+    """Digits below a column's largest value would drop the small values' bits: such columns are summed
+    in double-float, on a mesh whose triangles are graded 7 : 1 in size (so that the small values weigh in
+    the result); the coupling of order 3 and the nearfield of every order, beside even columns.  Order 4
+    only beyond 16 columns, where its coupling is double-float too.  Two opposite neighbours cancel to the
+    kernel's change over a triangle, a tenth of either or more: ten roundings of 2^-44 for those."""
+    n = 128 * leaf
+    v, f = I.icosphere(4)
+    v, f = v * np.exp(v[:, 2:3]), np.ascontiguousarray(f[:n])
+    o = oracle.Oracle(v, f, leaf_size=leaf, eta=2.0, order=order)
+    h = H2Matrix(v, f, leaf_size=leaf, eta=2.0, order=order, prec="f64")
+    assert h.stats["leaf_max"] == leaf and h.stats["tensor_near"] == 1
+    for nrhs in (1, 5, 16, 17, 40) if order < 4 else (17, 32):
+        x = _wide_columns(n, nrhs, 5500 + nrhs)
+        y, ref = h.matvec_host(x), o.matvec(x)
+        for c in range(nrhs):
+            assert _rel(y[:, c], ref[:, c]) <= (10 * 2.0**-44 if c % 5 == 1 else TOL), (nrhs, c)
+    h.close()
 
 
 def test_columns_with_infinity_or_nan(require_gpu):
