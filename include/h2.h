@@ -215,7 +215,9 @@ int h2_build_times(h2_handle h, double *ms);
  * their own where a column's values span many orders of magnitude, except in order-4
  * products of up to 16 columns with the coupling on the tensor cores: there
  * coefficients are rounded to 2^-48 of the column's largest of their tree level
- * (options.tensor = 1 has none of this).  Zero, infinite and NaN columns are passed as they are.
+ * (options.tensor = 1 has none of this).  A column with an infinity or a NaN gives NaN
+ * throughout, in H2_F64 and wherever the coupling runs on the tensor cores; the
+ * others are not touched by it.
  * Errors: H2_EINVAL (NULL, nrhs out of range), H2_ENOMEM (work buffers),
  * H2_ECUDA (launch failure). */
 int h2_matvec(h2_handle h, const void *x, void *y, int nrhs);

@@ -77,8 +77,13 @@ __device__ __forceinline__ double scale_pow2(double v, int e) {
 
 // a column with an infinity or a NaN: every output depends on every input (the
 // nearfield and the far field cover all pairs), so all its results are NaN;
-// digits cannot carry one, so the last permutation writes them
+// digits cannot carry one, so the last permutation writes them.  Double-float handles
+// find it in the input's maxima; the digit coupling of FP32 handles in the
+// coefficients' at the topmost level (bits of a float), which every leaf's
+// coefficients reach and where overflow on the way shows as well.
 __host__ __device__ inline bool not_finite(unsigned long long bits) { return ((bits >> 52) & 0x7ff) == 0x7ff; }
+
+__device__ __forceinline__ bool not_finite(unsigned bits) { return (bits & 0x7f800000u) == 0x7f800000u; }
 
 // the power of two by which column c is scaled (0: untouched; zero, infinite
 // and NaN columns are not scaled)
@@ -194,7 +199,8 @@ void permute_in(Ctx &c, bool ranged, unsigned grid, const Tin *x, int nrhs, int 
 template <class Tin, class Tout>
 __global__ void __launch_bounds__(256) k_permute_out(const Tin *__restrict__ ypad, int64_t n, int nrhs, int rp,
                                                      const int32_t *__restrict__ pad_src, int64_t npad,
-                                                     const unsigned long long *__restrict__ colmax, int acc,
+                                                     const unsigned long long *__restrict__ colmax,
+                                                     const unsigned *__restrict__ topmax, int acc,
                                                      Tout *__restrict__ y) {
   pdl_wait();
   pdl_go();
@@ -207,8 +213,9 @@ __global__ void __launch_bounds__(256) k_permute_out(const Tin *__restrict__ ypa
   const int64_t p0 = (int64_t)blockIdx.x * kPermRows;
   if (threadIdx.x < kPermRows) src[threadIdx.x] = p0 + threadIdx.x < npad ? pad_src[p0 + threadIdx.x] : -1;
   if (threadIdx.x < 64) shift[threadIdx.x] = (colmax && (int)threadIdx.x < nrhs) ? range_shift(colmax[threadIdx.x]) : 0;
-  if (threadIdx.x < 64)
-    poison[threadIdx.x] = colmax && (int)threadIdx.x < nrhs && not_finite(colmax[threadIdx.x]) ? __int_as_float(0x7fc00000) : 0.0f;
+  if ((int)threadIdx.x < nrhs)
+    poison[threadIdx.x] = (colmax && not_finite(colmax[threadIdx.x])) || (topmax && not_finite(topmax[threadIdx.x]))
+                              ? __int_as_float(0x7fc00000) : 0.0f;
   const int64_t rows = npad - p0 < kPermRows ? npad - p0 : kPermRows;
   for (int i = threadIdx.x; i < rows * rp; i += blockDim.x) {
     const int q = i / rp, c = i - q * rp;
@@ -1362,7 +1369,7 @@ int matvec_typed(Ctx &c, const Tio *x, Tio *y, int nrhs, bool acc) {
   }
   mk.mark(H2_PH_PERMUTE_OUT);
   pdl(k_permute_out<T, Tio>, perm_grid, 256, (size_t)kPermRows * (rp + 1) * sizeof(T), st, 
-      ypad, d.n, nrhs, rp, d.pad_src, d.npad, cmx, acc ? 1 : 0, y);
+      ypad, d.n, nrhs, rp, d.pad_src, d.npad, cmx, tcpath && !cmx ? d.tc_xmax + lmin * kLevelCols : nullptr, acc ? 1 : 0, y);
   mk.count(H2_PH_PERMUTE_OUT);
   mk.mark(H2_NPHASE);
   mk.finish();
@@ -1518,7 +1525,7 @@ int matvec_gca(Ctx &c, const Tio *x, Tio *y, int nrhs, bool acc) {
   }
   mk.mark(H2_PH_PERMUTE_OUT);
   pdl(k_permute_out<T, Tio>, perm_grid, 256, (size_t)kPermRows * (rp + 1) * sizeof(T), st, 
-      ypad, d.n, nrhs, rp, d.pad_src, d.npad, cmx, acc ? 1 : 0, y);
+      ypad, d.n, nrhs, rp, d.pad_src, d.npad, cmx, nullptr, acc ? 1 : 0, y);
   mk.count(H2_PH_PERMUTE_OUT);
   mk.mark(H2_NPHASE);
   mk.finish();
@@ -2044,7 +2051,7 @@ static bool capture_call(Ctx &c, CallGraph &g, const void *x, void *y) {
       g.nodes.push_back({nodes[i], 0, false});
       ++nin;
     } else if (std::find(std::begin(outs), std::end(outs), p.func) != std::end(outs)) {
-      g.nodes.push_back({nodes[i], 8, true});
+      g.nodes.push_back({nodes[i], 9, true});
       ++nout;
     }
   }
@@ -2070,7 +2077,7 @@ static cudaError_t aim_call(CallGraph &g, const void *x, void *y) {
     if (e != cudaSuccess) return e;
     // the node's own parameter values, with x or y exchanged
     void *args[10];
-    const int count = nd.out ? 9 : nd.arg + (p.func == (void *)k_colmax<double> ? 3 : 10);
+    const int count = nd.out ? 10 : nd.arg + (p.func == (void *)k_colmax<double> ? 3 : 10);
     for (int i = 0; i < count; ++i) args[i] = p.kernelParams[i];
     args[nd.arg] = nd.out ? (void *)&y : (void *)&x;
     p.kernelParams = args;

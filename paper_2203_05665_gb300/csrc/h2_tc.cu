@@ -205,13 +205,10 @@ __global__ void k_tc_slice_s(const int32_t *__restrict__ brow, const int32_t *__
 
 // ---------------------------------------------------------------- per product
 // xmax[j] = largest |x| (double-float: |hi|) of column j over rows [0, rows) of x
-// ([rows][rp], as float bits).  A warp reads 32 / LPR rows at a time with 16-byte
+// ([rows][rp], as float bits, infinities and NaN above all others).  A warp reads 32 / LPR rows at a time with 16-byte
 // loads (LPR lanes per row of 16 columns, lane l: row l / LPR, its EPV columns
 // from EPV (l % LPR)), so the reads are contiguous and every lane keeps fixed
 // columns; rp is a multiple of EPV (rows are padded to 16 bytes).
-__device__ __forceinline__ float mag(float v) { return fabsf(v); }
-__device__ __forceinline__ float mag(dd v) { return fabsf(v.hi); }
-
 template <class T>
 __global__ void k_tc_levmax(const T *__restrict__ x, int64_t rows, int rp, unsigned *__restrict__ xmax) {
   pdl_wait();
@@ -223,22 +220,22 @@ __global__ void k_tc_levmax(const T *__restrict__ x, int64_t rows, int rp, unsig
   const int lane = threadIdx.x & 31, sub = lane % LPR, nv = rp / EPV;
   const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
   const int64_t w = blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5);
-  float m[EPV];
+  unsigned m[EPV];
 #pragma unroll
-  for (int e = 0; e < EPV; ++e) m[e] = 0.0f;
+  for (int e = 0; e < EPV; ++e) m[e] = 0u;
   if (sub < nv)
     for (int64_t r = RPW * w + lane / LPR; r < rows; r += RPW * warps) {
       const T *p = x + r * rp + EPV * sub;
 #pragma unroll
-      for (int e = 0; e < EPV; ++e) m[e] = fmaxf(m[e], mag(p[e]));
+      for (int e = 0; e < EPV; ++e) m[e] = max(m[e], __float_as_uint(mag_of(p[e])));
     }
 #pragma unroll
   for (int e = 0; e < EPV; ++e)
-    for (int o = LPR; o < 32; o <<= 1) m[e] = fmaxf(m[e], __shfl_xor_sync(0xffffffffu, m[e], o));
+    for (int o = LPR; o < 32; o <<= 1) m[e] = max(m[e], __shfl_xor_sync(0xffffffffu, m[e], o));
   if (lane < nv)
 #pragma unroll
     for (int e = 0; e < EPV; ++e)
-      if (m[e] > 0.0f) atomicMax(&loc[EPV * lane + e], __float_as_uint(m[e]));
+      if (m[e]) atomicMax(&loc[EPV * lane + e], m[e]);
   __syncthreads();
   if (threadIdx.x < kTcN && loc[threadIdx.x]) atomicMax(&xmax[threadIdx.x], loc[threadIdx.x]);
 }

@@ -77,7 +77,8 @@ __device__ __forceinline__ void load_factors(const TS *__restrict__ Ef, int64_t 
 
 // Upward (Algorithm 1): x^_parent = sum over both children of E_c^T x^_c.
 // With xmax, also the largest |x^_parent| (|hi| for double-float) of every
-// column over the launch, as float bits (atomicMax).
+// column over the launch, as float bits (atomicMax; infinities and NaN are above all
+// others).
 __device__ __forceinline__ float mag_of(float v) { return fabsf(v); }
 __device__ __forceinline__ float mag_of(double v) { return (float)fabs(v); }
 __device__ __forceinline__ float mag_of(dd v) { return fabsf(v.hi); }
@@ -131,18 +132,18 @@ __global__ void __launch_bounds__(256, 2) k_up_reg(const TS *__restrict__ Ef, in
         out[jy][jx] = ch == 0 ? zero_of<T>() + r : out[jy][jx] + r;
       }
   }
-  float mx = 0.0f;
+  unsigned mx = 0u;
 #pragma unroll
   for (int jy = 0; jy < M; ++jy)
 #pragma unroll
     for (int jx = 0; jx < M; ++jx) {
       if (act) xhat[(par * K + jx + M * jy + M * M * jz) * rp + j] = out[jy][jx];
-      if (act) mx = fmaxf(mx, mag_of(out[jy][jx]));
+      if (act) mx = max(mx, __float_as_uint(mag_of(out[jy][jx])));
     }
   if (xmax) {
-    mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
-    mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
-    if (act && jz == 0 && mx > 0.0f) atomicMax(&loc[j & 15], __float_as_uint(mx));
+    mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
+    mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
+    if (act && jz == 0 && mx) atomicMax(&loc[j & 15], mx);
     __syncthreads();
     if (threadIdx.x < 16 && loc[threadIdx.x]) atomicMax(&xmax[16 * blockIdx.y + threadIdx.x], loc[threadIdx.x]);
   }
@@ -212,7 +213,7 @@ __global__ void __launch_bounds__(256, 2) k_up_split(const TS *__restrict__ Ef, 
 #pragma unroll
       for (int jx = 0; jx < M; ++jx) R[pl][jx + M * jy][t] = a[jy][jx];
   __syncthreads();
-  float mx = 0.0f;
+  unsigned mx = 0u;
   if (ch == 0)
 #pragma unroll
     for (int jy = 0; jy < M; ++jy)
@@ -220,12 +221,12 @@ __global__ void __launch_bounds__(256, 2) k_up_split(const TS *__restrict__ Ef, 
       for (int jx = 0; jx < M; ++jx) {
         const T o = (zero_of<T>() + a[jy][jx]) + R[pl][jx + M * jy][t];
         if (act) xhat[(par * K + jx + M * jy + M * M * jz) * rp + j] = o;
-        if (act) mx = fmaxf(mx, mag_of(o));
+        if (act) mx = max(mx, __float_as_uint(mag_of(o)));
       }
   if (xmax) {
-    mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
-    mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
-    if (ch == 0 && act && jz == 0 && mx > 0.0f) atomicMax(&loc[j & 15], __float_as_uint(mx));
+    mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
+    mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
+    if (ch == 0 && act && jz == 0 && mx) atomicMax(&loc[j & 15], mx);
     __syncthreads();
     if (threadIdx.x < 16 && loc[threadIdx.x]) atomicMax(&xmax[16 * blockIdx.y + threadIdx.x], loc[threadIdx.x]);
   }

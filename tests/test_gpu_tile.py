@@ -111,6 +111,26 @@ def test_columns_with_infinity_or_nan(require_gpu):
         h.close()
 
 
+@pytest.mark.parametrize("nrhs", [4, 9, 16])
+def test_columns_with_infinity_or_nan_f32(require_gpu, nrhs):
+    """The same for FP32 handles whose coupling cuts the coefficients into digits (order 4), with either
+    kind of transfer kernel (register kernels: more than 8 columns, 4,096 columns times parents)."""
+    import torch
+    v, f = I.icosphere(4)
+    n = f.shape[0]
+    h = H2Matrix(v, f, leaf_size=4, eta=2.0, order=4, prec="f32")
+    assert h.stats["tensor"] == 1
+    x = colmajor(torch.from_numpy(I.uniform_rhs(n, nrhs, 5200)).float().cuda())
+    y0, y1 = colmajor(torch.empty_like(x)), colmajor(torch.empty_like(x))
+    h.matvec(x, y0)
+    x[7, 1], x[n - 1, 3] = float("inf"), float("nan")
+    h.matvec(x, y1)
+    good = [c for c in range(nrhs) if c not in (1, 3)]
+    assert torch.isnan(y1[:, [1, 3]]).all()
+    assert torch.equal(y0[:, good], y1[:, good])
+    h.close()
+
+
 @pytest.mark.parametrize("mesh, leaf", [("patch", 32), ("cube", 16), ("cube", 40), ("ellipsoid", 24)])
 def test_order3_coupling(require_gpu, mesh, leaf):
     """The order-3 coupling: ragged leaves, leaves beyond the tensor-core nearfield (40), rows of up to
