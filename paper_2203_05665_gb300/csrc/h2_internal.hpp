@@ -9,6 +9,7 @@
 #include <vector>
 
 #include "../../include/h2.h"
+#include "h2_callgraph.hpp"
 
 namespace h2 {
 
@@ -225,27 +226,6 @@ struct StreamWork {
   cudaStream_t in = nullptr, out = nullptr;
   cudaEvent_t ev_in[2] = {nullptr, nullptr}, ev_done[2] = {nullptr, nullptr}, ev_out[2] = {nullptr, nullptr};
 };
-
-// A product captured as a CUDA graph for repeated calls with the same number of
-// right-hand sides (run_matvec): only the nodes that read x or write y change
-// from call to call
-struct CallGraph {
-  struct Node {
-    cudaGraphNode_t node;
-    int arg;                      // index of the x or y parameter
-    bool out;
-  };
-  int nrhs = 0;
-  bool io64 = false, acc = false;
-  int64_t work_gen = -1;          // work buffers the capture refers to
-  uint64_t used = 0;              // call count of the last use
-  cudaGraph_t graph = nullptr;
-  cudaGraphExec_t exec = nullptr; // NULL until the second call
-  const void *x = nullptr;
-  void *y = nullptr;
-  std::vector<Node> nodes;
-};
-constexpr int kMaxCallGraphs = 4;
 
 struct Ctx {
   CallGraph calls[kMaxCallGraphs];

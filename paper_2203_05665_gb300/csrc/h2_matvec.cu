@@ -2070,8 +2070,7 @@ static bool capture_call(Ctx &c, CallGraph &g, const void *x, void *y) {
 
 // Point the graph's nodes at this call's x and y.
 static cudaError_t aim_call(CallGraph &g, const void *x, void *y) {
-  for (const CallGraph::Node &nd : g.nodes) {
-    if (nd.out ? y == g.y : x == g.x) continue;
+  return aim_nodes(g, x, y, [&](const CallGraph::Node &nd) {
     cudaKernelNodeParams p{};
     cudaError_t e = cudaGraphKernelNodeGetParams(nd.node, &p);
     if (e != cudaSuccess) return e;
@@ -2081,11 +2080,8 @@ static cudaError_t aim_call(CallGraph &g, const void *x, void *y) {
     for (int i = 0; i < count; ++i) args[i] = p.kernelParams[i];
     args[nd.arg] = nd.out ? (void *)&y : (void *)&x;
     p.kernelParams = args;
-    if ((e = cudaGraphExecKernelNodeSetParams(g.exec, nd.node, &p)) != cudaSuccess) return e;
-  }
-  g.x = x;
-  g.y = y;
-  return cudaSuccess;
+    return cudaGraphExecKernelNodeSetParams(g.exec, nd.node, &p);
+  });
 }
 
 // y = G~ x (or y += G~ x).  A product is 15 to 30 launches, whose cost on the
