@@ -49,4 +49,20 @@ cudaError_t aim_nodes(CallGraph &g, const void *x, void *y, Set set) {
   return cudaSuccess;
 }
 
+// Run body with the handle's stream replaced by cap and put it back however body ends;
+// false where it failed or threw (an error message that could not be allocated), so that
+// the caller ends the capture on cap in any case.
+template <class Body>
+bool run_on(cudaStream_t &stream, cudaStream_t cap, Body body) {
+  const cudaStream_t own = stream;
+  stream = cap;
+  bool ok = false;
+  try {
+    ok = body();
+  } catch (...) {
+  }
+  stream = own;
+  return ok;
+}
+
 }  // namespace h2

@@ -2013,14 +2013,12 @@ void free_call_graphs(Ctx &c) {
 // Capture the product into g on a private stream and find the nodes that take
 // the caller's x and y.  On any failure nothing is kept and the status says so.
 static bool capture_call(Ctx &c, CallGraph &g, const void *x, void *y) {
-  cudaStream_t cap = nullptr, own = c.stream;
+  cudaStream_t cap = nullptr;
   if (cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking) != cudaSuccess) return false;
   const int slast = c.d.last_nrhs, slast_rp = c.d.last_rp;
   bool ok = cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal) == cudaSuccess;
   if (ok) {
-    c.stream = cap;
-    ok = launch_matvec(c, x, y, g.nrhs, g.io64, g.acc) == H2_OK;
-    c.stream = own;
+    ok = run_on(c.stream, cap, [&] { return launch_matvec(c, x, y, g.nrhs, g.io64, g.acc) == H2_OK; });
     ok = cudaStreamEndCapture(cap, &g.graph) == cudaSuccess && ok;
   }
   cudaStreamDestroy(cap);
@@ -2092,7 +2090,7 @@ static cudaError_t aim_call(CallGraph &g, const void *x, void *y) {
 // nodes have been given this call's x and y.  Launch by launch: the first call,
 // products while the stream is being captured or phases are timed, the
 // allocation-free entry point, the single-launch product, and whatever a
-// capture refuses.  5,120 triangles, one column: 102 -> 72 us per product;
+// capture or a change of vectors refuses.  5,120 triangles, one column: 102 -> 72 us per product;
 // 327,680, 16 columns 3,540 -> 3,476 us.
 int run_matvec(Ctx &c, const void *x, void *y, int nrhs, bool io64, bool acc) {
   Dev &d = c.d;
@@ -2130,13 +2128,14 @@ int run_matvec(Ctx &c, const void *x, void *y, int nrhs, bool io64, bool acc) {
   try {
     ok = ok || capture_call(c, *g, x, y);
   } catch (const std::bad_alloc &) {
-    drop_graph(*g);
+    ok = false;
   }
-  if (!ok) {
+  if (!ok || aim_call(*g, x, y) != cudaSuccess) {
+    cudaGetLastError();
+    drop_graph(*g);
     c.direct = true;
     return launch_matvec(c, x, y, nrhs, io64, acc);
   }
-  H2_CUDA_TRY(aim_call(*g, x, y));
   H2_CUDA_TRY(cudaGraphLaunch(g->exec, c.stream));
   d.last_nrhs = nrhs;
   d.last_rp = rp;

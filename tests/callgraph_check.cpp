@@ -2,6 +2,7 @@
 // with failing driver calls.  Exit status 0 on success.
 #include <cstdio>
 #include <map>
+#include <new>
 
 #include "h2_callgraph.hpp"
 
@@ -51,7 +52,17 @@ static void aim_after_failure(int failing) {
   CHECK(aim(x0, y1) == cudaSuccess && count == before);
 }
 
+// a product that throws while its stream is replaced
+static void stream_after_throw() {
+  cudaStream_t own = reinterpret_cast<cudaStream_t>(uintptr_t(8)), cap = reinterpret_cast<cudaStream_t>(uintptr_t(16));
+  cudaStream_t stream = own;
+  CHECK(!h2::run_on(stream, cap, [&]() -> bool { throw std::bad_alloc(); }) && stream == own);
+  CHECK(!h2::run_on(stream, cap, [&] { return stream != cap; }) && stream == own);
+  CHECK(h2::run_on(stream, cap, [&] { return stream == cap; }) && stream == own);
+}
+
 int main() {
+  stream_after_throw();
   for (int failing = 1; failing <= 3; ++failing) aim_after_failure(failing);
   return bad != 0;
 }
