@@ -6,6 +6,8 @@
 #include <cuda_runtime_api.h>
 
 #include <cstdint>
+#include <tuple>
+#include <type_traits>
 #include <vector>
 
 namespace h2 {
@@ -15,7 +17,7 @@ namespace h2 {
 struct CallGraph {
   struct Node {
     cudaGraphNode_t node;
-    int arg;                      // index of the x or y parameter
+    int arg, count;               // index of the x or y parameter, number of parameters
     bool out;
   };
   int nrhs = 0;
@@ -29,6 +31,27 @@ struct CallGraph {
   std::vector<Node> nodes;
 };
 constexpr int kMaxCallGraphs = 4;
+
+// How a kernel's node is pointed at a vector, from the kernel's own signature: x is the
+// first parameter of those that read it, y the last of those that write it.
+struct VectorKernel {
+  const void *kernel;
+  int arg, count;
+  bool out;
+};
+constexpr int kMaxParams = 16;
+template <class T, class... P>
+VectorKernel reads_x(void (*kernel)(const T *, P...)) {
+  static_assert(sizeof...(P) < kMaxParams, "parameters");
+  return {reinterpret_cast<const void *>(kernel), 0, 1 + (int)sizeof...(P), false};
+}
+template <class... P>
+VectorKernel writes_y(void (*kernel)(P...)) {
+  using Last = std::tuple_element_t<sizeof...(P) - 1, std::tuple<P...>>;
+  static_assert(sizeof...(P) <= kMaxParams, "parameters");
+  static_assert(std::is_pointer<Last>::value && !std::is_const<std::remove_pointer_t<Last>>::value, "y comes last");
+  return {reinterpret_cast<const void *>(kernel), (int)sizeof...(P) - 1, (int)sizeof...(P), true};
+}
 
 // Point the graph's nodes at this call's x and y: set(node) exchanges a node's
 // parameter.  After a failure some nodes point at the new vectors and some at the

@@ -2028,13 +2028,13 @@ static bool capture_call(Ctx &c, CallGraph &g, const void *x, void *y) {
   ok = ok && cudaGraphGetNodes(g.graph, nullptr, &n) == cudaSuccess;
   std::vector<cudaGraphNode_t> nodes(ok ? n : 0);
   ok = ok && cudaGraphGetNodes(g.graph, nodes.data(), &n) == cudaSuccess;
-  const void *ins[] = {(const void *)k_permute_in<double, dd, false>, (const void *)k_permute_in<double, dd, true>,
-                       (const void *)k_permute_in<double, double, false>,
-                       (const void *)k_permute_in<double, float, false>,
-                       (const void *)k_permute_in<float, float, false>};
-  const void *outs[] = {(const void *)k_permute_out<dd, double>, (const void *)k_permute_out<double, double>,
-                        (const void *)k_permute_out<float, double>, (const void *)k_permute_out<float, float>};
-  int nin = 0, nout = 0, nmax = 0;
+  const VectorKernel kernels[] = {reads_x(k_colmax<double>), reads_x(k_permute_in<double, dd, false>),
+                                  reads_x(k_permute_in<double, dd, true>), reads_x(k_permute_in<double, double, false>),
+                                  reads_x(k_permute_in<double, float, false>),
+                                  reads_x(k_permute_in<float, float, false>), writes_y(k_permute_out<dd, double>),
+                                  writes_y(k_permute_out<double, double>), writes_y(k_permute_out<float, double>),
+                                  writes_y(k_permute_out<float, float>)};
+  int nin = 0, nout = 0;
   for (size_t i = 0; ok && i < n; ++i) {
     cudaGraphNodeType type;
     ok = cudaGraphNodeGetType(nodes[i], &type) == cudaSuccess;
@@ -2042,18 +2042,14 @@ static bool capture_call(Ctx &c, CallGraph &g, const void *x, void *y) {
     cudaKernelNodeParams p{};
     ok = cudaGraphKernelNodeGetParams(nodes[i], &p) == cudaSuccess;
     if (!ok) break;
-    if (p.func == (void *)k_colmax<double>) {
-      g.nodes.push_back({nodes[i], 0, false});
-      ++nmax;
-    } else if (std::find(std::begin(ins), std::end(ins), p.func) != std::end(ins)) {
-      g.nodes.push_back({nodes[i], 0, false});
-      ++nin;
-    } else if (std::find(std::begin(outs), std::end(outs), p.func) != std::end(outs)) {
-      g.nodes.push_back({nodes[i], 9, true});
-      ++nout;
-    }
+    for (const VectorKernel &v : kernels)
+      if (p.func == v.kernel) {
+        g.nodes.push_back({nodes[i], v.arg, v.count, v.out});
+        ++(v.out ? nout : nin);
+      }
   }
-  ok = ok && nin == 1 && nout == 1 && nmax == (c.d.prec == H2_F64 ? 1 : 0) &&
+  // double-float products read x twice (column maxima, permutation)
+  ok = ok && nin == (c.d.prec == H2_F64 ? 2 : 1) && nout == 1 &&
        cudaGraphInstantiate(&g.exec, g.graph, 0) == cudaSuccess;
   if (!ok) {
     cudaGetLastError();
@@ -2073,9 +2069,8 @@ static cudaError_t aim_call(CallGraph &g, const void *x, void *y) {
     cudaError_t e = cudaGraphKernelNodeGetParams(nd.node, &p);
     if (e != cudaSuccess) return e;
     // the node's own parameter values, with x or y exchanged
-    void *args[10];
-    const int count = nd.out ? 10 : nd.arg + (p.func == (void *)k_colmax<double> ? 3 : 10);
-    for (int i = 0; i < count; ++i) args[i] = p.kernelParams[i];
+    void *args[kMaxParams];
+    for (int i = 0; i < nd.count; ++i) args[i] = p.kernelParams[i];
     args[nd.arg] = nd.out ? (void *)&y : (void *)&x;
     p.kernelParams = args;
     return cudaGraphExecKernelNodeSetParams(g.exec, nd.node, &p);

@@ -21,7 +21,7 @@ static void aim_after_failure(int failing) {
   void *y0 = &v[2], *y1 = &v[3];
   for (uintptr_t i = 1; i <= 3; ++i) {
     const cudaGraphNode_t n = reinterpret_cast<cudaGraphNode_t>(i);
-    g.nodes.push_back({n, 0, i == 3});
+    g.nodes.push_back({n, 0, 1, i == 3});
     at[n] = i == 3 ? y0 : x0;
   }
   g.x = x0;
@@ -61,7 +61,13 @@ static void stream_after_throw() {
   CHECK(h2::run_on(stream, cap, [&] { return stream == cap; }) && stream == own);
 }
 
+static void first(const float *, int, double *) {}
+static void last(const float *, int, int, double *) {}
+
 int main() {
+  const h2::VectorKernel in = h2::reads_x(first), out = h2::writes_y(last);
+  CHECK(!in.out && in.arg == 0 && in.count == 3 && in.kernel == reinterpret_cast<const void *>(first));
+  CHECK(out.out && out.arg == 3 && out.count == 4 && out.kernel == reinterpret_cast<const void *>(last));
   stream_after_throw();
   for (int failing = 1; failing <= 3; ++failing) aim_after_failure(failing);
   return bad != 0;
