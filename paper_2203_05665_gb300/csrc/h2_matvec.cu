@@ -2010,6 +2010,16 @@ void free_call_graphs(Ctx &c) {
   for (CallGraph &g : c.calls) drop_graph(g);
 }
 
+// While one lives, the calls of this thread that make and free graphs do not count as
+// unsafe beside a capture that somebody else has open (of another stream on this
+// thread, or with the global mode on any other): they concern this library's own
+// objects alone, and a product launched kernel by kernel makes none of them.
+struct RelaxedCapture {
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+  RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+  ~RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+};
+
 // Capture the product into g on a private stream and find the nodes that take
 // the caller's x and y.  On any failure nothing is kept and the status says so.
 static bool capture_call(Ctx &c, CallGraph &g, const void *x, void *y) {
@@ -2102,6 +2112,7 @@ int run_matvec(Ctx &c, const void *x, void *y, int nrhs, bool io64, bool acc) {
     if (cs == cudaStreamCaptureStatusNone) cudaGetLastError();
     return launch_matvec(c, x, y, nrhs, io64, acc);
   }
+  const RelaxedCapture relaxed;
   CallGraph *g = nullptr;
   for (CallGraph &q : c.calls)
     if (q.nrhs == nrhs && q.io64 == wide && q.acc == acc) g = &q;

@@ -69,3 +69,53 @@ def test_product_in_a_capture(require_gpu):
     assert torch.equal(y, 2.0 * ref)
     del g
     h.close()
+
+
+@pytest.mark.parametrize("where", ["thread", "other thread"])
+def test_products_beside_a_capture(require_gpu, where):
+    """Products on the handle's own stream while another stream is being captured in the global mode (by
+    this thread, or by another): neither disturbs the other, also where the product makes a graph (the
+    second with its number of right-hand sides) or drops one (the sixth number of them)."""
+    import threading
+    import torch
+    s, other = torch.cuda.Stream(), torch.cuda.Stream()
+    h = _mat("f64", stream=s.cuda_stream)
+    xs = {nrhs: _x(h.n, nrhs, 7300 + nrhs, torch.float64) for nrhs in (5, 1, 2, 3, 4, 6)}
+    ref = {nrhs: colmajor(torch.empty_like(x)) for nrhs, x in xs.items()}
+    ys = {nrhs: [colmajor(torch.empty_like(x)) for _ in range(3)] for nrhs, x in xs.items()}
+    z = torch.zeros(8, device="cuda")
+    torch.cuda.synchronize()
+    h.matvec(xs[6], ref[6])   # the work buffers exist
+    for nrhs, x in xs.items():
+        first = _mat("f64")
+        first.matvec(x, ref[nrhs])
+        first.close()
+    torch.cuda.synchronize()
+    errors = []
+
+    def products():
+        try:
+            for nrhs, x in xs.items():
+                for y in ys[nrhs]:
+                    h.matvec(x, y)
+        except Exception as e:   # raised by the test's own thread below
+            errors.append(e)
+
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=other):
+        z.add_(1)
+        if where == "thread":
+            products()
+        else:
+            t = threading.Thread(target=products)
+            t.start()
+            t.join()
+        z.add_(1)
+    assert not errors, errors
+    g.replay()
+    torch.cuda.synchronize()
+    assert z[0].item() == 2
+    for nrhs in xs:
+        assert all(torch.equal(y, ref[nrhs]) for y in ys[nrhs]), nrhs
+    del g
+    h.close()
