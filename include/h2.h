@@ -217,7 +217,10 @@ int h2_build_times(h2_handle h, double *ms);
  * coefficients are rounded to 2^-48 of the column's largest of their tree level
  * (options.tensor = 1 has none of this).  A column with an infinity or a NaN gives NaN
  * throughout, in H2_F64 and wherever the coupling runs on the tensor cores; the
- * others are not touched by it.
+ * others are not touched by it.  k nrhs and leaf_max nrhs (nrhs padded to 16
+ * bytes) must not exceed 4096; FP64 products whose tiles of 4 rows by 16 bytes
+ * exceed 256 run in equal groups of columns (order 5: beyond 16, order 4 and leaves
+ * of 64: beyond 32).
  * Errors: H2_EINVAL (NULL, nrhs out of range), H2_ENOMEM (work buffers),
  * H2_ECUDA (launch failure). */
 int h2_matvec(h2_handle h, const void *x, void *y, int nrhs);
@@ -281,7 +284,8 @@ int h2_matvec_host_stream(h2_handle h, const double *x, double *y, int nrhs, int
 /* Coefficients of the last product (diagnostics): which = 0 gives x^ after
  * the forward transformation, 1 gives y^ after the interaction and the
  * downward transfer (as used by the leaf backward step).  out: HOST double
- * array [clusters][k][nrhs] of the last product's nrhs. */
+ * array [clusters][k][nrhs] of the last product's nrhs.  H2_EINVAL after a product
+ * that ran in groups of columns (see h2_matvec). */
 int h2_coefficients(h2_handle h, int which, double *out);
 
 /* The stored representation as built on the device, converted to double

@@ -600,6 +600,7 @@ int h2_matvec_host_stream(h2_handle h, const double *x, double *y, int nrhs, int
 int h2_coefficients(h2_handle h, int which, double *out) {
   if (!h || !out || (which != 0 && which != 1)) return fail(H2_EINVAL, "bad argument");
   if (h->d.gca) return fail(H2_EINVAL, "GCA-H^2 handles have per-level ranks; use h2_export");
+  if (h->d.last_nrhs < 0) return fail(H2_EINVAL, "the last product ran in groups of columns; its coefficients are not kept");
   if (h->d.last_nrhs < 1) return fail(H2_EINVAL, "no product has run on this handle");
   H2_CUDA_TRY(cudaSetDevice(h->device));
   H2_CUDA_TRY(cudaStreamSynchronize(h->stream));

@@ -2087,6 +2087,16 @@ static cudaError_t aim_call(CallGraph &g, const void *x, void *y) {
   });
 }
 
+// Columns (padded) that one product takes: a block-row CTA has a thread per register
+// tile, so the larger of the coefficient and leaf tiles bounds them.  16 for order 5
+// in FP64 (128 rows), 32 for 64 rows, 64 up to 32 rows; FP32 always takes 64.
+static int pass_columns(const Dev &d) {
+  const int VN = 16 / (int)d.esize;
+  auto most = [&](int Mp) { return kThreads / (Mp / (4 * (d.esize == 4 && Mp % 8 == 0 ? 2 : 1))) * VN; };
+  const bool far = d.first_adm_level <= d.depth;
+  return std::max(VN, std::min(far ? most(d.kp) : 64, most((int)d.lp)));
+}
+
 // y = G~ x (or y += G~ x).  A product is 15 to 30 launches, whose cost on the
 // host and gaps on the device are those of one graph once it is captured: from
 // the second call with the same number of right-hand sides on, a graph kept on
@@ -2103,9 +2113,21 @@ int run_matvec(Ctx &c, const void *x, void *y, int nrhs, bool io64, bool acc) {
   const int rp = padded_rhs(nrhs, d.esize);
   if ((int64_t)d.k * rp > kThreads * kMaxOut || d.lmax * rp > kThreads * kMaxOut)
     return fail(H2_EINVAL, "k * nrhs and leaf_max * nrhs (nrhs padded to 16 bytes) must not exceed 4096");
-  int rc = ensure_work(c, nrhs);
-  if (rc) return rc;
+  int rc;
   const bool wide = io64 || d.esize == 8;   // the types of x and y
+  const int most = pass_columns(d);
+  if (rp > most && !d.gca && !single_launch(d)) {
+    // equal groups of columns, one product each
+    const int passes = (rp + most - 1) / most, width = padded_rhs((nrhs + passes - 1) / passes, d.esize);
+    const size_t col = (size_t)d.n * (wide ? 8 : 4);
+    for (int c0 = 0; c0 < nrhs; c0 += width)
+      if ((rc = run_matvec(c, (const char *)x + c0 * col, (char *)y + c0 * col, std::min(width, nrhs - c0), io64, acc)))
+        return rc;
+    if (c.prof.on) c.prof.products -= (nrhs + width - 1) / width - 1;
+    d.last_nrhs = -1;   // no one group's coefficients are those of the product
+    return H2_OK;
+  }
+  if ((rc = ensure_work(c, nrhs))) return rc;
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
   if (c.direct || c.prof.on || single_launch(d)) return launch_matvec(c, x, y, nrhs, io64, acc);
   if (cudaStreamIsCapturing(c.stream, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) {
