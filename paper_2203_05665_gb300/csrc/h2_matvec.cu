@@ -1010,26 +1010,23 @@ int launch_rows(const Rows &rows, const RowCfg &cfg, int threads, int R, int64_t
 
 
 // Leaf steps (Algorithm 1 at the leaves, x^_t = V_t^T x|t; Algorithm 2 at the
-// leaves, y|t = V_t y^_t) for leaves of at most 32 triangles and k <= 64, up to
-// 16 columns (c0 .. c0 + nc - 1) per launch: one CTA per leaf stages V_t
-// (converted to the arithmetic type) and the leaf's vector block in shared
-// memory; in the forward step thread
-// (nu, jq) forms x^[nu][jq + 4u], in the backward step thread (r, jo) forms
-// y[r][jo + 8u], each as one contraction with a single renormalisation, then
-// multiplied by the leaf's power-of-two scale (16-bit storage) if there is
-// one; with MAX the forward step also takes the largest |x^| (|hi|) of every
-// column, as float bits.  The generic block-row kernel pipelines many terms
+// leaves, y|t = V_t y^_t) of FP64 handles and of GCA-H^2 handles, for leaves of at
+// most 32 triangles and k <= 64, up to 16 columns (c0 .. c0 + nc - 1) per launch: one
+// CTA per leaf stages V_t and the leaf's vector block in shared memory; in the
+// forward step thread (nu, jq) forms x^[nu][jq + 4u], in the backward step thread
+// (r, jo) forms y[r][jo + 8u], each as one contraction with a single
+// renormalisation; with MAX the forward step also takes the largest |hi| of every
+// column of x^, as float bits.  The generic block-row kernel pipelines many terms
 // per row; a leaf row has one (more than 16 columns took one block-row launch
 // before: 81,920 triangles, order 3, 32 columns, FP64-accurate: product 891 ->
 // 881 us with two passes here).  Bound by the FP32 pipe.  The columns of a
 // thread are fixed at compile time, with indices clamped to the last column: a
 // test per column and term kept the double-float chains of a thread apart
-// (327,680 triangles, order 4, 16 columns: backward and nearfield 578 -> 563 us; 15,000,
+// (327,680 triangles, order 4, 16 columns: backward and nearfield 578 -> 563 us; 30,000,
 // order 3, 5 columns: forward 14.5 -> 12.3 us).
-template <class TS, class T, bool MAX>
-__global__ void __launch_bounds__(256) k_leaf_fwd_reg(const TS *__restrict__ V, const T *__restrict__ xpad,
-                                                      const float *__restrict__ vscale, int L, int kp, int k, int rp,
-                                                      int c0, int nc, T *__restrict__ xleaf,
+template <class T, bool MAX>
+__global__ void __launch_bounds__(256) k_leaf_fwd_reg(const T *__restrict__ V, const T *__restrict__ xpad, int L,
+                                                      int kp, int k, int rp, int c0, int nc, T *__restrict__ xleaf,
                                                       unsigned *__restrict__ xmax) {
   pdl_wait();
   pdl_go();
@@ -1039,14 +1036,13 @@ __global__ void __launch_bounds__(256) k_leaf_fwd_reg(const TS *__restrict__ V, 
   T *Vs = reinterpret_cast<T *>(lsm);   // [L][kp]
   T *xs = Vs + L * kp;                   // [L][nc]
   const int64_t t = blockIdx.x;
-  const TS *vt = V + t * (int64_t)L * kp;
+  const T *vt = V + t * (int64_t)L * kp;
   const T *xt = xpad + t * (int64_t)L * rp + c0;
-  for (int i = threadIdx.x; i < L * kp; i += blockDim.x) Vs[i] = to_compute<T>(vt[i]);
+  for (int i = threadIdx.x; i < L * kp; i += blockDim.x) Vs[i] = vt[i];
   for (int i = threadIdx.x; i < L * nc; i += blockDim.x) xs[i] = xt[i / nc * rp + i % nc];
   __syncthreads();
   const int nu = threadIdx.x >> 2, jq = threadIdx.x & 3;
   if (nu < k) {
-    const float sc = vscale ? vscale[t] : 1.0f;
     // NU columns jq + 4u; those beyond nc repeat the last one
     auto sum = [&](auto nuc) {
       constexpr int NU = decltype(nuc)::value;
@@ -1066,9 +1062,8 @@ __global__ void __launch_bounds__(256) k_leaf_fwd_reg(const TS *__restrict__ V, 
       for (int u = 0; u < NU; ++u)
         if (jq + 4 * u < nc) {
           acc_norm(acc[u]);
-          const T v = vscale ? acc[u] * from_double<T>(sc) : acc[u];
-          xleaf[(t * k + nu) * rp + c0 + jq + 4 * u] = v;
-          if (MAX) atomicMax(&smax[jq + 4 * u], __float_as_uint(mag_of(v)));
+          xleaf[(t * k + nu) * rp + c0 + jq + 4 * u] = acc[u];
+          if (MAX) atomicMax(&smax[jq + 4 * u], __float_as_uint(mag_of(acc[u])));
         }
     };
     if (nc > 8)
@@ -1085,24 +1080,22 @@ __global__ void __launch_bounds__(256) k_leaf_fwd_reg(const TS *__restrict__ V, 
   }
 }
 
-template <class TS, class T>
-__global__ void __launch_bounds__(256) k_leaf_bwd_reg(const TS *__restrict__ Vt, const T *__restrict__ yleaf,
-                                                      const float *__restrict__ vscale, int L, int Lp, int k, int rp,
-                                                      int c0, int nc, T *__restrict__ ypad) {
+template <class T>
+__global__ void __launch_bounds__(256) k_leaf_bwd_reg(const T *__restrict__ Vt, const T *__restrict__ yleaf, int L,
+                                                      int Lp, int k, int rp, int c0, int nc, T *__restrict__ ypad) {
   pdl_wait();
   pdl_go();
   extern __shared__ __align__(16) unsigned char lsm[];
   T *Vs = reinterpret_cast<T *>(lsm);   // [k][Lp]
   T *ys = Vs + k * Lp;                   // [k][nc]
   const int64_t t = blockIdx.x;
-  const TS *vt = Vt + t * (int64_t)k * Lp;
+  const T *vt = Vt + t * (int64_t)k * Lp;
   const T *yt = yleaf + t * (int64_t)k * rp + c0;
-  for (int i = threadIdx.x; i < k * Lp; i += blockDim.x) Vs[i] = to_compute<T>(vt[i]);
+  for (int i = threadIdx.x; i < k * Lp; i += blockDim.x) Vs[i] = vt[i];
   for (int i = threadIdx.x; i < k * nc; i += blockDim.x) ys[i] = yt[i / nc * rp + i % nc];
   __syncthreads();
   const int r = threadIdx.x >> 3, jo = threadIdx.x & 7;
   if (r >= L) return;
-  const float sc = vscale ? vscale[t] : 1.0f;
   auto sum = [&](auto nuc) {
     constexpr int NU = decltype(nuc)::value;
     T acc[NU];
@@ -1121,7 +1114,7 @@ __global__ void __launch_bounds__(256) k_leaf_bwd_reg(const TS *__restrict__ Vt,
     for (int u = 0; u < NU; ++u)
       if (jo + 8 * u < nc) {
         acc_norm(acc[u]);
-        ypad[(t * L + r) * rp + c0 + jo + 8 * u] = vscale ? acc[u] * from_double<T>(sc) : acc[u];
+        ypad[(t * L + r) * rp + c0 + jo + 8 * u] = acc[u];
       }
   };
   if (nc > 8)
@@ -1189,8 +1182,9 @@ int matvec_typed(Ctx &c, const Tio *x, Tio *y, int nrhs, bool acc) {
   bool leaf_max = leaf_tc;   // the leaf step takes its coefficients' column maxima
   // FP32 arithmetic, tiles of at most 64 rows: one or four warps per block row
   const bool lane = std::is_same<T, float>::value && L <= kLaneMax && k <= kLaneMax;
-  // leaf steps with one CTA per leaf
-  const bool leaf_reg = L <= 32 && k <= 64;
+  // leaf steps with one CTA per leaf (FP64; FP32 arithmetic of these sizes takes the rows above)
+  constexpr bool wide = sizeof(T) == 8;
+  const bool leaf_reg = wide && L <= 32 && k <= 64;
   if (leaf_tc) {
     ntc_input(c, xpad, rp, 0, rp, true);
     if ((rc = tc_leaf_forward(c, xhat, rp))) return rc;
@@ -1210,18 +1204,19 @@ int matvec_typed(Ctx &c, const Tio *x, Tio *y, int nrhs, bool acc) {
     if ((rc = lane_rows(g, d.v32 ? (int)H2_F32 : d.prec, false, &nl, st))) return rc;
     mk.count(H2_PH_LEAF_FORWARD, nl);
   } else if (far && leaf_reg) {
-    T *xl = xhat + leaf0 * (int64_t)k * rp;
-    leaf_max = cpl_tile || (std::is_same<T, dd>::value && tcpath && d.prec == H2_F64);
-    for (int c0 = 0; c0 < rp; c0 += 16) {
-      const int nc = std::min(16, rp - c0);
-      const size_t sm = (size_t)L * (kp + nc) * sizeof(T);
-      if (leaf_max)
-        pdl(k_leaf_fwd_reg<TV, T, true>, (unsigned)d.nleaf, 256, sm, st, (const TV *)d.V, xpad, vscale, L, kp, k, rp,
-            c0, nc, xl, d.tc_xmax + D * kLevelCols + c0);
-      else
-        pdl(k_leaf_fwd_reg<TV, T, false>, (unsigned)d.nleaf, 256, sm, st, (const TV *)d.V, xpad, vscale, L, kp, k, rp,
-            c0, nc, xl, nullptr);
-      mk.count(H2_PH_LEAF_FORWARD);
+    if constexpr (wide) {
+      T *xl = xhat + leaf0 * (int64_t)k * rp;
+      leaf_max = std::is_same<T, dd>::value && (cpl_tile || tcpath);
+      for (int c0 = 0; c0 < rp; c0 += 16) {
+        const int nc = std::min(16, rp - c0);
+        const size_t sm = (size_t)L * (kp + nc) * sizeof(T);
+        auto fwd = k_leaf_fwd_reg<T, false>;
+        if constexpr (std::is_same<T, dd>::value)
+          if (leaf_max) fwd = k_leaf_fwd_reg<T, true>;
+        pdl(fwd, (unsigned)d.nleaf, 256, sm, st, (const T *)d.V, xpad, L, kp, k, rp, c0, nc, xl,
+            leaf_max ? d.tc_xmax + D * kLevelCols + c0 : nullptr);
+        mk.count(H2_PH_LEAF_FORWARD);
+      }
     }
   } else if (far) {
     LeafForwardRows<TV, T> rows{(const TV *)d.V, xpad, vscale, L, kp, rp};
@@ -1310,13 +1305,14 @@ int matvec_typed(Ctx &c, const Tio *x, Tio *y, int nrhs, bool acc) {
     // FP32 arithmetic: the leaf backward step, the FP32 self blocks of bfloat16 handles and the
     // nearfield as one sum per leaf row
   } else if (far && leaf_reg) {
-    for (int c0 = 0; c0 < rp; c0 += 16) {
-      const int nc = std::min(16, rp - c0);
-      const size_t sm = (size_t)k * (Lp + nc) * sizeof(T);
-      pdl(k_leaf_bwd_reg<TV, T>, (unsigned)d.nleaf, 256, sm, st, (const TV *)d.Vt, yhat + leaf0 * (int64_t)k * rp,
-          vscale, L, Lp, k, rp, c0, nc, ypad);
-      mk.count(H2_PH_LEAF_NEAR);
-    }
+    if constexpr (wide)
+      for (int c0 = 0; c0 < rp; c0 += 16) {
+        const int nc = std::min(16, rp - c0);
+        const size_t sm = (size_t)k * (Lp + nc) * sizeof(T);
+        pdl(k_leaf_bwd_reg<T>, (unsigned)d.nleaf, 256, sm, st, (const T *)d.Vt, yhat + leaf0 * (int64_t)k * rp, L, Lp,
+            k, rp, c0, nc, ypad);
+        mk.count(H2_PH_LEAF_NEAR);
+      }
   } else if (far) {
     LeafBackwardRows<TV, T> rows{(const TV *)d.Vt, yhat, vscale, k, Lp, rp, leaf0};
     if ((rc = launch_rows<TV, T>(rows, cf_back, t_back, RL, d.nleaf, 0, ypad, st))) return rc;
@@ -1431,6 +1427,7 @@ int gca_rows_launch(const Rows &rows, int M, int Mp, int Kmax, int rp, int64_t n
 // padded rank.  Coefficients of level l start at gX[l] * rp.
 template <class TS, class T, class Tio>
 int matvec_gca(Ctx &c, const Tio *x, Tio *y, int nrhs, bool acc) {
+  static_assert(std::is_same<TS, T>::value, "stored in the arithmetic type");
   Dev &d = c.d;
   cudaStream_t st = c.stream;
   const int L = (int)d.lmax, Lp = (int)d.lp, D = d.depth, lmin = d.first_adm_level;
@@ -1470,8 +1467,8 @@ int matvec_gca(Ctx &c, const Tio *x, Tio *y, int nrhs, bool acc) {
   mk.mark(H2_PH_LEAF_FORWARD);
   if (far && leaf_reg) {
     const size_t sm = (size_t)L * (KD + rp) * sizeof(T);
-    pdl(k_leaf_fwd_reg<TS, T, false>, (unsigned)d.nleaf, 256, sm, st, (const TS *)d.V, xpad, nullptr, L, KD, KD, rp,
-        0, rp, X(xhat, D), nullptr);
+    pdl(k_leaf_fwd_reg<T, false>, (unsigned)d.nleaf, 256, sm, st, (const T *)d.V, xpad, L, KD, KD, rp, 0, rp,
+        X(xhat, D), nullptr);
     mk.count(H2_PH_LEAF_FORWARD);
   } else if (far) {
     LeafForwardRows<TS, T> rows{(const TS *)d.V, xpad, nullptr, L, KD, rp};
@@ -1506,8 +1503,7 @@ int matvec_gca(Ctx &c, const Tio *x, Tio *y, int nrhs, bool acc) {
   mk.mark(H2_PH_LEAF_NEAR);
   if (far && leaf_reg) {
     const size_t sm = (size_t)KD * (Lp + rp) * sizeof(T);
-    pdl(k_leaf_bwd_reg<TS, T>, (unsigned)d.nleaf, 256, sm, st, (const TS *)d.Vt, X(yhat, D), nullptr, L, Lp, KD, rp, 0,
-        rp, ypad);
+    pdl(k_leaf_bwd_reg<T>, (unsigned)d.nleaf, 256, sm, st, (const T *)d.Vt, X(yhat, D), L, Lp, KD, rp, 0, rp, ypad);
     mk.count(H2_PH_LEAF_NEAR);
   } else if (far) {
     LeafBackwardRows<TS, T> rows{(const TS *)d.Vt, X(yhat, D), nullptr, KD, Lp, rp, 0};

@@ -708,8 +708,8 @@ int tc_build_nd(Ctx &c) {
 }
 
 // Upward pass of a product on the tensor-core path: the transfers of
-// Algorithm 1, each level's column maxima taken on the way (k_up_reg /
-// k_up_split; the leaves' by k_tc_levmax), then the coefficient digits of
+// Algorithm 1, each level's column maxima taken on the way (launch_up; the leaves' by the
+// leaf step or k_tc_levmax), then the coefficient digits of
 // every far-field level in one launch (k_tc_slice_x, each cluster with its
 // level's maxima).  Cutting a level's digits inside the next level's
 // transfer launch was slower: the transfer threads are latency bound.

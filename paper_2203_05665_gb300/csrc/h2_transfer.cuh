@@ -44,10 +44,6 @@ __device__ __forceinline__ float to_compute<float, __half>(__half v) {
 constexpr int kRegParents = 4;   // parents per 256-thread CTA
 
 __device__ __forceinline__ float shfl_t(float v, int src) { return __shfl_sync(0xffffffffu, v, src); }
-__device__ __forceinline__ double shfl_t(double v, int src) { return __shfl_sync(0xffffffffu, v, src); }
-__device__ __forceinline__ dd shfl_t(dd v, int src) {
-  return dd{__shfl_sync(0xffffffffu, v.hi, src), __shfl_sync(0xffffffffu, v.lo, src)};
-}
 
 // out[a] = sum_b F[a][b] in[b] (plain, E) or sum_b F[b][a] in[b] (trans, E^T)
 template <class T, bool TRANS, int M>
@@ -152,7 +148,7 @@ __global__ void __launch_bounds__(256, 2) k_up_reg(const TS *__restrict__ Ef, in
 // Child-split variants: 128 threads per parent, the two 64-thread halves
 // taking one child each (two parents per 256-thread CTA), so every thread
 // forms half the mode products.  On levels with few parents a CTA's time is
-// the latency of one thread's chain of double-float operations, which this
+// the latency of one thread's chain of operations, which this
 // halves.  The second child's part is added to the first through shared memory
 // in the order of k_up_reg (same bits).
 constexpr int kSplitParents = 2;   // parents per 256-thread CTA
@@ -244,7 +240,7 @@ __global__ void __launch_bounds__(256, 2) k_up_split(const TS *__restrict__ Ef, 
 // operations in the same order as there, so the bits are the same.  Narrow
 // levels: 8 - 9 us per level with the register kernels (order 4, double-float),
 // 4 - 5 us here; 81,920 triangles, order 4, one column, all upward levels 122
-// -> 64 us.
+// -> 64 us (51 us with the shorter sums of mode_pair).
 template <class T>
 struct alignas(2 * sizeof(T)) Pair {
   T a, b;
@@ -430,7 +426,7 @@ void launch_up_m(const TS *Ef, int rp, int64_t par0, int64_t npar, T *xhat, unsi
         Ef, rp, np, pp, par0, npar, xhat, xmax);
     return;
   }
-  if constexpr (M == 3 || M == 4) {
+  if constexpr (sizeof(T) == 4 && (M == 3 || M == 4)) {   // the only ones pair_up leaves
     const int gy = (rp + 15) / 16;
     if (npar <= kUpSplitMax)
       pdl(k_up_split<TS, T, M>, dim3((unsigned)((npar + kSplitParents - 1) / kSplitParents), gy), 256, 0, st, 
