@@ -194,7 +194,7 @@ def run_ours(args):
     if args.prec == "f64n":
         roof = {"bound": "alu", "achieved": alg["coupling_flops"] / (cpl_ms * 1e-3) / 1e12, "peak": FP64_TFLOPS,
                 "unit": "TFLOP/s", "kernel": "k_blockrow (coupling, FP64 FMA pipe)"}
-    elif args.prec == "f64" and st.get("tensor", 0) and args.order == 4:
+    elif args.prec == "f64" and st.get("tensor", 0) and args.order == 4 and nrhs <= 16:
         # tensor-core coupling: a stream of the stored slices; algorithmic bytes are
         # those of the FP64 coupling matrices (k^2 x 8 B per block) and coefficients
         # stored_stream_frac: the E4M3 digit planes of S alone (10 B per entry), the part
@@ -206,10 +206,17 @@ def run_ours(args):
                 "stored_bytes_per_entry": 10,
                 "stored_stream_frac": (st["adm_blocks"] * 10 * st["rank"] ** 2 / (cpl_ms * 1e-3) / 1e9
                                        / peaks["hbm_gbs"])}
+    elif args.prec == "f64" and st.get("tensor", 0) and args.order == 3:
+        # the same with the small tiles: 280 rows of 32 bytes per block (8,960 B, ten digits
+        # of 27 x 27 entries padded to K = 32), read once per pass of 16 columns
+        roof = {"bound": "hbm", "achieved": alg["coupling_bytes"] / (cpl_ms * 1e-3) / 1e9, "peak": peaks["hbm_gbs"],
+                "unit": "GB/s", "kernel": "k_tile_tc (tcgen05 kind::f8f6f4, ten by eleven 5-bit E4M3 digits)",
+                "stored_bytes_per_block": 8960,
+                "stored_stream_frac": (st["adm_blocks"] * 8960 * -(-nrhs // 16) / (cpl_ms * 1e-3) / 1e9
+                                       / peaks["hbm_gbs"])}
     elif args.prec == "f64":
         roof = {"bound": "alu", "achieved": alg["coupling_flops"] / (cpl_ms * 1e-3) / 1e12, "peak": DD_TFLOPS,
-                "unit": "TFLOP/s", "kernel": ("k_tile_tc (coupling, tcgen05 digits)" if st.get("tensor", 0) else
-                                              "k_blockrow (coupling, double-float on the FP32 pipe)"),
+                "unit": "TFLOP/s", "kernel": "k_blockrow (coupling, double-float on the FP32 pipe)",
                 "hbm_frac": alg["coupling_bytes"] / (cpl_ms * 1e-3) / 1e9 / peaks["hbm_gbs"]}
     elif args.prec in ("bf16", "f16"):
         # regenerated coupling: 2 k^2 nrhs multiply-adds plus one kernel evaluation
@@ -227,13 +234,13 @@ def run_ours(args):
     # same kernel at level 5 (profiles/k_coupling_tc_icosphere_L5_m4_16rhs_f64.md,
     # profiles/k_blockrow_coupling_icosphere_L5_m4_16rhs_f64.md), scaled by
     # admissible blocks; None where no capture of the current kernel exists
-    tc = args.prec == "f64" and st.get("tensor", 0) and args.order == 4
+    tc = args.prec == "f64" and st.get("tensor", 0) and args.order == 4 and nrhs <= 16
     traffic_per_block = {"f64": 691.93e6 / 18876, "f64-tc": (794.690048e6 + 7.657472e6) / 18876}
     key = "f64-tc" if tc else args.prec
     roof["traffic"] = (traffic_per_block[key] * st["adm_blocks"]
                        if key in traffic_per_block and args.order == 4 and args.nrhs == 16 else None)
     roof["peak_source"] = {"f64n": "nominal FP64 rate",
-                           "f64": (f"{peaks['src']} HBM copy bandwidth" if tc else
+                           "f64": (f"{peaks['src']} HBM copy bandwidth" if roof["bound"] == "hbm" else
                                    "FP32 FMA rate (152 SMs x 128 lanes x 2.07 GHz) / 12 instructions per dd FMA"),
                            "f32": f"{peaks['src']} HBM copy bandwidth",
                            "bf16": "FP32 FMA rate (152 SMs x 128 lanes x 2 flop x 2.07 GHz)",

@@ -123,7 +123,8 @@ typedef struct h2_stats {
   int64_t near_blocks;    /* inadmissible leaves */
   int64_t near_entries;   /* sum over inadmissible leaves of |t| |s| */
   int64_t first_adm_level;/* smallest level holding an admissible block */
-  int64_t device_bytes;   /* device memory held by the handle (without work buffers) */
+  int64_t device_bytes;   /* device memory held by the handle (without work buffers, and without what
+                           * the driver takes for the graphs of repeated products, some 100 KB each) */
   int64_t prec;           /* enum h2_prec */
   int64_t coupling;       /* H2_COUPLING_STORED or H2_COUPLING_REGEN as built */
   int64_t tensor;         /* 1 if the tensor-core digits of the coupling were built */

@@ -48,7 +48,7 @@
 // (h2_tile.cu), so that the CTAs read the coefficient tiles of one
 // neighbourhood at a time and L2 holds them.  327,680 triangles, 16 right-hand
 // sides: FP64-accurate 2,197 -> 1,905 us (6.6 TB/s of stored digits, 0.97 of the
-// copy bandwidth), FP32 1,515 -> 1,184 us (6.4 TB/s).  Every wait is bounded; on a timeout the
+// copy bandwidth), FP32 1,515 -> 1,173 us (6.4 TB/s).  Every wait is bounded; on a timeout the
 // device error word is raised, every role stops, copies and MMAs in flight
 // are waited for and the tensor memory is released before the CTA exits.
 #include <cuda_fp8.h>

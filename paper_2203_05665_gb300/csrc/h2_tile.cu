@@ -57,12 +57,12 @@
 // What bounds it: the copy stream and the MMA warp's issue.  Nearfield of
 // 327,680 triangles (leaves of 20, 179,008 blocks of 6.4 KB and as many input
 // tiles of 5.6 KB), 16 columns: 480 us before (one epilogue group, separate
-// accumulator columns per plane group, single-stage commits), 354 us now, 6.1
+// accumulator columns per plane group, single-stage commits), 351 us now, 6.1
 // TB/s into shared memory.  Leaves of 30 (cube, 30,000 triangles, 5 columns):
 // 161 us in double-float block rows, 47 us now; 32 right-hand sides, 81,920
 // triangles: 414 us in double-float, 215 us now (two passes).  Order-3
 // coupling, double-float block rows before: 81,920 triangles, 32 right-hand
-// sides (75,224 blocks of 9.0 KB, two passes) 1,070 us, now 393 us with the
+// sides (75,224 blocks of 9.0 KB, two passes) 1,070 us, now 381 us with the
 // digit cuts; cube of 30,000 triangles, 5 columns 195 us, now 62 us; 5,120
 // triangles, one column 35 us, now 22 us.
 #include <algorithm>
@@ -291,8 +291,10 @@ __global__ void __launch_bounds__(kTileThreads, 1) k_tile_tc(const __grid_consta
   const uint32_t tbase = *tslot;
   const int64_t seg = tile_seg(R);
   pdl_wait();   // everything above is set-up data and this CTA's own
-  // narrow tiles: CTAs of the next kernel beside a long tail cost more than their early start gives
-  // (cube of 30,000 triangles, 5 columns 166 us with, 161 us without)
+  // narrow tiles: CTAs of the next kernel beside a long tail cost more than their early start
+  // gives.  Products of 5 columns with and without: 5,120 triangles 66 and 60 us, 20,480 124
+  // and 119, 81,920 337 and 334, cubes of 4,800 64 and 60, 30,000 155 and 150, 129,792 343
+  // and 340; one column the same either way
   if (W == 16) pdl_go();
   const bool wide =
       a.spread && __any_sync(0xffffffffu, lane < a.ncol && a.spread[min(lane, a.ncol - 1)] < 0);   // the same in every warp
