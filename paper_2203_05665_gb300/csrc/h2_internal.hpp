@@ -275,7 +275,7 @@ int tc_leaf_build(Ctx &c);
 // (the tensor-core leaf step reads those)
 bool ntc_eligible(const Dev &d);
 int ntc_build(Ctx &c);
-void ntc_input(Ctx &c, const void *xpad, int rp, int c0, int ncol, bool wide);
+void ntc_input(Ctx &c, const void *xpad, int rp, int c0, int ncol, bool wide, bool ranged);
 int ntc_near(Ctx &c, const void *xpad, void *ypad, int rp, int accumulate, int64_t *launches, bool ranged,
              bool have_input = false);
 int tile_take_error(cudaStream_t st);

@@ -1186,7 +1186,7 @@ int matvec_typed(Ctx &c, const Tio *x, Tio *y, int nrhs, bool acc) {
   constexpr bool wide = sizeof(T) == 8;
   const bool leaf_reg = wide && L <= 32 && k <= 64;
   if (leaf_tc) {
-    ntc_input(c, xpad, rp, 0, rp, true);
+    ntc_input(c, xpad, rp, 0, rp, true, ranged);
     if ((rc = tc_leaf_forward(c, xhat, rp))) return rc;
     mk.count(H2_PH_LEAF_FORWARD, 2);
   } else if (far && lane) {

@@ -21,9 +21,11 @@
 // digits if at least half of its non-zero entries reach 2^-5 of the largest
 // (k_permute_in counts): those keep their 48 bits, and in the 2-norm the rounding
 // is at most 2^-53 2^5 sqrt(2) = 2^-47.5 of the column.  Evenly distributed columns do by a wide margin (uniform 97 %, normal
-// 87 % at 10^6 entries), and so do unit vectors; a pass with a column that
-// does not (a few entries far above the rest, values over many orders of magnitude)
-// is summed in double-float by the same CTAs over the same rows (rows_dd).
+// 87 % at 10^6 entries), and so do unit vectors; a column that does not (a few
+// entries far above the rest, values over many orders of magnitude) is summed in
+// double-float by the same CTAs over the same rows (rows_dd), after the digits of
+// the pass's other columns (its own are cut as zeros), so that no column's result
+// depends on another's values.
 // Errors in the 2-norm, 5,120 triangles graded 55 : 1 in size, order 3, 20
 // columns of entries in [-1, 1] and one of 1e8: 1.0e-10 without that rule, 1.3e-14
 // now, 1.7e-14 in double-float block rows.  The rule and the eleventh digit cost even
@@ -116,8 +118,9 @@ struct TileArgs {
   const unsigned *xmax;       // column maxima (bits of a float)
   const int32_t *split;       // [gridDim.x + 1]: rows of every CTA
   dd *out;                    // [row][R][rp], at the first column of the pass
-  // the same rows in double-float (rows_dd), for the passes that need it; spread NULL: never
+  // the same rows in double-float (rows_dd), for the columns that need it; spread NULL: none
   const int *spread;          // per column: negative where too few entries come near the largest
+  const unsigned long long *colmax;   // per column: 0 where the input vanishes
   const dd *B, *Xd;           // blocks [K = R][Bp] (contraction index major), inputs [item][R][rp]
   const int64_t *bptr;        // CSR over the output rows (from row0 on)
   const int32_t *bcol;
@@ -128,11 +131,12 @@ struct TileArgs {
   uint32_t stage, xch;        // bytes of a stage, of one exchange area
 };
 
-// The CTA's rows in double-float: two blocks and their inputs at a time, staged three
+// The CTA's rows of the columns in mask in double-float: two blocks and their inputs at a time, staged three
 // deep (cp.async); one of 256 threads sums four output rows of two columns, spare ones
 // take further slices of the contraction, added in order.  Every four blocks are summed
 // from zero and then added to the row, so that long rows keep the rounding error of
-// short sums.  Bound by the FP32 pipe (two warps per scheduler; the other two warps only
+// short sums.  Threads and slices are those of all columns of the pass, whichever are
+// in mask.  Bound by the FP32 pipe (two warps per scheduler; the other two warps only
 // copy).  Whole products of wide columns, 81,920 triangles, order 3, 1 / 5 / 16 / 32
 // columns: 558 / 694 / 1,178 / 2,298 us; pipelined block rows on the same sums 531 / 637 / 1,053 / 1,871 us
 // (every product, before the digits).
@@ -140,12 +144,14 @@ constexpr int kDdStages = 3, kDdThreads = 256;
 __host__ __device__ inline uint32_t rows_dd_stage(int R, int Bp, int ncol) {
   return (uint32_t)(2 * R * (Bp + ncol) * (int)sizeof(dd));
 }
-__device__ __noinline__ void rows_dd(const TileArgs &a, int64_t r_begin, int64_t r_end, unsigned char *smem) {
+__device__ __noinline__ void rows_dd(const TileArgs &a, int64_t r_begin, int64_t r_end, unsigned char *smem,
+                                     uint32_t mask) {
   const int R = a.R, Bp = a.Bp, nc = a.ncol, tid = threadIdx.x;
   const uint32_t stage = rows_dd_stage(R, Bp, nc);
   dd *red = reinterpret_cast<dd *>(smem + kDdStages * stage);   // [slice][tile][8], at most 8 values per thread
   const int rg = (R + 3) / 4, tiles = rg * (nc / 2), slices = max(1, min(kDdThreads / tiles, R));
   const int ks = tid / tiles, q = tid - ks * tiles, nu = 4 * (q % rg), c = 2 * (q / rg);
+  const bool on = ks < slices && (mask >> c & 3u);
   const int xo = 2 * tid / nc * a.rp + 2 * tid % nc;   // this thread's two values of an input
   // The copies run ahead of the sums across rows: block pb (of blocks to pe - 1 of scheduled
   // row pr) comes next; the bounds of the row after and the row after that are on their way.
@@ -196,7 +202,7 @@ __device__ __noinline__ void rows_dd(const TileArgs &a, int64_t r_begin, int64_t
       cp_async_wait<kDdStages - 2>();
       __syncthreads();
       copy(step + kDdStages - 1);   // into the stage before this one
-      if (ks < slices) {
+      if (on) {
         const dd *sB = reinterpret_cast<const dd *>(smem + (step % kDdStages) * stage), *sX = sB + 2 * R * Bp;
         const int K = (i + 1 < nb ? 2 : 1) * R;
 #pragma unroll 2
@@ -223,12 +229,13 @@ __device__ __noinline__ void rows_dd(const TileArgs &a, int64_t r_begin, int64_t
       }
     }
     // the slices' sums, added in order by a thread per output
-    if (ks < slices)
+    if (on)
 #pragma unroll
       for (int u = 0; u < 8; ++u) red[(ks * tiles + q) * 8 + u] = s[u >> 1][u & 1];
     __syncthreads();
     for (int o = tid; o < R * nc; o += kTileThreads) {
       const int ro = o / nc, co = o - ro * nc;
+      if (!(mask >> co & 1u)) continue;
       const dd *v = red + ((co >> 1) * rg + (ro >> 2)) * 8 + (ro & 3) * 2 + (co & 1);
       dd sum = v[0];
       for (int z = 1; z < slices; ++z) sum = sum + v[z * tiles * 8];
@@ -256,8 +263,8 @@ __global__ void __launch_bounds__(kTileThreads, 1) k_tile_tc(const __grid_consta
   uint32_t *tslot = reinterpret_cast<uint32_t *>(done + 1);
   volatile int *abort = reinterpret_cast<volatile int *>(tslot + 1);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int64_t r_begin = a.split[blockIdx.x], r_end = a.split[blockIdx.x + 1];
-  const int64_t e_begin = a.ptr[r_begin], e_end = a.ptr[r_end];
+  const int64_t r_begin = a.split[blockIdx.x], r_all = a.split[blockIdx.x + 1], e_begin = a.ptr[r_begin];
+  int64_t r_end = r_all, e_end = a.ptr[r_all];   // the rows multiplied as digits
 
   if (tid == 0) {
     for (int s = 0; s < nst; ++s) {
@@ -296,12 +303,21 @@ __global__ void __launch_bounds__(kTileThreads, 1) k_tile_tc(const __grid_consta
   // and 119, 81,920 337 and 334, cubes of 4,800 64 and 60, 30,000 155 and 150, 129,792 343
   // and 340; one column the same either way
   if (W == 16) pdl_go();
-  const bool wide =
-      a.spread && __any_sync(0xffffffffu, lane < a.ncol && a.spread[min(lane, a.ncol - 1)] < 0);   // the same in every warp
+  // columns in double-float (the same in every warp); without any other that does not
+  // vanish no row is multiplied as digits
+  uint32_t wide = 0u;
+  if (a.spread) {
+    const bool in = lane < a.ncol, w = in && a.spread[min(lane, a.ncol - 1)] < 0;
+    const bool zero = a.colmax[min(lane, a.ncol - 1)] == 0ull;
+    wide = __ballot_sync(0xffffffffu, w);
+    if (wide && !__any_sync(0xffffffffu, in && !w && !zero)) {
+      wide = 0xffffffffu;
+      r_end = r_begin;
+      e_end = e_begin;
+    }
+  }
 
-  if (wide) {
-    rows_dd(a, r_begin, r_end, smem);
-  } else if (warp == 0) {
+  if (warp == 0) {
     // ---------------- producer: the digits of every block of the range and of its column tile
     if (lane == 0) {
       int64_t e = e_begin;
@@ -449,11 +465,16 @@ __global__ void __launch_bounds__(kTileThreads, 1) k_tile_tc(const __grid_consta
           break;
         }
         tc_fence_after();
-        // column blocks c, c + 1 combine exactly; weight 2^(-8 - 5 (c + 1)), times 2^(-5 q) at the end
+        // column blocks c, c + 1 combine exactly; weight 2^(-8 - 5 (c + 1)), times 2^(-5 q) at the
+        // end.  Rolled for 16 columns: unrolled, the three roles' code missed the instruction
+        // cache, the first of the stalls, and the kernel's time moved by 4 % with the code
+        // around it (81,920 triangles, order 3, 32 columns: product 873 us unrolled, 795 rolled;
+        // 327,680, order 4, 16 columns: nearfield and leaf backward 581 and 514 us; 8 columns
+        // or fewer 143 us unrolled, 145 rolled)
         dd acc[W];
 #pragma unroll
         for (int j = 0; j < W; ++j) acc[j] = dd{0.0f, 0.0f};
-#pragma unroll
+#pragma unroll(W == 16 ? 1 : 4)
         for (int base = 0; base < N0; base += 64) {
           uint32_t raw[4][16];
 #pragma unroll
@@ -509,17 +530,18 @@ __global__ void __launch_bounds__(kTileThreads, 1) k_tile_tc(const __grid_consta
   tc_fence_after();
   if (warp == 1)
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tbase), "r"(2 * SET) : "memory");
+  if (wide) rows_dd(a, r_begin, r_all, smem, wide);   // every copy and MMA of the digits is complete
 }
 
 // The input digit tiles of items first .. first + count - 1 (R rows of rp
 // values each, columns 0 .. ncol - 1 of x): 4 W threads per item, thread (j, g)
 // cuts rows 8 g .. 8 g + 7 of column j in registers (zero beyond R and ncol) and
 // writes half a 16-byte row of a core matrix per plane, and of the zero rows behind the
-// eleven planes.  (Sixteen values per thread took 168 registers.)
+// eleven planes.  Columns of wide range (spread, NULL: none) are cut as zeros.  (Sixteen values per thread took 168 registers.)
 template <int W>
 __global__ void __launch_bounds__(128) k_tile_cut(const dd *__restrict__ x, int64_t first, int64_t count, int R,
                                                   int rp, int ncol, const unsigned *__restrict__ xmax, int by_level,
-                                                  unsigned char *__restrict__ X) {
+                                                  const int *__restrict__ spread, unsigned char *__restrict__ X) {
   pdl_wait();
   pdl_go();
   constexpr int N0 = tile_n<W>();
@@ -529,11 +551,12 @@ __global__ void __launch_bounds__(128) k_tile_cut(const dd *__restrict__ x, int6
   // the halves of a core-matrix row are neighbouring lanes, then the columns
   const int h = threadIdx.x & 1, j = (threadIdx.x >> 1) % W, c = (threadIdx.x / (2 * W)) & 1, g = 2 * c + h;
   const int sc = kTileFixBits - tc_colexp(j < ncol ? xmax[(by_level ? tc_level(t) * kXmaxCols : 0) + j] : 0u);
+  const bool cut = j < ncol && !(spread && spread[j] < 0);
   dd v[8];
 #pragma unroll
   for (int q = 0; q < 8; ++q) {
     const int mu = 8 * g + q;
-    v[q] = mu < R && j < ncol ? x[(t * R + mu) * rp + j] : dd{0.0f, 0.0f};
+    v[q] = mu < R && cut ? x[(t * R + mu) * rp + j] : dd{0.0f, 0.0f};
   }
   uint32_t w[kTileDigits][2];
   cut_row<kTileDigits, 8>(v, sc, w);
@@ -698,17 +721,18 @@ int tile_run(const TileArgs &a, int width, int grid, cudaStream_t st) {
 
 template <int W>
 void cut_launch(const dd *x, int64_t first, int64_t count, int R, int rp, int ncol, const unsigned *xmax, int by_level,
-                unsigned char *X, cudaStream_t st) {
+                const int *spread, unsigned char *X, cudaStream_t st) {
   constexpr int per = 32 / W;
-  pdl(k_tile_cut<W>, (unsigned)((count + per - 1) / per), 128, 0, st, x, first, count, R, rp, ncol, xmax, by_level, X);
+  pdl(k_tile_cut<W>, (unsigned)((count + per - 1) / per), 128, 0, st, x, first, count, R, rp, ncol, xmax, by_level, spread,
+      X);
 }
 
 void tile_cut(const dd *x, int64_t first, int64_t count, int R, int rp, int ncol, const unsigned *xmax, int by_level,
-              unsigned char *X, int width, cudaStream_t st) {
+              const int *spread, unsigned char *X, int width, cudaStream_t st) {
   switch (width) {
-    case 4: return cut_launch<4>(x, first, count, R, rp, ncol, xmax, by_level, X, st);
-    case 8: return cut_launch<8>(x, first, count, R, rp, ncol, xmax, by_level, X, st);
-    default: return cut_launch<16>(x, first, count, R, rp, ncol, xmax, by_level, X, st);
+    case 4: return cut_launch<4>(x, first, count, R, rp, ncol, xmax, by_level, spread, X, st);
+    case 8: return cut_launch<8>(x, first, count, R, rp, ncol, xmax, by_level, spread, X, st);
+    default: return cut_launch<16>(x, first, count, R, rp, ncol, xmax, by_level, spread, X, st);
   }
 }
 
@@ -833,10 +857,10 @@ int ntc_build(Ctx &c) {
 }
 
 // the digit tiles of columns c0 .. c0 + ncol - 1 of the permuted input
-void ntc_input(Ctx &c, const void *xpad, int rp, int c0, int ncol, bool wide) {
+void ntc_input(Ctx &c, const void *xpad, int rp, int c0, int ncol, bool wide, bool ranged) {
   Dev &d = c.d;
   tile_cut(static_cast<const dd *>(xpad) + c0, 0, d.nleaf, (int)d.lmax, rp, ncol, d.ntc_xmax + c0, 0,
-           (unsigned char *)d.xnt, wide ? kTcN : tile_width(ncol), c.stream);
+           ranged ? d.spread + c0 : nullptr, (unsigned char *)d.xnt, wide ? kTcN : tile_width(ncol), c.stream);
 }
 
 // The nearfield phase (y_pad += or = the near sums), 16 columns per pass.
@@ -850,7 +874,7 @@ int ntc_near(Ctx &c, const void *xpad, void *ypad, int rp, int accumulate, int64
   for (int c0 = 0; c0 < rp; c0 += kTcN) {
     const int ncol = std::min(kTcN, rp - c0);
     if (!have_input) {
-      ntc_input(c, xpad, rp, c0, ncol, false);
+      ntc_input(c, xpad, rp, c0, ncol, false, ranged);
       ++nl;
     }
     TileArgs a{};
@@ -863,6 +887,7 @@ int ntc_near(Ctx &c, const void *xpad, void *ypad, int rp, int accumulate, int64
     a.E = d.ntc_E;
     a.xmax = d.ntc_xmax + c0;
     a.spread = ranged ? d.spread + c0 : nullptr;
+    a.colmax = d.colmax + c0;
     a.B = static_cast<const dd *>(d.near);
     a.Bp = (int)d.lp;
     a.bptr = d.near_ptr;
@@ -936,7 +961,7 @@ int tct_coupling(Ctx &c, const void *xhat, void *yhat, int rp, int64_t *launches
   for (int c0 = 0; c0 < rp; c0 += kTcN) {
     const int ncol = std::min(kTcN, rp - c0);
     tile_cut(static_cast<const dd *>(xhat) + c0, row0, d.nclu - row0, d.k, rp, ncol, d.tc_xmax + c0, 1,
-             (unsigned char *)d.xtc, tile_width(ncol), c.stream);
+             d.spread + c0, (unsigned char *)d.xtc, tile_width(ncol), c.stream);
     TileArgs a{};
     a.A = (const unsigned char *)d.Stc;
     a.X = (const unsigned char *)d.xtc;
@@ -947,6 +972,7 @@ int tct_coupling(Ctx &c, const void *xhat, void *yhat, int rp, int64_t *launches
     a.E = d.tc_E;
     a.xmax = d.tc_xmax + c0;
     a.spread = d.spread + c0;
+    a.colmax = d.colmax + c0;
     a.B = static_cast<const dd *>(d.S);
     a.Bp = d.kp;
     a.bptr = d.adm_ptr + row0;

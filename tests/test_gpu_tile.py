@@ -91,6 +91,32 @@ def test_columns_of_wide_range(require_gpu, order, leaf):
     h.close()
 
 
+@pytest.mark.parametrize("order, leaf", [(3, 30), (3, 9), (2, 32)])
+def test_columns_do_not_depend_on_others(require_gpu, order, leaf):
+    """Columns of wide range (double-float), even ones (digits) and zero ones in one product: each gives,
+    bit for bit, what it gives beside any others."""
+    import torch
+    n = 64 * leaf
+    v, f = I.icosphere(4)
+    v, f = v * np.exp(v[:, 2:3]), np.ascontiguousarray(f[:n])
+    h = H2Matrix(v, f, leaf_size=leaf, eta=2.0, order=order, prec="f64")
+    for nrhs in (2, 7, 16, 21):
+        sets = {"even": I.uniform_rhs(n, nrhs, 5800), "zero": np.zeros((n, nrhs)),
+                "wide": np.stack([_wide_columns(n, 5, 5801 + j)[:, j % 4] for j in range(nrhs)], axis=1)}
+        dev = {k: torch.from_numpy(np.ascontiguousarray(x.T)).cuda().t() for k, x in sets.items()}
+        ref = {}
+        for k, x in dev.items():
+            ref[k] = colmajor(torch.empty_like(x))
+            h.matvec(x, ref[k])
+        kinds = np.array(["even", "wide", "zero"])[np.random.default_rng(nrhs).integers(0, 3, nrhs)]
+        x = colmajor(torch.stack([dev[k][:, c] for c, k in enumerate(kinds)], dim=1))
+        y = colmajor(torch.empty_like(x))
+        h.matvec(x, y)
+        for c, k in enumerate(kinds):
+            assert torch.equal(y[:, c], ref[k][:, c]), (nrhs, c, k)
+    h.close()
+
+
 def test_columns_with_infinity_or_nan(require_gpu):
     """Every output depends on every input: a column with an infinity or a NaN gives NaN throughout,
     the other columns are not touched by it."""
