@@ -29,7 +29,7 @@
 // Errors in the 2-norm, 5,120 triangles graded 55 : 1 in size, order 3, 20
 // columns of entries in [-1, 1] and one of 1e8: 1.0e-10 without that rule, 1.3e-14
 // now, 1.7e-14 in double-float block rows.  The rule and the eleventh digit cost even
-// columns 0 to 1 % (81,920 triangles, 32 columns 853 -> 862 us; 5,120, one 62 us).
+// columns about 1 % (81,920 triangles, 32 columns).
 //
 // Layout.  The digit planes of a block are stacked four to a 128-row MMA
 // operand: digit i (from 0) of row nu lies in group i / 4, row (i mod 4) R +
@@ -59,14 +59,14 @@
 // What bounds it: the copy stream and the MMA warp's issue.  Nearfield of
 // 327,680 triangles (leaves of 20, 179,008 blocks of 6.4 KB and as many input
 // tiles of 5.6 KB), 16 columns: 480 us before (one epilogue group, separate
-// accumulator columns per plane group, single-stage commits), 351 us now, 6.1
+// accumulator columns per plane group, single-stage commits), 298 us now, 7.2
 // TB/s into shared memory.  Leaves of 30 (cube, 30,000 triangles, 5 columns):
-// 161 us in double-float block rows, 47 us now; 32 right-hand sides, 81,920
-// triangles: 414 us in double-float, 215 us now (two passes).  Order-3
+// 161 us in double-float block rows, 44 us now; 32 right-hand sides, 81,920
+// triangles: 414 us in double-float, 184 us now (two passes, with the digit cuts).  Order-3
 // coupling, double-float block rows before: 81,920 triangles, 32 right-hand
-// sides (75,224 blocks of 9.0 KB, two passes) 1,070 us, now 381 us with the
-// digit cuts; cube of 30,000 triangles, 5 columns 195 us, now 62 us; 5,120
-// triangles, one column 35 us, now 22 us.
+// sides (75,224 blocks of 9.0 KB, two passes) 1,070 us, now 339 us with the
+// digit cuts; cube of 30,000 triangles, 5 columns 195 us, now 54 us; 5,120
+// triangles, one column 35 us, now 17 us.
 #include <algorithm>
 #include <functional>
 #include <queue>
@@ -138,7 +138,7 @@ struct TileArgs {
 // short sums.  Threads and slices are those of all columns of the pass, whichever are
 // in mask.  Bound by the FP32 pipe (two warps per scheduler; the other two warps only
 // copy).  Whole products of wide columns, 81,920 triangles, order 3, 1 / 5 / 16 / 32
-// columns: 558 / 694 / 1,178 / 2,298 us; pipelined block rows on the same sums 531 / 637 / 1,053 / 1,871 us
+// columns: 573 / 714 / 1,185 / 2,310 us, one among even ones 572 / 882 / 1,359 / 2,677 us; pipelined block rows on the same sums 531 / 637 / 1,053 / 1,871 us
 // (every product, before the digits).
 constexpr int kDdStages = 3, kDdThreads = 256;
 __host__ __device__ inline uint32_t rows_dd_stage(int R, int Bp, int ncol) {
